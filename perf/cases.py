@@ -253,3 +253,133 @@ def run(s):
         out = sa.fwd(q, k, v, idx, cnt, block)
         out = sa.comp_apply(q, s["pq"], state, s["gate"], out, s["grid"], s["axis"], s["freq"])
     return out, state, idx, cnt
+
+
+EXACT_FLOPS = 1e13          # above it the 64-bit evaluation takes too long
+
+
+def _pooled(x, block, valid=None):
+    """Block means [nb, d] of [N, d], over the first valid[b] rows of block b (default: those below N)."""
+    n, d = x.shape
+    nb = -(-n // block)
+    rows = torch.arange(nb * block, device=x.device).view(nb, block)
+    real = rows < n if valid is None else (rows % block) < valid[:, None]
+    x = torch.nn.functional.pad(x, (0, 0, 0, nb * block - n)).view(nb, block, d)
+    return (x * real[..., None]).sum(1) / real.sum(1, keepdim=True)
+
+
+def _chosen(q, k, block, topk, valid=None, frame=0, window=0):
+    """Top-k key blocks of every query block of one head by the product of block means; -1 beyond the candidates."""
+    n = q.shape[0]
+    score = _pooled(q, block, valid) @ _pooled(k, block, valid).T
+    if frame:
+        first = torch.arange(0, n, block, device=q.device)
+        last = (first + block - 1).clamp(max=n - 1)
+        lo, hi = ((first // frame - window + 1).clamp(min=0) * frame)[:, None], (last // frame + 1)[:, None] * frame
+        score = score.masked_fill((first[None] >= hi) | (last[None] < lo), -math.inf)
+    best, idx = score.topk(topk, dim=1)
+    return torch.where(best == -math.inf, -1, idx)
+
+
+def _attend(q, k, v, idx, block, valid=None, frame=0, window=0):
+    """Softmax attention of one head over the listed key blocks, [N, d] in 64 bits -> output and log-sum-exp."""
+    n, d = q.shape
+    nb, topk = idx.shape
+    pad = (0, 0, 0, nb * block - n)
+    q, k, v = (torch.nn.functional.pad(t, pad).view(nb, block, d) for t in (q, k, v))
+    out, lse = torch.empty_like(q), torch.empty((nb, block), dtype=q.dtype, device=q.device)
+    lane = torch.arange(block, device=q.device)
+    step = max(1, int(1e8) // (topk * block * block))
+    for i in range(0, nb, step):
+        at = idx[i: i + step].clamp(min=0)
+        c = at.shape[0]
+        key = at[..., None] * block + lane                                     # [c, topk, block]
+        real = (idx[i: i + step] >= 0)[..., None] & (key < n)
+        if valid is not None:
+            real &= lane < valid[at][..., None]
+        real = real.view(c, 1, -1)
+        if frame:
+            row = (i + torch.arange(c, device=q.device))[:, None] * block + lane
+            fq, fk = (row.clamp(max=n - 1) // frame)[..., None], (key // frame).view(c, 1, -1)
+            real = real & (fk <= fq) & (fk > fq - window)
+        s = (q[i: i + step] @ k[at].view(c, -1, d).mT) * (1.0 / math.sqrt(d))
+        s.masked_fill_(~real, -math.inf)
+        lse[i: i + step] = torch.logsumexp(s, -1)
+        s.sub_(lse[i: i + step].nan_to_num(neginf=0.0)[..., None]).exp_()
+        out[i: i + step] = s @ v[at].view(c, -1, d)
+    return out.view(-1, d)[:n], lse.view(-1)[:n]
+
+
+def _dequantised(x, block):
+    """What one head's E4M3 codes with a scale per block stand for, in 64 bits."""
+    n, d = x.shape
+    x = torch.nn.functional.pad(x.float(), (0, 0, 0, -n % block)).view(-1, block, d)
+    amax = x.abs().amax((1, 2), keepdim=True).clamp(min=1e-12)
+    return ((x * (448.0 / amax)).to(torch.float8_e4m3fn).double() * (amax / 448.0).double()).view(-1, d)[:n]
+
+
+def _feature(x, p, grid, axis, freq):
+    """Rotated silu features [N, rank] of one head's rows."""
+    i = torch.arange(x.shape[0], device=x.device)
+    pos = torch.stack([i // (grid[1] * grid[2]), i // grid[2] % grid[1], i % grid[2]], 1).double()
+    a = pos[:, axis.long().to(x.device)] * freq.double().to(x.device)
+    z = torch.nn.functional.silu(x @ p.T).view(-1, RANK // 2, 2)
+    even, odd = z.unbind(2)
+    return torch.stack([even * a.cos() - odd * a.sin(), even * a.sin() + odd * a.cos()], 2).view(-1, RANK)
+
+
+def _brick_rows(case):
+    """(raster token at each row of the brick order, -1 for padding; tokens of each brick)."""
+    T, Hg, Wg, bt, bh, bw = (case[a] for a in ("T", "Hg", "Wg", "bt", "bh", "bw"))
+    n = torch.arange(T * Hg * Wg).view(T, Hg, Wg)
+    rows, valid = [], []
+    for t in range(0, T, bt):
+        for y in range(0, Hg, bh):
+            for x in range(0, Wg, bw):
+                cells = n[t: t + bt, y: y + bh, x: x + bw].reshape(-1)
+                valid.append(cells.numel())
+                rows.append(torch.nn.functional.pad(cells, (0, case["block"] - cells.numel()), value=-1))
+    return torch.cat(rows).cuda(), torch.tensor(valid, device="cuda")
+
+
+def exact(case, seed):
+    """What run() returns, in 64 bits from the same inputs; no counterpart for lists and codes."""
+    if work(case)["flops"] > EXACT_FLOPS:
+        return None
+    s = prepare(case, seed)
+    path, block = s["path"], s["block"]
+    if path == "activation":
+        return None, s["x"].double().abs().amax(-1).clamp(min=1e-12) / 448.0
+    q, k, v = (t.cuda() for t in (s["q"], s["k"], s["v"]))
+    B, H, n, d = q.shape
+    out = torch.empty((B, H, n, d), dtype=torch.float64, device="cuda")
+    lse, state = out.new_empty((B, H, n)), out.new_empty((B, H, RANK, d))
+    rows, valid = _brick_rows(case) if path == "bricks" else (None, None)
+    window = (s["frame"], s["window"]) if path == "causal" else (0, 0)
+    for b in range(B):
+        for h in range(H):
+            x, y, z = (t[b, h].double() for t in (q, k, v))
+            if path == "bricks":
+                x, y, z = (t[rows.clamp(min=0)] * (rows >= 0)[:, None] for t in (x, y, z))
+            idx = s["idx"][b, h].long() if path == "lists" else _chosen(x, y, block, s["topk"], valid, *window)
+            if path == "fp8":
+                x, y, z = (_dequantised(t, block) for t in (x, y, z))
+            o, lse[b, h] = _attend(x, y, z, idx, block, valid, *window) if path != "bricks" else (
+                _attend(x, y, z, idx, block, valid)[0], 0.0)
+            if path == "bricks":
+                out[b, h, rows[rows >= 0]] = o[rows >= 0]
+                continue
+            if path in ("module", "gated"):
+                args = s["grid"], s["axis"], s["freq"]
+                state[b, h] = _feature(y, s["pk"][h].double(), *args).T @ z
+                low = _feature(x, s["pq"][h].double(), *args) @ state[b, h]
+                low = low / (low.square().mean(-1, keepdim=True) + 1e-6).sqrt()
+                o = o + s["gate"][b, h].double()[:, None] * o.square().mean(-1, keepdim=True).sqrt() * low
+            out[b, h] = o
+    if path in ("lists", "host"):
+        return out
+    if path == "causal":
+        return out, lse, None, None
+    if path in ("module", "gated"):
+        return out, state, None, None
+    return out, None, None
