@@ -96,7 +96,7 @@ int select_impl(const sparkattn_shape_t* shape, const void* q_bf16, const void* 
   if (!aligned16(q_bf16) || !aligned16(k_bf16) || !aligned256(workspace)) return SPARKATTN_E_MISALIGNED;
   if (workspace_bytes < select_workspace_bytes(*shape)) return SPARKATTN_E_WORKSPACE_TOO_SMALL;
   cudaStream_t stream = static_cast<cudaStream_t>(cuda_stream);
-  if (cudaMemsetAsync(workspace, 0, kWorkspaceHeaderBytes, stream) != cudaSuccess) return SPARKATTN_E_CUDA;
+  // (the pooling kernel clears the workspace header)
   return launch_select(*shape, q_bf16, k_bf16, topk, frame_tokens, window, block_valid, kept_idx, kept_cnt, workspace,
                        stream);
 }

@@ -10,6 +10,24 @@
 
 namespace sparkattn {
 
+// Launches a kernel; with `overlap` it may start while the kernel before it on the stream is draining (it then calls
+// pdl_wait, common.cuh, before it touches memory).
+template <typename... Params, typename... Args>
+inline int launch_kernel(void (*kern)(Params...), unsigned grid, unsigned threads, size_t smem, bool overlap, cudaStream_t stream,
+                         const Args&... args) {
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3(grid);
+  cfg.blockDim = dim3(threads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = stream;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = overlap ? 1 : 0;
+  return cudaLaunchKernelEx(&cfg, kern, Params(args)...) == cudaSuccess ? SPARKATTN_OK : SPARKATTN_E_CUDA;
+}
+
 // quant.cu
 int launch_quant_fp8(const sparkattn_shape_t& s, const void* x, uint8_t* codes, float* scales,
                      cudaStream_t stream);

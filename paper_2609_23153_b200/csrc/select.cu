@@ -9,22 +9,23 @@
 // bit for bit; this is why scoring runs on the FMA pipe and not on tensor cores.
 //
 // Two kernels:
-//   pool_kernel    one warp per (tensor, batch, head, block); reads Q and K once
-//                  from HBM (the only HBM-heavy step: 2 bytes per element) and
-//                  writes pooled Q [BH][nb][d] and pooled K transposed [BH][d][nbp].
-//   topk_kernel    one CTA per 16 (8 for very long sequences) query blocks of one
-//                  (batch, head): scores against all key blocks as a 16 x 4 register
-//                  tile per thread (pooled K streamed from L2 in 16-byte loads along j,
-//                  packed fp32x2 FMAs over row pairs), then one warp per query block
-//                  does an exact radix select of the topk-th largest key (keys in
-//                  registers for nb <= 1280) and an ordered ballot compaction.
+//   pool_kernel       two resident CTAs per SM walk the (tensor, batch, head, block) items: a block's rows go to shared
+//                     memory in one go (asynchronous copies into one of two buffers) while thread c adds up two
+//                     channels of the block before.  The only HBM-heavy step (2 bytes per element); writes pooled Q
+//                     [BH][nb][d] and pooled K transposed [BH][d][nbp].
+//   topk_kernel       nb <= 256: one CTA per 8, 16 or 32 query blocks of one (batch, head): scores against all key
+//                     blocks as an RT x 4 register tile per thread (pooled K through a ring of asynchronous copies in
+//                     shared memory, packed fp32x2 FMAs over row pairs), then a warp per query block (or two) selects
+//                     the topk largest keys exactly (keys in registers for nb <= 1280) and compacts them in order.
+//   topk_wide_kernel  nb > 256: 16 or 8 query blocks per CTA of ten warps, pooled K straight from L2.
+// The second is launched before the first has drained (programmatic dependent launch) and waits inside.
 #include "common.cuh"
 #include "launch.h"
+#include "tmap.h"
 
 namespace sparkattn {
 
-constexpr int kPoolThreads = 256;
-constexpr int kTopkThreads = 160;  // 4 x 160 key-block slots per sweep (591 blocks of the 720P shape fit one sweep)
+constexpr int kTopkThreads = 256;
 
 static inline int round_up(int x, int m) { return (x + m - 1) / m * m; }
 
@@ -35,65 +36,95 @@ size_t select_workspace_bytes(const sparkattn_shape_t& s) {
   return kWorkspaceHeaderBytes + bh * nb * s.d * sizeof(float) + bh * s.d * nbp * sizeof(float);
 }
 
+// Bound by HBM.  A sum is a chain of additions over the block's tokens, so a warp that reads its rows as it adds
+// them waits for memory block / 16 times over; here a whole block (32 KB at most) is on its way at once, into one of
+// two buffers, while the block before it is added up.
+// 40 heads of 75,600 tokens: 225 us (6.9 TB/s) against 255 us for one warp per block with 16 rows in flight; 3 heads of
+// 1,200 tokens: a few us against 12, all of them latency.  Two CTAs of two buffers per SM; three take 238 us.
+constexpr int kPoolCtasPerSm = 2;
 template <int D>
-__global__ void __launch_bounds__(kPoolThreads)
+__global__ void __launch_bounds__(D / 2)
 pool_kernel(const __nv_bfloat16* __restrict__ q, const __nv_bfloat16* __restrict__ k, float* __restrict__ pq,
             float* __restrict__ pkT, int H, int N, int blk_size, int nb, int nbp, int64_t stride_b,
             int64_t stride_h, int64_t stride_n, int64_t n_items /* B*H*nb */,
-            const int32_t* __restrict__ block_valid /* [nb] real tokens per block, or NULL */) {
-  constexpr int VEC = D / 32;  // channels per lane: 4 (8-byte loads) or 2 (4-byte loads)
-  const int lane = threadIdx.x & 31;
-  const int64_t gw = (int64_t)blockIdx.x * (kPoolThreads / 32) + (threadIdx.x >> 5);
-  if (gw >= 2 * n_items) return;
-  const bool is_k = gw >= n_items;
-  const int64_t item = is_k ? gw - n_items : gw;
-  const int blk = (int)(item % nb);
-  const int64_t bh = item / nb;
-  const int h = (int)(bh % H), b = (int)(bh / H);
-  const int row0 = blk * blk_size;
-  int nvalid = min(blk_size, N - row0);
-  if (block_valid != nullptr) nvalid = max(1, min(nvalid, __ldg(block_valid + blk)));   // bricks padded to whole blocks
-  const __nv_bfloat16* src = (is_k ? k : q) + b * stride_b + h * stride_h + (int64_t)row0 * stride_n + lane * VEC;
+            const int32_t* __restrict__ block_valid /* [nb] real tokens per block, or NULL */,
+            int32_t* __restrict__ header) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];      // [2][blk_size][D] bf16
+  constexpr int kThreads = D / 2;
+  constexpr int kRowChunks = D / 8;                    // 16-byte chunks of a row
+  constexpr int kRowStep = kThreads / kRowChunks;      // rows the CTA covers with one copy per thread
+  const int buf_bytes = blk_size * D * 2;
+  const int chunk = threadIdx.x % kRowChunks, r0 = threadIdx.x / kRowChunks;
+  struct Item {
+    bool is_k;
+    int blk, nvalid;
+    int64_t bh;
+  };
+  auto item_at = [&](int64_t w) {
+    Item it;
+    it.is_k = w >= n_items;
+    const int64_t item = it.is_k ? w - n_items : w;
+    it.blk = (int)(item % nb);
+    it.bh = item / nb;
+    it.nvalid = min(blk_size, N - it.blk * blk_size);
+    if (block_valid != nullptr) it.nvalid = max(1, min(it.nvalid, __ldg(block_valid + it.blk)));   // bricks padded to whole blocks
+    return it;
+  };
+  auto fetch = [&](const Item& it, int buf) {
+    const int h = (int)(it.bh % H), b = (int)(it.bh / H);
+    const __nv_bfloat16* src =
+        (it.is_k ? k : q) + b * stride_b + h * stride_h + (int64_t)(it.blk * blk_size + r0) * stride_n + chunk * 8;
+    uint32_t dst = smem_u32(smem_raw) + buf * buf_bytes + r0 * (D * 2) + chunk * 16;
+#pragma unroll 8
+    for (int r = r0; r < it.nvalid; r += kRowStep, src += kRowStep * stride_n, dst += kRowStep * D * 2) cp_async16(dst, src);
+  };
 
-  float sum[VEC];
+  pdl_trigger();
+  pdl_wait();
+  if (blockIdx.x == 0)
+    for (int e = threadIdx.x; e < kWorkspaceHeaderBytes / 4; e += kThreads) header[e] = 0;
+  Item next = item_at(blockIdx.x);
+  fetch(next, 0);
+  cp_async_commit();
+  int buf = 0;
+  for (int64_t w = blockIdx.x; w < 2 * n_items; w += gridDim.x, buf ^= 1) {
+    const Item it = next;
+    if (w + gridDim.x < 2 * n_items) {
+      next = item_at(w + gridDim.x);
+      fetch(next, buf ^ 1);
+    }
+    cp_async_commit();
+    cp_async_wait<1>();
+    __syncthreads();
+    const uint32_t* col = reinterpret_cast<const uint32_t*>(smem_raw + buf * buf_bytes) + threadIdx.x;   // channels 2t and 2t + 1
+    float s0 = 0.0f, s1 = 0.0f;
+    constexpr int U = 16;
+    int r = 0;
+    for (; r + U <= it.nvalid; r += U) {
+      uint32_t x[U];
 #pragma unroll
-  for (int c = 0; c < VEC; ++c) sum[c] = 0.0f;
-
-  constexpr int U = 16;  // rows in flight per lane
-  int t = 0;
-  for (; t + U <= nvalid; t += U) {
-    float x[U][VEC];
+      for (int u = 0; u < U; ++u) x[u] = col[(r + u) * (D / 2)];
 #pragma unroll
-    for (int u = 0; u < U; ++u) {
-      const __nv_bfloat16* p = src + (int64_t)(t + u) * stride_n;
-      if constexpr (VEC == 4) {
-        const uint2 raw = __ldg(reinterpret_cast<const uint2*>(p));
-        const float2 a = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&raw.x));
-        const float2 c = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&raw.y));
-        x[u][0] = a.x; x[u][1] = a.y; x[u][2] = c.x; x[u][3] = c.y;
-      } else {
-        const uint32_t raw = __ldg(reinterpret_cast<const uint32_t*>(p));
-        const float2 a = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&raw));
-        x[u][0] = a.x; x[u][1] = a.y;
+      for (int u = 0; u < U; ++u) {
+        s0 = __fadd_rn(s0, __uint_as_float(x[u] << 16));
+        s1 = __fadd_rn(s1, __uint_as_float(x[u] & 0xffff0000u));
       }
     }
-#pragma unroll
-    for (int u = 0; u < U; ++u)
-#pragma unroll
-      for (int c = 0; c < VEC; ++c) sum[c] = __fadd_rn(sum[c], x[u][c]);
-  }
-  for (; t < nvalid; ++t) {
-    const __nv_bfloat16* p = src + (int64_t)t * stride_n;
-#pragma unroll
-    for (int c = 0; c < VEC; ++c) sum[c] = __fadd_rn(sum[c], __bfloat162float(p[c]));
-  }
-  const float nv = (float)nvalid;
-#pragma unroll
-  for (int c = 0; c < VEC; ++c) {
-    const float mean = __fdiv_rn(sum[c], nv);
-    const int ch = lane * VEC + c;
-    if (is_k) pkT[(bh * D + ch) * nbp + blk] = mean;
-    else pq[(bh * nb + blk) * D + ch] = mean;
+    for (; r < it.nvalid; ++r) {
+      const uint32_t x = col[r * (D / 2)];
+      s0 = __fadd_rn(s0, __uint_as_float(x << 16));
+      s1 = __fadd_rn(s1, __uint_as_float(x & 0xffff0000u));
+    }
+    const float nv = (float)it.nvalid;
+    const float m0 = __fdiv_rn(s0, nv), m1 = __fdiv_rn(s1, nv);
+    const int ch = 2 * threadIdx.x;
+    if (it.is_k) {
+      pkT[(it.bh * D + ch) * nbp + it.blk] = m0;
+      pkT[(it.bh * D + ch + 1) * nbp + it.blk] = m1;
+    } else {
+      *reinterpret_cast<float2*>(pq + (it.bh * nb + it.blk) * D + ch) = make_float2(m0, m1);
+    }
+    __syncthreads();                     // the buffer may be filled again
   }
 }
 
@@ -129,6 +160,7 @@ __device__ __forceinline__ void select_row(KeyAt key_at, int nb, int jlo, int jh
     for (int j = lane; j < nb; j += 32) cnt += (key_at(j) >= cand);
     cnt = __reduce_add_sync(0xffffffffu, cnt);
     if (cnt >= topk) thr = cand;
+    if (cnt == topk) break;          // exactly the keys wanted: the lower bits of the threshold do not matter
   }
   int ngreater = 0;
   for (int j = lane; j < nb; j += 32) ngreater += (key_at(j) > thr);
@@ -152,248 +184,457 @@ __device__ __forceinline__ void select_row(KeyAt key_at, int nb, int jlo, int jh
   }
 }
 
-// select_row with the row's keys held in KR registers per lane (nb <= 32 * KR): the key loops unroll
-// over registers.  Keys outside the candidate range are held as 0, below every candidate (candidates
-// are >= 1).
+// The same with a row's keys held in KR registers per lane (nb <= 32 * KR), for NR rows of a warp at once: the search
+// is a chain of warp reductions, and two rows' chains fill each other's gaps.  Keys outside the candidate range
+// are held as 0, below every candidate (candidates are >= 1).
 //
-// The threshold (the topk-th largest key) is first sought among the four largest keys of every lane,
-// 128 values: their topk-th largest, T, never exceeds the true threshold, and when no lane holds more
-// than four keys >= T every key >= T is among the 128, so T is the true threshold.  The bitwise search
-// then costs 4 compares per pass instead of KR.  Otherwise (a lane with five such keys, or topk > 128)
-// the search runs over all KR keys.  Either way the threshold is exact; only the cost differs.
-template <int KR, bool WINDOW>
-__device__ __forceinline__ void select_row_regs(const uint32_t* __restrict__ key, int nb, int jlo, int jhi, int topk,
-                                                int lane, int32_t* __restrict__ dst) {
+// The threshold is first sought among the four largest keys of every lane, 128 values, two bits per pass (the
+// counts of the three candidates share one reduction), and the search ends as soon as a candidate has exactly topk
+// keys at or above it.  When no lane holds more than four keys >= the threshold found, every key >= it is among the
+// 128 and it separates the row's topk largest keys.  Otherwise (a lane with five such keys, or topk > 128) the
+// search runs over all KR keys.  Either way the selection is exact; only the cost differs.
+template <int KR, bool WINDOW, int NR>
+__device__ __forceinline__ void select_rows_regs(const uint32_t* const (&key)[NR], int nb, const int (&jlo)[NR],
+                                                 const int (&jhi)[NR], const int (&topk)[NR], int lane,
+                                                 int32_t* const (&dst)[NR]) {
   constexpr uint32_t kFull = 0xffffffffu;
-  auto in_range = [&](int j) { return WINDOW ? (j >= jlo && j <= jhi) : (j < nb); };
-  uint32_t kr[KR];
+  uint32_t kr[NR][KR];
+  uint32_t m1[NR], m2[NR], m3[NR], m4[NR];                     // sorted four largest keys of the lane
+  uint32_t kmaxv[NR], thr[NR];
+  int sh[NR];
+  bool active[NR];
+  bool any = false;
 #pragma unroll
-  for (int u = 0; u < KR; ++u) {
-    const int j = lane + 32 * u;
-    kr[u] = in_range(j) ? key[j] : 0u;
-  }
-  // sorted four largest keys of the lane
-  uint32_t m1 = 0u, m2 = 0u, m3 = 0u, m4 = 0u;
-#pragma unroll
-  for (int u = 0; u < KR; ++u) {
-    uint32_t x = kr[u], t;
-    t = min(m1, x); m1 = max(m1, x); x = t;
-    t = min(m2, x); m2 = max(m2, x); x = t;
-    t = min(m3, x); m3 = max(m3, x); x = t;
-    m4 = max(m4, x);
-  }
-  const uint32_t kmaxv = __reduce_max_sync(kFull, m1);
-  uint32_t thr = 0u;
-  bool exact = false;
-  int nge = 0;
-  if (topk <= 128) {
-    // T lies between the smallest lane maximum (32 >= topk values are at least that) and the row maximum;
-    // the bits above the highest bit in which the two differ are common to both and need no pass
-    const uint32_t lo = (topk <= 32) ? __reduce_min_sync(kFull, m1) : 0u;
-    const int top_bit = 31 - __clz(lo ^ kmaxv);              // -1 when the two are equal
-    thr = (top_bit >= 31) ? 0u : (kmaxv & ~((2u << max(top_bit, 0)) - 1u));
-    if (top_bit < 0) thr = kmaxv;
-    for (int bit = top_bit; bit >= 0; --bit) {
-      const uint32_t cand = thr | (1u << bit);
-      int cnt = (m1 >= cand) + (m2 >= cand) + (m3 >= cand) + (m4 >= cand);
-      cnt = __reduce_add_sync(kFull, cnt);
-      if (cnt >= topk) thr = cand;
-    }
-    int c = 0;
-#pragma unroll
-    for (int u = 0; u < KR; ++u) c += (kr[u] >= thr);
-    exact = thr != 0u && __ballot_sync(kFull, c > 4) == 0u;
-    nge = c;
-  }
-  if (!exact) {
-    // bitwise search over all keys, from the highest bit in which the row's candidates differ
-    uint32_t kmin = 0xffffffffu;
-#pragma unroll
-    for (int u = 0; u < KR; ++u)
-      if (in_range(lane + 32 * u)) kmin = min(kmin, kr[u]);
-    kmin = __reduce_min_sync(kFull, kmin);
-    const int top_bit = 31 - __clz(kmin ^ kmaxv);
-    thr = (top_bit >= 31) ? 0u : (kmaxv & ~((2u << max(top_bit, 0)) - 1u));
-    if (top_bit < 0) thr = kmaxv;
-    for (int bit = top_bit; bit >= 0; --bit) {
-      const uint32_t cand = thr | (1u << bit);
-      int cnt = 0;
-#pragma unroll
-      for (int u = 0; u < KR; ++u) cnt += (kr[u] >= cand);
-      cnt = __reduce_add_sync(kFull, cnt);
-      if (cnt >= topk) thr = cand;
-    }
-    nge = 0;
-#pragma unroll
-    for (int u = 0; u < KR; ++u) nge += (kr[u] >= thr);
-  }
-  // ordered compaction: keys above the threshold, then the lowest-indexed keys equal to it.  With thr >= 1
-  // the zero keys that stand for blocks outside the candidate range never pass a comparison (thr = 0 only
-  // when a candidate's own key is 0, the key of one NaN pattern: the general path below handles it).
-  nge = __reduce_add_sync(kFull, nge);
-  const uint32_t lt_mask = (1u << lane) - 1u;
-  int out = 0;
-  if (nge == topk && thr != 0u) {   // no surplus of keys equal to the threshold: keep every key >= thr
+  for (int r = 0; r < NR; ++r) {
+    m1[r] = m2[r] = m3[r] = m4[r] = 0u;
 #pragma unroll
     for (int u = 0; u < KR; ++u) {
-      const uint32_t keep_ballot = __ballot_sync(kFull, kr[u] >= thr);
-      if (keep_ballot != 0u) {
-        if (kr[u] >= thr) dst[out + __popc(keep_ballot & lt_mask)] = lane + 32 * u;
-        out += __popc(keep_ballot);
+      const int j = lane + 32 * u;
+      kr[r][u] = (WINDOW ? (j >= jlo[r] && j <= jhi[r]) : (j < nb)) ? key[r][j] : 0u;
+    }
+#pragma unroll
+    for (int u = 0; u < KR; ++u) {
+      uint32_t x = kr[r][u], t;
+      t = min(m1[r], x); m1[r] = max(m1[r], x); x = t;
+      t = min(m2[r], x); m2[r] = max(m2[r], x); x = t;
+      t = min(m3[r], x); m3[r] = max(m3[r], x); x = t;
+      m4[r] = max(m4[r], x);
+    }
+    kmaxv[r] = __reduce_max_sync(kFull, m1[r]);
+    // the topk-th largest lies between the smallest of the lanes' p-th largest keys, p = ceil(topk / 32) (32 p values
+    // are at least that), and the row maximum; the bits above the highest bit in which the two differ are common to
+    // both and need no pass
+    const int p = (topk[r] + 31) / 32;
+    const uint32_t lo = __reduce_min_sync(kFull, p == 1 ? m1[r] : p == 2 ? m2[r] : p == 3 ? m3[r] : p == 4 ? m4[r] : 0u);
+    const int top_bit = 31 - __clz(lo ^ kmaxv[r]);             // -1 when the two are equal
+    sh[r] = max(top_bit, 0) & ~1;
+    thr[r] = sh[r] >= 30 ? 0u : (kmaxv[r] & ~((4u << sh[r]) - 1u));
+    active[r] = topk[r] <= 128 && top_bit >= 0;
+    if (top_bit < 0) thr[r] = kmaxv[r];
+    any = any || active[r];
+  }
+  while (any) {
+    any = false;
+    int cnt[NR];
+#pragma unroll
+    for (int r = 0; r < NR; ++r) {
+      const uint32_t c1 = thr[r] | (1u << sh[r]), c2 = thr[r] | (2u << sh[r]), c3 = thr[r] | (3u << sh[r]);
+      cnt[r] = (m1[r] >= c1) + (m2[r] >= c1) + (m3[r] >= c1) + (m4[r] >= c1) +
+               (((m1[r] >= c2) + (m2[r] >= c2) + (m3[r] >= c2) + (m4[r] >= c2)) << 10) +
+               (((m1[r] >= c3) + (m2[r] >= c3) + (m3[r] >= c3) + (m4[r] >= c3)) << 20);
+    }
+#pragma unroll
+    for (int r = 0; r < NR; ++r) cnt[r] = __reduce_add_sync(kFull, cnt[r]);
+#pragma unroll
+    for (int r = 0; r < NR; ++r) {
+      if (active[r]) {
+        const int n1 = cnt[r] & 1023, n2 = (cnt[r] >> 10) & 1023, n3 = cnt[r] >> 20;
+        int n = -1;
+        if (n3 >= topk[r]) { thr[r] |= 3u << sh[r]; n = n3; }
+        else if (n2 >= topk[r]) { thr[r] |= 2u << sh[r]; n = n2; }
+        else if (n1 >= topk[r]) { thr[r] |= 1u << sh[r]; n = n1; }
+        active[r] = n != topk[r] && sh[r] > 0;
+        sh[r] = max(sh[r] - 2, 0);
+        any = any || active[r];
       }
     }
-    return;
   }
-  int ngreater = 0;
 #pragma unroll
-  for (int u = 0; u < KR; ++u) ngreater += (kr[u] > thr);
-  ngreater = __reduce_add_sync(kFull, ngreater);
-  const int ties_allowed = topk - ngreater;  // >= 1: lowest indices among the keys equal to thr
-  int ties_seen = 0;
+  for (int r = 0; r < NR; ++r) {
+    const int k = topk[r];
+    uint32_t t = thr[r];
+    int nge = 0;
 #pragma unroll
-  for (int u = 0; u < KR; ++u) {
-    if (32 * u < nb) {
-      const int j = lane + 32 * u;
-      const bool valid = in_range(j);
-      const bool tie = valid && (kr[u] == thr);
-      const uint32_t tie_ballot = __ballot_sync(kFull, tie);
-      const int tie_rank = ties_seen + __popc(tie_ballot & lt_mask);
-      const bool keep = valid && ((kr[u] > thr) || (tie && tie_rank < ties_allowed));
-      const uint32_t keep_ballot = __ballot_sync(kFull, keep);
-      if (keep) dst[out + __popc(keep_ballot & lt_mask)] = j;
-      out += __popc(keep_ballot);
-      ties_seen += __popc(tie_ballot);
+    for (int u = 0; u < KR; ++u) nge += (kr[r][u] >= t);
+    if (k > 128 || t == 0u || __any_sync(kFull, nge > 4)) {
+      // bitwise search over all keys, from the highest bit in which the row's candidates differ
+      uint32_t kmin = 0xffffffffu;
+#pragma unroll
+      for (int u = 0; u < KR; ++u) {
+        const int j = lane + 32 * u;
+        if (WINDOW ? (j >= jlo[r] && j <= jhi[r]) : (j < nb)) kmin = min(kmin, kr[r][u]);
+      }
+      kmin = __reduce_min_sync(kFull, kmin);
+      const int top_bit = 31 - __clz(kmin ^ kmaxv[r]);
+      t = (top_bit >= 31) ? 0u : (kmaxv[r] & ~((2u << max(top_bit, 0)) - 1u));
+      if (top_bit < 0) t = kmaxv[r];
+      for (int bit = top_bit; bit >= 0; --bit) {
+        const uint32_t cand = t | (1u << bit);
+        int cnt = 0;
+#pragma unroll
+        for (int u = 0; u < KR; ++u) cnt += (kr[r][u] >= cand);
+        cnt = __reduce_add_sync(kFull, cnt);
+        if (cnt >= k) t = cand;
+        if (cnt == k) break;
+      }
+      nge = 0;
+#pragma unroll
+      for (int u = 0; u < KR; ++u) nge += (kr[r][u] >= t);
+    }
+    // ordered compaction: keys above the threshold, then the lowest-indexed keys equal to it.  With t >= 1 the
+    // zero keys that stand for blocks outside the candidate range never pass a comparison (t = 0 only when a
+    // candidate's own key is 0, the key of one NaN pattern: the general path below handles it).
+    nge = __reduce_add_sync(kFull, nge);
+    const uint32_t lt_mask = (1u << lane) - 1u;
+    int out = 0;
+    if (nge == k && t != 0u) {   // no surplus of keys equal to the threshold: keep every key >= t
+      // lane u takes the ballot of keys 32u .. 32u + 31 (and of the 32 ballots after the 32nd), an exclusive sum over
+      // the lanes gives its place in the list, and it writes its few indices itself
+#pragma unroll
+      for (int base = 0; base < KR; base += 32) {
+        uint32_t mine = 0u;
+#pragma unroll
+        for (int u = base; u < KR && u < base + 32; ++u) {
+          const uint32_t keep_ballot = __ballot_sync(kFull, kr[r][u] >= t);
+          if (lane == u - base) mine = keep_ballot;
+        }
+        int at = __popc(mine);
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+          const int before = __shfl_up_sync(kFull, at, o);
+          if (lane >= o) at += before;
+        }
+        const int total = __shfl_sync(kFull, at, 31);
+        int32_t* d = dst[r] + out + at - __popc(mine);
+        for (; mine != 0u; mine &= mine - 1u) *d++ = (base + lane) * 32 + __ffs(mine) - 1;
+        out += total;
+      }
+      continue;
+    }
+    int ngreater = 0;
+#pragma unroll
+    for (int u = 0; u < KR; ++u) ngreater += (kr[r][u] > t);
+    ngreater = __reduce_add_sync(kFull, ngreater);
+    const int ties_allowed = k - ngreater;  // >= 1: lowest indices among the keys equal to t
+    int ties_seen = 0;
+#pragma unroll
+    for (int u = 0; u < KR; ++u) {
+      if (32 * u < nb) {
+        const int j = lane + 32 * u;
+        const bool valid = WINDOW ? (j >= jlo[r] && j <= jhi[r]) : (j < nb);
+        const bool tie = valid && (kr[r][u] == t);
+        const uint32_t tie_ballot = __ballot_sync(kFull, tie);
+        const int tie_rank = ties_seen + __popc(tie_ballot & lt_mask);
+        const bool keep = valid && ((kr[r][u] > t) || (tie && tie_rank < ties_allowed));
+        const uint32_t keep_ballot = __ballot_sync(kFull, keep);
+        if (keep) dst[r][out + __popc(keep_ballot & lt_mask)] = j;
+        out += __popc(keep_ballot);
+        ties_seen += __popc(tie_ballot);
+      }
     }
   }
 }
 
-template <int D, int ROWS, bool WINDOW>
-__global__ void __launch_bounds__(kTopkThreads, ROWS == 16 ? 3 : 4)
+// Selection of a CTA's rows from their keys in shared memory: a warp takes rows WARPS apart, NR of them at a time.
+// SHORT: nb <= 256, otherwise more.
+template <bool WINDOW, int WARPS, int NR, bool SHORT>
+__device__ __forceinline__ void select_tile(const uint32_t* s_key, int nb, int nbp, int topk, int64_t bh, int i0, int nrows, int N,
+                                            int blk_size, int frame_tokens, int window, int32_t* __restrict__ kept_idx,
+                                            int32_t* __restrict__ kept_cnt) {
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const bool all = topk >= nb;        // with all candidates kept there is nothing to compare
+  for (int first = warp; first < nrows; first += WARPS * NR) {
+    const uint32_t* key[NR];
+    int32_t* dst[NR];
+    int jlo[NR], jhi[NR], k_row[NR];
+#pragma unroll
+    for (int r = 0; r < NR; ++r) {
+      const int row = first + WARPS * r < nrows ? first + WARPS * r : first;        // (beyond the last row: the first one again)
+      key[r] = s_key + (int64_t)row * nbp;
+      dst[r] = kept_idx + (bh * nb + i0 + row) * (int64_t)topk;
+      // Causal frame window (Sec. 1, auto-regressive extension): only the key blocks that hold a key some
+      // row of this query block may attend to are candidates, a contiguous run jlo..jhi.
+      jlo[r] = 0;
+      jhi[r] = nb - 1;
+      if constexpr (WINDOW) {
+        const int r0 = (i0 + row) * blk_size, r1 = min((i0 + row + 1) * blk_size, N) - 1;
+        const int f0 = max(r0 / frame_tokens - window + 1, 0);
+        const int kend = (int)min((long long)(r1 / frame_tokens + 1) * frame_tokens, (long long)N);
+        jlo[r] = (int)((long long)f0 * frame_tokens / blk_size);
+        jhi[r] = (kend - 1) / blk_size;
+      }
+      k_row[r] = min(topk, jhi[r] - jlo[r] + 1);
+      if constexpr (WINDOW)
+        for (int t = k_row[r] + lane; t < topk; t += 32) dst[r][t] = -1;    // unused tail of a list cut short by the window
+      if (lane == 0 && kept_cnt != nullptr) kept_cnt[bh * nb + i0 + row] = k_row[r];
+    }
+    if (all) {
+#pragma unroll
+      for (int r = 0; r < NR; ++r)
+        for (int t = lane; t < k_row[r]; t += 32) dst[r][t] = jlo[r] + t;
+    } else if constexpr (SHORT) {       // nb <= 256
+      select_rows_regs<8, WINDOW, NR>(key, nb, jlo, jhi, k_row, lane, dst);
+    } else if (nb <= 32 * 20) {
+      select_rows_regs<20, WINDOW, NR>(key, nb, jlo, jhi, k_row, lane, dst);
+    } else if (nb <= 32 * 40) {
+      select_rows_regs<40, WINDOW, NR>(key, nb, jlo, jhi, k_row, lane, dst);
+    } else {
+#pragma unroll
+      for (int r = 0; r < NR; ++r)
+        select_row([&](int j) { return (WINDOW ? (j >= jlo[r] && j <= jhi[r]) : (j < nb)) ? key[r][j] : 0u; }, nb, jlo[r],
+                   jhi[r], k_row[r], lane, dst[r]);
+    }
+  }
+}
+
+// the keys of a thread's 2 * PAIRS x 4 scores into the rows of the key tile
+template <int PAIRS>
+__device__ __forceinline__ void store_keys(const uint64_t (&acc)[4][PAIRS], uint32_t* out, int nbp) {
+#pragma unroll
+  for (int r = 0; r < PAIRS; ++r) {
+    uint4 lo, hi;
+    float2 a;
+    a = unpack_f32x2(acc[0][r]); lo.x = score_key(a.x); hi.x = score_key(a.y);
+    a = unpack_f32x2(acc[1][r]); lo.y = score_key(a.x); hi.y = score_key(a.y);
+    a = unpack_f32x2(acc[2][r]); lo.z = score_key(a.x); hi.z = score_key(a.y);
+    a = unpack_f32x2(acc[3][r]); lo.w = score_key(a.x); hi.w = score_key(a.y);
+    *reinterpret_cast<uint4*>(out + (2 * r) * nbp) = lo;
+    *reinterpret_cast<uint4*>(out + (2 * r + 1) * nbp) = hi;
+  }
+}
+
+// RT x 4 scores per thread; the CTA's 8 warps are RG groups of RT rows times 8 / RG groups of 128 key blocks.  NS ring
+// stages of KC channels.
+template <int RT, int RG, int KC, int NS>
+struct TopkShape {
+  static constexpr int kRows = RT * RG, kCols = 128 * (8 / RG);
+  static constexpr int kStageFloats = KC * kCols;
+  static constexpr size_t smem_bytes(int d, int nbp) {
+    return (size_t)(NS * kStageFloats + kRows * d) * sizeof(float) + (size_t)kRows * nbp * sizeof(uint32_t);
+  }
+};
+
+template <int D, int RT, int RG, int KC, int NS, bool WINDOW>
+__global__ void __launch_bounds__(kTopkThreads, 2)
 topk_kernel(const float* __restrict__ pq, const float* __restrict__ pkT, int32_t* __restrict__ kept_idx,
             int32_t* __restrict__ kept_cnt, int nb, int nbp, int topk, int groups_per_bh, int N, int blk_size,
             int frame_tokens, int window) {
+  using Shape = TopkShape<RT, RG, KC, NS>;
+  constexpr int R = Shape::kRows, JT = Shape::kCols;
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  // pooled Q of the CTA's ROWS query blocks, channel-major: s_pq[c][r], so that one 16-byte load
-  // yields four rows of one channel as two packed fp32x2 operands
-  float* s_pq = reinterpret_cast<float*>(smem_raw);                   // [D][ROWS]
-  uint32_t* s_key = reinterpret_cast<uint32_t*>(s_pq + ROWS * D);     // [ROWS][nbp]
+  float* s_ring = reinterpret_cast<float*>(smem_raw);                 // [NS][KC][JT] pooled K, channel-major
+  // pooled Q of the CTA's R query blocks, channel-major: s_pq[c][r], so that one 16-byte load yields four rows of one
+  // channel as two packed fp32x2 operands
+  float* s_pq = s_ring + NS * Shape::kStageFloats;                    // [D][R]
+  uint32_t* s_key = reinterpret_cast<uint32_t*>(s_pq + R * D);        // [R][nbp]
 
   const int64_t bh = blockIdx.x / groups_per_bh;
-  const int i0 = (blockIdx.x % groups_per_bh) * ROWS;
-  const int nrows = min(ROWS, nb - i0);
-
-  for (int e = threadIdx.x; e < ROWS * D; e += kTopkThreads) {
-    const int r = e / D, c = e % D;
-    s_pq[c * ROWS + r] = (r < nrows) ? pq[(bh * nb + i0 + r) * D + c] : 0.0f;
-  }
-  __syncthreads();
-
-  // scores: a thread owns 4 adjacent key blocks (one 16-byte load per channel) and walks the channels
-  // in ascending order for the CTA's ROWS query blocks at once: a ROWS x 4 register tile.
-  // fma.rn.f32x2 is a pair of IEEE fmaf over two rows, so every accumulator still sees exactly the
-  // chain a = fmaf(pq[i,c], pk[j,c], a), c ascending.  Columns nb..nbp-1 of pooled K are padding
-  // whose scores are stored but never read.
-  const float* kcol = pkT + bh * D * (int64_t)nbp;
-  const ulonglong2* s_pq2 = reinterpret_cast<const ulonglong2*>(s_pq);       // [D][ROWS / 4]
-  constexpr int kPairs = ROWS / 2;
-  constexpr int kCB = 4;   // channels per batch of loads; two batches (2 x 4 x 16 bytes) in flight per thread
-  for (int j0 = threadIdx.x * 4; j0 < nb; j0 += kTopkThreads * 4) {
-    uint64_t acc[4][kPairs];
-#pragma unroll
-    for (int u = 0; u < 4; ++u)
-#pragma unroll
-      for (int r = 0; r < kPairs; ++r) acc[u][r] = pack_f32x2(0.0f, 0.0f);
-    const float* kp = kcol + j0;
-    auto load_batch = [&](float4 (&kv)[kCB], int c0) {
-#pragma unroll
-      for (int cc = 0; cc < kCB; ++cc) kv[cc] = __ldg(reinterpret_cast<const float4*>(kp + (int64_t)(c0 + cc) * nbp));
-    };
-    auto fma_batch = [&](const float4 (&kv)[kCB], int c0) {
-#pragma unroll
-      for (int cc = 0; cc < kCB; ++cc) {
-        uint64_t q2[kPairs];
-#pragma unroll
-        for (int g = 0; g < ROWS / 4; ++g) {
-          const ulonglong2 t = s_pq2[(c0 + cc) * (ROWS / 4) + g];   // rows (4g, 4g+1), (4g+2, 4g+3)
-          q2[2 * g] = t.x;
-          q2[2 * g + 1] = t.y;
-        }
-        const uint64_t k2[4] = {pack_f32x2(kv[cc].x, kv[cc].x), pack_f32x2(kv[cc].y, kv[cc].y),
-                                pack_f32x2(kv[cc].z, kv[cc].z), pack_f32x2(kv[cc].w, kv[cc].w)};
-#pragma unroll
-        for (int u = 0; u < 4; ++u)
-#pragma unroll
-          for (int r = 0; r < kPairs; ++r) acc[u][r] = ffma2(q2[r], k2[u], acc[u][r]);
-      }
-    };
-    float4 kva[kCB], kvb[kCB];
-    load_batch(kva, 0);
-#pragma unroll 1
-    for (int c0 = 0; c0 < D; c0 += 2 * kCB) {
-      load_batch(kvb, c0 + kCB);
-      fma_batch(kva, c0);
-      if (c0 + 2 * kCB < D) load_batch(kva, c0 + 2 * kCB);
-      fma_batch(kvb, c0 + kCB);
-    }
-#pragma unroll
-    for (int r = 0; r < kPairs; ++r) {
-      uint4 lo, hi;
-      float2 a;
-      a = unpack_f32x2(acc[0][r]); lo.x = score_key(a.x); hi.x = score_key(a.y);
-      a = unpack_f32x2(acc[1][r]); lo.y = score_key(a.x); hi.y = score_key(a.y);
-      a = unpack_f32x2(acc[2][r]); lo.z = score_key(a.x); hi.z = score_key(a.y);
-      a = unpack_f32x2(acc[3][r]); lo.w = score_key(a.x); hi.w = score_key(a.y);
-      *reinterpret_cast<uint4*>(s_key + (2 * r) * nbp + j0) = lo;
-      *reinterpret_cast<uint4*>(s_key + (2 * r + 1) * nbp + j0) = hi;
-    }
-  }
-  __syncthreads();
-
-  // selection: the CTA's warps take the rows round-robin, one warp per row
+  const int i0 = (blockIdx.x % groups_per_bh) * R;
+  const int nrows = min(R, nb - i0);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  for (int row = warp; row < nrows; row += kTopkThreads / 32) {
-    const uint32_t* key = s_key + row * nbp;
-    int32_t* dst = kept_idx + (bh * nb + i0 + row) * (int64_t)topk;
-    // Causal frame window (Sec. 1, auto-regressive extension): only the key blocks that hold a key some
-    // row of this query block may attend to are candidates, a contiguous run jlo..jhi.
-    int jlo = 0, jhi = nb - 1;
-    if constexpr (WINDOW) {
-      const int r0 = (i0 + row) * blk_size, r1 = min((i0 + row + 1) * blk_size, N) - 1;
-      const int f0 = max(r0 / frame_tokens - window + 1, 0);
-      const int kend = (int)min((long long)(r1 / frame_tokens + 1) * frame_tokens, (long long)N);
-      jlo = (int)((long long)f0 * frame_tokens / blk_size);
-      jhi = (kend - 1) / blk_size;
+  const float* kcol = pkT + bh * D * (int64_t)nbp;
+
+  constexpr int kSteps = D / KC;                                      // stages per sweep over JT key blocks
+  const int steps = (nbp + JT - 1) / JT * kSteps;
+  // with all candidates kept there is nothing to compare
+  const bool all = topk >= nb;
+  auto issue = [&](int step) {
+    if (step < steps) {
+      const int j0 = step / kSteps * JT, c0 = step % kSteps * KC;
+      const int w4 = min(JT, nbp - j0) / 4;
+      const uint32_t dst = smem_u32(s_ring + step % NS * Shape::kStageFloats);
+      const float* src = kcol + (int64_t)c0 * nbp + j0;
+#pragma unroll
+      for (int e = threadIdx.x; e < KC * JT / 4; e += kTopkThreads) {
+        const int c = e / (JT / 4), x = e % (JT / 4);
+        if (x < w4) cp_async16(dst + (c * JT + 4 * x) * 4, src + (int64_t)c * nbp + 4 * x);
+      }
     }
-    const int k_row = min(topk, jhi - jlo + 1);
-    if (nb <= 32 * 8) {
-      select_row_regs<8, WINDOW>(key, nb, jlo, jhi, k_row, lane, dst);
-    } else if (nb <= 32 * 20) {
-      select_row_regs<20, WINDOW>(key, nb, jlo, jhi, k_row, lane, dst);
-    } else if (nb <= 32 * 40) {
-      select_row_regs<40, WINDOW>(key, nb, jlo, jhi, k_row, lane, dst);
-    } else {
-      select_row([&](int j) { return (WINDOW ? (j >= jlo && j <= jhi) : (j < nb)) ? key[j] : 0u; }, nb, jlo, jhi, k_row,
-                 lane, dst);
+    cp_async_commit();
+  };
+
+  pdl_wait();
+  if (!all) {
+#pragma unroll
+    for (int p = 0; p < NS - 1; ++p) issue(p);
+    for (int e = threadIdx.x; e < R * (D / 4); e += kTopkThreads) {
+      const int r = e % R, c = e / R * 4;
+      const float4 x = r < nrows ? __ldg(reinterpret_cast<const float4*>(pq + (bh * nb + i0 + r) * D + c))
+                                 : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+      s_pq[c * R + r] = x.x; s_pq[(c + 1) * R + r] = x.y; s_pq[(c + 2) * R + r] = x.z; s_pq[(c + 3) * R + r] = x.w;
     }
-    if constexpr (WINDOW)
-      for (int t = k_row + lane; t < topk; t += 32) dst[t] = -1;    // unused tail of a list cut short by the window
-    if (lane == 0 && kept_cnt != nullptr) kept_cnt[bh * nb + i0 + row] = k_row;
+
+    // scores: a thread owns 4 adjacent key blocks and RT query blocks and walks the channels in ascending order.
+    // fma.rn.f32x2 is a pair of IEEE fmaf over two rows, so every accumulator sees exactly the chain
+    // a = fmaf(pq[i,c], pk[j,c], a), c ascending.  Columns nb..nbp-1 of pooled K are padding whose scores are stored
+    // but never read.
+    constexpr int kPairs = RT / 2;
+    const int rg = warp % RG, jc = warp / RG * 128 + lane * 4;        // first row of the thread: rg * RT; its column in the sweep
+    for (int j0 = 0, step = 0; j0 < nbp; j0 += JT) {
+      uint64_t acc[4][kPairs];
+#pragma unroll
+      for (int u = 0; u < 4; ++u)
+#pragma unroll
+        for (int r = 0; r < kPairs; ++r) acc[u][r] = pack_f32x2(0.0f, 0.0f);
+      const bool mine = j0 + warp / RG * 128 < nbp;                   // the warp has a key block in this sweep
+#pragma unroll 1
+      for (int s = 0; s < kSteps; ++s, ++step) {
+        cp_async_wait<NS - 2>();
+        __syncthreads();                 // this stage has landed for everybody, and the slot of the last one is free
+        issue(step + NS - 1);
+        if (mine) {
+          const float* kst = s_ring + step % NS * Shape::kStageFloats + jc;
+          const float* qst = s_pq + s * KC * R + rg * RT;
+#pragma unroll
+          for (int cc = 0; cc < KC; ++cc) {
+            uint64_t q2[kPairs];
+            if constexpr (RT >= 4) {
+#pragma unroll
+              for (int g = 0; g < RT / 4; ++g) {
+                const ulonglong2 t = *reinterpret_cast<const ulonglong2*>(qst + cc * R + 4 * g);   // rows (4g, 4g+1), (4g+2, 4g+3)
+                q2[2 * g] = t.x;
+                q2[2 * g + 1] = t.y;
+              }
+            } else {
+              q2[0] = *reinterpret_cast<const uint64_t*>(qst + cc * R);
+            }
+            const float4 kv = *reinterpret_cast<const float4*>(kst + cc * JT);
+            const uint64_t k2[4] = {pack_f32x2(kv.x, kv.x), pack_f32x2(kv.y, kv.y), pack_f32x2(kv.z, kv.z),
+                                    pack_f32x2(kv.w, kv.w)};
+#pragma unroll
+            for (int u = 0; u < 4; ++u)
+#pragma unroll
+              for (int r = 0; r < kPairs; ++r) acc[u][r] = ffma2(q2[r], k2[u], acc[u][r]);
+          }
+        }
+      }
+      if (j0 + jc < nbp) {
+        store_keys<kPairs>(acc, s_key + (int64_t)(rg * RT) * nbp + j0 + jc, nbp);
+      }
+    }
+    __syncthreads();
   }
+
+  select_tile<WINDOW, 8, (R >= 16 ? 2 : 1), true>(s_key, nb, nbp, topk, bh, i0, nrows, N, blk_size, frame_tokens, window, kept_idx, kept_cnt);
 }
 
-template <int D, int ROWS>
+// The same for long rows of key blocks: a CTA of WARPS warps takes R query blocks, a thread owns an RT x 4 register tile
+// and reads its own pooled K columns straight from L2 (two batches of 4 channels in flight), so that a warp never
+// waits for another one until the scores are complete.  Bound by the FMA pipe and, in the selection, by latency: what
+// helps both is warps, so the tile is 8 x 4 (96 registers, two CTAs of ten warps per SM) although 16 x 4 needs fewer
+// shared loads per FMA.  40 heads of 591 blocks: 126 us (16 x 4 with five warps, three CTAs: 121; with one row searched
+// bit by bit at a time, as it was: 147); of 1182: 439 us (484; 596).  The FMAs alone are 50 and 200 us.
+template <int D, int R, int RT, int WARPS, int CTAS, bool WINDOW>
+__global__ void __launch_bounds__(WARPS * 32, CTAS)
+topk_wide_kernel(const float* __restrict__ pq, const float* __restrict__ pkT, int32_t* __restrict__ kept_idx,
+                 int32_t* __restrict__ kept_cnt, int nb, int nbp, int topk, int groups_per_bh, int N, int blk_size,
+                 int frame_tokens, int window) {
+  constexpr int kThreads = WARPS * 32;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  float* s_pq = reinterpret_cast<float*>(smem_raw);                   // [D][R], see topk_kernel
+  uint32_t* s_key = reinterpret_cast<uint32_t*>(s_pq + R * D);        // [R][nbp]
+  const int64_t bh = blockIdx.x / groups_per_bh;
+  const int i0 = (blockIdx.x % groups_per_bh) * R;
+  const int nrows = min(R, nb - i0);
+
+  pdl_wait();
+  if (topk < nb) {
+    for (int e = threadIdx.x; e < R * (D / 4); e += kThreads) {
+      const int r = e % R, c = e / R * 4;
+      const float4 x = r < nrows ? __ldg(reinterpret_cast<const float4*>(pq + (bh * nb + i0 + r) * D + c))
+                                 : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+      s_pq[c * R + r] = x.x; s_pq[(c + 1) * R + r] = x.y; s_pq[(c + 2) * R + r] = x.z; s_pq[(c + 3) * R + r] = x.w;
+    }
+    __syncthreads();
+    const float* kcol = pkT + bh * D * (int64_t)nbp;
+    const ulonglong2* s_pq2 = reinterpret_cast<const ulonglong2*>(s_pq);       // [D][R / 4]
+    constexpr int RG = R / RT, kPairs = RT / 2;
+    constexpr int kCB = 4;   // channels per batch of loads
+    const int rg = (threadIdx.x >> 5) % RG;
+    for (int j0 = (threadIdx.x / (32 * RG) * 32 + (threadIdx.x & 31)) * 4; j0 < nb; j0 += kThreads / RG * 4) {
+      uint64_t acc[4][kPairs];
+#pragma unroll
+      for (int u = 0; u < 4; ++u)
+#pragma unroll
+        for (int r = 0; r < kPairs; ++r) acc[u][r] = pack_f32x2(0.0f, 0.0f);
+      const float* kp = kcol + j0;
+      auto load_batch = [&](float4 (&kv)[kCB], int c0) {
+#pragma unroll
+        for (int cc = 0; cc < kCB; ++cc) kv[cc] = __ldg(reinterpret_cast<const float4*>(kp + (int64_t)(c0 + cc) * nbp));
+      };
+      auto fma_batch = [&](const float4 (&kv)[kCB], int c0) {
+#pragma unroll
+        for (int cc = 0; cc < kCB; ++cc) {
+          uint64_t q2[kPairs];
+#pragma unroll
+          for (int g = 0; g < RT / 4; ++g) {
+            const ulonglong2 t = s_pq2[(c0 + cc) * (R / 4) + rg * (RT / 4) + g];   // rows (4g, 4g+1), (4g+2, 4g+3)
+            q2[2 * g] = t.x;
+            q2[2 * g + 1] = t.y;
+          }
+          const uint64_t k2[4] = {pack_f32x2(kv[cc].x, kv[cc].x), pack_f32x2(kv[cc].y, kv[cc].y),
+                                  pack_f32x2(kv[cc].z, kv[cc].z), pack_f32x2(kv[cc].w, kv[cc].w)};
+#pragma unroll
+          for (int u = 0; u < 4; ++u)
+#pragma unroll
+            for (int r = 0; r < kPairs; ++r) acc[u][r] = ffma2(q2[r], k2[u], acc[u][r]);
+        }
+      };
+      float4 kva[kCB], kvb[kCB];
+      load_batch(kva, 0);
+#pragma unroll 1
+      for (int c0 = 0; c0 < D; c0 += 2 * kCB) {
+        load_batch(kvb, c0 + kCB);
+        fma_batch(kva, c0);
+        if (c0 + 2 * kCB < D) load_batch(kva, c0 + 2 * kCB);
+        fma_batch(kvb, c0 + kCB);
+      }
+      store_keys<kPairs>(acc, s_key + (int64_t)(rg * RT) * nbp + j0, nbp);
+    }
+    __syncthreads();
+  }
+  select_tile<WINDOW, WARPS, 1, false>(s_key, nb, nbp, topk, bh, i0, nrows, N, blk_size, frame_tokens, window, kept_idx, kept_cnt);
+}
+
+template <int D, int RT, int RG, int KC, int NS>
 static int launch_topk(const float* pq, const float* pkT, int32_t* kept_idx, int32_t* kept_cnt, int nb, int nbp, int topk,
-                       int64_t bh, int N, int block, int frame_tokens, int window, cudaStream_t stream) {
-  const int groups = (nb + ROWS - 1) / ROWS;
+                       int64_t bh, int N, int block, int frame_tokens, int window, bool overlap, cudaStream_t stream) {
+  using Shape = TopkShape<RT, RG, KC, NS>;
+  const int groups = (nb + Shape::kRows - 1) / Shape::kRows;
   const int64_t ctas = bh * groups;
   if (ctas > 0x7fffffffLL) return SPARKATTN_E_UNSUPPORTED_SHAPE;
-  const size_t smem = (size_t)ROWS * D * sizeof(float) + (size_t)ROWS * nbp * sizeof(uint32_t);
-  auto kern = frame_tokens > 0 ? topk_kernel<D, ROWS, true> : topk_kernel<D, ROWS, false>;
+  const size_t smem = Shape::smem_bytes(D, nbp);
+  auto kern = frame_tokens > 0 ? topk_kernel<D, RT, RG, KC, NS, true> : topk_kernel<D, RT, RG, KC, NS, false>;
   if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
     return SPARKATTN_E_CUDA;
-  kern<<<(unsigned)ctas, kTopkThreads, smem, stream>>>(pq, pkT, kept_idx, kept_cnt, nb, nbp, topk, groups, N, block,
-                                                       frame_tokens, window);
-  return SPARKATTN_OK;
+  return launch_kernel(kern, (unsigned)ctas, kTopkThreads, smem, overlap, stream, pq, pkT, kept_idx, kept_cnt, nb, nbp, topk,
+                       groups, N, block, frame_tokens, window);
+}
+
+static size_t wide_smem(int rows, int d, int nbp) { return (size_t)rows * (d + nbp) * sizeof(float); }
+
+template <int D, int R, int RT, int WARPS, int CTAS>
+static int launch_topk_wide(const float* pq, const float* pkT, int32_t* kept_idx, int32_t* kept_cnt, int nb, int nbp, int topk,
+                            int64_t bh, int N, int block, int frame_tokens, int window, bool overlap, cudaStream_t stream) {
+  const int groups = (nb + R - 1) / R;
+  const int64_t ctas = bh * groups;
+  if (ctas > 0x7fffffffLL) return SPARKATTN_E_UNSUPPORTED_SHAPE;
+  const size_t smem = wide_smem(R, D, nbp);
+  auto kern = frame_tokens > 0 ? topk_wide_kernel<D, R, RT, WARPS, CTAS, true> : topk_wide_kernel<D, R, RT, WARPS, CTAS, false>;
+  if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
+    return SPARKATTN_E_CUDA;
+  return launch_kernel(kern, (unsigned)ctas, WARPS * 32, smem, overlap, stream, pq, pkT, kept_idx, kept_cnt, nb, nbp, topk,
+                       groups, N, block, frame_tokens, window);
 }
 
 // Where the pooled means live in a selection workspace: pooled Q [B*H][nb][d] right behind the header, pooled K
@@ -404,24 +645,42 @@ float* select_pooled_ptr(const sparkattn_shape_t& s, void* workspace, bool key_s
   return key_side ? pq + (int64_t)s.B * s.H * nb * s.d : pq;
 }
 
-// scores + top-k on pooled means that are already in the workspace
-static int launch_topk_any(const sparkattn_shape_t& s, int topk, int frame_tokens, int window, int32_t* kept_idx,
-                           int32_t* kept_cnt, void* workspace, cudaStream_t stream) {
+// scores + top-k on pooled means that are already in the workspace (overlap: the kernel that pools them is the last
+// launch on the stream)
+template <int D>
+static int launch_topk_d(const sparkattn_shape_t& s, int topk, int frame_tokens, int window, int32_t* kept_idx,
+                         int32_t* kept_cnt, void* workspace, bool overlap, cudaStream_t stream) {
   const int nb = (s.N + s.block - 1) / s.block;
   const int nbp = round_up(nb, 32);
   const int64_t bh = (int64_t)s.B * s.H;
   const float* pq = select_pooled_ptr(s, workspace, false);
   const float* pkT = select_pooled_ptr(s, workspace, true);
-  // 16 query blocks per CTA while two CTAs' score rows fit one SM's shared memory and the grid still
-  // fills the device several times over (small problems are bound by the latency of one CTA), else 8
-  constexpr int kNumSMs = 148;   // B200; another count only moves the point where the CTAs get smaller
-  const bool rows16 = (size_t)16 * nbp * sizeof(uint32_t) <= 100u * 1024u && bh * ((nb + 15) / 16) >= 6 * kNumSMs;
-  if (s.d == 128)
-    return rows16 ? launch_topk<128, 16>(pq, pkT, kept_idx, kept_cnt, nb, nbp, topk, bh, s.N, s.block, frame_tokens, window, stream)
-                  : launch_topk<128, 8>(pq, pkT, kept_idx, kept_cnt, nb, nbp, topk, bh, s.N, s.block, frame_tokens, window, stream);
-  if (s.d == 64)
-    return rows16 ? launch_topk<64, 16>(pq, pkT, kept_idx, kept_cnt, nb, nbp, topk, bh, s.N, s.block, frame_tokens, window, stream)
-                  : launch_topk<64, 8>(pq, pkT, kept_idx, kept_cnt, nb, nbp, topk, bh, s.N, s.block, frame_tokens, window, stream);
+  auto go = [&](auto launch) {
+    return launch(pq, pkT, kept_idx, kept_cnt, nb, nbp, topk, bh, s.N, s.block, frame_tokens, window, overlap, stream);
+  };
+  constexpr size_t kOne = 227 * 1024, kTwo = 113 * 1024;       // shared memory of a CTA alone on its SM, and of one of two
+  constexpr int kNumSMs = 148;   // B200; another count only moves the points where the CTAs get smaller
+  const int64_t ctas32 = bh * ((nb + 31) / 32), ctas16 = bh * ((nb + 15) / 16);
+  // More than 256 key blocks (d = 128, one launch): the wide kernel, which the other one matches at best (1 head of 591
+  // blocks 20.8 against 22.5 us, but 4 heads 26.8 against 22.8, 12 heads 55.5 against 45.4, 8 heads of 1182 166 against
+  // 111), with 16 rows while two CTAs' key rows fit an SM and 8 beyond.  Up to 256: the other one (its column split
+  // leaves no warp idle there), with as many rows per CTA as still leave 1.5 CTAs (32 rows) or one CTA (16) per SM:
+  // 80 heads of 250 blocks 63.9 us with 32 rows, 69.9 with 16, 94.6 with 8; 12 heads of 256 22.0 / 20.8 / 22.2; 3 heads
+  // of 50 16.9 / 12.5 / 10.4.
+  if (nb > 256) {
+    if (wide_smem(16, D, nbp) <= kTwo) return go(launch_topk_wide<D, 16, 8, 10, 2>);
+    return go(launch_topk_wide<D, 8, 8, 10, 2>);               // at most 132 KB
+  }
+  static_assert(TopkShape<8, 4, 16, 4>::smem_bytes(D, 256) <= kOne, "the tile of 32 rows of 256 keys");
+  if (2 * ctas32 >= 3 * kNumSMs) return go(launch_topk<D, 8, 4, 16, 4>);
+  if (ctas16 >= kNumSMs) return go(launch_topk<D, 4, 4, 16, 4>);
+  return go(launch_topk<D, 2, 4, 16, 4>);
+}
+
+static int launch_topk_any(const sparkattn_shape_t& s, int topk, int frame_tokens, int window, int32_t* kept_idx,
+                           int32_t* kept_cnt, void* workspace, bool overlap, cudaStream_t stream) {
+  if (s.d == 128) return launch_topk_d<128>(s, topk, frame_tokens, window, kept_idx, kept_cnt, workspace, overlap, stream);
+  if (s.d == 64) return launch_topk_d<64>(s, topk, frame_tokens, window, kept_idx, kept_cnt, workspace, overlap, stream);
   return SPARKATTN_E_UNSUPPORTED_SHAPE;
 }
 
@@ -429,7 +688,7 @@ int launch_select_pooled(const sparkattn_shape_t& s, int topk, int32_t* kept_idx
                          cudaStream_t stream) {
   const int nb = (s.N + s.block - 1) / s.block;
   if (nb > kSelectMaxBlocks) return SPARKATTN_E_UNSUPPORTED_SHAPE;
-  const int rc = launch_topk_any(s, topk, 0, 0, kept_idx, kept_cnt, workspace, stream);
+  const int rc = launch_topk_any(s, topk, 0, 0, kept_idx, kept_cnt, workspace, false, stream);
   if (rc != SPARKATTN_OK) return rc;
   return cudaGetLastError() == cudaSuccess ? SPARKATTN_OK : SPARKATTN_E_CUDA;
 }
@@ -444,18 +703,19 @@ int launch_select(const sparkattn_shape_t& s, const void* q, const void* k, int 
   float* pkT = select_pooled_ptr(s, workspace, true);
   const __nv_bfloat16* qb = static_cast<const __nv_bfloat16*>(q);
   const __nv_bfloat16* kb = static_cast<const __nv_bfloat16*>(k);
-  const int64_t pool_ctas = (2 * n_items + kPoolThreads / 32 - 1) / (kPoolThreads / 32);
-  if (pool_ctas > 0x7fffffffLL) return SPARKATTN_E_UNSUPPORTED_SHAPE;
-  if (s.d == 128) {
-    pool_kernel<128><<<(unsigned)pool_ctas, kPoolThreads, 0, stream>>>(
-        qb, kb, pq, pkT, s.H, s.N, s.block, nb, nbp, s.stride_b, s.stride_h, s.stride_n, n_items, block_valid);
-  } else if (s.d == 64) {
-    pool_kernel<64><<<(unsigned)pool_ctas, kPoolThreads, 0, stream>>>(
-        qb, kb, pq, pkT, s.H, s.N, s.block, nb, nbp, s.stride_b, s.stride_h, s.stride_n, n_items, block_valid);
-  } else {
-    return SPARKATTN_E_UNSUPPORTED_SHAPE;
-  }
-  const int rc = launch_topk_any(s, topk, frame_tokens, window, kept_idx, kept_cnt, workspace, stream);
+  if (s.d != 128 && s.d != 64) return SPARKATTN_E_UNSUPPORTED_SHAPE;
+  const int sm_count = current_sm_count();
+  if (sm_count < 1) return SPARKATTN_E_CUDA;
+  const size_t pool_smem = (size_t)2 * s.block * s.d * 2;
+  auto pool = s.d == 128 ? pool_kernel<128> : pool_kernel<64>;
+  if (cudaFuncSetAttribute(pool, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)pool_smem) != cudaSuccess)
+    return SPARKATTN_E_CUDA;
+  const int64_t resident = (int64_t)sm_count * kPoolCtasPerSm * (65536 / (int)pool_smem);
+  const int64_t pool_ctas = 2 * n_items < resident ? 2 * n_items : resident;
+  const int rc0 = launch_kernel(pool, (unsigned)pool_ctas, s.d / 2, pool_smem, true, stream, qb, kb, pq, pkT, s.H, s.N, s.block, nb,
+                                nbp, s.stride_b, s.stride_h, s.stride_n, n_items, block_valid, static_cast<int32_t*>(workspace));
+  if (rc0 != SPARKATTN_OK) return rc0;
+  const int rc = launch_topk_any(s, topk, frame_tokens, window, kept_idx, kept_cnt, workspace, true, stream);
   if (rc != SPARKATTN_OK) return rc;
   return cudaGetLastError() == cudaSuccess ? SPARKATTN_OK : SPARKATTN_E_CUDA;
 }

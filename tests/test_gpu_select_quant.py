@@ -98,6 +98,32 @@ def test_select_crafted_scores_with_window(pattern):
     assert torch.equal(cnt[0].cpu(), ref_cnt)
 
 
+# (heads, key blocks, missing tokens of the last block, block, d): one side and the other of every line of the dispatch
+# (256 key blocks; CTAs of 8, 16 and 32 rows; 16 and 8 rows of the wide kernel at 1680 blocks of d = 128, 1744 of d = 64)
+# and of the key registers (640, 1280), with remainders of the row tiles and of the last block
+@pytest.mark.parametrize("H,nb,tail,block,d", [(1, 1, 63, 64, 64), (1, 9, 1, 64, 64), (10, 241, 5, 64, 64), (30, 250, 63, 64, 64),
+                                               (3, 256, 0, 64, 128), (2, 257, 17, 64, 64), (1, 640, 1, 64, 64), (1, 641, 0, 64, 64),
+                                               (1, 1281, 30, 64, 64), (1, 1680, 3, 64, 128), (1, 1745, 9, 64, 64)])
+def test_select_kernel_variants_match_oracle(H, nb, tail, block, d):
+    g = torch.Generator().manual_seed(nb)
+    N = nb * block - tail
+    q, k = (torch.randn((1, H, N, d), generator=g).to(torch.bfloat16) for _ in range(2))
+    qd, kd = q.to(DEV), k.to(DEV)
+    for topk in sorted({t for t in (1, 32, 33, 128, 129, nb - 1, nb) if 1 <= t <= nb}):
+        ref_idx, ref_cnt = oracle.select(q[0], k[0], block, topk)
+        idx, cnt = sa.select(qd, kd, block, topk)
+        assert torch.equal(idx[0].cpu(), ref_idx) and torch.equal(cnt[0].cpu(), ref_cnt), topk
+    # the two launches under capture: same lists from a replay
+    ws = sa.alloc_workspace(sa.make_shape(qd, block), 0, topk, DEV)
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        sa.select(qd, kd, block, topk, kept_idx=idx, kept_cnt=cnt, workspace=ws)
+    idx.zero_(), cnt.zero_()
+    graph.replay()
+    assert torch.equal(idx[0].cpu(), ref_idx) and torch.equal(cnt[0].cpu(), ref_cnt)
+    assert sa.read_status(ws) == sa.OK
+
+
 def test_select_strided_layout_and_batch():
     # [B, N, H, d] storage viewed as [B, H, N, d]; two batches
     w = workloads.small_structured(H=2, d=128, grid=(2, 10, 26), block=128, sparsity=0.75, cfg_id=16)
