@@ -203,6 +203,30 @@ def test_persistent_path_short_and_empty_lists(seed, kmax, block):
                 assert torch.all(out[0, h, rows] == 0) and torch.all(torch.isneginf(lse[0, h, rows]))
 
 
+@pytest.mark.parametrize("H,window", [(3, 0), (7, 0), (3, 2)])
+def test_d64_chains_of_every_length(H, window):
+    """d = 64: the tiles of an item go to four chains (H = 3: 123 items, no SM gets a second one) or two (H = 7), so lists
+    of 0 .. 9 blocks leave chains empty, level and one tile apart; ragged last block, and rows whose tiles are all
+    masked in some chains (causal window).  Scores large enough that references are raised on the way."""
+    nbk, block, frame = 41, 64, 300
+    N = nbk * block - 21
+    g = torch.Generator().manual_seed(H + window)
+    q, k, v = (torch.randn((1, H, N, 64), generator=g) for _ in range(3))
+    q, k, v = (3.0 * q).to(torch.bfloat16), (k * (1.0 + torch.arange(N)[None, None, :, None] / N)).to(torch.bfloat16), v.to(torch.bfloat16)
+    idx = torch.stack([torch.stack([torch.randperm(nbk, generator=g)[:9] for _ in range(nbk)]) for _ in range(H)]).to(torch.int32)
+    cnt = (torch.arange(H * nbk) % 10).reshape(H, nbk).to(torch.int32)
+    kw = dict(frame_tokens=frame, window=window) if window else {}
+    out, lse = sa.fwd(q.to(DEV), k.to(DEV), v.to(DEV), idx[None].to(DEV), cnt[None].to(DEV), block, return_lse=True,
+                      check_status=True, **kw)
+    ref_out, ref_lse = oracle.attention(q[0], k[0], v[0], idx, cnt, block, **kw)
+    got, ref = out[0].cpu().double(), ref_out.reshape(H, -1, 64)[:, :N]
+    gl, rl = lse[0].cpu().double(), ref_lse.reshape(H, -1)[:, :N]
+    empty = torch.isneginf(rl) | (cnt.repeat_interleave(block, 1)[:, :N] == 0)
+    assert torch.equal(torch.isneginf(gl), empty) and torch.all(got[empty] == 0)
+    relrms, maxabs = _errors(got[~empty], ref[~empty])
+    assert relrms <= BF16_RELRMS and maxabs <= BF16_MAXABS and float((gl - rl)[~empty].abs().max()) <= LSE_ABS
+
+
 @pytest.mark.parametrize("block,fp8", [(128, False), (128, True), (64, False)])
 def test_long_permuted_lists_own_block_anywhere(block, fp8):
     """Kept lists of 70-100 entries in random order: the forward's list pre-pass moves the query block's own
