@@ -33,15 +33,21 @@
 // compacted by a small pre-pass into the workspace; every role reads the clean lists from there.
 // Every wait is bounded; nothing here waits on another CTA.
 //
-// EPI variant (kept lists of at most kEpiMaxKept blocks): 512 threads, warps 12-15 are a closing
-// warpgroup.  At the end of an item the softmax warpgroups only leave their partial row sums (the
-// warpgroup of the last tile in the first KB of the item's dead Q slot, the other one in s_lsum) and go
-// on to the next item's tiles; the closing warpgroup waits for the last PV, reads O, normalises it into
-// the Q slot, hands O back to the PV issuer, writes lse and stores the tile.  That takes the wait for the
-// last PV, the O read and the store off the warpgroup whose next tile the pipeline needs (bf16 -2.6 %,
-// FP8 -1 % at 18 tiles per item, 6-8 % at 6); with four more warps resident, and 40 registers for the
-// control warps, the tile loop itself runs 3 % slower, so the launcher keeps the 384-thread kernel for
-// longer lists.
+// EPI variant (512 threads): warps 12-15 are a closing warpgroup.  At the end of an item the softmax warpgroups only
+// leave their partial row sums (the warpgroup of the last tile in the first KB of the item's dead Q slot, the other
+// one in s_lsum) and go on to the next item's tiles; the closing warpgroup waits for the last PV, reads O, normalises
+// it into the Q slot, hands O back to the PV issuer, writes lse and stores the tile.  That takes the wait for the last
+// PV, the O read and the store off the warpgroup whose next tile the pipeline needs; the price is 40 registers for
+// the control and closing warps and another register allocation of the tile loop (see launch_pipe for who gets it).
+//
+// What bounds it: bf16 with 128-token blocks runs at the chip's power limit (1.42-1.50 GHz, whatever happened before the
+// launch); the others at 1.8 GHz by the softmax warps' chain of short steps and the special-function unit.  The
+// kernel's code is larger than the SM's instruction cache and its warps stream through it, so what the hot loops are
+// compiled to matters as much as their order: the control warps run their loops as whole warps with one elected thread
+// issuing (descriptors and coordinates in uniform registers), masks are a bit per column, items are taken apart by a
+// multiplication, waits have the shortest polling loop.  Measured over the version without these (12 heads of 32,760
+// tokens, 18 of 256 blocks kept): 177 -> 159 million warp instructions, 620,000 -> 582,000 clocks; 40 heads of 75,600
+// tokens, 97 %: bf16 2.97 -> 2.86 ms, FP8 2.77 -> 2.60 ms, 64-token blocks 4.30 -> 3.55 ms.
 //
 // GATE variant (sparkattn_fwd_gated; bf16, 128-token blocks, 384 threads): the closing softmax warpgroup
 // adds the gated low-rank term of Sec. 4.1 before the store.  Once the last PV of the item is complete it
@@ -65,9 +71,8 @@ namespace sparkattn {
 
 constexpr int kPipeThreads = 384;                           // GATE variant: 4 control warps + 2 softmax warpgroups
 constexpr int kPipeSoftmaxRegs = 216, kPipeCtrlRegs = 64;   // 2*128*216 + 128*64 <= 384*168
-// short kept lists (EPI): a third warpgroup (warps 12-15) closes the items, see below
+// EPI: a third warpgroup (warps 12-15) closes the items, see above
 constexpr int kEpiThreads = 512;
-constexpr int kEpiMaxKept = 32;                             // longest kept list the launcher gives to that variant
 constexpr int kEpiSoftmaxRegs = 216, kEpiCtrlRegs = 40, kEpiCloseRegs = 40;   // 2*128*216 + 128*40 + 128*40 = 512*128
 constexpr int kPD = 128, kPBLK = 128;
 constexpr float kPipeLazyLog2 = 8.0f;        // bf16: P may exceed 1 by up to 2^8 before O is rescaled
@@ -77,6 +82,18 @@ constexpr float kPipeFp8LazyLog2 = 4.0f, kPipeFp8PScaleLog2 = 4.0f;
 constexpr int kTile = 32768;                               // bytes of one 128 x 128 bf16 tile (two 64-column slabs)
 constexpr int kOffQ = 0, kOffK = 2 * kTile, kOffMisc = 7 * kTile;     // Q slots | K ring, V ring (5 x 32 KB) | barriers ...
 constexpr int kPipeSmem = kOffMisc + 512 /*barriers*/ + 2 * 128 * 4 /*reference maxima*/ + 128 * 8 /*row sums*/ + 64;
+
+// x / d for 0 <= x < 2^31 without the division's twenty-odd instructions at every place that takes an item apart
+struct FastDiv {
+  uint32_t mul, shift;
+};
+static FastDiv make_fast_div(uint32_t d) {
+  FastDiv f{0, 0};
+  while ((1ull << f.shift) < d) ++f.shift;
+  f.mul = (uint32_t)(((1ull << 32) * ((1ull << f.shift) - d)) / d + 1);
+  return f;
+}
+__device__ __forceinline__ int fast_div(int x, FastDiv f) { return (int)((__umulhi((uint32_t)x, f.mul) + (uint32_t)x) >> f.shift); }
 
 struct PipeParams {
   const int32_t* clean_cnt;    // [items] valid kept blocks per item
@@ -88,7 +105,11 @@ struct PipeParams {
   __nv_bfloat16* out;
   float* lse;
   int32_t* status;
+  const int32_t* kept_idx;     // the caller's lists, looked at again only when an index has to be reported
+  const int32_t* kept_cnt;
+  int kmax;
   int H, N, nb, items;
+  FastDiv by_nbq, by_H;
   int nbq;                     // work items per (batch, head): query blocks, or pairs of 64-token query blocks
   int lstride;                 // list entries per item in clean_list
   int frame_tokens, window;    // causal frame window (0 = none): key frame in (query frame - window, query frame]
@@ -103,10 +124,30 @@ struct PipeParams {
   float eps;
 };
 
-// one warp per item: drop (and report) kept indices outside [0, nb), clamp the count, own block first
+// The list pre-passes are also what clears the workspace header, so they cannot report into it themselves (their CTAs
+// run in no order): an item with an index outside [0, nb) gets this flag in its count, and the forward kernel looks the
+// index up and reports it.
+constexpr int32_t kBadFlag = 0x40000000;
+__device__ __forceinline__ int clean_count(const int32_t* clean_cnt, int item) { return __ldg(clean_cnt + item) & ~kBadFlag; }
+__device__ __forceinline__ void report_bad_index(const PipeParams& p, int item, bool pair) {
+  const int bh = item / p.nbq, first = pair ? 2 * (item % p.nbq) : item % p.nbq;
+  for (int qb = first; qb < min(first + (pair ? 2 : 1), p.nb); ++qb) {
+    const int64_t list = (int64_t)bh * p.nb + qb;
+    const int cnt = p.kept_cnt ? min(max(__ldg(p.kept_cnt + list), 0), p.kmax) : p.kmax;
+    for (int t = 0; t < cnt; ++t) {
+      const int kb = __ldg(p.kept_idx + list * p.kmax + t);
+      if (kb < 0 || kb >= p.nb) report_status(p.status, SPARKATTN_E_BAD_INDEX, kb);
+    }
+  }
+}
+
+// one warp per item: drop (and flag) kept indices outside [0, nb), clamp the count, own block first
 __global__ void compact_lists_kernel(const int32_t* __restrict__ kept_idx, const int32_t* __restrict__ kept_cnt,
                                      int32_t* __restrict__ clean_cnt, int32_t* __restrict__ clean_list, int items,
                                      int nb, int kmax, int32_t* status) {
+  pdl_trigger();
+  pdl_wait();
+  if (blockIdx.x == 0 && threadIdx.x < kWorkspaceHeaderBytes / 4) status[threadIdx.x] = 0;
   const int item = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
   const int lane = threadIdx.x & 31;
   if (item >= items) return;
@@ -114,26 +155,29 @@ __global__ void compact_lists_kernel(const int32_t* __restrict__ kept_idx, const
   const int32_t* src = kept_idx + (int64_t)item * kmax;
   int32_t* dst = clean_list + (int64_t)item * kmax;
   int out = 0;
+  bool bad = false;
   for (int base = 0; base < cnt; base += 32) {
     const int t = base + lane;
     const int kb = (t < cnt) ? __ldg(src + t) : 0;
     const bool valid = (t < cnt) && kb >= 0 && kb < nb;
-    if (t < cnt && !valid) report_status(status, SPARKATTN_E_BAD_INDEX, kb);
+    bad = __any_sync(0xffffffffu, (t < cnt) && !valid) || bad;
     const uint32_t ballot = __ballot_sync(0xffffffffu, valid);
     if (valid) dst[out + __popc(ballot & ((1u << lane) - 1u))] = kb;
     out += __popc(ballot);
   }
-  if (lane == 0) clean_cnt[item] = out;
+  if (lane == 0) clean_cnt[item] = out | (bad ? kBadFlag : 0);
   // The query block's own key block goes first.  The result does not depend on the order of the tiles, the
   // work does: a row's running maximum is usually set by its own block, and when that block comes late (it is
   // the last entry of an ascending list under a causal window) nearly every row's maximum jumps past the lazy
   // threshold there and the whole O tile is rescaled; with it first the later tiles stay below the reference.
+  // (The list is read back past L1: the forward kernel may already be resident, and must find no line of it there that
+  // was fetched before a neighbouring item's warp had written its part.)
   __syncwarp();
   const int qb = item % nb;
   int p = -1;
   for (int base = 0; base < out && p < 0; base += 32) {
     const int t = base + lane;
-    const uint32_t hit = __ballot_sync(0xffffffffu, t < out && dst[t] == qb);
+    const uint32_t hit = __ballot_sync(0xffffffffu, t < out && __ldcg(dst + t) == qb);
     if (hit) p = base + __ffs(hit) - 1;
   }
   if (p > 0) {
@@ -141,7 +185,7 @@ __global__ void compact_lists_kernel(const int32_t* __restrict__ kept_idx, const
       const int t = base + lane;
       const bool mine = t <= p;
       int val = 0;
-      if (mine) val = (t == 0) ? qb : dst[t - 1];
+      if (mine) val = (t == 0) ? qb : __ldcg(dst + t - 1);
       __syncwarp();
       if (mine) dst[t] = val;
       __syncwarp();
@@ -159,6 +203,9 @@ __global__ void __launch_bounds__(kPairWarps * 32)
 pair_lists_kernel(const int32_t* __restrict__ kept_idx, const int32_t* __restrict__ kept_cnt,
                   int32_t* __restrict__ clean_cnt, int32_t* __restrict__ clean_list, int pairs, int nb, int nbq,
                   int kmax, int32_t* status) {
+  pdl_trigger();
+  pdl_wait();
+  if (blockIdx.x == 0 && threadIdx.x < kWorkspaceHeaderBytes / 4) status[threadIdx.x] = 0;
   extern __shared__ uint32_t s_bits[];                      // [kPairWarps][2][words]
   const int words = (nb + 31) / 32;
   const int wl = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -168,16 +215,18 @@ pair_lists_kernel(const int32_t* __restrict__ kept_idx, const int32_t* __restric
   for (int i = lane; i < 2 * words; i += 32) bits[i] = 0u;
   __syncwarp();
   const int bh = pair / nbq, qp = pair % nbq;
+  bool bad = false;
   for (int side = 0; side < 2; ++side) {
     const int qb = 2 * qp + side;
     if (qb >= nb) break;
     const int64_t item = (int64_t)bh * nb + qb;
     const int cnt = kept_cnt ? min(max(__ldg(kept_cnt + item), 0), kmax) : kmax;
     const int32_t* src = kept_idx + item * kmax;
-    for (int t = lane; t < cnt; t += 32) {
-      const int kb = __ldg(src + t);
-      if (kb >= 0 && kb < nb) atomicOr(bits + side * words + (kb >> 5), 1u << (kb & 31));
-      else report_status(status, SPARKATTN_E_BAD_INDEX, kb);
+    for (int base = 0; base < cnt; base += 32) {
+      const int kb = base + lane < cnt ? __ldg(src + base + lane) : 0;
+      const bool valid = kb >= 0 && kb < nb;
+      if (base + lane < cnt && valid) atomicOr(bits + side * words + (kb >> 5), 1u << (kb & 31));
+      bad = __any_sync(0xffffffffu, !valid) || bad;
     }
   }
   __syncwarp();
@@ -205,12 +254,14 @@ pair_lists_kernel(const int32_t* __restrict__ kept_idx, const int32_t* __restric
   __syncwarp();
   if (lane == 0) {
     if (out & 1) { dst[out] = dst[out - 1] & 0x3fffffff; }   // odd tail: second half of the last tile is nobody's
-    clean_cnt[pair] = (out + 1) >> 1;
+    clean_cnt[pair] = ((out + 1) >> 1) | (bad ? kBadFlag : 0);
   }
 }
 
 // FP8: largest V block scale of every (batch, head); one warp each
 __global__ void head_vmax_kernel(const float* __restrict__ v_scale, float* __restrict__ v_max, int bh_count, int nb) {
+  pdl_trigger();
+  pdl_wait();
   const int bh = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
   const int lane = threadIdx.x & 31;
   if (bh >= bh_count) return;
@@ -227,6 +278,44 @@ __device__ __forceinline__ void pipe_tma_store_4d(const void* tmap, const void* 
       ::"l"(reinterpret_cast<uint64_t>(tmap)), "r"(smem_u32(smem_src)), "r"(c0), "r"(c1), "r"(c2), "r"(c3)
       : "memory");
 }
+
+// mbar_wait (common.cuh) in the shortest form: this kernel has some twenty of these waits, and what its warps run does
+// not fit the SM's instruction cache as it is.  The limit is the same; on expiry only the wait's id goes to the abort
+// flag, and the teardown reports it.
+constexpr int kAbortTimeout = 256;
+__device__ __forceinline__ uint32_t global_timer_lo() {
+  uint32_t t;
+  asm volatile("mov.u32 %0, %%globaltimer_lo;" : "=r"(t));
+  return t;
+}
+__device__ __forceinline__ bool pipe_wait(uint64_t* bar, uint32_t parity, volatile int* abort_flag, int wait_id) {
+  if (mbar_try_wait(bar, parity)) return true;
+  static_assert(kWaitLimitNs < 0xf0000000ull, "the limit is counted in 32 bits");
+  const uint32_t t0 = global_timer_lo();
+  for (uint32_t it = 1;; ++it) {
+    if (mbar_try_wait(bar, parity)) return true;
+    if ((it & 63u) == 0u) {
+      if (*abort_flag) return false;
+      if (global_timer_lo() - t0 > (uint32_t)kWaitLimitNs) {
+        *abort_flag = kAbortTimeout + wait_id;
+        return false;
+      }
+    }
+  }
+}
+
+// One thread of a converged warp; and a value that is the same in all its threads, told to the compiler as such.
+__device__ __forceinline__ bool elect_one() {
+  uint32_t one;
+  asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(one));
+  return one != 0;
+}
+// a truth value that is known when it is compiled
+template <bool V>
+struct Const {
+  __device__ constexpr operator bool() const { return V; }
+};
+__device__ __forceinline__ int uniform(int x) { return __shfl_sync(0xffffffffu, x, 0); }
 
 // PAIR: 64-token blocks; a work item is a pair of query blocks, a tile two key blocks (see pair_lists_kernel).
 // GATE (bf16, 128-token blocks, no window): the closing warpgroup of an item also computes the low-rank branch
@@ -274,7 +363,7 @@ fwd_pipe_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
   volatile int* s_abort = reinterpret_cast<volatile int*>(s_tmem + 1);
   volatile int* s_gate_bh = s_abort + 1;      // GATE: (batch, head) whose P_q and C are in shared memory
 
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = uniform(threadIdx.x >> 5), lane = threadIdx.x & 31;
   constexpr int kTileTx = FP8 ? kTile / 2 : kTile;
   constexpr int kEnt = PAIR ? 2 : 1;              // list entries per tile
   constexpr int kKeyBlk = PAIR ? 64 : 128;        // tokens per key block
@@ -295,12 +384,6 @@ fwd_pipe_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
     for (int i = 0; i < RK; ++i) { mbar_init(bar_k_full + i, 1); mbar_init(bar_k_free + i, 1); }
     for (int i = 0; i < RV; ++i) { mbar_init(bar_v_full + i, 1); mbar_init(bar_v_free + i, 1); }
     mbar_init(bar_o_free, 128); mbar_init(bar_lsum, 128); mbar_init(bar_lsum_ack, 128);
-    int dead = (*reinterpret_cast<volatile int32_t*>(p.status) == SPARKATTN_E_DEVICE_TIMEOUT) ? 1 : 0;
-    if ((smem_u32(smem) & 1023u) != 0u) {       // the swizzled tiles need a 1024-byte aligned base
-      report_status(p.status, SPARKATTN_E_MISALIGNED, (int)(smem_u32(smem) & 1023u));
-      dead = 1;
-    }
-    *s_abort = dead;
     mbar_fence_init();
   }
   if (warp == 0) {
@@ -312,6 +395,15 @@ fwd_pipe_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
     tmem_alloc(s_tmem, 512);
     tmem_relinquish();
   }
+  pdl_wait();                                   // everything above runs while the list pre-pass drains
+  if (threadIdx.x == 0) {
+    int dead = (*reinterpret_cast<volatile int32_t*>(p.status) == SPARKATTN_E_DEVICE_TIMEOUT) ? 1 : 0;
+    if ((smem_u32(smem) & 1023u) != 0u) {       // the swizzled tiles need a 1024-byte aligned base
+      report_status(p.status, SPARKATTN_E_MISALIGNED, (int)(smem_u32(smem) & 1023u));
+      dead = 1;
+    }
+    *s_abort = dead;
+  }
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
@@ -320,6 +412,15 @@ fwd_pipe_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
   const uint32_t tmem_O = tmem + 3 * kPBLK;
   const bool dead = *s_abort != 0;
   const int first_item = blockIdx.x, item_step = gridDim.x;
+  // A wait of a control warp.  bf16 with 128-token blocks runs at the chip's power limit: there one thread polls and
+  // all learn of it (720p shape at 97 %: 2.86 ms, against 3.00 with 32 polling threads in 3 % fewer clocks).  The
+  // others run at full clock and take the shorter way.
+  constexpr bool kLone = !FP8 && !PAIR;
+  auto ctrl_wait = [&](uint64_t* bar, uint32_t parity, int id) {
+    bool done = true;
+    if (!kLone || lane == 0) done = pipe_wait(bar, parity, s_abort, id);
+    return kLone ? __all_sync(0xffffffffu, done) != 0 : done;
+  };
 
   static_assert(!EPI || !GATE, "the gated variant closes its items in the softmax warpgroups");
   if constexpr (EPI) {
@@ -332,150 +433,158 @@ fwd_pipe_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
     // fall through to the teardown
   } else if (warp == 0 || warp == 3) {
     // ------------------------------------------------------------ TMA producers: warp 0 Q + the K ring, warp 3 the V ring
-    // One thread each, walking the CTA's tile stream across item boundaries.  A producer only ever waits for
-    // one thing, the release of the slot it fills next, so it sleeps in that barrier wait (a loop polling
-    // several barriers with a back-off reacts to a freed slot up to a microsecond late, which is exposed
-    // latency on a two-slot ring).  List entries and item counts are fetched one step ahead of their use.
-    if (lane == 0) {
-      const bool is_v = warp == 3;
-      unsigned char* ring = is_v ? sV : sK;
-      const CUtensorMap* map = is_v ? &tmap_v : &tmap_k;
-      uint64_t* bar_full = is_v ? bar_v_full : bar_k_full;
-      uint64_t* bar_free = is_v ? bar_v_free : bar_k_free;
+    // One warp each, walking the CTA's tile stream across item boundaries (see the issuers for why the whole warp).  A
+    // producer only ever waits for one thing, the release of the slot it fills next, so it sleeps in that barrier
+    // wait (a loop polling several barriers with a back-off reacts to a freed slot up to a microsecond late, which is
+    // exposed latency on a two-slot ring).  List entries and item counts are fetched one step ahead of their use.
+    auto produce = [&](auto which) {
+      const bool is_v = which;
       const int R = is_v ? RV : RK;
-      int ord = 0, t = 0;                               // items seen, tiles loaded so far
+      int ord = 0, slot = 0, use = 0;                   // items seen; ring slot of the next tile and how often the ring has been filled
       int item = first_item;
+      const int32_t* lst = p.clean_list + (int64_t)item * p.lstride;
       int cnt = item < p.items ? __ldg(p.clean_cnt + item) : 0;
-      int kb = item < p.items ? __ldg(p.clean_list + (int64_t)item * p.lstride) : 0;
-      int kb2 = (PAIR && item < p.items) ? __ldg(p.clean_list + (int64_t)item * p.lstride + 1) : 0;
+      int kb = item < p.items ? __ldg(lst) : 0;
+      int kb2 = (PAIR && item < p.items) ? __ldg(lst + 1) : 0;
       bool ok = true;
       while (ok && item < p.items) {
         // the next item's count and first entries, needed when this item is done
         const int nxt = item + item_step;
+        const int32_t* lst_next = p.clean_list + (int64_t)nxt * p.lstride;
         const int cnt_next = nxt < p.items ? __ldg(p.clean_cnt + nxt) : 0;
-        const int kb_next = nxt < p.items ? __ldg(p.clean_list + (int64_t)nxt * p.lstride) : 0;
-        const int kb2_next = (PAIR && nxt < p.items) ? __ldg(p.clean_list + (int64_t)nxt * p.lstride + 1) : 0;
-        const int bh = item / p.nbq;
-        const int hh = bh % p.H, bb = bh / p.H;
-        if (!is_v) {
-          const int qslot = ord & 1;
-          if (cnt > 0) {
-            if (ord >= 2) ok = mbar_wait(bar_q_free + qslot, ((ord >> 1) - 1) & 1, s_abort, p.status, 1);
-            if (!ok) break;
-            const int qb = item % p.nbq;
-            mbar_expect_tx(bar_q_full + qslot, kTileTx);
-            tma_load_4d(sQ + qslot * kTile, &tmap_q, bar_q_full + qslot, 0, qb * kPBLK, hh, bb);
-            if constexpr (!FP8) tma_load_4d(sQ + qslot * kTile + kTile / 2, &tmap_q, bar_q_full + qslot, 64, qb * kPBLK, hh, bb);
-          } else {
-            mbar_arrive(bar_q_full + qslot);            // empty item: nothing to load, consumers still step through it
-          }
+        const int kb_next = nxt < p.items ? __ldg(lst_next) : 0;
+        const int kb2_next = (PAIR && nxt < p.items) ? __ldg(lst_next + 1) : 0;
+        const int bh = fast_div(item, p.by_nbq);
+        const int bb = fast_div(bh, p.by_H), hh = bh - bb * p.H;
+        cnt = uniform(cnt);
+        if (cnt & kBadFlag) {
+          cnt &= ~kBadFlag;
+          if (!is_v && lane == 0) report_bad_index(p, item, PAIR);
         }
-        for (int n = 0; ok && n < cnt; ++n, ++t) {
-          const int slot = t % R;
+        if (!is_v) {
+          const int qslot = ord & 1, qb = item - bh * p.nbq;
+          if (cnt > 0 && ord >= 2) ok = __all_sync(0xffffffffu, ctrl_wait(bar_q_free + qslot, ((ord >> 1) - 1) & 1, 1));
+          if (!ok) break;
+          if (elect_one()) {
+            if (cnt > 0) {
+              mbar_expect_tx(bar_q_full + qslot, kTileTx);
+              tma_load_4d(sQ + qslot * kTile, &tmap_q, bar_q_full + qslot, 0, qb * kPBLK, hh, bb);
+              if constexpr (!FP8) tma_load_4d(sQ + qslot * kTile + kTile / 2, &tmap_q, bar_q_full + qslot, 64, qb * kPBLK, hh, bb);
+            } else {
+              mbar_arrive(bar_q_full + qslot);            // empty item: nothing to load, consumers still step through it
+            }
+          }
+          __syncwarp();
+        }
+        for (int n = 0; n < cnt; ++n) {
           // the entries of the tile after this one (used one step later)
           int kb_n = 0, kb2_n = 0;
           if (n + 1 < cnt) {
-            kb_n = __ldg(p.clean_list + (int64_t)item * p.lstride + (n + 1) * kEnt);
-            if constexpr (PAIR) kb2_n = __ldg(p.clean_list + (int64_t)item * p.lstride + (n + 1) * kEnt + 1);
+            kb_n = __ldg(lst + (n + 1) * kEnt);
+            if constexpr (PAIR) kb2_n = __ldg(lst + (n + 1) * kEnt + 1);
           }
-          if (t >= R) ok = mbar_wait(bar_free + slot, ((t / R) - 1) & 1, s_abort, p.status, is_v ? 16 : 1);
+          if (use > 0) ok = __all_sync(0xffffffffu, ctrl_wait((is_v ? bar_v_free : bar_k_free) + slot, (use - 1) & 1, is_v ? 16 : 1));
           if (!ok) break;
-          unsigned char* dst = ring + slot * kSlot;
-          uint64_t* bar = bar_full + slot;
-          mbar_expect_tx(bar, kTileTx);
-          // one K or V tile: 128 key rows of one block, or 64 + 64 rows of the tile's two 64-token blocks
-          if constexpr (PAIR) {
-            const int r0 = (kb & 0x3fffffff) * 64, r1 = (kb2 & 0x3fffffff) * 64;
+          const int r0 = uniform(PAIR ? (kb & 0x3fffffff) * 64 : kb * kPBLK);
+          [[maybe_unused]] const int r1 = PAIR ? uniform((kb2 & 0x3fffffff) * 64) : 0;
+          if (elect_one()) {
+            unsigned char* dst = (is_v ? sV : sK) + slot * kSlot;
+            uint64_t* bar = (is_v ? bar_v_full : bar_k_full) + slot;
+            const CUtensorMap* map = is_v ? &tmap_v : &tmap_k;
+            mbar_expect_tx(bar, kTileTx);
+            // one K or V tile: 128 key rows of one block, or 64 + 64 rows of the tile's two 64-token blocks
             tma_load_4d(dst, map, bar, 0, r0, hh, bb);
-            tma_load_4d(dst + 8192, map, bar, 0, r1, hh, bb);
+            if constexpr (PAIR) tma_load_4d(dst + 8192, map, bar, 0, r1, hh, bb);
             if constexpr (!FP8) {
               tma_load_4d(dst + kTile / 2, map, bar, 64, r0, hh, bb);
-              tma_load_4d(dst + kTile / 2 + 8192, map, bar, 64, r1, hh, bb);
+              if constexpr (PAIR) tma_load_4d(dst + kTile / 2 + 8192, map, bar, 64, r1, hh, bb);
             }
-          } else {
-            tma_load_4d(dst, map, bar, 0, kb * kPBLK, hh, bb);
-            if constexpr (!FP8) tma_load_4d(dst + kTile / 2, map, bar, 64, kb * kPBLK, hh, bb);
           }
+          __syncwarp();
           kb = kb_n; kb2 = kb2_n;
+          if (++slot == R) { slot = 0; ++use; }
         }
         item = nxt; ++ord;
+        lst = p.clean_list + (int64_t)item * p.lstride;
         cnt = cnt_next; kb = kb_next; kb2 = kb2_next;
       }
-    }
+    };
+    if constexpr (FP8) produce(warp == 3);            // (one piece of code for both: 1 % at long lists; bf16 would spill)
+    else if (warp == 0) produce(Const<false>{});
+    else produce(Const<true>{});
   } else if (warp == 1) {
     // -------------------------------------------------------------- S issuer: S = Q K^T of the next tile
-    if (lane == 0) {
-      constexpr uint32_t idesc_qk = make_idesc(FP8 ? 0u : 1u, 128, kPBLK, false);
-      int si = 0, s_item = first_item, s_n = 0, s_cnt = -1, s_t = 0;
-      bool ok = true;
-      while (ok && s_item < p.items) {
-        if (s_cnt < 0) s_cnt = __ldg(p.clean_cnt + s_item);
-        if (s_n >= s_cnt) {
-          s_item += item_step; ++si; s_n = 0; s_cnt = -1;
-          continue;
-        }
-        const int sbuf = s_t & 1, kslot = s_t % RK, qslot = si & 1;
-        const uint64_t dQ = make_smem_desc_sw128(smem_u32(sQ + qslot * kTile), 16);
-        const uint64_t dK = make_smem_desc_sw128(smem_u32(sK + kslot * kSlot), 16);
-        const uint32_t q_lo = (uint32_t)dQ, q_hi = (uint32_t)(dQ >> 32), k_lo = (uint32_t)dK, k_hi = (uint32_t)(dK >> 32);
-        // The product needs all three (its S buffer free, K landed, Q landed), so the thread sleeps in one barrier
+    // The issuers' loops are run by the whole warp and only the MMAs by one thread, so that everything the
+    // MMAs are given lives in uniform registers (with the loop inside the one thread every descriptor word is moved
+    // there again for every MMA: 100 clocks an instruction next to two softmax warps).
+    constexpr uint32_t idesc_qk = make_idesc(FP8 ? 0u : 1u, 128, kPBLK, false);
+    const uint32_t q_hi = (uint32_t)(make_smem_desc_sw128(0, 16) >> 32);
+    const uint32_t q_lo = (uint32_t)make_smem_desc_sw128(smem_u32(sQ), 16), k_lo = (uint32_t)make_smem_desc_sw128(smem_u32(sK), 16);
+    int si = 0, t = 0;
+    bool ok = true;
+    for (int item = first_item; ok && item < p.items; item += item_step, ++si) {
+      const int cnt = uniform(clean_count(p.clean_cnt, item));
+      for (int n = 0; n < cnt; ++n, ++t) {
+        const int sbuf = t & 1, kslot = t % RK, qslot = si & 1;
+        // The product needs all three (its S buffer free, K landed, Q landed), so the warp sleeps in one barrier
         // wait after the other instead of polling them with a back-off: the K tile, which is waited for longest,
         // comes first; the others have normally happened by then.
-        ok = mbar_wait(bar_k_full + kslot, (s_t / RK) & 1, s_abort, p.status, 2);
-        if (ok && s_n == 0) ok = mbar_wait(bar_q_full + qslot, (si >> 1) & 1, s_abort, p.status, 17);
-        if (ok && s_t >= 2) ok = mbar_wait(bar_s_free + sbuf, ((s_t >> 1) - 1) & 1, s_abort, p.status, 18);   // row of tile s_t - 2 is in registers
+        ok = ctrl_wait(bar_k_full + kslot, (t / RK) & 1, 2);
+        if (ok && n == 0) ok = ctrl_wait(bar_q_full + qslot, (si >> 1) & 1, 17);
+        if (ok && t >= 2) ok = ctrl_wait(bar_s_free + sbuf, ((t >> 1) - 1) & 1, 18);   // row of tile t - 2 is in registers
+        if constexpr (!kLone) ok = __all_sync(0xffffffffu, ok);
         if (!ok) break;
-        {
-          tc_fence_after();
+        tc_fence_after();
+        if (elect_one()) {
+          const uint32_t qa = q_lo + ((qslot * kTile) >> 4), ka = k_lo + ((kslot * kSlot) >> 4);
           // 32 bytes of the channel dimension per MMA: 16 bf16 (8 MMAs over two slabs) or 32 E4M3 (4 MMAs)
 #pragma unroll
           for (int sl = 0; sl < (FP8 ? 1 : 2); ++sl)
 #pragma unroll
             for (int kk = 0; kk < 4; ++kk)
-              mma_ss<FP8>(tmem + sbuf * kPBLK, make_desc(q_lo + ((sl * (kTile / 2) + kk * 32) >> 4), q_hi),
-                          make_desc(k_lo + ((sl * (kTile / 2) + kk * 32) >> 4), k_hi), idesc_qk, (sl | kk) != 0 ? 1u : 0u);
+              mma_ss<FP8>(tmem + sbuf * kPBLK, make_desc(qa + ((sl * (kTile / 2) + kk * 32) >> 4), q_hi),
+                          make_desc(ka + ((sl * (kTile / 2) + kk * 32) >> 4), q_hi), idesc_qk, (sl | kk) != 0 ? 1u : 0u);
           tc_commit(bar_s_full + sbuf);
           tc_commit(bar_k_free + kslot);
-          ++s_n; ++s_t;
         }
+        __syncwarp();
       }
     }
   } else if (warp == 2) {
     // -------------------------------------------------------------- PV issuer: O += P V of the oldest pending tile
     // (its own warp on another scheduler: an issuing thread shares its scheduler with two softmax
     // warps that are almost always ready, and gets an issue slot only when they stall)
-    if (lane == 0) {
-      constexpr uint32_t idesc_pv = make_idesc(FP8 ? 0u : 1u, 128, kPD, true);
-      constexpr int kPvSteps = FP8 ? 4 : 8;          // 32 bytes of P per row per MMA: 16 bf16 or 32 E4M3 keys
-      int p_item = first_item, p_n = 0, p_cnt = -1, p_t = 0, p_nonempty = 0;
-      bool ok = true;
-      while (ok && p_item < p.items) {
-        if (p_cnt < 0) p_cnt = __ldg(p.clean_cnt + p_item);
-        if (p_n >= p_cnt) {
-          if (p_cnt > 0) ++p_nonempty;
-          p_item += item_step; p_n = 0; p_cnt = -1;
-          continue;
-        }
-        const int pbuf = p_t & 1, vslot = p_t % RV;
-        const uint64_t dV = make_smem_desc_sw128(smem_u32(sV + vslot * kSlot), kTile / 2);
-        const uint32_t v_lo = (uint32_t)dV, v_hi = (uint32_t)(dV >> 32);
+    constexpr uint32_t idesc_pv = make_idesc(FP8 ? 0u : 1u, 128, kPD, true);
+    constexpr int kPvSteps = FP8 ? 4 : 8;          // 32 bytes of P per row per MMA: 16 bf16 or 32 E4M3 keys
+    const uint32_t v_hi = (uint32_t)(make_smem_desc_sw128(0, kTile / 2) >> 32);
+    const uint32_t v_lo = (uint32_t)make_smem_desc_sw128(smem_u32(sV), kTile / 2);
+    int t = 0, nonempty = 0, vslot = 0, vphase = 0;
+    bool ok = true;
+    for (int item = first_item; ok && item < p.items; item += item_step) {
+      const int cnt = uniform(clean_count(p.clean_cnt, item));
+      for (int n = 0; n < cnt; ++n, ++t) {
+        const int pbuf = t & 1;
         // (see the S issuer) the V tile and the previous item's closer first, P, which arrives last, last
-        ok = mbar_wait(bar_v_full + vslot, (p_t / RV) & 1, s_abort, p.status, 10);
+        ok = ctrl_wait(bar_v_full + vslot, vphase, 10);
         // first tile of an item only: O of the previous item must have been read by its closer
-        if (ok && p_n == 0 && p_nonempty > 0) ok = mbar_wait(bar_o_free, (p_nonempty - 1) & 1, s_abort, p.status, 19);
-        if (ok) ok = mbar_wait(bar_p_full + pbuf, (p_t >> 1) & 1, s_abort, p.status, 20);
+        if (ok && n == 0 && nonempty > 0) ok = ctrl_wait(bar_o_free, (nonempty - 1) & 1, 19);
+        if (ok) ok = ctrl_wait(bar_p_full + pbuf, (t >> 1) & 1, 20);
+        if constexpr (!kLone) ok = __all_sync(0xffffffffu, ok);
         if (!ok) break;
-        {
-          tc_fence_after();
+        tc_fence_after();
+        if (elect_one()) {
+          const uint32_t va = v_lo + ((vslot * kSlot) >> 4);
 #pragma unroll
           for (int kk = 0; kk < kPvSteps; ++kk)
-            mma_ts<FP8>(tmem_O, tmem_P + pbuf * 64 + kk * 8, make_desc(v_lo + ((kk * (128 / kPvSteps) * 128) >> 4), v_hi),
-                        idesc_pv, (p_n == 0 && kk == 0) ? 0u : 1u);
+            mma_ts<FP8>(tmem_O, tmem_P + pbuf * 64 + kk * 8, make_desc(va + ((kk * (128 / kPvSteps) * 128) >> 4), v_hi),
+                        idesc_pv, (n == 0 && kk == 0) ? 0u : 1u);
           tc_commit(bar_pv_done + pbuf);
           tc_commit(bar_v_free + vslot);
-          ++p_n; ++p_t;
         }
+        __syncwarp();
+        if (++vslot == RV) { vslot = 0; vphase ^= 1; }
       }
+      nonempty += cnt > 0;
     }
   } else if (warp >= 4 && warp < 12) {
     // ----------------------------------------------------------------- softmax
@@ -512,12 +621,12 @@ fwd_pipe_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
     };
     for (int item = first_item; ok && item < p.items; item += item_step, ++io) {
       const int qslot = io & 1;
-      const int cnt = __ldg(p.clean_cnt + item);
+      const int cnt = clean_count(p.clean_cnt, item);
       if constexpr (kDeferStoreWait) {
         if (row == 0 && store_slot >= 0 && io >= store_io + 2) store_flush();
       }
-      const int qb = item % p.nbq, bh = item / p.nbq;     // PAIR: qb counts pairs of 64-token query blocks
-      const int h = bh % p.H, b = bh / p.H;
+      const int bh = fast_div(item, p.by_nbq), b = fast_div(bh, p.by_H);
+      const int qb = item - bh * p.nbq, h = bh - b * p.H;  // PAIR: qb counts pairs of 64-token query blocks
       const int q_row = qb * kPBLK + row;
       const bool row_valid = q_row < p.N;
       // keys this row may attend to: [klo, khi) (everything up to N without a causal window)
@@ -530,11 +639,11 @@ fwd_pipe_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
       if (cnt == 0) {
         if (g == 0) {
           // empty kept list: zero output, lse = -inf; release the item's Q slot
-          ok = __all_sync(0xffffffffu, mbar_wait(bar_q_full + qslot, (io >> 1) & 1, s_abort, p.status, 3));
+          ok = __all_sync(0xffffffffu, pipe_wait(bar_q_full + qslot, (io >> 1) & 1, s_abort, 3));
           if (!ok) break;
           if (row_valid) {
             __nv_bfloat16* orow = p.out + b * p.stride_b + h * p.stride_h + (int64_t)q_row * p.stride_n;
-#pragma unroll
+#pragma unroll 1
             for (int ch = 0; ch < kPD / 8; ++ch) reinterpret_cast<uint4*>(orow)[ch] = make_uint4(0u, 0u, 0u, 0u);
             if (p.lse) p.lse[(int64_t)bh * p.N + q_row] = -INFINITY;
           }
@@ -621,7 +730,7 @@ fwd_pipe_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
         // [c_lo1, c_hi1) of its second 64 columns (empty when the block is not in this query block's list)
         const int c_lo = klo - kb * kKeyBlk, c_hi = PAIR ? (mem0 ? min(khi - kb * 64, bv0) : 0) : min(khi - kb * kPBLK, bv0);
         const int c_lo1 = klo - kb1 * 64, c_hi1 = mem1 ? min(khi - kb1 * 64, bv1) : 0;
-        ok = __all_sync(0xffffffffu, mbar_wait(bar_s_full + buf, (tt >> 1) & 1, s_abort, p.status, 4));
+        ok = __all_sync(0xffffffffu, pipe_wait(bar_s_full + buf, (tt >> 1) & 1, s_abort, 4));
         if (!ok) break;
         tc_fence_after();
         const uint32_t tS = tmem + buf * kPBLK + lane_off;
@@ -631,23 +740,21 @@ fwd_pipe_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
         tc_wait_ld();
         tc_fence_before();
         mbar_arrive(bar_s_free + buf);    // the S buffer can take the next-but-one tile
-        if constexpr (PAIR) {
-          if ((WINDOW && (c_lo > 0 || c_lo1 > 0)) || c_hi < 64 || c_hi1 < 64) {
+        // ragged last key block / padding rows of a brick / keys outside the causal window get weight 0: a bit per column,
+        // 32 columns at a time (a short tail touches the last 32 only)
+        if ((WINDOW && (c_lo > 0 || (PAIR && c_lo1 > 0))) || c_hi < kKeyBlk || (PAIR && c_hi1 < kKeyBlk)) {
+          auto below = [](int x) { return x >= 32 ? 0xffffffffu : x <= 0 ? 0u : (1u << x) - 1u; };
 #pragma unroll
-            for (int i = 0; i < 64; ++i) {
-              if ((WINDOW && i < c_lo) || i >= c_hi) sr[i] = 0xff800000u;
-              if ((WINDOW && i < c_lo1) || i >= c_hi1) sr[64 + i] = 0xff800000u;
+          for (int ch = 0; ch < kPBLK / 32; ++ch) {
+            const bool second = PAIR && ch >= 2;
+            const int at = (second ? ch - 2 : ch) * 32;
+            uint32_t keep = below((second ? c_hi1 : c_hi) - at);
+            if constexpr (WINDOW) keep &= ~below((second ? c_lo1 : c_lo) - at);
+            if (keep != 0xffffffffu) {
+#pragma unroll
+              for (int i = 0; i < 32; ++i)
+                if (!(keep & (1u << i))) sr[ch * 32 + i] = 0xff800000u;
             }
-          }
-        } else if ((WINDOW && c_lo > 0) || c_hi < kPBLK) {   // ragged last key block / padding rows of a brick / keys outside the causal window get weight 0
-          if (!WINDOW && c_hi >= kPBLK - 32) {                // a short tail (every tile of a padded brick layout): 32 tests, not 128
-#pragma unroll
-            for (int i = kPBLK - 32; i < kPBLK; ++i)
-              if (i >= c_hi) sr[i] = 0xff800000u;
-          } else {
-#pragma unroll
-            for (int i = 0; i < kPBLK; ++i)
-              if ((WINDOW && i < c_lo) || i >= c_hi) sr[i] = 0xff800000u;
           }
         }
         float mx0 = __uint_as_float(sr[0]), mx1 = __uint_as_float(sr[1]);
@@ -674,7 +781,7 @@ fwd_pipe_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
 
         // reference maximum: token from the warpgroup of tile tt-1 (also orders the reuse of s_mref[g])
         if (tt > 0) {
-          ok = __all_sync(0xffffffffu, mbar_wait(bar_tok + (g ^ 1), ((tt - 1) >> 1) & 1, s_abort, p.status, 5));
+          ok = __all_sync(0xffffffffu, pipe_wait(bar_tok + (g ^ 1), ((tt - 1) >> 1) & 1, s_abort, 5));
           if (!ok) break;
         }
         float m_new;
@@ -703,25 +810,25 @@ fwd_pipe_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
           // waited for PV of tile tt-3 yet; PVs complete in order, so PV of tile tt-2 (this warpgroup's
           // own barrier, whose previous completion it has already seen) is waited for first.
           if (tt >= 2) {
-            ok = __all_sync(0xffffffffu, mbar_wait(bar_pv_done + buf, ((tt >> 1) - 1) & 1, s_abort, p.status, 12));
+            ok = __all_sync(0xffffffffu, pipe_wait(bar_pv_done + buf, ((tt >> 1) - 1) & 1, s_abort, 12));
             if (!ok) break;
           }
-          ok = __all_sync(0xffffffffu, mbar_wait(bar_pv_done + ((tt - 1) & 1), ((tt - 1) >> 1) & 1, s_abort, p.status, 6));
+          ok = __all_sync(0xffffffffu, pipe_wait(bar_pv_done + ((tt - 1) & 1), ((tt - 1) >> 1) & 1, s_abort, 6));
           if (!ok) break;
           tc_fence_after();
           const uint64_t a2 = pack_f32x2(alpha, alpha);
 #pragma unroll 1
-          for (int ch = 0; ch < kPD / 32; ++ch) {
-            uint32_t r[32];
-            tmem_ld32(tmem_O + lane_off + ch * 32, r);
+          for (int ch = 0; ch < kPD / 16; ++ch) {
+            uint32_t r[16];
+            tmem_ld16(tmem_O + lane_off + ch * 16, r);
             tc_wait_ld();
 #pragma unroll
-            for (int i = 0; i < 32; i += 2) {
+            for (int i = 0; i < 16; i += 2) {
               const float2 o2 = unpack_f32x2(fmul2(pack_f32x2(__uint_as_float(r[i]), __uint_as_float(r[i + 1])), a2));
               r[i] = __float_as_uint(o2.x);
               r[i + 1] = __float_as_uint(o2.y);
             }
-            tmem_st32(tmem_O + lane_off + ch * 32, r);
+            tmem_st16(tmem_O + lane_off + ch * 16, r);
           }
           tc_wait_st();
           tc_fence_before();
@@ -768,7 +875,7 @@ fwd_pipe_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
           }
           if (ch == 0 && tt >= 2) {
             // this warpgroup's P buffer is free once PV of tile tt-2 is complete (normally long ago)
-            ok = __all_sync(0xffffffffu, mbar_wait(bar_pv_done + buf, ((tt >> 1) - 1) & 1, s_abort, p.status, 11));
+            ok = __all_sync(0xffffffffu, pipe_wait(bar_pv_done + buf, ((tt >> 1) - 1) & 1, s_abort, 11));
           }
           if constexpr (FP8) tmem_st8(tP + ch * 8, w);
           else tmem_st16(tP + ch * 16, w);
@@ -799,7 +906,7 @@ fwd_pipe_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
         // S product of the item is complete and Q is dead), the other one in s_lsum.
         if ((t_last & 1) != g) {
           if (nonempty > 0) {
-            ok = __all_sync(0xffffffffu, mbar_wait(bar_lsum_ack, (nonempty - 1) & 1, s_abort, p.status, 7));
+            ok = __all_sync(0xffffffffu, pipe_wait(bar_lsum_ack, (nonempty - 1) & 1, s_abort, 7));
             if (!ok) break;
           }
           s_lsum[row] = make_float2(l, m_used);
@@ -811,7 +918,7 @@ fwd_pipe_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
       } else if ((t_last & 1) != g) {
         // not the closer: hand the partial row sum over (after the previous hand-over was read)
         if (nonempty > 0) {
-          ok = __all_sync(0xffffffffu, mbar_wait(bar_lsum_ack, (nonempty - 1) & 1, s_abort, p.status, 7));
+          ok = __all_sync(0xffffffffu, pipe_wait(bar_lsum_ack, (nonempty - 1) & 1, s_abort, 7));
           if (!ok) break;
         }
         s_lsum[row] = make_float2(l, m_used);
@@ -823,14 +930,14 @@ fwd_pipe_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
         ok = wg_line_up(13);
         if (!ok) break;
       } else {
-        ok = __all_sync(0xffffffffu, mbar_wait(bar_lsum, nonempty & 1, s_abort, p.status, 8));
+        ok = __all_sync(0xffffffffu, pipe_wait(bar_lsum, nonempty & 1, s_abort, 8));
         if (!ok) break;
         const float2 other = s_lsum[row];
         mbar_arrive(bar_lsum_ack);
         ok = wg_line_up(14);                                            // see the note at the hand-over above
         if (!ok) break;
         if (other.x != 0.0f) l += other.x * fast_exp2(other.y - m_used);
-        ok = __all_sync(0xffffffffu, mbar_wait(bar_pv_done + (t_last & 1), (t_last >> 1) & 1, s_abort, p.status, 9));
+        ok = __all_sync(0xffffffffu, pipe_wait(bar_pv_done + (t_last & 1), (t_last >> 1) & 1, s_abort, 9));
         if (!ok) break;
         tc_fence_after();
         // normalised O row as bf16 into the item's Q slot (all S MMAs of the item are complete), 128-byte swizzle
@@ -859,7 +966,7 @@ fwd_pipe_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
                              *reinterpret_cast<const uint32_t*>(&h2), *reinterpret_cast<const uint32_t*>(&h3));
             }
             asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-            ok = __all_sync(0xffffffffu, mbar_wait(bar_pq + g, gate_loads & 1, s_abort, p.status, 21));
+            ok = __all_sync(0xffffffffu, pipe_wait(bar_pq + g, gate_loads & 1, s_abort, 21));
             ++gate_loads;
             if (ok) ok = wg_line_up(22);
             if (!ok) break;
@@ -896,7 +1003,7 @@ fwd_pipe_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
             }
           }
           const float gte = row_valid ? __ldg(p.gate + (int64_t)bh * p.N + q_row) : 0.0f;
-          ok = __all_sync(0xffffffffu, mbar_wait(bar_gt + g, closings & 1, s_abort, p.status, 23));
+          ok = __all_sync(0xffffffffu, pipe_wait(bar_gt + g, closings & 1, s_abort, 23));
           if (!ok) break;
           tc_fence_after();
           // ---- q~ = R(p) silu(T) as bf16 over the first 32 columns of T (a thread only touches its own row)
@@ -951,7 +1058,7 @@ fwd_pipe_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
               mma_ts<false>(tmem_O, tT + kk * 8, make_desc(c_lo + ((kk * 2048) >> 4), c_hi), idesc_y, kk != 0 ? 1u : 0u);
             tc_commit(bar_gy + g);
           }
-          ok = __all_sync(0xffffffffu, mbar_wait(bar_gy + g, closings & 1, s_abort, p.status, 25));
+          ok = __all_sync(0xffffffffu, pipe_wait(bar_gy + g, closings & 1, s_abort, 25));
           ++closings;
           if (!ok) break;
           tc_fence_after();
@@ -1045,11 +1152,11 @@ fwd_pipe_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
     int slot_use[2] = {0, 0};                         // non-empty items that have used Q slot i
     bool ok = true;
     for (int item = first_item; ok && item < p.items; item += item_step, ++io) {
-      const int cnt = __ldg(p.clean_cnt + item);
+      const int cnt = clean_count(p.clean_cnt, item);
       if (cnt == 0) continue;                          // warpgroup 0 writes the zero rows of an empty list
       const int qslot = io & 1;
-      const int qb = item % p.nbq, bh = item / p.nbq;
-      const int h = bh % p.H, b = bh / p.H;
+      const int bh = fast_div(item, p.by_nbq), b = fast_div(bh, p.by_H);
+      const int qb = item - bh * p.nbq, h = bh - b * p.H;
       const int q_row = qb * kPBLK + row;
       const bool row_valid = q_row < p.N;
       const int t_last = t + cnt - 1;
@@ -1058,8 +1165,8 @@ fwd_pipe_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
       if constexpr (FP8) v_max = __ldg(p.v_max + bh);
       // the slot's barrier completes once per non-empty item that uses the slot; this item's Q could only be
       // loaded after the previous user's output had left, so the wait is never more than one phase behind
-      ok = __all_sync(0xffffffffu, mbar_wait(bar_cl + qslot, slot_use[qslot] & 1, s_abort, p.status, 8));
-      if (ok) ok = __all_sync(0xffffffffu, mbar_wait(bar_lsum, nonempty & 1, s_abort, p.status, 27));
+      ok = __all_sync(0xffffffffu, pipe_wait(bar_cl + qslot, slot_use[qslot] & 1, s_abort, 8));
+      if (ok) ok = __all_sync(0xffffffffu, pipe_wait(bar_lsum, nonempty & 1, s_abort, 27));
       if (!ok) break;
       const float2 mine = reinterpret_cast<const float2*>(slot)[row];
       const float2 other = s_lsum[row];
@@ -1069,7 +1176,7 @@ fwd_pipe_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
       const float m_used = mine.y;
       if (other.x != 0.0f) l += other.x * fast_exp2(other.y - m_used);
       ok = line_up();                                  // every row's sums are read before O rows overwrite them
-      if (ok) ok = __all_sync(0xffffffffu, mbar_wait(bar_pv_done + (t_last & 1), (t_last >> 1) & 1, s_abort, p.status, 9));
+      if (ok) ok = __all_sync(0xffffffffu, pipe_wait(bar_pv_done + (t_last & 1), (t_last >> 1) & 1, s_abort, 9));
       if (!ok) break;
       tc_fence_after();
       float inv = l > 0.0f ? 1.0f / l : 0.0f;          // no admissible key at all: zero row, lse = -inf
@@ -1117,6 +1224,7 @@ fwd_pipe_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
   // ------------------------------------------------------------------ teardown
   tc_fence_before();
   __syncthreads();
+  if (threadIdx.x == 0 && *s_abort >= kAbortTimeout) report_status(p.status, SPARKATTN_E_DEVICE_TIMEOUT, *s_abort - kAbortTimeout);
   if (warp == 0) {
     if (*s_abort) __nanosleep(200000);  // let copies / MMAs in flight land before the CTA's resources go
     tc_fence_after();
@@ -1223,7 +1331,9 @@ static int launch_pipe(const sparkattn_shape_t& s, bool fp8, const void* q, cons
   prm.out = static_cast<__nv_bfloat16*>(out);
   prm.lse = lse;
   prm.status = static_cast<int32_t*>(workspace);
+  prm.kept_idx = kept_idx; prm.kept_cnt = kept_cnt; prm.kmax = kmax;
   prm.H = s.H; prm.N = s.N; prm.nb = nb; prm.items = (int)items; prm.nbq = nbq; prm.lstride = lstride;
+  prm.by_nbq = make_fast_div((uint32_t)nbq); prm.by_H = make_fast_div((uint32_t)s.H);
   prm.frame_tokens = frame_tokens; prm.window = window;
   prm.blk_valid = block_valid;
   prm.stride_b = s.stride_b; prm.stride_h = s.stride_h; prm.stride_n = s.stride_n;
@@ -1231,7 +1341,6 @@ static int launch_pipe(const sparkattn_shape_t& s, bool fp8, const void* q, cons
   prm.scale_log2 = sc * 1.4426950408889634f;
   const int sm_count = current_sm_count();
   if (sm_count < 1) return SPARKATTN_E_CUDA;
-  if (cudaMemsetAsync(workspace, 0, kWorkspaceHeaderBytes, stream) != cudaSuccess) return SPARKATTN_E_CUDA;
   if (ga) {
     for (int m = 0; m < kCompRank / 2; ++m) { prm.rope.axis[m] = ga->axis[m]; prm.rope.freq[m] = ga->freq[m]; }
     prm.rope.T = ga->grid[0]; prm.rope.Hg = ga->grid[1]; prm.rope.Wg = ga->grid[2];
@@ -1242,34 +1351,41 @@ static int launch_pipe(const sparkattn_shape_t& s, bool fp8, const void* q, cons
   }
   if (pair) {
     const size_t bits = (size_t)kPairWarps * 2 * ((nb + 31) / 32) * sizeof(uint32_t);
-    pair_lists_kernel<<<(unsigned)((items + kPairWarps - 1) / kPairWarps), kPairWarps * 32, bits, stream>>>(
-        kept_idx, kept_cnt, clean_cnt, clean_list, (int)items, nb, nbq, kmax, prm.status);
+    rc = launch_kernel(pair_lists_kernel, (unsigned)((items + kPairWarps - 1) / kPairWarps), kPairWarps * 32, bits, true, stream,
+                       kept_idx, kept_cnt, clean_cnt, clean_list, (int)items, nb, nbq, kmax, prm.status);
   } else {
-    compact_lists_kernel<<<(unsigned)((items + 7) / 8), 256, 0, stream>>>(kept_idx, kept_cnt, clean_cnt, clean_list,
-                                                                        (int)items, nb, kmax, prm.status);
+    rc = launch_kernel(compact_lists_kernel, (unsigned)((items + 7) / 8), 256, 0, true, stream, kept_idx, kept_cnt, clean_cnt,
+                       clean_list, (int)items, nb, kmax, prm.status);
   }
-  if (fp8) head_vmax_kernel<<<(unsigned)((s.B * s.H + 7) / 8), 256, 0, stream>>>(v_scale, v_max, s.B * s.H, nb);
+  if (rc != SPARKATTN_OK) return rc;
+  if (fp8 && (rc = launch_kernel(head_vmax_kernel, (unsigned)((s.B * s.H + 7) / 8), 256, 0, true, stream, v_scale, v_max,
+                                 s.B * s.H, nb)) != SPARKATTN_OK)
+    return rc;
   const bool win = frame_tokens > 0;
-  auto kern = pair ? (fp8 ? (win ? fwd_pipe_kernel<true, true, true> : fwd_pipe_kernel<true, false, true>)
-                          : (win ? fwd_pipe_kernel<false, true, true> : fwd_pipe_kernel<false, false, true>))
-                   : (fp8 ? (win ? fwd_pipe_kernel<true, true, false> : fwd_pipe_kernel<true, false, false>)
-                          : (win ? fwd_pipe_kernel<false, true, false> : fwd_pipe_kernel<false, false, false>));
-  // short lists: the variant with a closing warpgroup (it takes the item boundary off the softmax warpgroups: 2.6 %
-  // bf16 / 1 % FP8 at 18 tiles per item, 6-8 % at 6; but its tile loop is 3 % slower, and the two are level near 60
-  // tiles per item)
-  const bool epi = !ga && kmax <= kEpiMaxKept;
-  if (epi && !fp8)
-    kern = pair ? (win ? fwd_pipe_kernel<false, true, true, false, true> : fwd_pipe_kernel<false, false, true, false, true>)
-                : (win ? fwd_pipe_kernel<false, true, false, false, true> : fwd_pipe_kernel<false, false, false, false, true>);
-  if (epi && fp8)
-    kern = pair ? (win ? fwd_pipe_kernel<true, true, true, false, true> : fwd_pipe_kernel<true, false, true, false, true>)
-                : (win ? fwd_pipe_kernel<true, true, false, false, true> : fwd_pipe_kernel<true, false, false, false, true>);
+  // The variant with a closing warpgroup: bf16 with 128-token blocks always (12 heads of 32,760 tokens; 6 / 18 / 26 / 64 / 256
+  // kept blocks: 163 / 387 / 541 / 1275 / 5023 us against 170 / 400 / 557 / 1293 / 5059), 64-token blocks up to 64 kept
+  // blocks (6 / 35 / 70: 150 / 528 / 961 against 163 / 534 / 965; 140 / 512: 1791 / 5196 against 1784 / 5088), FP8 up to 32
+  // (18 / 40 blocks of 128: 351 / 786 against 363 / 786; 64 / 256: 1183 / 4613 against 1164 / 4519; 64-token blocks 35: 532
+  // against 534, 70: 947 against 941).
+  const bool epi = !ga && (fp8 ? kmax <= 32 : !pair || kmax <= 64);
+  using Kern = void (*)(CUtensorMap, CUtensorMap, CUtensorMap, CUtensorMap, CUtensorMap, PipeParams);
+  Kern kern;
+  if (fp8 && pair)
+    kern = epi ? (win ? fwd_pipe_kernel<true, true, true, false, true> : fwd_pipe_kernel<true, false, true, false, true>)
+               : (win ? fwd_pipe_kernel<true, true, true> : fwd_pipe_kernel<true, false, true>);
+  else if (fp8)
+    kern = epi ? (win ? fwd_pipe_kernel<true, true, false, false, true> : fwd_pipe_kernel<true, false, false, false, true>)
+               : (win ? fwd_pipe_kernel<true, true, false> : fwd_pipe_kernel<true, false, false>);
+  else if (pair)
+    kern = epi ? (win ? fwd_pipe_kernel<false, true, true, false, true> : fwd_pipe_kernel<false, false, true, false, true>)
+               : (win ? fwd_pipe_kernel<false, true, true> : fwd_pipe_kernel<false, false, true>);
+  else
+    kern = win ? fwd_pipe_kernel<false, true, false, false, true> : fwd_pipe_kernel<false, false, false, false, true>;
   if (ga) kern = fwd_pipe_kernel<false, false, false, true>;
   if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kPipeSmem) != cudaSuccess)
     return SPARKATTN_E_CUDA;
   const unsigned grid = (unsigned)(items < sm_count ? items : sm_count);
-  kern<<<grid, epi ? kEpiThreads : kPipeThreads, kPipeSmem, stream>>>(mq, mk, mv, mo, mp, prm);
-  return cudaGetLastError() == cudaSuccess ? SPARKATTN_OK : SPARKATTN_E_CUDA;
+  return launch_kernel(kern, grid, epi ? kEpiThreads : kPipeThreads, kPipeSmem, true, stream, mq, mk, mv, mo, mp, prm);
 }
 
 }  // namespace sparkattn

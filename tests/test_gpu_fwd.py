@@ -203,6 +203,29 @@ def test_persistent_path_short_and_empty_lists(seed, kmax, block):
                 assert torch.all(out[0, h, rows] == 0) and torch.all(torch.isneginf(lse[0, h, rows]))
 
 
+@pytest.mark.parametrize("block,kmax", [(128, 33), (128, 4), (64, 5), (64, 40)])
+def test_bad_indices_are_dropped_and_reported(block, kmax):
+    """d = 128: an index outside [0, nb) is dropped by the list pre-pass and reported by the forward kernel (64-token
+    blocks: pairs of lists, one with a bad index, an odd number of blocks left).  The output is that of the lists
+    without it, bit for bit; the next call's status is clean."""
+    nbk, H = 41, 5
+    N = nbk * block - 5
+    g = torch.Generator().manual_seed(kmax)
+    q, k, v = (torch.randn((1, H, N, 128), generator=g).to(torch.bfloat16).to(DEV) for _ in range(3))
+    idx = torch.stack([torch.stack([torch.randperm(nbk, generator=g)[:kmax] for _ in range(nbk)]) for _ in range(H)]).to(torch.int32)
+    cnt = torch.full((H, nbk), kmax - 1, dtype=torch.int32)
+    bad, bad_cnt = idx.clone(), cnt.clone()
+    for h, i, at, value in [(0, 0, 0, -1), (1, 7, kmax - 1, nbk), (2, 40, 1, 1 << 30), (4, 11, 2, -(1 << 31))]:
+        bad[h, i] = torch.cat([idx[h, i, :at], torch.tensor([value], dtype=torch.int32), idx[h, i, at:kmax - 1]])
+        bad_cnt[h, i] = kmax
+    ws = sa.alloc_workspace(sa.make_shape(q, block), 1, kmax, DEV)
+    out = sa.fwd(q, k, v, bad[None].to(DEV), bad_cnt[None].to(DEV), block, workspace=ws)
+    assert sa.read_status(ws) == sa.E_BAD_INDEX
+    ref = sa.fwd(q, k, v, idx[None].to(DEV), cnt[None].to(DEV), block, workspace=ws)
+    assert sa.read_status(ws) == sa.OK
+    assert torch.equal(out.view(torch.int16), ref.view(torch.int16))
+
+
 @pytest.mark.parametrize("H,window", [(3, 0), (7, 0), (3, 2)])
 def test_d64_chains_of_every_length(H, window):
     """d = 64: the tiles of an item go to four chains (H = 3: 123 items, no SM gets a second one) or two (H = 7), so lists
