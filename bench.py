@@ -416,7 +416,7 @@ def run_ours(args, w):
     kernels = {
         "select": {"ms": ms_sel, "launches_per_step": 2, "algorithmic_bytes": sel_bytes,
                    "GBps": sel_bytes / (ms_sel * 1e-3) / 1e9, "frac_of_hbm_peak": sel_bytes / (ms_sel * 1e-3) / 1e9 / peaks["hbm"]},
-        "fwd_bf16": {"ms": ms_fwd, "launches_per_step": 2 if (w.d == 128 and w.block in (64, 128)) else 1, "TFLOPs": fwd_tflops},
+        "fwd_bf16": {"ms": ms_fwd, "launches_per_step": 2, "TFLOPs": fwd_tflops},
     }
     pipelined = w.d == 128 and w.block in (64, 128)   # d = 128 runs the persistent pipelined kernel (+ list pre-pass)
     roofline = {"kernel": f"fwd_pipe_kernel (bf16, d=128, {w.block}x{w.block} blocks)" if pipelined else f"fwd_kernel<{w.d},{w.block},bf16>", "bound": "tensor", "achieved": fwd_tflops, "peak": peaks["bf16"],
@@ -719,7 +719,7 @@ def run_ours(args, w):
             "metric": METRIC, "value": value, "unit": UNIT, "n_gpus": world, "steps": K, "warmup": args.warmup,
             "ms_per_step": ms_step, "higher_is_better": True, "scaling": "strong" if shard_heads else "weak", "vs_baseline": None,
             "dtype": "bf16", "data": "synthetic", "config": config_dict(w, "bf16", shard_heads, world),
-            "kept_flops_per_step_per_gpu": flops, "clocks": clocks, "gpu_launches": (4 if pipelined else 3) * K,
+            "kept_flops_per_step_per_gpu": flops, "clocks": clocks, "gpu_launches": 4 * K,
             "kernels": kernels, "roofline": roofline, "fp8": fp8, "sweep": sweep, "second_workload": second,
             "compensation": comp, "bricks": bricks, "e2e": e2e, "cpu_baseline": cpu, "peaks_in_run": run_peaks,
         }

@@ -17,8 +17,8 @@
 //                    warpgroup keeps its own partial row sum relative to the last reference it
 //                    saw; the warpgroup of the item's last tile combines them, normalises O into
 //                    the item's (now dead) Q slot and stores it with one TMA copy.
-//   warp 0           TMA producer (one thread): Q (2 slots) and the K ring (2 slots; FP8: 4).
-//   warp 3           TMA producer (one thread): the V ring (3 slots; FP8: 6).  Each producer sleeps in
+//   warp 0           TMA producer (one elected thread issues): Q (2 slots) and the K ring (2 slots; FP8: 4).
+//   warp 3           TMA producer (the same): the V ring (3 slots; FP8: 6).  Each producer sleeps in
 //                    the wait for the slot it fills next (one thread polling all rings with a
 //                    back-off answered a freed slot up to a microsecond late).
 //   warp 1           S issuer: S = Q K^T of the next tile once its K has landed and its S buffer is
