@@ -905,10 +905,13 @@ fwd_pipe_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
         // warpgroup of the item's last tile in the first KB of the item's Q slot (it has read the last S, so every
         // S product of the item is complete and Q is dead), the other one in s_lsum.
         if ((t_last & 1) != g) {
-          if (nonempty > 0) {
-            ok = __all_sync(0xffffffffu, pipe_wait(bar_lsum_ack, (nonempty - 1) & 1, s_abort, 7));
-            if (!ok) break;
-          }
+          // The closer must have read the previous hand-over.  This warpgroup may have closed that item itself and then
+          // has not waited for the one before it, which a parity cannot tell from the one wanted: both in turn.
+          // (The one before that is known to be read: whichever warpgroup did not close that item waited for it, and
+          // this one's last tile needed that one's.)
+          if (nonempty > 1) ok = __all_sync(0xffffffffu, pipe_wait(bar_lsum_ack, nonempty & 1, s_abort, 7));
+          if (ok && nonempty > 0) ok = __all_sync(0xffffffffu, pipe_wait(bar_lsum_ack, (nonempty - 1) & 1, s_abort, 7));
+          if (!ok) break;
           s_lsum[row] = make_float2(l, m_used);
           mbar_arrive(bar_lsum);
         } else {

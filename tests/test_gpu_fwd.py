@@ -331,3 +331,76 @@ def test_both_kernels_agree_bitwise(block, window, fp8):
         _compare_items(b[0], lb[0], ref_out, ref_lse, items, w.block, w.N, FP8_RELRMS, None)
     else:
         _compare_items(b[0], None if window else lb[0], ref_out, ref_lse, items, w.block, w.N, BF16_RELRMS, BF16_MAXABS)
+
+
+def _stream_of_short_items(streams, block, stride, H=16, N=74 * 128 - 17):
+    """Kept lists whose item i has streams[i % SMs % len][i // SMs % 8] tiles: what the persistent kernel's CTA c works
+    through (items c, c + SMs, ...).  Both query blocks of a 64-token pair keep the same blocks."""
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    nb, per = -(-N // block), 128 // block
+    nbq = -(-nb // per)
+    g = torch.Generator().manual_seed(block + stride + len(streams))
+    idx = torch.full((H, nb, stride), -7, dtype=torch.int32)          # entries past the count are never read
+    cnt = torch.zeros((H, nb), dtype=torch.int32)
+    for h in range(H):
+        for i in range(nb):
+            item = h * nbq + i // per
+            if i % per == 0:
+                n = streams[item % sms % len(streams)][item // sms % 8] * per
+                keep = torch.randperm(nb, generator=g)[:n].to(torch.int32)
+            cnt[h, i] = n
+            idx[h, i, :n] = keep
+    q, k, v = (torch.randn((1, H, N, 128), generator=g).to(torch.bfloat16).to(DEV) for _ in range(3))
+    return q, k, v, idx[None].to(DEV), cnt[None].to(DEV), sms // nbq
+
+
+STREAM_CASES = [(128, 6, "bf16"), (64, 6, "bf16"), (64, 72, "bf16"), (128, 6, "fp8"), (128, 40, "fp8"), (64, 6, "fp8"),
+                (64, 40, "fp8"), (128, 6, "gated")]
+
+
+def _check_stream(streams, block, stride, kind):
+    """All items in one call, against the same items a few heads at a time, no CTA with more than one: bit for bit (an item's
+    arithmetic does not depend on what its CTA did before), and those against fp32 attention over the lists."""
+    q, k, v, idx, cnt, heads = _stream_of_short_items(streams, block, stride)
+    H, N = q.shape[1], q.shape[2]
+    if kind == "fp8":
+        (q, sq), (k, sk), (v, sv) = (sa.quant_fp8(t, block) for t in (q, k, v))
+    if kind == "gated":
+        w = workloads.Workload("gatedstream", 83, 1, H, 128, (1, 1, N), 128, 0.0)
+        pq, pk, gate = workloads.compensation_params(w, 64, device=DEV)
+        axis, freq = workloads.rope_schedule(128, 64)
+        state = sa.comp_state(k, v, pk, w.grid, axis, freq)
+
+    def run(h):
+        args = [t[:, h] for t in (q, k, v)] + [t[:, h].contiguous() for t in (idx, cnt)]
+        if kind == "gated":
+            return sa.fwd_gated(*args, pq[h], state[:, h].contiguous(), gate[:, h].contiguous(), (1, 1, N), axis, freq,
+                                return_lse=True, check_status=True)
+        kw = dict(scales=tuple(s[:, h].contiguous() for s in (sq, sk, sv))) if kind == "fp8" else {}
+        return sa.fwd(*args, block, return_lse=True, check_status=True, **kw)
+
+    out, lse = run(slice(0, H))
+    for h0 in range(0, H, heads):
+        h = slice(h0, min(H, h0 + heads))
+        one, lse_one = run(h)
+        assert torch.equal(out[:, h].view(torch.int16), one.view(torch.int16))
+        assert torch.equal(lse[:, h].view(torch.int32), lse_one.view(torch.int32))
+    if kind != "bf16":
+        return
+    nb = idx.shape[2]
+    for h in (0, H // 2, H - 1):
+        keep = torch.zeros((nb, nb + 8), dtype=torch.bool, device=DEV)
+        keep.scatter_(1, torch.where(torch.arange(stride, device=DEV) < cnt[0, h][:, None], idx[0, h], nb).long(), True)
+        keep = keep[:, :nb].repeat_interleave(block, 0).repeat_interleave(block, 1)[:N, :N]
+        s = (q[0, h].float() @ k[0, h].float().T / math.sqrt(128)).masked_fill(~keep, -math.inf)
+        ref, empty = torch.softmax(s, -1).nan_to_num(0.0) @ v[0, h].float(), ~keep.any(1)
+        assert torch.all(out[0, h][empty] == 0) and torch.all(torch.isneginf(lse[0, h][empty]))
+        if not bool(empty.all()):
+            assert _errors(out[0, h].cpu(), ref.cpu())[0] <= BF16_RELRMS
+
+
+@pytest.mark.parametrize("block,stride,kind", STREAM_CASES)
+def test_streams_of_short_items(block, stride, kind):
+    """Every item one tile, or one and two or three in turn: the warpgroups swap the roles of the item's last tile at each
+    item and run as far ahead of the closing warpgroup as they can."""
+    _check_stream([[1] * 8, [2, 1] * 4, [1, 2] * 4, [3, 1, 1, 1, 2, 1, 1, 1], [1, 3] * 4], block, stride, kind)
