@@ -333,7 +333,7 @@ fwd_pipe_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
   unsigned char* sK = smem + kOffK;
   uint64_t* bars = reinterpret_cast<uint64_t*>(smem + kOffMisc);
   uint64_t* bar_q_full = bars + 0;     // [2]
-  uint64_t* bar_q_free = bars + 2;     // [2] the item's output store has read the slot (or the item was empty)
+  uint64_t* bar_q_free = bars + 2;     // [2] the item's output store has read the slot
   // An input tile is 128 rows x 128 channels: two 64-channel slabs of 16 KB in bf16, one slab in FP8, where the
   // same bytes hold rings twice as deep (the Q slots keep their 32 KB: the item's output is staged there).
   constexpr int kSlot = FP8 ? kTile / 2 : kTile;
@@ -440,7 +440,7 @@ fwd_pipe_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
     auto produce = [&](auto which) {
       const bool is_v = which;
       const int R = is_v ? RV : RK;
-      int ord = 0, slot = 0, use = 0;                   // items seen; ring slot of the next tile and how often the ring has been filled
+      int ord = 0, slot = 0, use = 0;                   // non-empty items seen; ring slot of the next tile and how often the ring has been filled
       int item = first_item;
       const int32_t* lst = p.clean_list + (int64_t)item * p.lstride;
       int cnt = item < p.items ? __ldg(p.clean_cnt + item) : 0;
@@ -461,20 +461,17 @@ fwd_pipe_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
           cnt &= ~kBadFlag;
           if (!is_v && lane == 0) report_bad_index(p, item, PAIR);
         }
-        if (!is_v) {
+        if (!is_v && cnt > 0) {
           const int qslot = ord & 1, qb = item - bh * p.nbq;
-          if (cnt > 0 && ord >= 2) ok = __all_sync(0xffffffffu, ctrl_wait(bar_q_free + qslot, ((ord >> 1) - 1) & 1, 1));
+          if (ord >= 2) ok = __all_sync(0xffffffffu, ctrl_wait(bar_q_free + qslot, ((ord >> 1) - 1) & 1, 1));
           if (!ok) break;
           if (elect_one()) {
-            if (cnt > 0) {
-              mbar_expect_tx(bar_q_full + qslot, kTileTx);
-              tma_load_4d(sQ + qslot * kTile, &tmap_q, bar_q_full + qslot, 0, qb * kPBLK, hh, bb);
-              if constexpr (!FP8) tma_load_4d(sQ + qslot * kTile + kTile / 2, &tmap_q, bar_q_full + qslot, 64, qb * kPBLK, hh, bb);
-            } else {
-              mbar_arrive(bar_q_full + qslot);            // empty item: nothing to load, consumers still step through it
-            }
+            mbar_expect_tx(bar_q_full + qslot, kTileTx);
+            tma_load_4d(sQ + qslot * kTile, &tmap_q, bar_q_full + qslot, 0, qb * kPBLK, hh, bb);
+            if constexpr (!FP8) tma_load_4d(sQ + qslot * kTile + kTile / 2, &tmap_q, bar_q_full + qslot, 64, qb * kPBLK, hh, bb);
           }
           __syncwarp();
+          ++ord;
         }
         for (int n = 0; n < cnt; ++n) {
           // the entries of the tile after this one (used one step later)
@@ -504,7 +501,7 @@ fwd_pipe_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
           kb = kb_n; kb2 = kb2_n;
           if (++slot == R) { slot = 0; ++use; }
         }
-        item = nxt; ++ord;
+        item = nxt;
         lst = p.clean_list + (int64_t)item * p.lstride;
         cnt = cnt_next; kb = kb_next; kb2 = kb2_next;
       }
@@ -520,9 +517,9 @@ fwd_pipe_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
     constexpr uint32_t idesc_qk = make_idesc(FP8 ? 0u : 1u, 128, kPBLK, false);
     const uint32_t q_hi = (uint32_t)(make_smem_desc_sw128(0, 16) >> 32);
     const uint32_t q_lo = (uint32_t)make_smem_desc_sw128(smem_u32(sQ), 16), k_lo = (uint32_t)make_smem_desc_sw128(smem_u32(sK), 16);
-    int si = 0, t = 0;
+    int si = 0, t = 0;                              // non-empty items and tiles so far
     bool ok = true;
-    for (int item = first_item; ok && item < p.items; item += item_step, ++si) {
+    for (int item = first_item; ok && item < p.items; item += item_step) {
       const int cnt = uniform(clean_count(p.clean_cnt, item));
       for (int n = 0; n < cnt; ++n, ++t) {
         const int sbuf = t & 1, kslot = t % RK, qslot = si & 1;
@@ -549,6 +546,7 @@ fwd_pipe_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
         }
         __syncwarp();
       }
+      si += cnt > 0;
     }
   } else if (warp == 2) {
     // -------------------------------------------------------------- PV issuer: O += P V of the oldest pending tile
@@ -597,7 +595,6 @@ fwd_pipe_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
     int t = 0;                                        // global tile counter at the start of the item
     int nonempty = 0;                                 // non-empty items finished so far
     bool ok = true;
-    int io = 0;
     int closings = 0, gate_loads = 0;                 // GATE: items this warpgroup has closed, heads it has staged (barrier phases)
     // Line-up of the warpgroup's 128 threads on a named barrier.  A hardware barrier has no time limit, so it
     // is fenced by the abort flag: no warp enters it once the flag is up, and a warp that leaves its loop
@@ -613,17 +610,17 @@ fwd_pipe_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
     // it releases the slot after its next tile, or, should the item after the next come first (its Q goes into
     // this very slot), before that.
     constexpr bool kDeferStoreWait = GATE;            // (elsewhere the extra test per tile costs more than the wait: lists are long, or FP8)
-    int store_slot = -1, store_io = 0;                // row 0: Q slot whose output store is in flight, and its item
+    int store_slot = -1, store_io = 0;                // row 0: Q slot whose output store is in flight, and its item (non-empty ones counted)
     auto store_flush = [&]() {
       asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
       mbar_arrive(bar_q_free + store_slot);
       store_slot = -1;
     };
-    for (int item = first_item; ok && item < p.items; item += item_step, ++io) {
-      const int qslot = io & 1;
+    for (int item = first_item; ok && item < p.items; item += item_step) {
+      const int qslot = nonempty & 1;
       const int cnt = clean_count(p.clean_cnt, item);
       if constexpr (kDeferStoreWait) {
-        if (row == 0 && store_slot >= 0 && io >= store_io + 2) store_flush();
+        if (row == 0 && store_slot >= 0 && nonempty >= store_io + 2) store_flush();
       }
       const int bh = fast_div(item, p.by_nbq), b = fast_div(bh, p.by_H);
       const int qb = item - bh * p.nbq, h = bh - b * p.H;  // PAIR: qb counts pairs of 64-token query blocks
@@ -637,17 +634,14 @@ fwd_pipe_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
         khi = (int)min((long long)(fi + 1) * p.frame_tokens, (long long)p.N);
       }
       if (cnt == 0) {
-        if (g == 0) {
-          // empty kept list: zero output, lse = -inf; release the item's Q slot
-          ok = __all_sync(0xffffffffu, pipe_wait(bar_q_full + qslot, (io >> 1) & 1, s_abort, 3));
-          if (!ok) break;
-          if (row_valid) {
-            __nv_bfloat16* orow = p.out + b * p.stride_b + h * p.stride_h + (int64_t)q_row * p.stride_n;
+        // empty kept list: zero output, lse = -inf.  Such an item takes no Q slot and no phase of any barrier: the
+        // roles pass it at different times, and a phase that one of them steps over without waiting is
+        // mistaken for the one two items later.
+        if (g == 0 && row_valid) {
+          __nv_bfloat16* orow = p.out + b * p.stride_b + h * p.stride_h + (int64_t)q_row * p.stride_n;
 #pragma unroll 1
-            for (int ch = 0; ch < kPD / 8; ++ch) reinterpret_cast<uint4*>(orow)[ch] = make_uint4(0u, 0u, 0u, 0u);
-            if (p.lse) p.lse[(int64_t)bh * p.N + q_row] = -INFINITY;
-          }
-          if (row == 0) mbar_arrive(bar_q_free + qslot);
+          for (int ch = 0; ch < kPD / 8; ++ch) reinterpret_cast<uint4*>(orow)[ch] = make_uint4(0u, 0u, 0u, 0u);
+          if (p.lse) p.lse[(int64_t)bh * p.N + q_row] = -INFINITY;
         }
         continue;
       }
@@ -1128,7 +1122,7 @@ fwd_pipe_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
           pipe_tma_store_4d(&tmap_o, slot, 0, qb * kPBLK, h, b);
           pipe_tma_store_4d(&tmap_o, slot + kTile / 2, 64, qb * kPBLK, h, b);
           asm volatile("cp.async.bulk.commit_group;" ::: "memory");
-          store_slot = qslot; store_io = io;
+          store_slot = qslot; store_io = nonempty;
           if constexpr (!kDeferStoreWait) store_flush();
         }
       }
@@ -1151,13 +1145,12 @@ fwd_pipe_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
       asm volatile("bar.sync 3, 128;" ::: "memory");
       return true;
     };
-    int t = 0, nonempty = 0, io = 0;
-    int slot_use[2] = {0, 0};                         // non-empty items that have used Q slot i
+    int t = 0, nonempty = 0;
     bool ok = true;
-    for (int item = first_item; ok && item < p.items; item += item_step, ++io) {
+    for (int item = first_item; ok && item < p.items; item += item_step) {
       const int cnt = clean_count(p.clean_cnt, item);
       if (cnt == 0) continue;                          // warpgroup 0 writes the zero rows of an empty list
-      const int qslot = io & 1;
+      const int qslot = nonempty & 1;
       const int bh = fast_div(item, p.by_nbq), b = fast_div(bh, p.by_H);
       const int qb = item - bh * p.nbq, h = bh - b * p.H;
       const int q_row = qb * kPBLK + row;
@@ -1166,15 +1159,14 @@ fwd_pipe_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
       unsigned char* slot = sQ + qslot * kTile;
       float v_max = 1.0f;
       if constexpr (FP8) v_max = __ldg(p.v_max + bh);
-      // the slot's barrier completes once per non-empty item that uses the slot; this item's Q could only be
+      // the slot's barrier completes once per item that uses the slot; this item's Q could only be
       // loaded after the previous user's output had left, so the wait is never more than one phase behind
-      ok = __all_sync(0xffffffffu, pipe_wait(bar_cl + qslot, slot_use[qslot] & 1, s_abort, 8));
+      ok = __all_sync(0xffffffffu, pipe_wait(bar_cl + qslot, (nonempty >> 1) & 1, s_abort, 8));
       if (ok) ok = __all_sync(0xffffffffu, pipe_wait(bar_lsum, nonempty & 1, s_abort, 27));
       if (!ok) break;
       const float2 mine = reinterpret_cast<const float2*>(slot)[row];
       const float2 other = s_lsum[row];
       mbar_arrive(bar_lsum_ack);
-      ++slot_use[qslot];
       float l = mine.x;
       const float m_used = mine.y;
       if (other.x != 0.0f) l += other.x * fast_exp2(other.y - m_used);

@@ -404,3 +404,14 @@ def test_streams_of_short_items(block, stride, kind):
     """Every item one tile, or one and two or three in turn: the warpgroups swap the roles of the item's last tile at each
     item and run as far ahead of the closing warpgroup as they can."""
     _check_stream([[1] * 8, [2, 1] * 4, [1, 2] * 4, [3, 1, 1, 1, 2, 1, 1, 1], [1, 3] * 4], block, stride, kind)
+
+
+STREAMS = [[1, 0, 0, 0, 1, 0, 0, 2], [2, 0, 0, 1, 0, 0, 0, 1], [0, 0, 1, 0, 0, 0, 1, 1], [1, 0, 1, 0, 1, 0, 0, 0],
+           [0, 1, 0, 0, 1, 1, 0, 3], [0, 0, 0, 0, 0, 0, 0, 0]]     # tiles of the items that one CTA takes in turn
+
+
+@pytest.mark.parametrize("block,stride,kind", STREAM_CASES)
+def test_empty_lists_between_short_ones(block, stride, kind):
+    """Items with an empty list between items of one to three tiles, so that the roles of a CTA are several items apart:
+    an empty item must neither release nor take a Q slot that another item still uses."""
+    _check_stream(STREAMS, block, stride, kind)
