@@ -898,14 +898,15 @@ fwd_pipe_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
         // partial row sums and the reference they are relative to, and go on to the next item's tiles: the
         // warpgroup of the item's last tile in the first KB of the item's Q slot (it has read the last S, so every
         // S product of the item is complete and Q is dead), the other one in s_lsum.
-        if ((t_last & 1) != g) {
-          // The closer must have read the previous hand-over.  This warpgroup may have closed that item itself and then
-          // has not waited for the one before it, which a parity cannot tell from the one wanted: both in turn.
-          // (The one before that is known to be read: whichever warpgroup did not close that item waited for it, and
-          // this one's last tile needed that one's.)
-          if (nonempty > 1) ok = __all_sync(0xffffffffu, pipe_wait(bar_lsum_ack, nonempty & 1, s_abort, 7));
-          if (ok && nonempty > 0) ok = __all_sync(0xffffffffu, pipe_wait(bar_lsum_ack, (nonempty - 1) & 1, s_abort, 7));
+        // The closer must have read the item before, and both warpgroups wait for that although only one of them writes
+        // s_lsum: the acknowledgement takes an arrival of either of them per item, so with both in step the phase waited
+        // for is never two away, which a parity could not tell (one-tile items bring a warpgroup that only waited
+        // when it hands over that far).
+        if (nonempty > 0) {
+          ok = __all_sync(0xffffffffu, pipe_wait(bar_lsum_ack, (nonempty - 1) & 1, s_abort, 7));
           if (!ok) break;
+        }
+        if ((t_last & 1) != g) {
           s_lsum[row] = make_float2(l, m_used);
           mbar_arrive(bar_lsum);
         } else {
