@@ -101,6 +101,9 @@ __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_gr
 // Programmatic dependent launch.  A kernel that may be launched while the one before it on the stream is still
 // running (launch_kernel with overlap) calls pdl_wait before its first access to device memory: it returns when
 // everything earlier on the stream is complete and visible.  pdl_trigger lets the next such kernel be launched.
+// Such a kernel reads device memory with ordinary loads only: a read-only load (__ldg, or through a const __restrict__
+// parameter) is for data that nothing writes during the whole life of the kernel, and the compiler may move it ahead of
+// the wait.
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 

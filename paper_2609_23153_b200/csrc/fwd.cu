@@ -124,12 +124,12 @@ fwd_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant__ C
   if (threadIdx.x == 0) *s_abort = (*reinterpret_cast<volatile int32_t*>(p.status) == SPARKATTN_E_DEVICE_TIMEOUT) ? 1 : 0;
   if (warp == 6) {
     // Stage the kept list in shared memory, in order, dropping (and reporting) indices outside [0, nb).
-    const int cnt = p.kept_cnt ? min(max(__ldg(p.kept_cnt + (int64_t)bh * p.nb + qb), 0), p.kmax) : p.kmax;
+    const int cnt = p.kept_cnt ? min(max(p.kept_cnt[(int64_t)bh * p.nb + qb], 0), p.kmax) : p.kmax;
     const int32_t* list = p.kept_idx + ((int64_t)bh * p.nb + qb) * p.kmax;
     int out = 0;
     for (int base = 0; base < cnt; base += 32) {
       const int t = base + lane;
-      const int kb = (t < cnt) ? __ldg(list + t) : 0;
+      const int kb = (t < cnt) ? list[t] : 0;
       const bool valid = (t < cnt) && kb >= 0 && kb < p.nb;
       if (t < cnt && !valid) report_status(p.status, SPARKATTN_E_BAD_INDEX, kb);
       const uint32_t ballot = __ballot_sync(0xffffffffu, valid);

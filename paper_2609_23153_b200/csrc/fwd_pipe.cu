@@ -128,21 +128,21 @@ struct PipeParams {
 // run in no order): an item with an index outside [0, nb) gets this flag in its count, and the forward kernel looks the
 // index up and reports it.
 constexpr int32_t kBadFlag = 0x40000000;
-__device__ __forceinline__ int clean_count(const int32_t* clean_cnt, int item) { return __ldg(clean_cnt + item) & ~kBadFlag; }
+__device__ __forceinline__ int clean_count(const int32_t* clean_cnt, int item) { return clean_cnt[item] & ~kBadFlag; }
 __device__ __forceinline__ void report_bad_index(const PipeParams& p, int item, bool pair) {
   const int bh = item / p.nbq, first = pair ? 2 * (item % p.nbq) : item % p.nbq;
   for (int qb = first; qb < min(first + (pair ? 2 : 1), p.nb); ++qb) {
     const int64_t list = (int64_t)bh * p.nb + qb;
-    const int cnt = p.kept_cnt ? min(max(__ldg(p.kept_cnt + list), 0), p.kmax) : p.kmax;
+    const int cnt = p.kept_cnt ? min(max(p.kept_cnt[list], 0), p.kmax) : p.kmax;
     for (int t = 0; t < cnt; ++t) {
-      const int kb = __ldg(p.kept_idx + list * p.kmax + t);
+      const int kb = p.kept_idx[list * p.kmax + t];
       if (kb < 0 || kb >= p.nb) report_status(p.status, SPARKATTN_E_BAD_INDEX, kb);
     }
   }
 }
 
 // one warp per item: drop (and flag) kept indices outside [0, nb), clamp the count, own block first
-__global__ void compact_lists_kernel(const int32_t* __restrict__ kept_idx, const int32_t* __restrict__ kept_cnt,
+__global__ void compact_lists_kernel(const int32_t* kept_idx, const int32_t* kept_cnt,
                                      int32_t* __restrict__ clean_cnt, int32_t* __restrict__ clean_list, int items,
                                      int nb, int kmax, int32_t* status) {
   pdl_trigger();
@@ -151,14 +151,14 @@ __global__ void compact_lists_kernel(const int32_t* __restrict__ kept_idx, const
   const int item = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
   const int lane = threadIdx.x & 31;
   if (item >= items) return;
-  const int cnt = kept_cnt ? min(max(__ldg(kept_cnt + item), 0), kmax) : kmax;
+  const int cnt = kept_cnt ? min(max(kept_cnt[item], 0), kmax) : kmax;
   const int32_t* src = kept_idx + (int64_t)item * kmax;
   int32_t* dst = clean_list + (int64_t)item * kmax;
   int out = 0;
   bool bad = false;
   for (int base = 0; base < cnt; base += 32) {
     const int t = base + lane;
-    const int kb = (t < cnt) ? __ldg(src + t) : 0;
+    const int kb = (t < cnt) ? src[t] : 0;
     const bool valid = (t < cnt) && kb >= 0 && kb < nb;
     bad = __any_sync(0xffffffffu, (t < cnt) && !valid) || bad;
     const uint32_t ballot = __ballot_sync(0xffffffffu, valid);
@@ -200,7 +200,7 @@ __global__ void compact_lists_kernel(const int32_t* __restrict__ kept_idx, const
 constexpr int kPairMaxBlocks = 16384;    // key blocks per head the merge can mark in shared memory
 constexpr int kPairWarps = 4;
 __global__ void __launch_bounds__(kPairWarps * 32)
-pair_lists_kernel(const int32_t* __restrict__ kept_idx, const int32_t* __restrict__ kept_cnt,
+pair_lists_kernel(const int32_t* kept_idx, const int32_t* kept_cnt,
                   int32_t* __restrict__ clean_cnt, int32_t* __restrict__ clean_list, int pairs, int nb, int nbq,
                   int kmax, int32_t* status) {
   pdl_trigger();
@@ -220,10 +220,10 @@ pair_lists_kernel(const int32_t* __restrict__ kept_idx, const int32_t* __restric
     const int qb = 2 * qp + side;
     if (qb >= nb) break;
     const int64_t item = (int64_t)bh * nb + qb;
-    const int cnt = kept_cnt ? min(max(__ldg(kept_cnt + item), 0), kmax) : kmax;
+    const int cnt = kept_cnt ? min(max(kept_cnt[item], 0), kmax) : kmax;
     const int32_t* src = kept_idx + item * kmax;
     for (int base = 0; base < cnt; base += 32) {
-      const int kb = base + lane < cnt ? __ldg(src + base + lane) : 0;
+      const int kb = base + lane < cnt ? src[base + lane] : 0;
       const bool valid = kb >= 0 && kb < nb;
       if (base + lane < cnt && valid) atomicOr(bits + side * words + (kb >> 5), 1u << (kb & 31));
       bad = __any_sync(0xffffffffu, !valid) || bad;
@@ -259,14 +259,14 @@ pair_lists_kernel(const int32_t* __restrict__ kept_idx, const int32_t* __restric
 }
 
 // FP8: largest V block scale of every (batch, head); one warp each
-__global__ void head_vmax_kernel(const float* __restrict__ v_scale, float* __restrict__ v_max, int bh_count, int nb) {
+__global__ void head_vmax_kernel(const float* v_scale, float* __restrict__ v_max, int bh_count, int nb) {
   pdl_trigger();
   pdl_wait();
   const int bh = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
   const int lane = threadIdx.x & 31;
   if (bh >= bh_count) return;
   float m = 0.0f;
-  for (int j = lane; j < nb; j += 32) m = fmaxf(m, __ldg(v_scale + (int64_t)bh * nb + j));
+  for (int j = lane; j < nb; j += 32) m = fmaxf(m, v_scale[(int64_t)bh * nb + j]);
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
   if (lane == 0) v_max[bh] = m;
@@ -443,17 +443,17 @@ fwd_pipe_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
       int ord = 0, slot = 0, use = 0;                   // non-empty items seen; ring slot of the next tile and how often the ring has been filled
       int item = first_item;
       const int32_t* lst = p.clean_list + (int64_t)item * p.lstride;
-      int cnt = item < p.items ? __ldg(p.clean_cnt + item) : 0;
-      int kb = item < p.items ? __ldg(lst) : 0;
-      int kb2 = (PAIR && item < p.items) ? __ldg(lst + 1) : 0;
+      int cnt = item < p.items ? p.clean_cnt[item] : 0;
+      int kb = item < p.items ? *lst : 0;
+      int kb2 = (PAIR && item < p.items) ? lst[1] : 0;
       bool ok = true;
       while (ok && item < p.items) {
         // the next item's count and first entries, needed when this item is done
         const int nxt = item + item_step;
         const int32_t* lst_next = p.clean_list + (int64_t)nxt * p.lstride;
-        const int cnt_next = nxt < p.items ? __ldg(p.clean_cnt + nxt) : 0;
-        const int kb_next = nxt < p.items ? __ldg(lst_next) : 0;
-        const int kb2_next = (PAIR && nxt < p.items) ? __ldg(lst_next + 1) : 0;
+        const int cnt_next = nxt < p.items ? p.clean_cnt[nxt] : 0;
+        const int kb_next = nxt < p.items ? *lst_next : 0;
+        const int kb2_next = (PAIR && nxt < p.items) ? lst_next[1] : 0;
         const int bh = fast_div(item, p.by_nbq);
         const int bb = fast_div(bh, p.by_H), hh = bh - bb * p.H;
         cnt = uniform(cnt);
@@ -477,8 +477,8 @@ fwd_pipe_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
           // the entries of the tile after this one (used one step later)
           int kb_n = 0, kb2_n = 0;
           if (n + 1 < cnt) {
-            kb_n = __ldg(lst + (n + 1) * kEnt);
-            if constexpr (PAIR) kb2_n = __ldg(lst + (n + 1) * kEnt + 1);
+            kb_n = lst[(n + 1) * kEnt];
+            if constexpr (PAIR) kb2_n = lst[(n + 1) * kEnt + 1];
           }
           if (use > 0) ok = __all_sync(0xffffffffu, ctrl_wait((is_v ? bar_v_free : bar_k_free) + slot, (use - 1) & 1, is_v ? 16 : 1));
           if (!ok) break;
@@ -648,8 +648,8 @@ fwd_pipe_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
       l = 0.0f;
       float q_sc = 1.0f, v_max = 1.0f;
       if constexpr (FP8) {
-        q_sc = PAIR ? __ldg(p.q_scale + (int64_t)bh * p.nb + min(2 * qb + (row >> 6), p.nb - 1)) : __ldg(p.q_scale + item);
-        v_max = __ldg(p.v_max + bh);
+        q_sc = PAIR ? p.q_scale[(int64_t)bh * p.nb + min(2 * qb + (row >> 6), p.nb - 1)] : p.q_scale[item];
+        v_max = p.v_max[bh];
       }
       // This warpgroup's tiles are n0, n0 + 2, ...  List entries are fetched two of its tiles ahead and the FP8
       // scales of a tile one tile ahead, so that neither load (nor the two in a row, entry then scale) is waited
@@ -658,21 +658,21 @@ fwd_pipe_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
       const int32_t* lst = p.clean_list + (int64_t)item * p.lstride;
       const float* ksc = FP8 ? p.k_scale + (int64_t)bh * p.nb : nullptr;
       const float* vsc = FP8 ? p.v_scale + (int64_t)bh * p.nb : nullptr;
-      auto ld_ent = [&](int n, int e) { return n < cnt ? __ldg(lst + n * kEnt + e) : 0; };
+      auto ld_ent = [&](int n, int e) { return n < cnt ? lst[n * kEnt + e] : 0; };
       int e_cur0 = ld_ent(n0, 0), e_cur1 = PAIR ? ld_ent(n0, 1) : 0;
       int e_nx0 = ld_ent(n0 + 2, 0), e_nx1 = PAIR ? ld_ent(n0 + 2, 1) : 0;
       float ks_cur0 = 1.0f, vs_cur0 = 1.0f, ks_cur1 = 1.0f, vs_cur1 = 1.0f;
       int bv_cur = kKeyBlk, bv_cur1 = kKeyBlk;     // real tokens of the tile's key block(s) (bricks padded to whole blocks)
       if (p.blk_valid != nullptr) {
-        bv_cur = __ldg(p.blk_valid + (e_cur0 & 0x3fffffff));
-        if constexpr (PAIR) bv_cur1 = __ldg(p.blk_valid + (e_cur1 & 0x3fffffff));
+        bv_cur = p.blk_valid[e_cur0 & 0x3fffffff];
+        if constexpr (PAIR) bv_cur1 = p.blk_valid[e_cur1 & 0x3fffffff];
       }
       if constexpr (FP8) {
-        ks_cur0 = __ldg(ksc + (e_cur0 & 0x3fffffff));
-        vs_cur0 = __ldg(vsc + (e_cur0 & 0x3fffffff));
+        ks_cur0 = ksc[e_cur0 & 0x3fffffff];
+        vs_cur0 = vsc[e_cur0 & 0x3fffffff];
         if constexpr (PAIR) {
-          ks_cur1 = __ldg(ksc + (e_cur1 & 0x3fffffff));
-          vs_cur1 = __ldg(vsc + (e_cur1 & 0x3fffffff));
+          ks_cur1 = ksc[e_cur1 & 0x3fffffff];
+          vs_cur1 = vsc[e_cur1 & 0x3fffffff];
         }
       }
       const float inv_vmax = 1.0f / v_max;
@@ -684,16 +684,16 @@ fwd_pipe_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
         const float ks0 = ks_cur0, vs0 = vs_cur0, ks1 = ks_cur1, vs1 = vs_cur1;
         const int bv0 = bv_cur, bv1 = bv_cur1;
         if (p.blk_valid != nullptr) {
-          bv_cur = __ldg(p.blk_valid + (e_nx0 & 0x3fffffff));
-          if constexpr (PAIR) bv_cur1 = __ldg(p.blk_valid + (e_nx1 & 0x3fffffff));
+          bv_cur = p.blk_valid[e_nx0 & 0x3fffffff];
+          if constexpr (PAIR) bv_cur1 = p.blk_valid[e_nx1 & 0x3fffffff];
         }
         // next tile of this warpgroup: its scales (its entries arrived a tile ago), and the entries of the one after
         if constexpr (FP8) {
-          ks_cur0 = __ldg(ksc + (e_nx0 & 0x3fffffff));
-          vs_cur0 = __ldg(vsc + (e_nx0 & 0x3fffffff));
+          ks_cur0 = ksc[e_nx0 & 0x3fffffff];
+          vs_cur0 = vsc[e_nx0 & 0x3fffffff];
           if constexpr (PAIR) {
-            ks_cur1 = __ldg(ksc + (e_nx1 & 0x3fffffff));
-            vs_cur1 = __ldg(vsc + (e_nx1 & 0x3fffffff));
+            ks_cur1 = ksc[e_nx1 & 0x3fffffff];
+            vs_cur1 = vsc[e_nx1 & 0x3fffffff];
           }
         }
         e_cur0 = e_nx0; e_cur1 = e_nx1;
@@ -955,8 +955,8 @@ fwd_pipe_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
             const float* src = p.state + ((int64_t)bh * kCompRank + a) * kPD + half * 64;
 #pragma unroll
             for (int c = 0; c < 8; ++c) {
-              const float4 lo = __ldg(reinterpret_cast<const float4*>(src + 8 * c));
-              const float4 hi = __ldg(reinterpret_cast<const float4*>(src + 8 * c + 4));
+              const float4 lo = *reinterpret_cast<const float4*>(src + 8 * c);
+              const float4 hi = *reinterpret_cast<const float4*>(src + 8 * c + 4);
               const __nv_bfloat162 h0 = __floats2bfloat162_rn(lo.x, lo.y), h1 = __floats2bfloat162_rn(lo.z, lo.w);
               const __nv_bfloat162 h2 = __floats2bfloat162_rn(hi.x, hi.y), h3 = __floats2bfloat162_rn(hi.z, hi.w);
               *reinterpret_cast<uint4*>(sC + half * 8192 + a * 128 + ((c ^ (a & 7)) << 4)) =
@@ -997,10 +997,10 @@ fwd_pipe_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
 #pragma unroll
             for (int m = 0; m < kCompRank / 2; ++m) {
               const int ax = p.rope.axis[m];
-              cs[m] = __ldg((ax == 0 ? row_t : (ax == 1 ? row_y : row_x)) + m);
+              cs[m] = (ax == 0 ? row_t : (ax == 1 ? row_y : row_x))[m];
             }
           }
-          const float gte = row_valid ? __ldg(p.gate + (int64_t)bh * p.N + q_row) : 0.0f;
+          const float gte = row_valid ? p.gate[(int64_t)bh * p.N + q_row] : 0.0f;
           ok = __all_sync(0xffffffffu, pipe_wait(bar_gt + g, closings & 1, s_abort, 23));
           if (!ok) break;
           tc_fence_after();
@@ -1159,7 +1159,7 @@ fwd_pipe_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
       const int t_last = t + cnt - 1;
       unsigned char* slot = sQ + qslot * kTile;
       float v_max = 1.0f;
-      if constexpr (FP8) v_max = __ldg(p.v_max + bh);
+      if constexpr (FP8) v_max = p.v_max[bh];
       // the slot's barrier completes once per item that uses the slot; this item's Q could only be
       // loaded after the previous user's output had left, so the wait is never more than one phase behind
       ok = __all_sync(0xffffffffu, pipe_wait(bar_cl + qslot, (nonempty >> 1) & 1, s_abort, 8));

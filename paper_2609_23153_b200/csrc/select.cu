@@ -44,10 +44,10 @@ size_t select_workspace_bytes(const sparkattn_shape_t& s) {
 constexpr int kPoolCtasPerSm = 2;
 template <int D>
 __global__ void __launch_bounds__(D / 2)
-pool_kernel(const __nv_bfloat16* __restrict__ q, const __nv_bfloat16* __restrict__ k, float* __restrict__ pq,
+pool_kernel(const __nv_bfloat16* q, const __nv_bfloat16* k, float* __restrict__ pq,
             float* __restrict__ pkT, int H, int N, int blk_size, int nb, int nbp, int64_t stride_b,
             int64_t stride_h, int64_t stride_n, int64_t n_items /* B*H*nb */,
-            const int32_t* __restrict__ block_valid /* [nb] real tokens per block, or NULL */,
+            const int32_t* block_valid /* [nb] real tokens per block, or NULL */,
             int32_t* __restrict__ header) {
   extern __shared__ __align__(16) unsigned char smem_raw[];      // [2][blk_size][D] bf16
   constexpr int kThreads = D / 2;
@@ -67,7 +67,7 @@ pool_kernel(const __nv_bfloat16* __restrict__ q, const __nv_bfloat16* __restrict
     it.blk = (int)(item % nb);
     it.bh = item / nb;
     it.nvalid = min(blk_size, N - it.blk * blk_size);
-    if (block_valid != nullptr) it.nvalid = max(1, min(it.nvalid, __ldg(block_valid + it.blk)));   // bricks padded to whole blocks
+    if (block_valid != nullptr) it.nvalid = max(1, min(it.nvalid, block_valid[it.blk]));   // bricks padded to whole blocks
     return it;
   };
   auto fetch = [&](const Item& it, int buf) {
@@ -426,7 +426,7 @@ struct TopkShape {
 
 template <int D, int RT, int RG, int KC, int NS, bool WINDOW>
 __global__ void __launch_bounds__(kTopkThreads, 2)
-topk_kernel(const float* __restrict__ pq, const float* __restrict__ pkT, int32_t* __restrict__ kept_idx,
+topk_kernel(const float* pq, const float* pkT, int32_t* __restrict__ kept_idx,
             int32_t* __restrict__ kept_cnt, int nb, int nbp, int topk, int groups_per_bh, int N, int blk_size,
             int frame_tokens, int window) {
   using Shape = TopkShape<RT, RG, KC, NS>;
@@ -469,7 +469,7 @@ topk_kernel(const float* __restrict__ pq, const float* __restrict__ pkT, int32_t
     for (int p = 0; p < NS - 1; ++p) issue(p);
     for (int e = threadIdx.x; e < R * (D / 4); e += kTopkThreads) {
       const int r = e % R, c = e / R * 4;
-      const float4 x = r < nrows ? __ldg(reinterpret_cast<const float4*>(pq + (bh * nb + i0 + r) * D + c))
+      const float4 x = r < nrows ? *reinterpret_cast<const float4*>(pq + (bh * nb + i0 + r) * D + c)
                                  : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
       s_pq[c * R + r] = x.x; s_pq[(c + 1) * R + r] = x.y; s_pq[(c + 2) * R + r] = x.z; s_pq[(c + 3) * R + r] = x.w;
     }
@@ -536,7 +536,7 @@ topk_kernel(const float* __restrict__ pq, const float* __restrict__ pkT, int32_t
 // bit by bit at a time, as it was: 147); of 1182: 439 us (484; 596).  The FMAs alone are 50 and 200 us.
 template <int D, int R, int RT, int WARPS, int CTAS, bool WINDOW>
 __global__ void __launch_bounds__(WARPS * 32, CTAS)
-topk_wide_kernel(const float* __restrict__ pq, const float* __restrict__ pkT, int32_t* __restrict__ kept_idx,
+topk_wide_kernel(const float* pq, const float* pkT, int32_t* __restrict__ kept_idx,
                  int32_t* __restrict__ kept_cnt, int nb, int nbp, int topk, int groups_per_bh, int N, int blk_size,
                  int frame_tokens, int window) {
   constexpr int kThreads = WARPS * 32;
@@ -551,7 +551,7 @@ topk_wide_kernel(const float* __restrict__ pq, const float* __restrict__ pkT, in
   if (topk < nb) {
     for (int e = threadIdx.x; e < R * (D / 4); e += kThreads) {
       const int r = e % R, c = e / R * 4;
-      const float4 x = r < nrows ? __ldg(reinterpret_cast<const float4*>(pq + (bh * nb + i0 + r) * D + c))
+      const float4 x = r < nrows ? *reinterpret_cast<const float4*>(pq + (bh * nb + i0 + r) * D + c)
                                  : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
       s_pq[c * R + r] = x.x; s_pq[(c + 1) * R + r] = x.y; s_pq[(c + 2) * R + r] = x.z; s_pq[(c + 3) * R + r] = x.w;
     }
@@ -570,7 +570,7 @@ topk_wide_kernel(const float* __restrict__ pq, const float* __restrict__ pkT, in
       const float* kp = kcol + j0;
       auto load_batch = [&](float4 (&kv)[kCB], int c0) {
 #pragma unroll
-        for (int cc = 0; cc < kCB; ++cc) kv[cc] = __ldg(reinterpret_cast<const float4*>(kp + (int64_t)(c0 + cc) * nbp));
+        for (int cc = 0; cc < kCB; ++cc) kv[cc] = *reinterpret_cast<const float4*>(kp + (int64_t)(c0 + cc) * nbp);
       };
       auto fma_batch = [&](const float4 (&kv)[kCB], int c0) {
 #pragma unroll

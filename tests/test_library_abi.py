@@ -270,3 +270,23 @@ def test_gated_forward_validates_on_the_host(lib):
     assert call(nbytes=need - 1) == sa.E_WORKSPACE_TOO_SMALL
     assert lib.sparkattn_fwd_gated_workspace_bytes(ctypes.byref(_shape(N=2048, d=128, block=64)), 4, grid) == 0
     assert lib.sparkattn_fwd_gated_workspace_bytes(ctypes.byref(s), 4, (ctypes.c_int32 * 3)(2, 32, 31)) == 0
+
+
+def test_early_launched_kernels_read_with_ordinary_loads():
+    """A kernel that calls pdl_wait may be resident while the kernels before it write what it reads.  A read-only load
+    is only defined for data that nothing writes during the kernel's life, so neither __ldg nor a const __restrict__
+    parameter may stand in such a kernel or in what it calls."""
+    src = os.path.join(ROOT, "paper_2609_23153_b200", "csrc")
+    kernels = 0
+    for name in sorted(f for f in os.listdir(src) if f.endswith(".cu")):
+        text = re.sub(r"//[^\n]*", "", open(os.path.join(src, name)).read())
+        if "pdl_wait" not in text:
+            continue
+        assert "__ldg" not in text, name
+        for kernel in re.split(r"\b__global__\b", text)[1:]:
+            if "pdl_wait" not in kernel:
+                continue
+            kernels += 1
+            params = kernel[:kernel.index("{")]
+            assert not re.search(r"const[^,]*__restrict__", params), (name, params.split("(")[0])
+    assert kernels >= 7
