@@ -90,6 +90,38 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, volati
   return false;
 }
 
+// mbar_wait in the shortest form, for a kernel with some twenty waits whose code does not fit the SM's instruction cache
+// as it is.  The limit is the same; on expiry only the wait's id goes to the abort flag (the first one stays), and
+// report_abort takes it to the status words when the CTA winds down.
+constexpr int kAbortTimeout = 256;
+__device__ __forceinline__ uint32_t global_timer_lo() {
+  uint32_t t;
+  asm volatile("mov.u32 %0, %%globaltimer_lo;" : "=r"(t));
+  return t;
+}
+__device__ __forceinline__ void abort_timeout(volatile int* abort_flag, int wait_id) {
+  atomicCAS(const_cast<int*>(abort_flag), 0, kAbortTimeout + wait_id);
+}
+__device__ __forceinline__ bool pipe_wait(uint64_t* bar, uint32_t parity, volatile int* abort_flag, int wait_id,
+                                          uint32_t limit_ns = (uint32_t)kWaitLimitNs) {
+  if (mbar_try_wait(bar, parity)) return true;
+  static_assert(kWaitLimitNs < 0xf0000000ull, "the limit is counted in 32 bits");
+  const uint32_t t0 = global_timer_lo();
+  for (uint32_t it = 1;; ++it) {
+    if (mbar_try_wait(bar, parity)) return true;
+    if ((it & 63u) == 0u) {
+      if (*abort_flag) return false;
+      if (global_timer_lo() - t0 > limit_ns) {
+        abort_timeout(abort_flag, wait_id);
+        return false;
+      }
+    }
+  }
+}
+__device__ __forceinline__ void report_abort(int32_t* status, int abort_flag) {
+  if (abort_flag >= kAbortTimeout) report_status(status, SPARKATTN_E_DEVICE_TIMEOUT, abort_flag - kAbortTimeout);
+}
+
 // Asynchronous 16-byte copies global -> shared (both sides 16-byte aligned) and their groups.
 __device__ __forceinline__ void cp_async16(uint32_t smem_dst, const void* src) {
   asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_dst), "l"(src) : "memory");

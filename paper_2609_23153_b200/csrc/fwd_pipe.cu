@@ -279,31 +279,6 @@ __device__ __forceinline__ void pipe_tma_store_4d(const void* tmap, const void* 
       : "memory");
 }
 
-// mbar_wait (common.cuh) in the shortest form: this kernel has some twenty of these waits, and what its warps run does
-// not fit the SM's instruction cache as it is.  The limit is the same; on expiry only the wait's id goes to the abort
-// flag, and the teardown reports it.
-constexpr int kAbortTimeout = 256;
-__device__ __forceinline__ uint32_t global_timer_lo() {
-  uint32_t t;
-  asm volatile("mov.u32 %0, %%globaltimer_lo;" : "=r"(t));
-  return t;
-}
-__device__ __forceinline__ bool pipe_wait(uint64_t* bar, uint32_t parity, volatile int* abort_flag, int wait_id) {
-  if (mbar_try_wait(bar, parity)) return true;
-  static_assert(kWaitLimitNs < 0xf0000000ull, "the limit is counted in 32 bits");
-  const uint32_t t0 = global_timer_lo();
-  for (uint32_t it = 1;; ++it) {
-    if (mbar_try_wait(bar, parity)) return true;
-    if ((it & 63u) == 0u) {
-      if (*abort_flag) return false;
-      if (global_timer_lo() - t0 > (uint32_t)kWaitLimitNs) {
-        *abort_flag = kAbortTimeout + wait_id;
-        return false;
-      }
-    }
-  }
-}
-
 // One thread of a converged warp; and a value that is the same in all its threads, told to the compiler as such.
 __device__ __forceinline__ bool elect_one() {
   uint32_t one;
@@ -1220,7 +1195,7 @@ fwd_pipe_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
   // ------------------------------------------------------------------ teardown
   tc_fence_before();
   __syncthreads();
-  if (threadIdx.x == 0 && *s_abort >= kAbortTimeout) report_status(p.status, SPARKATTN_E_DEVICE_TIMEOUT, *s_abort - kAbortTimeout);
+  if (threadIdx.x == 0) report_abort(p.status, *s_abort);
   if (warp == 0) {
     if (*s_abort) __nanosleep(200000);  // let copies / MMAs in flight land before the CTA's resources go
     tc_fence_after();

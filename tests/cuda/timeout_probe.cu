@@ -1,8 +1,8 @@
-// Test-only kernel (built by tests/test_gpu_timeout.py, not part of the library): one warp calls the
-// library's bounded barrier wait on an mbarrier that nothing ever arrives at, with a limit of about a
-// millisecond instead of the library's default.  The wait runs out, records SPARKATTN_E_DEVICE_TIMEOUT and
-// the wait id in the status words of the workspace, and the kernel returns normally: no trap, no fault,
-// nothing left spinning.
+// Test-only kernels (built by tests/test_gpu_timeout.py, not part of the library): they call the library's two
+// bounded barrier waits on an mbarrier that nothing ever arrives at, with a limit of about a millisecond
+// instead of the library's default.  The wait runs out, SPARKATTN_E_DEVICE_TIMEOUT and the wait id end up in
+// the status words of the workspace, and the kernel returns normally: no trap, no fault, nothing left
+// spinning.
 #include "../../paper_2609_23153_b200/csrc/common.cuh"
 
 using namespace sparkattn;
@@ -21,9 +21,31 @@ __global__ void timeout_probe_kernel(int32_t* status, unsigned long long limit_n
   atomicAdd(status + (ok ? 3 : 2), 1);
 }
 
-extern "C" int timeout_probe(void* workspace, unsigned long long limit_ns, int wait_id, void* stream) {
+// The wait of the pipelined kernels: two warps wait, the second with four times the limit, so it leaves because the first
+// one has given up; then a second expiry is recorded, which must not replace the first.
+__global__ void pipe_timeout_probe_kernel(int32_t* status, unsigned limit_ns, int wait_id) {
+  __shared__ uint64_t bar;
+  __shared__ int abort_flag;
+  if (threadIdx.x == 0) {
+    mbar_init(&bar, 1);
+    abort_flag = 0;
+    mbar_fence_init();
+  }
+  __syncthreads();
+  const int warp = threadIdx.x >> 5;
+  const bool ok = pipe_wait(&bar, 0, &abort_flag, wait_id + warp, limit_ns << (2 * warp));
+  atomicAdd(status + (ok ? 3 : 2), 1);
+  __syncthreads();
+  if (threadIdx.x == 32) abort_timeout(&abort_flag, wait_id + 1);
+  __syncthreads();
+  if (threadIdx.x == 0) report_abort(status, abort_flag);
+}
+
+extern "C" int timeout_probe(void* workspace, unsigned long long limit_ns, int wait_id, int pipelined, void* stream) {
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   if (cudaMemsetAsync(workspace, 0, kWorkspaceHeaderBytes, s) != cudaSuccess) return -1;
-  timeout_probe_kernel<<<1, 32, 0, s>>>(static_cast<int32_t*>(workspace), limit_ns, wait_id);
+  int32_t* status = static_cast<int32_t*>(workspace);
+  if (pipelined) pipe_timeout_probe_kernel<<<1, 64, 0, s>>>(status, (unsigned)limit_ns, wait_id);
+  else timeout_probe_kernel<<<1, 32, 0, s>>>(status, limit_ns, wait_id);
   return cudaGetLastError() == cudaSuccess ? 0 : -1;
 }
