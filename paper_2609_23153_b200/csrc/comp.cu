@@ -639,8 +639,8 @@ static int comp_chunks(const sparkattn_shape_t& s) {
   return best;
 }
 
-void launch_rope_table(const RopeTable& rope, float2* table, cudaStream_t stream) {
-  rope_table_kernel<<<(unsigned)(rope.T + rope.Hg + rope.Wg), kRank / 2, 0, stream>>>(rope, table);
+int launch_rope_table(const RopeTable& rope, float2* table, cudaStream_t stream) {
+  return launch_kernel(rope_table_kernel, (unsigned)(rope.T + rope.Hg + rope.Wg), kRank / 2, 0, false, stream, rope, table);
 }
 
 size_t rope_table_bytes(const int32_t* grid) {
@@ -661,8 +661,7 @@ static int prepare_workspace(CompParams& prm, const int32_t* grid, void* workspa
   prm.rope_table = table;
   prm.partial = reinterpret_cast<float*>(base + kWorkspaceHeaderBytes + rope_table_bytes(grid));
   if (cudaMemsetAsync(workspace, 0, kWorkspaceHeaderBytes, stream) != cudaSuccess) return SPARKATTN_E_CUDA;
-  rope_table_kernel<<<(unsigned)(grid[0] + grid[1] + grid[2]), kRank / 2, 0, stream>>>(prm.rope, table);
-  return SPARKATTN_OK;
+  return launch_rope_table(prm.rope, table, stream);
 }
 
 static void fill_rope(CompParams& prm, const int32_t* grid, const int32_t* axis, const float* freq) {

@@ -1316,7 +1316,7 @@ static int launch_pipe(const sparkattn_shape_t& s, bool fp8, const void* q, cons
     for (int m = 0; m < kCompRank / 2; ++m) { prm.rope.axis[m] = ga->axis[m]; prm.rope.freq[m] = ga->freq[m]; }
     prm.rope.T = ga->grid[0]; prm.rope.Hg = ga->grid[1]; prm.rope.Wg = ga->grid[2];
     float2* table = reinterpret_cast<float2*>(base + (fwd_pipe_workspace_bytes(s, kmax) + 255) / 256 * 256);
-    launch_rope_table(prm.rope, table, stream);
+    if ((rc = launch_rope_table(prm.rope, table, stream)) != SPARKATTN_OK) return rc;
     prm.rope_table = table;
     prm.state = ga->state; prm.gate = ga->gate; prm.eps = ga->eps;
   }

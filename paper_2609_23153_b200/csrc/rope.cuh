@@ -18,7 +18,7 @@ struct RopeTable {
 // Bytes of the position-major cos / sin table of a (T, Hg, Wg) grid, and the launch that fills it:
 // table[(base(axis) + e) * rank/2 + m] = (cos, sin)(e * freq[m]), base(t) = 0, base(y) = T, base(x) = T + Hg.
 size_t rope_table_bytes(const int32_t* grid);
-void launch_rope_table(const RopeTable& rope, float2* table, cudaStream_t stream);
+int launch_rope_table(const RopeTable& rope, float2* table, cudaStream_t stream);
 
 __device__ __forceinline__ float fast_rcp(float x) {
   float y;

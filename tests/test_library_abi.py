@@ -290,3 +290,14 @@ def test_early_launched_kernels_read_with_ordinary_loads():
             params = kernel[:kernel.index("{")]
             assert not re.search(r"const[^,]*__restrict__", params), (name, params.split("(")[0])
     assert kernels >= 7
+
+
+def test_failed_rotary_table_launch_is_reported(lib):
+    """A grid of no positions is a launch without blocks: the runtime refuses it on the host, with or without a device,
+    and the launcher has to hand that on (the gated forward would read a table that nothing wrote)."""
+    name = "_ZN9sparkattn17launch_rope_tableERKNS_9RopeTableEP6float2P11CUstream_st"
+    launch = getattr(ctypes.CDLL(sa.LIB_PATH), name)
+    launch.restype = ctypes.c_int
+    launch.argtypes = [ctypes.c_void_p] * 3
+    rope = (ctypes.c_int32 * 67)()                            # axis[32], freq[32], T, Hg, Wg
+    assert launch(rope, None, None) == sa.E_CUDA
