@@ -25,7 +25,9 @@ inline int launch_kernel(void (*kern)(Params...), unsigned grid, unsigned thread
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = overlap ? 1 : 0;
-  return cudaLaunchKernelEx(&cfg, kern, Params(args)...) == cudaSuccess ? SPARKATTN_OK : SPARKATTN_E_CUDA;
+  if (cudaLaunchKernelEx(&cfg, kern, Params(args)...) == cudaSuccess) return SPARKATTN_OK;
+  cudaGetLastError();          // reported here: a later call's own check must not find it again
+  return SPARKATTN_E_CUDA;
 }
 
 // quant.cu

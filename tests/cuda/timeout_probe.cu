@@ -4,6 +4,7 @@
 // the status words of the workspace, and the kernel returns normally: no trap, no fault, nothing left
 // spinning.
 #include "../../paper_2609_23153_b200/csrc/common.cuh"
+#include "../../paper_2609_23153_b200/csrc/launch.h"
 
 using namespace sparkattn;
 
@@ -48,4 +49,13 @@ extern "C" int timeout_probe(void* workspace, unsigned long long limit_ns, int w
   if (pipelined) pipe_timeout_probe_kernel<<<1, 64, 0, s>>>(status, (unsigned)limit_ns, wait_id);
   else timeout_probe_kernel<<<1, 32, 0, s>>>(status, limit_ns, wait_id);
   return cudaGetLastError() == cudaSuccess ? 0 : -1;
+}
+
+// A launch without blocks, which the runtime refuses on the host, through the library's launch helper.  Bit 0: the helper
+// did not report it; bit 1: the runtime still holds the error.
+__global__ void never_run_kernel(int) {}
+
+extern "C" int launch_probe(int overlap) {
+  const int rc = launch_kernel(never_run_kernel, 0, 32, 0, overlap != 0, nullptr, 1);
+  return (rc != SPARKATTN_E_CUDA ? 1 : 0) | (cudaGetLastError() != cudaSuccess ? 2 : 0);
 }

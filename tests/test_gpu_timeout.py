@@ -47,3 +47,10 @@ def test_expired_wait_sets_timeout_status_and_returns(probe, pipelined, threads)
     # the context is still usable and a later library call on the same workspace starts clean
     x = torch.ones(1024, device="cuda:0")
     assert float(x.sum()) == 1024.0
+
+
+@pytest.mark.parametrize("overlap", [0, 1])
+def test_failed_launch_is_reported_once(probe, overlap):
+    """A launch that the runtime refuses on the host: the library's launch helper reports it and takes the runtime's
+    last error with it, so that the check after a later, unrelated launch does not find it again."""
+    assert probe.launch_probe(overlap) == 0
