@@ -301,3 +301,17 @@ def test_failed_rotary_table_launch_is_reported(lib):
     launch.argtypes = [ctypes.c_void_p] * 3
     rope = (ctypes.c_int32 * 67)()                            # axis[32], freq[32], T, Hg, Wg
     assert launch(rope, None, None) == sa.E_CUDA
+
+
+def test_current_stream_without_the_private_name(monkeypatch):
+    """The binding takes the current stream's handle through a name that torch may drop; the public way stays."""
+    class Stream:
+        cuda_stream = 0x1230
+
+    monkeypatch.setattr(torch.cuda, "current_stream", lambda: Stream)
+    monkeypatch.setattr(sa, "_raw_stream", None)
+    assert sa._stream_ptr(None) == 0x1230
+    monkeypatch.setattr(torch.cuda, "current_device", lambda: 3)
+    monkeypatch.setattr(sa, "_raw_stream", lambda device: 0x4560 + device)
+    assert sa._stream_ptr(None) == 0x4563
+    assert sa._stream_ptr(Stream) == 0x1230
