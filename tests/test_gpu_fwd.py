@@ -293,13 +293,15 @@ def test_long_permuted_lists_own_block_anywhere(block, fp8):
     assert (num / den) ** 0.5 <= (5e-2 if fp8 else 1e-2)
 
 
-@pytest.mark.parametrize("block,window,fp8", [(128, 0, False), (64, 0, False), (128, 2, False), (128, 0, True), (64, 0, True)])
-def test_both_kernels_agree_bitwise(block, window, fp8):
-    """d = 128: kept lists of at most 32 entries run the kernel with a closing warpgroup, longer list strides the
-    two-warpgroup kernel.  The same lists padded to a stride of 40 (the counts say how many entries are real)
-    must give the same output and lse bit for bit: both kernels take every step in the same arithmetic and order.
-    More items than SMs, counts 0 ... kmax, a ragged last block; with a causal window the same through the masked
-    instantiations; bf16 and FP8."""
+@pytest.mark.parametrize("block,window,fp8,stride", [(64, 0, False, 72), (64, 2, False, 72), (128, 0, True, 40), (128, 2, True, 40),
+                                                     (64, 0, True, 40), (64, 2, True, 40), (128, 0, False, 40), (128, 2, False, 40)])
+def test_both_kernels_agree_bitwise(block, window, fp8, stride):
+    """d = 128: list strides of at most 64 (bf16, 64-token blocks) or 32 (FP8) run the kernel with a closing warpgroup,
+    longer ones the two-warpgroup kernel.  The same lists padded to a stride beyond that line (the counts say how
+    many entries are real) must give the same output and lse bit for bit: both kernels take every step in the same
+    arithmetic and order.  (bf16 with 128-token blocks has one kernel for every stride: there the padding alone must not
+    matter.)  More items than SMs, counts 0 ... kmax, a ragged last block; with a causal window the same through the
+    masked instantiations."""
     grid = (15, 18, 19)                                        # N = 5130: 41 blocks of 128 (last: 10 tokens) / 81 of 64
     w = _small(71 + block + window + int(fp8), 6, 128, grid, block, 0.0)
     q, k, v = workloads.structured_qkv(w)
@@ -308,7 +310,7 @@ def test_both_kernels_agree_bitwise(block, window, fp8):
     idx = torch.stack([torch.stack([torch.randperm(w.nb, generator=g)[:kmax] for _ in range(w.nb)]) for _ in range(w.H)]).to(torch.int32)
     cnt = torch.randint(0, kmax + 1, (w.H, w.nb), generator=g, dtype=torch.int32)
     cnt[0, 0] = 0; cnt[0, 1] = 1; cnt[0, 2] = 2; cnt[0, 3] = kmax
-    wide = torch.full((w.H, w.nb, 40), -7, dtype=torch.int32)  # entries past the count are never read
+    wide = torch.full((w.H, w.nb, stride), -7, dtype=torch.int32)  # entries past the count are never read
     wide[:, :, :kmax] = idx
     qd, kd, vd = q.to(DEV), k.to(DEV), v.to(DEV)
     kw = dict(frame_tokens=18 * 19, window=window) if window else {}
@@ -328,7 +330,7 @@ def test_both_kernels_agree_bitwise(block, window, fp8):
     # (random lists under a causal window leave some rows without any admissible key: lse = -inf on both sides,
     # which test_gpu_window.py checks; here the output alone is compared with the oracle in that case)
     if fp8:
-        _compare_items(b[0], lb[0], ref_out, ref_lse, items, w.block, w.N, FP8_RELRMS, None)
+        _compare_items(b[0], None if window else lb[0], ref_out, ref_lse, items, w.block, w.N, FP8_RELRMS, None)
     else:
         _compare_items(b[0], None if window else lb[0], ref_out, ref_lse, items, w.block, w.N, BF16_RELRMS, BF16_MAXABS)
 
