@@ -390,10 +390,13 @@ fwd_pipe_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
   // A wait of a control warp.  bf16 with 128-token blocks runs at the chip's power limit: there one thread polls and
   // all learn of it (720p shape at 97 %: 2.86 ms, against 3.00 with 32 polling threads in 3 % fewer clocks).  The
   // others run at full clock and take the shorter way (the gated kernel: 8-11 % faster with it).
+  // The thread that polls is the one that issues: elect.sync picks the same one for the same mask every time, and only
+  // the thread that has seen the barrier flip is ordered behind what it stands for.
   constexpr bool kLone = !FP8 && !PAIR && !GATE;
+  const bool leader = elect_one();
   auto ctrl_wait = [&](uint64_t* bar, uint32_t parity, int id) {
     bool done = true;
-    if (!kLone || lane == 0) done = pipe_wait(bar, parity, s_abort, id);
+    if (!kLone || leader) done = pipe_wait(bar, parity, s_abort, id);
     return kLone ? __all_sync(0xffffffffu, done) != 0 : done;
   };
 
