@@ -358,7 +358,7 @@ fwd_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant__ C
           }
           reinterpret_cast<uint4*>(orow)[i] = make_uint4(ww[0], ww[1], ww[2], ww[3]);
         }
-        if (p.lse && chain == 0) p.lse[(int64_t)bh * p.N + q_row] = (m + log2f(total)) * 0.6931471805599453f;
+        if (p.lse && chain == 0) p.lse[(int64_t)bh * p.N + q_row] = fmaf(m, 0.6931471805599453f, log2f(total) * 0.6931471805599453f);   // one rounding
       }
     }
   }

@@ -417,3 +417,21 @@ def test_empty_lists_between_short_ones(block, stride, kind):
     """Items with an empty list between items of one to three tiles, so that the roles of a CTA are several items apart:
     an empty item must neither release nor take a Q slot that another item still uses."""
     _check_stream(STREAMS, block, stride, kind)
+
+
+@pytest.mark.parametrize("H", [28, 56])
+def test_lse_of_merged_chains_is_rounded_once(H):
+    """d = 64: scores that fp32 holds exactly and one key that outweighs the others, so that the log-sum-exp is off by its
+    own rounding (at most 2^-24 of it) and by what ln 2 and log2 e lose as fp32 constants (1.1e-8 together).  112 items
+    run four chains each, 224 two."""
+    N, nb = 256, 4
+    a = 128 + torch.arange(N) % 128
+    b = (200 + torch.arange(H))[:, None] - 16 * torch.ones((H, N), dtype=torch.int64)
+    b[torch.arange(H), 37 * torch.arange(H) % N] += 16
+    q, k = torch.zeros((1, H, N, 64)), torch.zeros((1, H, N, 64))
+    q[0, :, :, 0], k[0, :, :, 0] = a, b                                    # integers below 256: exact in bf16
+    idx = torch.arange(nb, dtype=torch.int32).expand(1, H, nb, nb).contiguous()
+    q, k = (t.to(torch.bfloat16).to(DEV) for t in (q, k))
+    _, lse = sa.fwd(q, k, k, idx.to(DEV), None, 64, return_lse=True, check_status=True)
+    ref = torch.logsumexp(a.double()[None, :, None] * b.double()[:, None] / 8, -1)
+    assert float(((lse[0].cpu().double() - ref) / ref).abs().max()) <= 2.0 ** -24 + 1.2e-8
