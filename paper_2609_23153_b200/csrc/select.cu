@@ -661,14 +661,19 @@ static int launch_topk_d(const sparkattn_shape_t& s, int topk, int frame_tokens,
   constexpr size_t kOne = 227 * 1024, kTwo = 113 * 1024;       // shared memory of a CTA alone on its SM, and of one of two
   constexpr int kNumSMs = 148;   // B200; another count only moves the points where the CTAs get smaller
   const int64_t ctas32 = bh * ((nb + 31) / 32), ctas16 = bh * ((nb + 15) / 16);
-  // More than 256 key blocks (d = 128, one launch): the wide kernel, which the other one matches at best (1 head of 591
-  // blocks 20.8 against 22.5 us, but 4 heads 26.8 against 22.8, 12 heads 55.5 against 45.4, 8 heads of 1182 166 against
-  // 111), with 16 rows while two CTAs' key rows fit an SM and 8 beyond.  Up to 256: the other one (its column split
-  // leaves no warp idle there), with as many rows per CTA as still leave 1.5 CTAs (32 rows) or one CTA (16) per SM:
+  // More than 256 key blocks: the wide kernel, with 8 rows while 16 would leave SMs idle or do not fit twice into an SM,
+  // else 16.  8 against 16 rows, whole selection (pooling included), d = 128: 1 head of 260 / 591 / 1182 blocks of 128
+  // 16.5 / 23.5 / 35 us against 21.1 / 26.7 / 71, 4 of 591 (148 CTAs of 16) 47.6 against 52.6, 3 of 1000 (189) 69 against 82,
+  // but 12 of 257 (204) 64.7 against 57.3, 12 of 591 132 against 127, 40 of 591 425 against 389; d = 64: 1 of 260 / 591 10.6 /
+  // 13.6 against 14.0 / 17.1, 4 of 591 22.0 against 25.9, 12 of 257 26.7 against 25.9, 40 of 591 197 against 178.  The other
+  // kernel on these rows: d = 128 1 head of 260 / 591 15.9 / 33.5, 12 of 257 / 591 59.9 / 154, 40 of 591 463; d = 64 1 of 260 /
+  // 591 10.1 / 14.4, 12 of 257 / 591 26.8 / 80, 40 of 591 232.  Up to 256 blocks: the other one (its column split leaves
+  // no warp idle there; wide with 16 rows: 1 / 12 / 40 heads of 256 20.6 / 54 / 158 against 12.8 / 51 / 143, d = 64 14.7 / 23.9 /
+  // 65 against 9.1 / 20.8 / 59), with as many rows per CTA as still leave 1.5 CTAs (32 rows) or one CTA (16) per SM:
   // 80 heads of 250 blocks 63.9 us with 32 rows, 69.9 with 16, 94.6 with 8; 12 heads of 256 22.0 / 20.8 / 22.2; 3 heads
   // of 50 16.9 / 12.5 / 10.4.
   if (nb > 256) {
-    if (wide_smem(16, D, nbp) <= kTwo) return go(launch_topk_wide<D, 16, 8, 10, 2>);
+    if (ctas16 > kNumSMs && wide_smem(16, D, nbp) <= kTwo) return go(launch_topk_wide<D, 16, 8, 10, 2>);
     return go(launch_topk_wide<D, 8, 8, 10, 2>);               // at most 132 KB
   }
   static_assert(TopkShape<8, 4, 16, 4>::smem_bytes(D, 256) <= kOne, "the tile of 32 rows of 256 keys");

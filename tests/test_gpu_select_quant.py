@@ -260,3 +260,18 @@ def test_quant_with_pooling_strided_batch_equals_separate_calls():
     assert torch.equal(cq, rq) and torch.equal(ck, rk)
     assert torch.equal(sq.view(torch.int32), rsq.view(torch.int32)) and torch.equal(sk.view(torch.int32), rsk.view(torch.int32))
     assert torch.equal(idx, ridx) and torch.equal(cnt, rcnt)
+
+
+@pytest.mark.parametrize("H,nb,d,window", [(1, 257, 128, 0), (1, 263, 64, 0), (3, 300, 64, 0), (1, 1290, 64, 3), (8, 289, 128, 0), (8, 305, 64, 0)])
+def test_few_heads_of_many_blocks(H, nb, d, window):
+    """More than 256 key blocks, on either side of the number of query blocks from which a CTA takes 16 of them instead
+    of 8 (8 heads of 289 blocks: 152 CTAs of 16): the oracle's lists."""
+    g = torch.Generator().manual_seed(nb + d)
+    N = nb * 64 - 29
+    q, k = ((torch.randn((H, N, d), generator=g) + torch.randn((H, nb, 1, d), generator=g).expand(H, nb, 64, d).reshape(H, -1, d)[:, :N])
+            .to(torch.bfloat16) for _ in range(2))
+    kw = dict(frame_tokens=1000, window=window) if window else {}
+    for topk in (1, nb // 30, nb // 2):
+        idx, cnt = sa.select(q[None].to(DEV), k[None].to(DEV), 64, topk, **kw)
+        ref_idx, ref_cnt = oracle.select(q, k, 64, topk, **kw)
+        assert torch.equal(idx[0].cpu(), ref_idx) and torch.equal(cnt[0].cpu(), ref_cnt)
