@@ -47,7 +47,7 @@
 // issuing (descriptors and coordinates in uniform registers), masks are a bit per column, items are taken apart by a
 // multiplication, waits have the shortest polling loop.  Measured over the version without these (12 heads of 32,760
 // tokens, 18 of 256 blocks kept): 177 -> 159 million warp instructions, 620,000 -> 582,000 clocks; 40 heads of 75,600
-// tokens, 97 %: bf16 2.97 -> 2.86 ms, FP8 2.77 -> 2.60 ms, 64-token blocks 4.30 -> 3.55 ms.
+// tokens, 97 %, after idle: bf16 3.08 -> 2.99 ms (in turn on one board), FP8 2.80 -> 2.60 ms, 64-token blocks 4.30 -> 3.55 ms.
 //
 // GATE variant (sparkattn_fwd_gated; bf16, 128-token blocks, 384 threads): the closing softmax warpgroup
 // adds the gated low-rank term of Sec. 4.1 before the store.  Once the last PV of the item is complete it
@@ -58,7 +58,9 @@
 // and order are those of comp.cu's apply pass, so the result equals the two separate calls bit for
 // bit.  Measured (720p shape, 97 % sparsity): the closing grows from ~1300 to ~7200 clocks per item
 // (two dependent tensor-core round trips, 128 special-function operations per row, three passes over
-// TMEM), during which the pipeline drains: the fused call takes as long as the two calls it replaces.
+// TMEM), during which the pipeline drains: the fused call takes 2 % longer than the two calls it replaces (3.44
+// against 3.37 ms after idle, in turn; 480p shape 0.623 against 0.610) and less only where launches are what
+// counts (3 heads of 1,200 tokens: 33 against 47 us).
 #include <cuda.h>
 #include <cuda_fp8.h>
 
@@ -83,7 +85,8 @@ constexpr int kTile = 32768;                               // bytes of one 128 x
 constexpr int kOffQ = 0, kOffK = 2 * kTile, kOffMisc = 7 * kTile;     // Q slots | K ring, V ring (5 x 32 KB) | barriers ...
 constexpr int kPipeSmem = kOffMisc + 512 /*barriers*/ + 2 * 128 * 4 /*reference maxima*/ + 128 * 8 /*row sums*/ + 64;
 
-// x / d for 0 <= x < 2^31 without the division's twenty-odd instructions at every place that takes an item apart
+// x / d for 0 <= x < 2^31 without the division's twenty-odd instructions at every place that takes an item apart: division
+// by an invariant integer through multiplication, after Granlund and Montgomery
 struct FastDiv {
   uint32_t mul, shift;
 };
