@@ -57,8 +57,9 @@ struct CompParams {
 // pairs of one axis sit in one 256-byte row: table[(base(axis) + e) * 32 + m] = (cos, sin)(e * freq[m])
 // with base(t) = 0, base(y) = T, base(x) = T + Hg (entries of pairs that rotate by another axis are
 // unused).  A few thousand entries; the feature loops read it through L1 instead of running a
-// full-range sincosf per (token, pair).
-__global__ void rope_table_kernel(const RopeTable rope, float2* __restrict__ table) {
+// full-range sincosf per (token, pair).  `header` (may be NULL): a workspace header to clear on the way.
+__global__ void rope_table_kernel(const RopeTable rope, float2* __restrict__ table, int32_t* __restrict__ header) {
+  pdl_trigger();
   const int m = threadIdx.x;                         // rank/2 threads
   const int ax = rope.axis[m];
   const int e = blockIdx.x;                          // T + Hg + Wg blocks
@@ -66,6 +67,9 @@ __global__ void rope_table_kernel(const RopeTable rope, float2* __restrict__ tab
   const int hi = ax == 0 ? rope.T : (ax == 1 ? rope.T + rope.Hg : rope.T + rope.Hg + rope.Wg);
   float sn = 0.0f, cs = 1.0f;
   if (e >= lo && e < hi) sincosf((float)(e - lo) * rope.freq[m], &sn, &cs);
+  pdl_wait();
+  if (header != nullptr && e == 0)
+    for (int i = m; i < kWorkspaceHeaderBytes / 4; i += kRank / 2) header[i] = 0;
   table[e * (kRank / 2) + m] = make_float2(cs, sn);
 }
 
@@ -76,7 +80,7 @@ __device__ __forceinline__ void fence_proxy_async_smem() {
 // The (cos, sin) pairs of one token's rank/2 feature pairs, requested from the position-major table.  Called
 // before the wait for the token tile's projection, so that the table's L2 latency is not on the row's path.
 __device__ __forceinline__ void rope_factors(float2 (&cs)[kRank / 2], const RopeTable& rope,
-                                             const float2* __restrict__ table, int token) {
+                                             const float2* table, int token) {
   const int x = token % rope.Wg;
   const int yy = token / rope.Wg;
   const int y = yy % rope.Hg;
@@ -87,7 +91,7 @@ __device__ __forceinline__ void rope_factors(float2 (&cs)[kRank / 2], const Rope
 #pragma unroll
   for (int m = 0; m < kRank / 2; ++m) {
     const int ax = rope.axis[m];
-    cs[m] = __ldg((ax == 0 ? row_t : (ax == 1 ? row_y : row_x)) + m);
+    cs[m] = (ax == 0 ? row_t : (ax == 1 ? row_y : row_x))[m];
   }
 }
 
@@ -213,6 +217,8 @@ comp_state_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid_const
     tmem_alloc(s_tmem, 256);
     tmem_relinquish();
   }
+  pdl_trigger();
+  pdl_wait();                                      // everything above runs while the kernel before this one drains
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
@@ -342,15 +348,36 @@ comp_state_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid_const
   }
 }
 
-// state[bh][r][d] = sum over chunks (ascending) of partial[bh][chunk][d][r]
-__global__ void comp_reduce_kernel(const float* __restrict__ partial, float* __restrict__ state, int nchunks) {
-  const int bh = blockIdx.x;
-  for (int e = threadIdx.x; e < kRank * kCD; e += blockDim.x) {
-    const int a = e / kCD, c = e % kCD;
-    float acc = 0.0f;
-    for (int k = 0; k < nchunks; ++k) acc += partial[(((int64_t)bh * nchunks + k) * kCD + c) * kRank + a];
-    state[((int64_t)bh * kRank + a) * kCD + c] = acc;
+// state[bh][r][d] = sum over chunks (ascending) of partial[bh][chunk][d][r].  Bound by the latency of one thread's chain
+// of loads: a CTA takes 8 channels (2 KB of every chunk, 16 contiguous bytes per thread), 16 chunks' loads in flight, so
+// that few heads (which have many chunks: 148 of one head) still spread over 16 CTAs each.  One CTA per head walking the
+// chunks element by element, 256 bytes apart, took most of a small state pass: whole pass with this and with the launches
+// overlapped, 3 heads of 1,200 tokens 64 -> 7.7 us, of 32,760 203 -> 16, 12 heads of 32,760 97 -> 38, 40 of 75,600 270 -> 232.
+constexpr int kReduceChannels = 8, kReduceThreads = kReduceChannels * kRank / 4;
+__global__ void __launch_bounds__(kReduceThreads) comp_reduce_kernel(const float* partial, float* __restrict__ state, int nchunks) {
+  pdl_trigger();
+  pdl_wait();
+  constexpr int kGroups = kCD / kReduceChannels;
+  const int bh = blockIdx.x / kGroups, c0 = blockIdx.x % kGroups * kReduceChannels;
+  const int c = threadIdx.x / (kRank / 4), a = threadIdx.x % (kRank / 4) * 4;
+  const float* src = partial + ((int64_t)bh * nchunks * kCD + c0 + c) * kRank + a;
+  constexpr int64_t kStep = (int64_t)kCD * kRank;
+  float4 acc = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+  constexpr int U = 16;
+  for (int k = 0; k < nchunks; k += U) {
+    float4 x[U];
+#pragma unroll
+    for (int u = 0; u < U; ++u)
+      if (k + u < nchunks) x[u] = *reinterpret_cast<const float4*>(src + (k + u) * kStep);
+#pragma unroll
+    for (int u = 0; u < U; ++u)
+      if (k + u < nchunks) { acc.x += x[u].x; acc.y += x[u].y; acc.z += x[u].z; acc.w += x[u].w; }
   }
+  __shared__ float s_out[kRank][kReduceChannels + 1];
+  s_out[a][c] = acc.x; s_out[a + 1][c] = acc.y; s_out[a + 2][c] = acc.z; s_out[a + 3][c] = acc.w;
+  __syncthreads();
+  for (int e = threadIdx.x; e < kRank * kReduceChannels; e += kReduceThreads)
+    state[((int64_t)bh * kRank + e / kReduceChannels) * kCD + c0 + e % kReduceChannels] = s_out[e / kReduceChannels][e % kReduceChannels];
 }
 
 // TMA store of a [128 rows x 64 columns] bf16 slab from shared memory (rows past the tensor's end are clipped)
@@ -414,6 +441,8 @@ comp_apply_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_const
     tmem_alloc(s_tmem, 512);
     tmem_relinquish();
   }
+  pdl_trigger();
+  pdl_wait();                                      // everything above runs while the kernel before this one drains
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
@@ -511,8 +540,8 @@ comp_apply_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_const
         const float* src = p.state + ((int64_t)bh * kRank + a) * kCD + half * 64;
 #pragma unroll
         for (int c = 0; c < 8; ++c) {
-          const float4 lo = __ldg(reinterpret_cast<const float4*>(src + 8 * c));
-          const float4 hi = __ldg(reinterpret_cast<const float4*>(src + 8 * c + 4));
+          const float4 lo = *reinterpret_cast<const float4*>(src + 8 * c);
+          const float4 hi = *reinterpret_cast<const float4*>(src + 8 * c + 4);
           const __nv_bfloat162 h0 = __floats2bfloat162_rn(lo.x, lo.y), h1 = __floats2bfloat162_rn(lo.z, lo.w);
           const __nv_bfloat162 h2 = __floats2bfloat162_rn(hi.x, hi.y), h3 = __floats2bfloat162_rn(hi.z, hi.w);
           *reinterpret_cast<uint4*>(sC + half * 8192 + a * 128 + ((c ^ (a & 7)) << 4)) =
@@ -529,7 +558,7 @@ comp_apply_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_const
       const int token = tile_row + row;
       float2 cs[kRank / 2];
       rope_factors(cs, p.rope, p.rope_table, min(token, p.N - 1));
-      const float gte = token < p.N ? __ldg(p.gate + (int64_t)bh * p.N + token) : 0.0f;
+      const float gte = token < p.N ? p.gate[(int64_t)bh * p.N + token] : 0.0f;
       ok = __all_sync(0xffffffffu, mbar_wait(bar_t_full + g, u & 1, s_abort, p.status, 64));
       if (!ok) break;
       tc_fence_after();
@@ -639,8 +668,12 @@ static int comp_chunks(const sparkattn_shape_t& s) {
   return best;
 }
 
+int launch_rope_table(const RopeTable& rope, float2* table, int32_t* header, cudaStream_t stream) {
+  return launch_kernel(rope_table_kernel, (unsigned)(rope.T + rope.Hg + rope.Wg), kRank / 2, 0, true, stream, rope, table, header);
+}
+
 int launch_rope_table(const RopeTable& rope, float2* table, cudaStream_t stream) {
-  return launch_kernel(rope_table_kernel, (unsigned)(rope.T + rope.Hg + rope.Wg), kRank / 2, 0, false, stream, rope, table);
+  return launch_rope_table(rope, table, nullptr, stream);
 }
 
 size_t rope_table_bytes(const int32_t* grid) {
@@ -660,8 +693,7 @@ static int prepare_workspace(CompParams& prm, const int32_t* grid, void* workspa
   float2* table = reinterpret_cast<float2*>(base + kWorkspaceHeaderBytes);
   prm.rope_table = table;
   prm.partial = reinterpret_cast<float*>(base + kWorkspaceHeaderBytes + rope_table_bytes(grid));
-  if (cudaMemsetAsync(workspace, 0, kWorkspaceHeaderBytes, stream) != cudaSuccess) return SPARKATTN_E_CUDA;
-  return launch_rope_table(prm.rope, table, stream);
+  return launch_rope_table(prm.rope, table, prm.status, stream);
 }
 
 static void fill_rope(CompParams& prm, const int32_t* grid, const int32_t* axis, const float* freq) {
@@ -686,10 +718,10 @@ int launch_comp_state(const sparkattn_shape_t& s, const void* k, const void* v, 
   if ((rc = prepare_workspace(prm, grid, workspace, stream)) != SPARKATTN_OK) return rc;
   if (cudaFuncSetAttribute(comp_state_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kStateSmem) != cudaSuccess)
     return SPARKATTN_E_CUDA;
-  const dim3 grid_dim((unsigned)prm.nchunks, (unsigned)(s.B * s.H));
-  comp_state_kernel<<<grid_dim, kCompThreads, kStateSmem, stream>>>(mk, mv, mp, prm);
-  comp_reduce_kernel<<<(unsigned)(s.B * s.H), 256, 0, stream>>>(prm.partial, state, prm.nchunks);
-  return cudaGetLastError() == cudaSuccess ? SPARKATTN_OK : SPARKATTN_E_CUDA;
+  const unsigned bh = (unsigned)(s.B * s.H);
+  if ((rc = launch_kernel(comp_state_kernel, dim3((unsigned)prm.nchunks, bh), kCompThreads, kStateSmem, true, stream, mk, mv, mp, prm)) != SPARKATTN_OK)
+    return rc;
+  return launch_kernel(comp_reduce_kernel, bh * (kCD / kReduceChannels), kReduceThreads, 0, true, stream, prm.partial, state, prm.nchunks);
 }
 
 int launch_comp_apply(const sparkattn_shape_t& s, const void* q, const void* pq, const int32_t* grid,
@@ -715,9 +747,8 @@ int launch_comp_apply(const sparkattn_shape_t& s, const void* q, const void* pq,
   if ((rc = prepare_workspace(prm, grid, workspace, stream)) != SPARKATTN_OK) return rc;
   if (cudaFuncSetAttribute(comp_apply_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kApplySmem) != cudaSuccess)
     return SPARKATTN_E_CUDA;
-  const dim3 grid_dim((unsigned)prm.nchunks, (unsigned)(s.B * s.H));
-  comp_apply_kernel<<<grid_dim, kCompThreads, kApplySmem, stream>>>(mq, mp, mos, mout, prm);
-  return cudaGetLastError() == cudaSuccess ? SPARKATTN_OK : SPARKATTN_E_CUDA;
+  return launch_kernel(comp_apply_kernel, dim3((unsigned)prm.nchunks, (unsigned)(s.B * s.H)), kCompThreads, kApplySmem, true, stream, mq,
+                       mp, mos, mout, prm);
 }
 
 }  // namespace sparkattn

@@ -13,10 +13,10 @@ namespace sparkattn {
 // Launches a kernel; with `overlap` it may start while the kernel before it on the stream is draining (it then calls
 // pdl_wait, common.cuh, before it touches memory).
 template <typename... Params, typename... Args>
-inline int launch_kernel(void (*kern)(Params...), unsigned grid, unsigned threads, size_t smem, bool overlap, cudaStream_t stream,
+inline int launch_kernel(void (*kern)(Params...), dim3 grid, unsigned threads, size_t smem, bool overlap, cudaStream_t stream,
                          const Args&... args) {
   cudaLaunchConfig_t cfg{};
-  cfg.gridDim = dim3(grid);
+  cfg.gridDim = grid;
   cfg.blockDim = dim3(threads);
   cfg.dynamicSmemBytes = smem;
   cfg.stream = stream;

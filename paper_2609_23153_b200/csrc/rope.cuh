@@ -17,8 +17,10 @@ struct RopeTable {
 
 // Bytes of the position-major cos / sin table of a (T, Hg, Wg) grid, and the launch that fills it:
 // table[(base(axis) + e) * rank/2 + m] = (cos, sin)(e * freq[m]), base(t) = 0, base(y) = T, base(x) = T + Hg.
+// `header`: a workspace header that the same launch clears.
 size_t rope_table_bytes(const int32_t* grid);
 int launch_rope_table(const RopeTable& rope, float2* table, cudaStream_t stream);
+int launch_rope_table(const RopeTable& rope, float2* table, int32_t* header, cudaStream_t stream);
 
 __device__ __forceinline__ float fast_rcp(float x) {
   float y;

@@ -60,6 +60,17 @@ def test_small_full(grid, H, B, layout):
         _check_out(out[b].cpu(), ref)
 
 
+@pytest.mark.parametrize("tiles,H", [(1, 1), (15, 1), (16, 1), (17, 1), (149, 1), (17, 37)])
+def test_state_over_chunk_counts(tiles, H):
+    """The sum over a head's chunks at the edges of its batches of 16: 1, 15, 16, 17 and (two tiles each) 75 chunks of one
+    head, 4 of 37 heads."""
+    w = workloads.Workload("compchunks", 41 + tiles, 1, H, 128, (1, tiles, 128), 128, 0.5)
+    q, k, v, osp, pq, pk, gate, axis, freq = _inputs(w)
+    state = sa.comp_state(k, v, pk, w.grid, axis, freq, check_status=True)
+    ref = oracle.comp_state(k[0].cpu().contiguous(), v[0].cpu().contiguous(), pk.cpu(), w.grid, axis, freq)
+    assert _relrms(state[0].cpu(), ref) <= 1e-2
+
+
 def test_state_is_deterministic_and_apply_in_place():
     w = workloads.Workload("compdet", 17, 1, 2, 128, (4, 10, 16), 128, 0.5)
     q, k, v, osp, pq, pk, gate, axis, freq = _inputs(w)
