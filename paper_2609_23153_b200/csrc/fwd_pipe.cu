@@ -17,7 +17,9 @@
 //                    warpgroup keeps its own partial row sum relative to the last reference it
 //                    saw; the warpgroup of the item's last tile combines them, normalises O into
 //                    the item's (now dead) Q slot and stores it with one TMA copy.
-//   warp 0           TMA producer (one elected thread issues): Q (2 slots) and the K ring (2 slots; FP8: 4).
+//   warp 0           TMA producer (one elected thread issues): Q (2 slots) and the K ring (2 slots; FP8: 4).  It also leaves
+//                    a descriptor of every tile (real columns, FP8 scales) in a ring in shared memory, so that the
+//                    softmax warps read no lists and no scales and take no logarithms.
 //   warp 3           TMA producer (the same): the V ring (3 slots; FP8: 6).  Each producer sleeps in
 //                    the wait for the slot it fills next (one thread polling all rings with a
 //                    back-off answered a freed slot up to a microsecond late).
@@ -83,7 +85,9 @@ constexpr float kPipeLazyLog2 = 8.0f;        // bf16: P may exceed 1 by up to 2^
 constexpr float kPipeFp8LazyLog2 = 4.0f, kPipeFp8PScaleLog2 = 4.0f;
 constexpr int kTile = 32768;                               // bytes of one 128 x 128 bf16 tile (two 64-column slabs)
 constexpr int kOffQ = 0, kOffK = 2 * kTile, kOffMisc = 7 * kTile;     // Q slots | K ring, V ring (5 x 32 KB) | barriers ...
-constexpr int kPipeSmem = kOffMisc + 512 /*barriers*/ + 2 * 128 * 4 /*reference maxima*/ + 128 * 8 /*row sums*/ + 64;
+constexpr int kTileRing = 8;                               // tile descriptors the K producer leaves for the softmax warpgroups
+constexpr int kPipeSmem = kOffMisc + 512 /*barriers*/ + 2 * 128 * 4 /*reference maxima*/ + 128 * 8 /*row sums*/ + 64 +
+                          kTileRing * 32 /*tile descriptors*/;
 
 // x / d for 0 <= x < 2^31 without the division's twenty-odd instructions at every place that takes an item apart: division
 // by an invariant integer through multiplication, after Granlund and Montgomery
@@ -340,6 +344,15 @@ fwd_pipe_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
   uint32_t* s_tmem = reinterpret_cast<uint32_t*>(s_lsum + 128);
   volatile int* s_abort = reinterpret_cast<volatile int*>(s_tmem + 1);
   volatile int* s_gate_bh = s_abort + 1;      // GATE: (batch, head) whose P_q and C are in shared memory
+  // What the softmax warpgroups need to know of a tile, written by the K producer in the slot tile % 8 before it requests
+  // the K tile: the number of real columns (WINDOW: the key block), PAIR with the flags of the two query blocks in bits
+  // 30 and 31; FP8: K scale, log2 of the factor folded into P, its inverse.  PAIR: the same of the tile's second block.
+  // Tile t's entry is overwritten with tile t + 8's: K of that tile is requested when S of tile t + 8 - RK is complete,
+  // which needs the row of tile t + 6 - RK >= t + 2 in registers.
+  // (Loading list entries two tiles and scales one tile ahead in every softmax thread, and the logarithm there, took 490 us
+  // where this takes 472, FP8, 12 heads of 32,760 tokens, 26 of 256 blocks; 64-token blocks at 40 x 75,600, 97 %, 3602 -> 3513;
+  // plain bf16 546 -> 542.)
+  int* s_desc = reinterpret_cast<int*>(s_lsum + 128) + 16;       // [kTileRing][8]
 
   const int warp = uniform(threadIdx.x >> 5), lane = threadIdx.x & 31;
   constexpr int kTileTx = FP8 ? kTile / 2 : kTile;
@@ -422,6 +435,25 @@ fwd_pipe_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
       const bool is_v = which;
       const int R = is_v ? RV : RK;
       int ord = 0, slot = 0, use = 0;                   // non-empty items seen; ring slot of the next tile and how often the ring has been filled
+      int t = 0;                                        // K: tiles so far
+      struct Desc { int x; float ks, off, inv; };
+      auto describe = [&](int e, int bh, float inv_vmax) {
+        Desc d{};
+        [[maybe_unused]] const int b = e & 0x3fffffff;
+        if constexpr (WINDOW) {
+          d.x = e;
+        } else {
+          d.x = min(p.N - b * kKeyBlk, kKeyBlk);
+          if (p.blk_valid != nullptr) d.x = min(d.x, p.blk_valid[b]);
+          if constexpr (PAIR) d.x = max(d.x, 0) | (e & 0xc0000000);
+        }
+        if constexpr (FP8) {
+          d.ks = p.k_scale[(int64_t)bh * p.nb + b];
+          d.off = kPipeFp8PScaleLog2 + log2f(p.v_scale[(int64_t)bh * p.nb + b] * inv_vmax);
+          d.inv = fast_exp2(-d.off);
+        }
+        return d;
+      };
       int item = first_item;
       const int32_t* lst = p.clean_list + (int64_t)item * p.lstride;
       int cnt = item < p.items ? p.clean_cnt[item] : 0;
@@ -441,6 +473,13 @@ fwd_pipe_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
         if (cnt & kBadFlag) {
           cnt &= ~kBadFlag;
           if (!is_v && lane == 0) report_bad_index(p, item, PAIR);
+        }
+        float inv_vmax = 1.0f;
+        Desc d0{}, d1{};
+        if (!is_v && cnt > 0) {
+          if constexpr (FP8) inv_vmax = 1.0f / p.v_max[bh];
+          d0 = describe(kb, bh, inv_vmax);
+          if constexpr (PAIR) d1 = describe(kb2, bh, inv_vmax);
         }
         if (!is_v && cnt > 0) {
           const int qslot = ord & 1, qb = item - bh * p.nbq;
@@ -469,6 +508,13 @@ fwd_pipe_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
             unsigned char* dst = (is_v ? sV : sK) + slot * kSlot;
             uint64_t* bar = (is_v ? bar_v_full : bar_k_full) + slot;
             const CUtensorMap* map = is_v ? &tmap_v : &tmap_k;
+            if (!is_v) {
+              int* e = s_desc + (t & (kTileRing - 1)) * 8;
+              if constexpr (FP8) *reinterpret_cast<int4*>(e) = make_int4(d0.x, __float_as_int(d0.ks), __float_as_int(d0.off), __float_as_int(d0.inv));
+              else if constexpr (PAIR) *reinterpret_cast<int2*>(e) = make_int2(d0.x, d1.x);
+              else *e = d0.x;
+              if constexpr (FP8 && PAIR) *reinterpret_cast<int4*>(e + 4) = make_int4(d1.x, __float_as_int(d1.ks), __float_as_int(d1.off), __float_as_int(d1.inv));
+            }
             mbar_expect_tx(bar, kTileTx);
             // one K or V tile: 128 key rows of one block, or 64 + 64 rows of the tile's two 64-token blocks
             tma_load_4d(dst, map, bar, 0, r0, hh, bb);
@@ -480,6 +526,11 @@ fwd_pipe_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
           }
           __syncwarp();
           kb = kb_n; kb2 = kb2_n;
+          if (!is_v) {
+            ++t;
+            d0 = describe(kb, bh, inv_vmax);
+            if constexpr (PAIR) d1 = describe(kb2, bh, inv_vmax);
+          }
           if (++slot == R) { slot = 0; ++use; }
         }
         item = nxt;
@@ -586,6 +637,17 @@ fwd_pipe_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
       asm volatile("bar.sync %0, 128;" ::"r"(1 + g) : "memory");
       return true;
     };
+    // The exponentials go in chunks of kChunk columns.  Where the softmax warps bound the kernel (all but plain bf16), the
+    // token is passed after chunk kTokenAfter and not before the first: the two warps of a scheduler otherwise start
+    // their exponentials at the same time, share the special-function unit through all of them and then leave it idle
+    // together; apart, one's maxima run under the other's exponentials.  Passed much later the token itself becomes the
+    // chain.  The wait for the P buffer then stands before the chunks, so that they are one straight piece of code.
+    // 12 heads of 32,760 tokens: FP8, 26 of 256 blocks 472 -> 416 us (token after 32 columns 427, after 64 436, after 96
+    // 532), 64 of 256 1104 -> 987; 64-token blocks, 128 of 512: bf16 1640 -> 1587, FP8 (51 of 512) 678 -> 637.  Plain bf16
+    // runs at the power limit and is as fast either way (538 against 539-542).
+    constexpr bool kApart = FP8 || PAIR;
+    constexpr int kChunk = kApart ? 16 : 32;
+    constexpr int kTokenAfter = !kApart ? -1 : PAIR ? 1 : 0;
     // GATE (a softmax warpgroup closes the item, lists are short): the thread that stores an item's output does not wait
     // until the copy has read the Q slot (about 1300 clocks, on the path to the closing warpgroup's next tile);
     // it releases the slot after its next tile, or, should the item after the next come first (its Q goes into
@@ -632,79 +694,10 @@ fwd_pipe_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
         q_sc = PAIR ? p.q_scale[(int64_t)bh * p.nb + min(2 * qb + (row >> 6), p.nb - 1)] : p.q_scale[item];
         v_max = p.v_max[bh];
       }
-      // This warpgroup's tiles are n0, n0 + 2, ...  List entries are fetched two of its tiles ahead and the FP8
-      // scales of a tile one tile ahead, so that neither load (nor the two in a row, entry then scale) is waited
-      // for inside the tile loop.
-      const int n0 = (g ^ t) & 1;
-      const int32_t* lst = p.clean_list + (int64_t)item * p.lstride;
-      const float* ksc = FP8 ? p.k_scale + (int64_t)bh * p.nb : nullptr;
-      const float* vsc = FP8 ? p.v_scale + (int64_t)bh * p.nb : nullptr;
-      auto ld_ent = [&](int n, int e) { return n < cnt ? lst[n * kEnt + e] : 0; };
-      int e_cur0 = ld_ent(n0, 0), e_cur1 = PAIR ? ld_ent(n0, 1) : 0;
-      int e_nx0 = ld_ent(n0 + 2, 0), e_nx1 = PAIR ? ld_ent(n0 + 2, 1) : 0;
-      float ks_cur0 = 1.0f, vs_cur0 = 1.0f, ks_cur1 = 1.0f, vs_cur1 = 1.0f;
-      int bv_cur = kKeyBlk, bv_cur1 = kKeyBlk;     // real tokens of the tile's key block(s) (bricks padded to whole blocks)
-      if (p.blk_valid != nullptr) {
-        bv_cur = p.blk_valid[e_cur0 & 0x3fffffff];
-        if constexpr (PAIR) bv_cur1 = p.blk_valid[e_cur1 & 0x3fffffff];
-      }
-      if constexpr (FP8) {
-        ks_cur0 = ksc[e_cur0 & 0x3fffffff];
-        vs_cur0 = vsc[e_cur0 & 0x3fffffff];
-        if constexpr (PAIR) {
-          ks_cur1 = ksc[e_cur1 & 0x3fffffff];
-          vs_cur1 = vsc[e_cur1 & 0x3fffffff];
-        }
-      }
-      const float inv_vmax = 1.0f / v_max;
+      const int n0 = (g ^ t) & 1;                       // this warpgroup's tiles are n0, n0 + 2, ...
       for (int n = n0; ok && n < cnt; n += 2) {
         const int tt = t + n;
         const int buf = g;                          // (tt & 1) == g: this warpgroup's S and P buffers
-        // the tile's key block(s); PAIR: two 64-token blocks, each with a flag per query block of the pair
-        const int e0 = e_cur0, e1 = e_cur1;
-        const float ks0 = ks_cur0, vs0 = vs_cur0, ks1 = ks_cur1, vs1 = vs_cur1;
-        const int bv0 = bv_cur, bv1 = bv_cur1;
-        if (p.blk_valid != nullptr) {
-          bv_cur = p.blk_valid[e_nx0 & 0x3fffffff];
-          if constexpr (PAIR) bv_cur1 = p.blk_valid[e_nx1 & 0x3fffffff];
-        }
-        // next tile of this warpgroup: its scales (its entries arrived a tile ago), and the entries of the one after
-        if constexpr (FP8) {
-          ks_cur0 = ksc[e_nx0 & 0x3fffffff];
-          vs_cur0 = vsc[e_nx0 & 0x3fffffff];
-          if constexpr (PAIR) {
-            ks_cur1 = ksc[e_nx1 & 0x3fffffff];
-            vs_cur1 = vsc[e_nx1 & 0x3fffffff];
-          }
-        }
-        e_cur0 = e_nx0; e_cur1 = e_nx1;
-        e_nx0 = ld_ent(n + 4, 0);
-        if constexpr (PAIR) e_nx1 = ld_ent(n + 4, 1);
-        int kb, kb1 = 0;
-        bool mem0 = true, mem1 = true;
-        if constexpr (PAIR) {
-          kb = e0 & 0x3fffffff;
-          kb1 = e1 & 0x3fffffff;
-          mem0 = (((uint32_t)e0 >> (30 + (row >> 6))) & 1u) != 0u;
-          mem1 = (((uint32_t)e1 >> (30 + (row >> 6))) & 1u) != 0u;
-        } else {
-          kb = e0;
-        }
-        float c = p.scale_log2;                      // logit -> log2 units
-        float p_off = 0.0f;                          // log2 of the factor folded into P
-        float c1 = c, p_off1 = 0.0f;                 // PAIR + FP8: the second key block of the tile has its own scales
-        if constexpr (FP8) {
-          c *= q_sc * ks0;
-          p_off = kPipeFp8PScaleLog2 + log2f(vs0 * inv_vmax);
-          if constexpr (PAIR) {
-            c1 *= q_sc * ks1;
-            p_off1 = kPipeFp8PScaleLog2 + log2f(vs1 * inv_vmax);
-          }
-        }
-        // this row's valid columns: [c_lo, c_hi) of the tile, or (PAIR) [c_lo, c_hi) of its first 64 and
-        // [c_lo1, c_hi1) of its second 64 columns (empty when the block is not in this query block's list)
-        const int c_lo = klo - kb * kKeyBlk, c_hi = PAIR ? (mem0 ? min(khi - kb * 64, bv0) : 0) : min(khi - kb * kPBLK, bv0);
-        const int c_lo1 = klo - kb1 * 64, c_hi1 = mem1 ? min(khi - kb1 * 64, bv1) : 0;
         ok = __all_sync(0xffffffffu, pipe_wait(bar_s_full + buf, (tt >> 1) & 1, s_abort, 4));
         if (!ok) break;
         tc_fence_after();
@@ -712,6 +705,52 @@ fwd_pipe_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
         uint32_t sr[kPBLK];
 #pragma unroll
         for (int ch = 0; ch < kPBLK / 32; ++ch) tmem_ld32(tS + ch * 32, *reinterpret_cast<uint32_t(*)[32]>(&sr[ch * 32]));
+        // the tile's descriptor (see s_desc)
+        const volatile int* desc = s_desc + (tt & (kTileRing - 1)) * 8;
+        int x0, x1 = 0;
+        float c = p.scale_log2, p_off = 0.0f, p_inv = 1.0f;       // logit -> log2 units; log2 of the factor folded into P; its inverse
+        float c1 = c, p_off1 = 0.0f, p_inv1 = 1.0f;               // PAIR + FP8: the second key block of the tile has its own scales
+        if constexpr (FP8) {
+          const int4 e = *reinterpret_cast<const int4*>(const_cast<const int*>(desc));
+          x0 = e.x;
+          c *= q_sc * __int_as_float(e.y);
+          p_off = __int_as_float(e.z);
+          p_inv = __int_as_float(e.w);
+          if constexpr (PAIR) {
+            const int4 f = *reinterpret_cast<const int4*>(const_cast<const int*>(desc + 4));
+            x1 = f.x;
+            c1 *= q_sc * __int_as_float(f.y);
+            p_off1 = __int_as_float(f.z);
+            p_inv1 = __int_as_float(f.w);
+          }
+        } else if constexpr (PAIR) {
+          x0 = desc[0];
+          x1 = desc[1];
+        } else {
+          x0 = desc[0];
+        }
+        // this row's valid columns: [c_lo, c_hi) of the tile, or (PAIR) [c_lo, c_hi) of its first 64 and
+        // [c_lo1, c_hi1) of its second 64 columns (empty when the block is not in this query block's list)
+        int c_lo = 0, c_hi, c_lo1 = 0, c_hi1 = kKeyBlk;
+        bool mem0 = true, mem1 = true;
+        if constexpr (PAIR) {
+          mem0 = (((uint32_t)x0 >> (30 + (row >> 6))) & 1u) != 0u;
+          mem1 = (((uint32_t)x1 >> (30 + (row >> 6))) & 1u) != 0u;
+          x0 &= 0x3fffffff;
+          x1 &= 0x3fffffff;
+        }
+        if constexpr (WINDOW) {
+          c_lo = klo - x0 * kKeyBlk;
+          c_hi = khi - x0 * kKeyBlk;
+          if constexpr (PAIR) { c_lo1 = klo - x1 * 64; c_hi1 = khi - x1 * 64; }
+        } else {
+          c_hi = x0;
+          if constexpr (PAIR) c_hi1 = x1;
+        }
+        if constexpr (PAIR) {
+          if (!mem0) c_hi = 0;
+          if (!mem1) c_hi1 = 0;
+        }
         tc_wait_ld();
         tc_fence_before();
         mbar_arrive(bar_s_free + buf);    // the S buffer can take the next-but-one tile
@@ -754,6 +793,10 @@ fwd_pipe_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
           m_tile = fmaxf(ma * c, mb * c1);
         }
 
+        auto pass_token = [&]() {
+          s_mref[g * 128 + row] = m_used;
+          mbar_arrive(bar_tok + g);
+        };
         // reference maximum: token from the warpgroup of tile tt-1 (also orders the reuse of s_mref[g])
         if (tt > 0) {
           ok = __all_sync(0xffffffffu, pipe_wait(bar_tok + (g ^ 1), ((tt - 1) >> 1) & 1, s_abort, 5));
@@ -808,8 +851,7 @@ fwd_pipe_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
           tc_wait_st();
           tc_fence_before();
         }
-        s_mref[g * 128 + row] = m_used;
-        mbar_arrive(bar_tok + g);
+        if constexpr (kTokenAfter < 0) pass_token();
 
         // P = exp2(S*c - m) as bf16 into this warpgroup's P buffer
         const uint32_t tP = tmem_P + buf * 64 + lane_off;
@@ -818,17 +860,21 @@ fwd_pipe_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
         const uint64_t c2a = pack_f32x2(c, c), nm2a = pack_f32x2(neg_m, neg_m);
         const uint64_t c2b = pack_f32x2(c1, c1), nm2b = pack_f32x2(neg_m1, neg_m1);
         uint64_t lsum0 = pack_f32x2(0.0f, 0.0f), lsum1 = lsum0;
-        constexpr int kWords = FP8 ? 8 : 16;        // 32-bit words of P per 32 S columns
+        auto wait_p = [&]() {      // this warpgroup's P buffer is free once PV of tile tt-2 is complete (normally long ago)
+          if (tt >= 2) ok = __all_sync(0xffffffffu, pipe_wait(bar_pv_done + buf, ((tt >> 1) - 1) & 1, s_abort, 11));
+        };
+        if constexpr (kApart) wait_p();
+        constexpr int kWords = FP8 ? kChunk / 4 : kChunk / 2;        // 32-bit words of P per chunk
 #pragma unroll
-        for (int ch = 0; ch < kPBLK / 32; ++ch) {
+        for (int ch = 0; ch < kPBLK / kChunk; ++ch) {
           uint32_t w[kWords];
-          float e[32];
-          const bool second = PAIR && FP8 && ch >= 2;       // the tile's second key block: its own scales, its own sum
+          float e[kChunk];
+          const bool second = PAIR && FP8 && ch >= 64 / kChunk;       // the tile's second key block: its own scales, its own sum
           const uint64_t c2 = second ? c2b : c2a, nm2 = second ? nm2b : nm2a;
 #pragma unroll
-          for (int i = 0; i < 32; i += 2) {
+          for (int i = 0; i < kChunk; i += 2) {
             const float2 x = unpack_f32x2(
-                ffma2(pack_f32x2(__uint_as_float(sr[ch * 32 + i]), __uint_as_float(sr[ch * 32 + i + 1])), c2, nm2));
+                ffma2(pack_f32x2(__uint_as_float(sr[ch * kChunk + i]), __uint_as_float(sr[ch * kChunk + i + 1])), c2, nm2));
             e[i] = fast_exp2(x.x);
             e[i + 1] = fast_exp2(x.y);
             if ((PAIR && FP8) ? second : (((i >> 1) & 1) != 0)) lsum1 = fadd2(lsum1, pack_f32x2(e[i], e[i + 1]));
@@ -836,31 +882,32 @@ fwd_pipe_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
           }
           if constexpr (FP8) {
 #pragma unroll
-            for (int i = 0; i < 8; ++i) {
+            for (int i = 0; i < kWords; ++i) {
               const uint32_t lo = __nv_cvt_float2_to_fp8x2(make_float2(e[4 * i], e[4 * i + 1]), __NV_SATFINITE, __NV_E4M3);
               const uint32_t hi = __nv_cvt_float2_to_fp8x2(make_float2(e[4 * i + 2], e[4 * i + 3]), __NV_SATFINITE, __NV_E4M3);
               w[i] = lo | (hi << 16);
             }
           } else {
 #pragma unroll
-            for (int i = 0; i < 16; ++i) {
+            for (int i = 0; i < kWords; ++i) {
               const __nv_bfloat162 h2 = __floats2bfloat162_rn(e[2 * i], e[2 * i + 1]);
               w[i] = *reinterpret_cast<const uint32_t*>(&h2);
             }
           }
-          if (ch == 0 && tt >= 2) {
-            // this warpgroup's P buffer is free once PV of tile tt-2 is complete (normally long ago)
-            ok = __all_sync(0xffffffffu, pipe_wait(bar_pv_done + buf, ((tt >> 1) - 1) & 1, s_abort, 11));
+          if constexpr (!kApart) {
+            if (ch == 0) wait_p();
           }
-          if constexpr (FP8) tmem_st8(tP + ch * 8, w);
-          else tmem_st16(tP + ch * 16, w);
+          if constexpr (kWords == 4) tmem_st4(tP + ch * kWords, w);
+          else if constexpr (kWords == 8) tmem_st8(tP + ch * kWords, w);
+          else tmem_st16(tP + ch * kWords, w);
+          if (ch == kTokenAfter) pass_token();
         }
         if constexpr (PAIR && FP8) {       // the row sum is kept without the factors folded into P, one per key block
           const float2 la = unpack_f32x2(lsum0), lb = unpack_f32x2(lsum1);
-          l += (la.x + la.y) * fast_exp2(-p_off) + (lb.x + lb.y) * fast_exp2(-p_off1);
+          l += (la.x + la.y) * p_inv + (lb.x + lb.y) * p_inv1;
         } else {
           const float2 ls = unpack_f32x2(fadd2(lsum0, lsum1));
-          if constexpr (FP8) l += (ls.x + ls.y) * fast_exp2(-p_off);
+          if constexpr (FP8) l += (ls.x + ls.y) * p_inv;
           else l += ls.x + ls.y;
         }
         tc_wait_st();

@@ -335,6 +335,40 @@ def test_both_kernels_agree_bitwise(block, window, fp8, stride):
         _compare_items(b[0], None if window else lb[0], ref_out, ref_lse, items, w.block, w.N, BF16_RELRMS, BF16_MAXABS)
 
 
+@pytest.mark.parametrize("block,fp8,window", [(128, True, 0), (64, True, 0), (64, True, 3), (128, True, 3), (128, False, 0), (64, False, 3)])
+def test_tile_descriptors_around_their_ring(block, fp8, window):
+    """The K producer hands the softmax warps a descriptor per tile through a ring of eight: items of 7, 8, 9, 15, 16 and 17
+    tiles, eight or more of them per CTA, so that every item starts somewhere else in the ring; K and V blocks of
+    different magnitude, so that a descriptor of another tile gives another result."""
+    grid = (15, 18, 19)                                        # N = 5130: 41 blocks of 128 (last: 10 tokens) / 81 of 64
+    w = _small(91 + block + window + int(fp8), 30, 128, grid, block, 0.0)
+    q, k, v = workloads.structured_qkv(w)
+    g = torch.Generator().manual_seed(700 + block + window)
+    size = lambda: (2.0 ** torch.randint(-1, 2, (w.H, w.nb), generator=g)).repeat_interleave(block, 1)[None, :, : w.N, None]
+    k, v = (k * size()).to(torch.bfloat16), (v * size()).to(torch.bfloat16)
+    per = 128 // block
+    kmax = 17 * per
+    own = torch.arange(w.nb)[None, :, None].expand(w.H, w.nb, 1)
+    idx = torch.stack([torch.stack([torch.randperm(w.nb, generator=g)[:kmax] for _ in range(w.nb)]) for _ in range(w.H)])
+    idx = torch.where((idx == own).any(-1, keepdim=True), idx, torch.cat([own, idx[..., 1:]], -1)).to(torch.int32)
+    cnt = (torch.tensor([7, 8, 9, 15, 16, 17])[torch.randint(0, 6, (w.H, w.nb), generator=g)] * per).to(torch.int32)
+    idx[..., 0], keep = idx.gather(-1, (idx == own).int().argmax(-1, keepdim=True))[..., 0], idx[..., 0].clone()
+    at = (idx[..., 1:] == own).int()                           # the own block comes first, what stood there takes its place
+    idx[..., 1:] = torch.where(at.bool(), keep[..., None], idx[..., 1:])
+    qd, kd, vd = q.to(DEV), k.to(DEV), v.to(DEV)
+    kw = dict(frame_tokens=18 * 19, window=window) if window else {}
+    okw = dict(kw)
+    if fp8:
+        cs = [sa.quant_fp8(t, block) for t in (qd, kd, vd)]
+        qd, kd, vd = (c for c, _ in cs)
+        kw["scales"] = tuple(s for _, s in cs)
+        okw["scales"] = tuple(s[0].cpu() for _, s in cs)
+    out = sa.fwd(qd, kd, vd, idx[None].to(DEV), cnt[None].to(DEV), block, check_status=True, **kw)
+    items = [(h, i) for h in (0, w.H // 2, w.H - 1) for i in list(range(0, w.nb, 7)) + [w.nb - 1]]
+    ref, _ = oracle.attention(qd[0].cpu(), kd[0].cpu(), vd[0].cpu(), idx, cnt, block, items=items, **okw)
+    _compare_items(out[0], None, ref, None, items, block, w.N, FP8_RELRMS if fp8 else BF16_RELRMS, None)
+
+
 def _stream_of_short_items(streams, block, stride, H=16, N=74 * 128 - 17):
     """Kept lists whose item i has streams[i % SMs % len][i // SMs % 8] tiles: what the persistent kernel's CTA c works
     through (items c, c + SMs, ...).  Both query blocks of a 64-token pair keep the same blocks."""
