@@ -1,10 +1,11 @@
 """Python binding of the sparkattn C-ABI library (``libsparkattn.so``).
 
-Argument marshalling only: every step of the path (block selection, FP8
-quantisation, block-sparse attention) runs in the CUDA kernels behind the
-``extern "C"`` entry points declared in ``include/sparkattn.h``.  PyTorch is
-used for device memory and streams.  There is no CPU fallback: if the shared
-library is missing or cannot be loaded, every call raises.
+Argument marshalling only, for the per-layer calls in native code
+(``_sparkattn.so``, ``csrc/binding.cpp``), for the others through ctypes: every
+step of the path (block selection, FP8 quantisation, block-sparse attention)
+runs in the CUDA kernels behind the ``extern "C"`` entry points declared in
+``include/sparkattn.h``.  PyTorch is used for device memory and streams.  There
+is no CPU fallback: if the shared library is missing or cannot be loaded, every call raises.
 """
 from __future__ import annotations
 
@@ -62,12 +63,19 @@ class SparkAttnError(RuntimeError):
         super().__init__(f"{where}: {status_string(status)} ({status})")
 
 
+# What the native marshalling of the per-layer calls (csrc/binding.cpp) calls, in its order.
+_BOUND = ("workspace_bytes", "select", "select_window", "select_padded", "select_pooled", "quant_fp8", "quant_fp8_pooled",
+          "quant_fp8_per_token", "fwd", "fwd_window", "fwd_padded", "gather_tokens", "comp_workspace_bytes", "comp_state", "comp_apply",
+          "fwd_gated_workspace_bytes", "fwd_gated")
+_NO_WORKSPACE = 1        # the library does not serve the shape: the workspace query returned 0
+
 _lib = None
+_native = None
 
 
 def lib() -> ctypes.CDLL:
     """Loads the shared library (once).  Raises if it has not been built."""
-    global _lib
+    global _lib, _native
     if _lib is None:
         if not os.path.exists(LIB_PATH):
             raise ImportError(
@@ -129,8 +137,17 @@ def lib() -> ctypes.CDLL:
         L.sparkattn_fwd_gated.restype = ctypes.c_int
         L.sparkattn_fwd_gated.argtypes = [sp, vp, vp, vp, vp, vp, i32, vp, i32, vp, vp, vp, vp, vp, ctypes.c_float, vp,
                                           vp, vp, sz, vp]
+        from . import _sparkattn
+        _sparkattn.bind(*(ctypes.cast(getattr(L, "sparkattn_" + name), vp).value for name in _BOUND))
+        _native = _sparkattn
         _lib = L
     return _lib
+
+
+def _calls():
+    if _lib is None:
+        lib()
+    return _native
 
 
 def status_string(status: int) -> str:
@@ -139,6 +156,8 @@ def status_string(status: int) -> str:
 
 def _check(rc: int, where: str) -> None:
     if rc != OK:
+        if rc == _NO_WORKSPACE:
+            raise SparkAttnError(E_UNSUPPORTED_SHAPE, "sparkattn_workspace_bytes")
         raise SparkAttnError(rc, where)
 
 
@@ -195,32 +214,13 @@ def select(q: torch.Tensor, k: torch.Tensor, block: int, topk: int, *,
     """``sparkattn_select`` (``sparkattn_select_window`` when ``frame_tokens`` > 0, ``sparkattn_select_padded``
     with ``block_valid``, device int32 [nb]): q, k bf16 [B,H,N,d] on the device -> (kept_idx int32
     [B,H,nb,topk] ascending, kept_cnt int32 [B,H,nb])."""
-    _same_layout(q, k)
-    shape = make_shape(q, block)
-    B, H, N, _ = q.shape
-    nb = (N + block - 1) // block
-    if kept_idx is None:
-        kept_idx = torch.empty((B, H, nb, max(topk, 1)), dtype=torch.int32, device=q.device)
-    if kept_cnt is None:
-        kept_cnt = torch.empty((B, H, nb), dtype=torch.int32, device=q.device)
-    if workspace is None:
-        workspace = alloc_workspace(shape, 0, topk, q.device)
-    if block_valid is not None:
-        if frame_tokens > 0:
-            raise ValueError("block_valid and a causal window cannot be combined")
-        rc = lib().sparkattn_select_padded(ctypes.byref(shape), _ptr(q), _ptr(k), topk, _ptr(block_valid), _ptr(kept_idx),
-                                           _ptr(kept_cnt), _ptr(workspace), workspace.numel(), _stream_ptr(stream))
-        _check(rc, "sparkattn_select_padded")
-        return kept_idx, kept_cnt
-    if frame_tokens > 0:
-        rc = lib().sparkattn_select_window(ctypes.byref(shape), _ptr(q), _ptr(k), topk, frame_tokens, window,
-                                           _ptr(kept_idx), _ptr(kept_cnt), _ptr(workspace), workspace.numel(),
-                                           _stream_ptr(stream))
-        _check(rc, "sparkattn_select_window")
-        return kept_idx, kept_cnt
-    rc = lib().sparkattn_select(ctypes.byref(shape), _ptr(q), _ptr(k), topk, _ptr(kept_idx), _ptr(kept_cnt),
-                                _ptr(workspace), workspace.numel(), _stream_ptr(stream))
-    _check(rc, "sparkattn_select")
+    if block_valid is not None and frame_tokens > 0:
+        raise ValueError("block_valid and a causal window cannot be combined")
+    rc, kept_idx, kept_cnt = _calls().select(q, k, block, topk, kept_idx, kept_cnt, workspace,
+                                             None if stream is None else stream.cuda_stream, frame_tokens, window, block_valid)
+    if rc != OK:
+        _check(rc, "sparkattn_select_padded" if block_valid is not None else
+               "sparkattn_select_window" if frame_tokens > 0 else "sparkattn_select")
     return kept_idx, kept_cnt
 
 
@@ -242,14 +242,7 @@ def quant_fp8(x: torch.Tensor, block: int, *, codes: Optional[torch.Tensor] = No
               scales: Optional[torch.Tensor] = None, stream: Optional[torch.cuda.Stream] = None,
               ) -> Tuple[torch.Tensor, torch.Tensor]:
     """``sparkattn_quant_fp8``: x bf16 [B,H,N,d] -> (codes uint8, same strides; scales fp32 [B,H,nb])."""
-    shape = make_shape(x, block)
-    B, H, N, _ = x.shape
-    nb = (N + block - 1) // block
-    if codes is None:
-        codes = torch.empty_strided(x.shape, x.stride(), dtype=torch.uint8, device=x.device)
-    if scales is None:
-        scales = torch.empty((B, H, nb), dtype=torch.float32, device=x.device)
-    rc = lib().sparkattn_quant_fp8(ctypes.byref(shape), _ptr(x), _ptr(codes), _ptr(scales), 0, _stream_ptr(stream))
+    rc, codes, scales = _calls().quant(x, block, -1, None, codes, scales, None if stream is None else stream.cuda_stream)
     _check(rc, "sparkattn_quant_fp8")
     return codes, scales
 
@@ -259,15 +252,8 @@ def quant_fp8_pooled(x: torch.Tensor, block: int, key_side: bool, select_workspa
                      stream: Optional[torch.cuda.Stream] = None) -> Tuple[torch.Tensor, torch.Tensor]:
     """``sparkattn_quant_fp8_pooled``: :func:`quant_fp8` that also leaves the pooled block means of ``x`` (the query
     tensor, or the key tensor with ``key_side``) in ``select_workspace`` for :func:`select_pooled`."""
-    shape = make_shape(x, block)
-    B, H, N, _ = x.shape
-    nb = (N + block - 1) // block
-    if codes is None:
-        codes = torch.empty_strided(x.shape, x.stride(), dtype=torch.uint8, device=x.device)
-    if scales is None:
-        scales = torch.empty((B, H, nb), dtype=torch.float32, device=x.device)
-    rc = lib().sparkattn_quant_fp8_pooled(ctypes.byref(shape), _ptr(x), _ptr(codes), _ptr(scales), 1 if key_side else 0,
-                                          _ptr(select_workspace), select_workspace.numel(), _stream_ptr(stream))
+    rc, codes, scales = _calls().quant(x, block, 1 if key_side else 0, select_workspace, codes, scales,
+                                       None if stream is None else stream.cuda_stream)
     _check(rc, "sparkattn_quant_fp8_pooled")
     return codes, scales
 
@@ -277,15 +263,8 @@ def select_pooled(ref: torch.Tensor, block: int, topk: int, workspace: torch.Ten
                   stream: Optional[torch.cuda.Stream] = None) -> Tuple[torch.Tensor, torch.Tensor]:
     """``sparkattn_select_pooled``: scores + top-k on the pooled means two :func:`quant_fp8_pooled` calls left in
     ``workspace``; ``ref`` is any [B,H,N,d] tensor of the problem (for the shape)."""
-    shape = make_shape(ref, block)
-    B, H, N, _ = ref.shape
-    nb = (N + block - 1) // block
-    if kept_idx is None:
-        kept_idx = torch.empty((B, H, nb, max(topk, 1)), dtype=torch.int32, device=ref.device)
-    if kept_cnt is None:
-        kept_cnt = torch.empty((B, H, nb), dtype=torch.int32, device=ref.device)
-    rc = lib().sparkattn_select_pooled(ctypes.byref(shape), topk, _ptr(kept_idx), _ptr(kept_cnt), _ptr(workspace),
-                                       workspace.numel(), _stream_ptr(stream))
+    rc, kept_idx, kept_cnt = _calls().select_pooled(ref, block, topk, workspace, kept_idx, kept_cnt,
+                                                    None if stream is None else stream.cuda_stream)
     _check(rc, "sparkattn_select_pooled")
     return kept_idx, kept_cnt
 
@@ -294,13 +273,7 @@ def quant_fp8_per_token(x: torch.Tensor, *, codes: Optional[torch.Tensor] = None
                         scales: Optional[torch.Tensor] = None, stream: Optional[torch.cuda.Stream] = None,
                         ) -> Tuple[torch.Tensor, torch.Tensor]:
     """``sparkattn_quant_fp8_per_token``: x bf16 [B,H,N,d] -> (codes uint8, same strides; scales fp32 [B,H,N])."""
-    shape = make_shape(x, 64 if x.shape[-1] == 64 else 128)
-    B, H, N, _ = x.shape
-    if codes is None:
-        codes = torch.empty_strided(x.shape, x.stride(), dtype=torch.uint8, device=x.device)
-    if scales is None:
-        scales = torch.empty((B, H, N), dtype=torch.float32, device=x.device)
-    rc = lib().sparkattn_quant_fp8_per_token(ctypes.byref(shape), _ptr(x), _ptr(codes), _ptr(scales), _stream_ptr(stream))
+    rc, codes, scales = _calls().quant(x, 0, -1, None, codes, scales, None if stream is None else stream.cuda_stream)
     _check(rc, "sparkattn_quant_fp8_per_token")
     return codes, scales
 
@@ -316,31 +289,12 @@ def fwd(q: torch.Tensor, k: torch.Tensor, v: torch.Tensor, kept_idx: torch.Tenso
     ``block_valid``, device int32 [nb]).  bf16 q,k,v, or uint8
     E4M3 codes with ``scales=(q_scale, k_scale, v_scale)``.  Returns out bf16 [B,H,N,d] (and lse
     fp32 [B,H,N])."""
-    _same_layout(q, k, v)
-    shape = make_shape(q, block, softmax_scale)
-    B, H, N, _ = q.shape
-    dtype = BF16 if scales is None else FP8_E4M3
-    kmax = kept_idx.shape[-1]
-    if out is None:
-        out = torch.empty_strided(q.shape, q.stride(), dtype=torch.bfloat16, device=q.device)
-    lse = torch.empty((B, H, N), dtype=torch.float32, device=q.device) if return_lse else None
-    if workspace is None:
-        workspace = alloc_workspace(shape, 1, kmax, q.device)
+    if block_valid is not None and frame_tokens > 0:
+        raise ValueError("block_valid and a causal window cannot be combined")
     sq, sk, sv = scales if scales is not None else (None, None, None)
-    if block_valid is not None:
-        if frame_tokens > 0:
-            raise ValueError("block_valid and a causal window cannot be combined")
-        rc = lib().sparkattn_fwd_padded(ctypes.byref(shape), dtype, _ptr(q), _ptr(k), _ptr(v), _ptr(sq), _ptr(sk), _ptr(sv),
-                                        _ptr(kept_idx), _ptr(kept_cnt), kmax, _ptr(block_valid), _ptr(out), _ptr(lse),
-                                        _ptr(workspace), workspace.numel(), _stream_ptr(stream))
-    elif frame_tokens > 0:
-        rc = lib().sparkattn_fwd_window(ctypes.byref(shape), dtype, _ptr(q), _ptr(k), _ptr(v), _ptr(sq), _ptr(sk),
-                                        _ptr(sv), _ptr(kept_idx), _ptr(kept_cnt), kmax, frame_tokens, window,
-                                        _ptr(out), _ptr(lse), _ptr(workspace), workspace.numel(), _stream_ptr(stream))
-    else:
-        rc = lib().sparkattn_fwd(ctypes.byref(shape), dtype, _ptr(q), _ptr(k), _ptr(v), _ptr(sq), _ptr(sk), _ptr(sv),
-                                 _ptr(kept_idx), _ptr(kept_cnt), kmax, _ptr(out), _ptr(lse), _ptr(workspace),
-                                 workspace.numel(), _stream_ptr(stream))
+    rc, out, lse, workspace = _calls().fwd(q, k, v, kept_idx, kept_cnt, block, BF16 if scales is None else FP8_E4M3, sq, sk, sv,
+                                           softmax_scale, out, return_lse, workspace,
+                                           None if stream is None else stream.cuda_stream, frame_tokens, window, block_valid)
     _check(rc, "sparkattn_fwd")
     if check_status:
         _check(read_status(workspace, stream), "sparkattn_fwd (device status)")
@@ -370,17 +324,7 @@ def gather_tokens(x: torch.Tensor, index: torch.Tensor, *, out: Optional[torch.T
                   check_status: bool = False) -> torch.Tensor:
     """``sparkattn_gather_tokens``: out[b,h,i,:] = x[b,h,index[i],:] (zero row for index -1); x bf16 [B,H,N,d],
     index int32 [N_out] on the device, out bf16 [B,H,N_out,d]."""
-    blk = 64 if x.shape[-1] == 64 else 128
-    B, H, _, d = x.shape
-    if index.dtype != torch.int32 or index.dim() != 1 or not index.is_contiguous():
-        raise ValueError("index must be a contiguous 1-D int32 tensor")
-    if out is None:
-        out = torch.empty((B, H, index.numel(), d), dtype=x.dtype, device=x.device)
-    src, dst = make_shape(x, blk), make_shape(out, blk)
-    if workspace is None:
-        workspace = torch.empty(256, dtype=torch.uint8, device=x.device)
-    rc = lib().sparkattn_gather_tokens(ctypes.byref(src), _ptr(x), ctypes.byref(dst), _ptr(index), _ptr(out), _ptr(workspace),
-                                       workspace.numel(), _stream_ptr(stream))
+    rc, out, workspace = _calls().gather_tokens(x, index, out, workspace, None if stream is None else stream.cuda_stream)
     _check(rc, "sparkattn_gather_tokens")
     if check_status:
         _check(read_status(workspace, stream), "sparkattn_gather_tokens (device status)")
@@ -411,15 +355,6 @@ def attention_host(q: torch.Tensor, k: torch.Tensor, v: torch.Tensor, block: int
     return out
 
 
-def _rope_host(grid, axis: torch.Tensor, freq: torch.Tensor):
-    g = (ctypes.c_int32 * 3)(*[int(x) for x in grid])
-    a = axis.detach().to("cpu", torch.int32).contiguous()
-    f = freq.detach().to("cpu", torch.float32).contiguous()
-    if a.numel() != f.numel():
-        raise ValueError("rope axis and frequency tables must have rank/2 entries each")
-    return g, a, f
-
-
 def comp_workspace_bytes(shape: Shape, grid) -> int:
     g = (ctypes.c_int32 * 3)(*[int(x) for x in grid])
     return int(lib().sparkattn_comp_workspace_bytes(ctypes.byref(shape), g))
@@ -430,19 +365,9 @@ def comp_state(k: torch.Tensor, v: torch.Tensor, pk: torch.Tensor, grid, axis: t
                stream: Optional[torch.cuda.Stream] = None, check_status: bool = False) -> torch.Tensor:
     """``sparkattn_comp_state``: k, v bf16 [B,H,N,d]; pk bf16 [H,r,d]; grid (T,Hg,Wg); axis/freq the
     rotary tables (rank/2 entries, any device).  Returns the state fp32 [B,H,r,d]."""
-    _same_layout(k, v)
-    shape = make_shape(k, 128)
-    B, H, _, d = k.shape
-    rank = pk.shape[1]
-    g, a, f = _rope_host(grid, axis, freq)
-    if not pk.is_contiguous() or pk.shape != (H, rank, d):
-        raise ValueError("pk must be contiguous [H, rank, d]")
-    if state is None:
-        state = torch.empty((B, H, rank, d), dtype=torch.float32, device=k.device)
-    if workspace is None:
-        workspace = torch.empty(max(comp_workspace_bytes(shape, grid), 256), dtype=torch.uint8, device=k.device)
-    rc = lib().sparkattn_comp_state(ctypes.byref(shape), _ptr(k), _ptr(v), _ptr(pk), rank, g, _ptr(a), _ptr(f),
-                                    _ptr(state), _ptr(workspace), workspace.numel(), _stream_ptr(stream))
+    T, Hg, Wg = grid
+    rc, state, workspace = _calls().comp_state(k, v, pk, int(T), int(Hg), int(Wg), axis, freq, state, workspace,
+                                               None if stream is None else stream.cuda_stream)
     _check(rc, "sparkattn_comp_state")
     if check_status:
         _check(read_status(workspace, stream), "sparkattn_comp_state (device status)")
@@ -455,24 +380,9 @@ def comp_apply(q: torch.Tensor, pq: torch.Tensor, state: torch.Tensor, gate: tor
                stream: Optional[torch.cuda.Stream] = None, check_status: bool = False) -> torch.Tensor:
     """``sparkattn_comp_apply``: q, o_sparse bf16 [B,H,N,d]; pq bf16 [H,r,d]; state fp32 [B,H,r,d];
     gate fp32 [B,H,N].  Returns the fused output bf16 [B,H,N,d]."""
-    _same_layout(q, o_sparse)
-    shape = make_shape(q, 128)
-    B, H, N, d = q.shape
-    rank = pq.shape[1]
-    g, a, f = _rope_host(grid, axis, freq)
-    if not pq.is_contiguous() or pq.shape != (H, rank, d):
-        raise ValueError("pq must be contiguous [H, rank, d]")
-    if not state.is_contiguous() or state.shape != (B, H, rank, d) or state.dtype != torch.float32:
-        raise ValueError("state must be contiguous fp32 [B, H, rank, d]")
-    if not gate.is_contiguous() or gate.shape != (B, H, N) or gate.dtype != torch.float32:
-        raise ValueError("gate must be contiguous fp32 [B, H, N]")
-    if out is None:
-        out = torch.empty_strided(q.shape, q.stride(), dtype=torch.bfloat16, device=q.device)
-    if workspace is None:
-        workspace = torch.empty(max(comp_workspace_bytes(shape, grid), 256), dtype=torch.uint8, device=q.device)
-    rc = lib().sparkattn_comp_apply(ctypes.byref(shape), _ptr(q), _ptr(pq), rank, g, _ptr(a), _ptr(f), _ptr(state),
-                                    _ptr(gate), _ptr(o_sparse), _ptr(out), ctypes.c_float(eps), _ptr(workspace),
-                                    workspace.numel(), _stream_ptr(stream))
+    T, Hg, Wg = grid
+    rc, out, workspace = _calls().comp_apply(q, pq, state, gate, o_sparse, int(T), int(Hg), int(Wg), axis, freq, eps, out, workspace,
+                                             None if stream is None else stream.cuda_stream)
     _check(rc, "sparkattn_comp_apply")
     if check_status:
         _check(read_status(workspace, stream), "sparkattn_comp_apply (device status)")
@@ -492,27 +402,10 @@ def fwd_gated(q: torch.Tensor, k: torch.Tensor, v: torch.Tensor, kept_idx: torch
     """``sparkattn_fwd_gated``: the bf16 forward over 128-token blocks whose epilogue adds the gated
     compensation term.  Arguments as in ``fwd`` and ``comp_apply``; returns the module output bf16
     [B,H,N,d] (and the lse of the sparse branch, fp32 [B,H,N])."""
-    _same_layout(q, k, v)
-    shape = make_shape(q, 128, softmax_scale)
-    B, H, N, d = q.shape
-    rank = pq.shape[1]
-    kmax = kept_idx.shape[-1]
-    g, a, f = _rope_host(grid, axis, freq)
-    if not pq.is_contiguous() or pq.shape != (H, rank, d):
-        raise ValueError("pq must be contiguous [H, rank, d]")
-    if not state.is_contiguous() or state.shape != (B, H, rank, d) or state.dtype != torch.float32:
-        raise ValueError("state must be contiguous fp32 [B, H, rank, d]")
-    if not gate.is_contiguous() or gate.shape != (B, H, N) or gate.dtype != torch.float32:
-        raise ValueError("gate must be contiguous fp32 [B, H, N]")
-    if out is None:
-        out = torch.empty_strided(q.shape, q.stride(), dtype=torch.bfloat16, device=q.device)
-    lse = torch.empty((B, H, N), dtype=torch.float32, device=q.device) if return_lse else None
-    if workspace is None:
-        workspace = torch.empty(max(fwd_gated_workspace_bytes(shape, kmax, grid), 256), dtype=torch.uint8,
-                                device=q.device)
-    rc = lib().sparkattn_fwd_gated(ctypes.byref(shape), _ptr(q), _ptr(k), _ptr(v), _ptr(kept_idx), _ptr(kept_cnt), kmax,
-                                   _ptr(pq), rank, g, _ptr(a), _ptr(f), _ptr(state), _ptr(gate), ctypes.c_float(eps),
-                                   _ptr(out), _ptr(lse), _ptr(workspace), workspace.numel(), _stream_ptr(stream))
+    T, Hg, Wg = grid
+    rc, out, lse, workspace = _calls().fwd_gated(q, k, v, kept_idx, kept_cnt, pq, state, gate, int(T), int(Hg), int(Wg), axis, freq,
+                                                 eps, softmax_scale, out, return_lse, workspace,
+                                                 None if stream is None else stream.cuda_stream)
     _check(rc, "sparkattn_fwd_gated")
     if check_status:
         _check(read_status(workspace, stream), "sparkattn_fwd_gated (device status)")

@@ -315,3 +315,28 @@ def test_current_stream_without_the_private_name(monkeypatch):
     monkeypatch.setattr(sa, "_raw_stream", lambda device: 0x4560 + device)
     assert sa._stream_ptr(None) == 0x4563
     assert sa._stream_ptr(Stream) == 0x1230
+
+
+def test_binding_refuses_what_it_refused(lib):
+    """Errors of the native marshalling, which come before any device work: layouts that differ, a strided last dimension,
+    arguments that are no tensors, shapes that the library does not serve, and operands of the compensation branch."""
+    q = torch.zeros((1, 2, 256, 128), dtype=torch.bfloat16)
+    idx, cnt = torch.zeros((1, 2, 2, 1), dtype=torch.int32), torch.ones((1, 2, 2), dtype=torch.int32)
+    pk, axis, freq = torch.zeros((2, 64, 128), dtype=torch.bfloat16), torch.zeros(32, dtype=torch.int32), torch.zeros(32)
+    state, gate = torch.zeros((1, 2, 64, 128)), torch.zeros((1, 2, 256))
+    other = torch.zeros((1, 256, 2, 128), dtype=torch.bfloat16).transpose(1, 2)      # the same shape, other strides
+    turned = q.transpose(2, 3)
+    for call in (lambda: sa.select(q, other, 128, 1), lambda: sa.fwd(q, q, other, idx, cnt, 128), lambda: sa.quant_fp8(turned, 128),
+                 lambda: sa.select(turned, turned, 128, 1), lambda: sa.gather_tokens(q, cnt), lambda: sa.comp_state(q, other, pk, (1, 1, 256), axis, freq),
+                 lambda: sa.comp_state(q, q, pk, (1, 1, 256), axis, freq[:16]), lambda: sa.comp_state(q, q, pk[:1], (1, 1, 256), axis, freq),
+                 lambda: sa.comp_apply(q, pk, state[:, :1], gate, q, (1, 1, 256), axis, freq),
+                 lambda: sa.fwd_gated(q, q, q, idx, cnt, pk, state, gate.double(), (1, 1, 256), axis, freq),
+                 lambda: sa.fwd(q, q, q, idx, cnt, 128, frame_tokens=64, window=1, block_valid=cnt[0, 0])):
+        with pytest.raises(ValueError):
+            call()
+    with pytest.raises(TypeError):
+        sa.fwd(q, q, [1.0], idx, cnt, 128)
+    for call in (lambda: sa.select(q, q, 96, 1), lambda: sa.fwd(q, q, q, idx, cnt, 96)):
+        with pytest.raises(sa.SparkAttnError) as e:
+            call()
+        assert e.value.status == sa.E_UNSUPPORTED_SHAPE
