@@ -369,6 +369,40 @@ def test_tile_descriptors_around_their_ring(block, fp8, window):
     _compare_items(out[0], None, ref, None, items, block, w.N, FP8_RELRMS if fp8 else BF16_RELRMS, None)
 
 
+@pytest.mark.parametrize("fp8,window", [(False, 0), (True, 0), (False, 4), (True, 4)])
+@pytest.mark.parametrize("shared", [0, 1, 5])
+def test_pairs_whose_lists_differ(shared, fp8, window):
+    """64-token blocks: the two query blocks of a pair share 0, 1 or all 5 of their blocks, so that tiles hold two blocks of
+    one, of the other, one of each and (an odd number in all) a half that is nobody's; the last pair is a single
+    query block with a ragged tail.  A half tile that a query block does not list adds nothing to its rows, whatever stands in it:
+    the blocks that only the other one lists hold keys with far larger scores."""
+    H, nbk, block = 3, 33, 64
+    N = nbk * block - 23
+    g = torch.Generator().manual_seed(77 + shared + window)
+    q, k, v = (torch.randn((1, H, N, 128), generator=g) for _ in range(3))
+    idx = torch.empty((H, nbk, 5), dtype=torch.int32)
+    for h in range(H):
+        for i in range(0, nbk, 2):
+            rest = [j for j in torch.randperm(nbk, generator=g).tolist() if j not in (i, i + 1)]
+            both = ([i] + rest[:shared - 1]) if shared else []
+            idx[h, i] = torch.tensor((both + [j for j in ([i] + rest[8:16]) if j not in both])[:5])
+            if i + 1 < nbk:
+                idx[h, i + 1] = torch.tensor((both + [j for j in ([i + 1] + rest[16:24]) if j not in both])[:5])
+    cnt = torch.full((H, nbk), 5, dtype=torch.int32)
+    cnt[:, 3::4] = 4                                            # an odd number of blocks in the pair's merged list
+    k = k * (1.0 + 3.0 * (torch.arange(N) // block % 2))[None, None, :, None]      # odd blocks: larger scores
+    q, k, v = (t.to(torch.bfloat16) for t in (q, k, v))
+    t, kw = (q.to(DEV), k.to(DEV), v.to(DEV)), dict(frame_tokens=150, window=window) if window else {}
+    okw = dict(kw)
+    if fp8:
+        t, sc = zip(*(sa.quant_fp8(x, block) for x in t))
+        kw["scales"], okw["scales"] = sc, tuple(x[0].cpu() for x in sc)
+    out = sa.fwd(*t, idx[None].to(DEV), cnt[None].to(DEV), block, check_status=True, **kw)
+    items = [(h, i) for h in range(H) for i in range(nbk)]
+    ref, _ = oracle.attention(*(x[0].cpu() for x in t), idx, cnt, block, items=items, **okw)
+    _compare_items(out[0], None, ref, None, items, block, N, FP8_RELRMS if fp8 else BF16_RELRMS, None)
+
+
 def _stream_of_short_items(streams, block, stride, H=16, N=74 * 128 - 17):
     """Kept lists whose item i has streams[i % SMs % len][i // SMs % 8] tiles: what the persistent kernel's CTA c works
     through (items c, c + SMs, ...).  Both query blocks of a 64-token pair keep the same blocks."""
