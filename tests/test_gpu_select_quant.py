@@ -242,6 +242,25 @@ def test_quant_with_pooling_and_select_from_pooled_match_oracle(w):
         assert torch.equal(idx[0].cpu(), ref_idx) and torch.equal(cnt[0].cpu(), ref_cnt)
 
 
+@pytest.mark.parametrize("d,block", [(128, 128), (128, 64), (64, 64)])
+@pytest.mark.parametrize("tail", [0, 1, 15, 16, 17])
+def test_quant_with_pooling_at_every_tail(d, block, tail):
+    """The last block holds a batch of the addition chain's 16 rows, one less, one more, one row or all of them: codes, scales and
+    means against the oracle, bit for bit, with more CTAs than fit the chip at once."""
+    H, nb = 40, 33
+    N = (nb - 1) * block + (tail or block)
+    x = torch.randn((1, H, N, d), generator=torch.Generator().manual_seed(d + block + tail)).to(torch.bfloat16)
+    xd = x.to(DEV)
+    ws = sa.alloc_workspace(sa.make_shape(xd, block), 0, 1, DEV)
+    for key_side in (False, True):
+        codes, scales = sa.quant_fp8_pooled(xd, block, key_side, ws)
+        rc, rs = oracle.quant_fp8(x[0], block)
+        assert torch.equal(codes[0].cpu(), rc) and torch.equal(scales[0].cpu().view(torch.int32), rs.view(torch.int32))
+    want = oracle.pool(x[0], block).view(torch.int32)
+    for pooled in _pooled_from_workspace(ws, H, nb, d):
+        assert torch.equal(pooled.view(torch.int32), want)
+
+
 def test_quant_with_pooling_strided_batch_equals_separate_calls():
     """[B, N, H, d] buffers viewed as [B, H, N, d], two batch entries: the fused pass must reproduce the separate
     sparkattn_quant_fp8 / sparkattn_select calls bit for bit."""
