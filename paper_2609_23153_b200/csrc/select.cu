@@ -606,6 +606,11 @@ topk_wide_kernel(const float* pq, const float* pkT, int32_t* __restrict__ kept_i
   select_tile<WINDOW, WARPS, 1, false>(s_key, nb, nbp, topk, bh, i0, nrows, N, blk_size, frame_tokens, window, kept_idx, kept_cnt);
 }
 
+// The limit of a kernel's dynamic shared memory belongs to the kernel, not to a launch: it is always set to the most that any
+// launch of the kernel asks for.  Set to what this launch needs, it could be lowered by another thread before the
+// launch, which then fails.
+constexpr int kSmemOfOne = 227 * 1024, kSmemOfTwo = 113 * 1024;      // of a CTA alone on its SM, and of one of two
+
 template <int D, int RT, int RG, int KC, int NS>
 static int launch_topk(const float* pq, const float* pkT, int32_t* kept_idx, int32_t* kept_cnt, int nb, int nbp, int topk,
                        int64_t bh, int N, int block, int frame_tokens, int window, bool overlap, cudaStream_t stream) {
@@ -615,7 +620,7 @@ static int launch_topk(const float* pq, const float* pkT, int32_t* kept_idx, int
   if (ctas > 0x7fffffffLL) return SPARKATTN_E_UNSUPPORTED_SHAPE;
   const size_t smem = Shape::smem_bytes(D, nbp);
   auto kern = frame_tokens > 0 ? topk_kernel<D, RT, RG, KC, NS, true> : topk_kernel<D, RT, RG, KC, NS, false>;
-  if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
+  if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Shape::smem_bytes(D, 256)) != cudaSuccess)
     return SPARKATTN_E_CUDA;
   return launch_kernel(kern, (unsigned)ctas, kTopkThreads, smem, overlap, stream, pq, pkT, kept_idx, kept_cnt, nb, nbp, topk,
                        groups, N, block, frame_tokens, window);
@@ -631,7 +636,7 @@ static int launch_topk_wide(const float* pq, const float* pkT, int32_t* kept_idx
   if (ctas > 0x7fffffffLL) return SPARKATTN_E_UNSUPPORTED_SHAPE;
   const size_t smem = wide_smem(R, D, nbp);
   auto kern = frame_tokens > 0 ? topk_wide_kernel<D, R, RT, WARPS, CTAS, true> : topk_wide_kernel<D, R, RT, WARPS, CTAS, false>;
-  if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
+  if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, CTAS == 2 && R == 16 ? kSmemOfTwo : kSmemOfOne) != cudaSuccess)
     return SPARKATTN_E_CUDA;
   return launch_kernel(kern, (unsigned)ctas, WARPS * 32, smem, overlap, stream, pq, pkT, kept_idx, kept_cnt, nb, nbp, topk,
                        groups, N, block, frame_tokens, window);
@@ -658,7 +663,6 @@ static int launch_topk_d(const sparkattn_shape_t& s, int topk, int frame_tokens,
   auto go = [&](auto launch) {
     return launch(pq, pkT, kept_idx, kept_cnt, nb, nbp, topk, bh, s.N, s.block, frame_tokens, window, overlap, stream);
   };
-  constexpr size_t kOne = 227 * 1024, kTwo = 113 * 1024;       // shared memory of a CTA alone on its SM, and of one of two
   constexpr int kNumSMs = 148;   // B200; another count only moves the points where the CTAs get smaller
   const int64_t ctas32 = bh * ((nb + 31) / 32), ctas16 = bh * ((nb + 15) / 16);
   // More than 256 key blocks: the wide kernel, with 8 rows while 16 would leave SMs idle or do not fit twice into an SM,
@@ -673,10 +677,10 @@ static int launch_topk_d(const sparkattn_shape_t& s, int topk, int frame_tokens,
   // 80 heads of 250 blocks 63.9 us with 32 rows, 69.9 with 16, 94.6 with 8; 12 heads of 256 22.0 / 20.8 / 22.2; 3 heads
   // of 50 16.9 / 12.5 / 10.4.
   if (nb > 256) {
-    if (ctas16 > kNumSMs && wide_smem(16, D, nbp) <= kTwo) return go(launch_topk_wide<D, 16, 8, 10, 2>);
+    if (ctas16 > kNumSMs && wide_smem(16, D, nbp) <= kSmemOfTwo) return go(launch_topk_wide<D, 16, 8, 10, 2>);
     return go(launch_topk_wide<D, 8, 8, 10, 2>);               // at most 132 KB
   }
-  static_assert(TopkShape<8, 4, 16, 4>::smem_bytes(D, 256) <= kOne, "the tile of 32 rows of 256 keys");
+  static_assert(TopkShape<8, 4, 16, 4>::smem_bytes(D, 256) <= kSmemOfOne, "the tile of 32 rows of 256 keys");
   if (2 * ctas32 >= 3 * kNumSMs) return go(launch_topk<D, 8, 4, 16, 4>);
   if (ctas16 >= kNumSMs) return go(launch_topk<D, 4, 4, 16, 4>);
   return go(launch_topk<D, 2, 4, 16, 4>);
@@ -713,7 +717,7 @@ int launch_select(const sparkattn_shape_t& s, const void* q, const void* k, int 
   if (sm_count < 1) return SPARKATTN_E_CUDA;
   const size_t pool_smem = (size_t)2 * s.block * s.d * 2;
   auto pool = s.d == 128 ? pool_kernel<128> : pool_kernel<64>;
-  if (cudaFuncSetAttribute(pool, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)pool_smem) != cudaSuccess)
+  if (cudaFuncSetAttribute(pool, cudaFuncAttributeMaxDynamicSharedMemorySize, 2 * 128 * s.d * 2) != cudaSuccess)    // (see kSmemOfOne)
     return SPARKATTN_E_CUDA;
   const int64_t resident = (int64_t)sm_count * kPoolCtasPerSm * (65536 / (int)pool_smem);
   const int64_t pool_ctas = 2 * n_items < resident ? 2 * n_items : resident;

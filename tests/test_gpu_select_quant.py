@@ -1,4 +1,6 @@
 """GPU parity: sparkattn_select and sparkattn_quant_fp8 against the CPU oracle, bit for bit."""
+import threading
+
 import pytest
 import torch
 
@@ -294,3 +296,34 @@ def test_few_heads_of_many_blocks(H, nb, d, window):
         idx, cnt = sa.select(q[None].to(DEV), k[None].to(DEV), 64, topk, **kw)
         ref_idx, ref_cnt = oracle.select(q, k, 64, topk, **kw)
         assert torch.equal(idx[0].cpu(), ref_idx) and torch.equal(cnt[0].cpu(), ref_cnt)
+
+
+def test_selections_of_several_threads():
+    """Threads with a stream each select at different sizes at the same time: a kernel's limit of dynamic shared memory is one
+    for the whole process, and no thread may lower it between another one's setting and launch."""
+    g = torch.Generator(device=DEV).manual_seed(9)
+    cases = []
+    for N, d, block, topk in ((1500, 128, 128, 3), (900, 128, 64, 4), (20000, 128, 64, 9), (6400, 128, 128, 7), (17000, 64, 64, 5), (700, 64, 64, 2)):
+        q, k = (torch.randn((1, 2, N, d), generator=g, device=DEV).to(torch.bfloat16) for _ in range(2))
+        cases.append((q, k, block, topk, sa.select(q, k, block, topk)))
+    torch.cuda.synchronize()
+    wrong = []
+
+    def work(first):
+        try:
+            with torch.cuda.stream(torch.cuda.Stream()):
+                for n in range(400):
+                    q, k, block, topk, (idx, cnt) = cases[(first + n) % len(cases)]
+                    i, c = sa.select(q, k, block, topk)
+                    if n % 40 == 0 and not (torch.equal(i, idx) and torch.equal(c, cnt)):
+                        wrong.append((first, n))
+        except Exception as e:                      # a thread's exception would otherwise end the thread alone
+            wrong.append(repr(e))
+
+    threads = [threading.Thread(target=work, args=(j,)) for j in range(len(cases))]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    torch.cuda.synchronize()
+    assert not wrong, wrong[:5]
