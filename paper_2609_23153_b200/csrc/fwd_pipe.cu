@@ -1398,11 +1398,11 @@ static int launch_pipe(const sparkattn_shape_t& s, bool fp8, const void* q, cons
     return rc;
   const bool win = frame_tokens > 0;
   // The variant with a closing warpgroup: bf16 with 128-token blocks always (12 heads of 32,760 tokens; 6 / 18 / 26 / 64 / 256
-  // kept blocks: 163 / 387 / 541 / 1275 / 5023 us against 170 / 400 / 557 / 1293 / 5059), 64-token blocks up to 64 kept
-  // blocks (6 / 35 / 70: 150 / 528 / 961 against 163 / 534 / 965; 140 / 512: 1791 / 5196 against 1784 / 5088), FP8 up to 32
-  // (18 / 40 blocks of 128: 351 / 786 against 363 / 786; 64 / 256: 1183 / 4613 against 1164 / 4519; 64-token blocks 35: 532
-  // against 534, 70: 947 against 941).
-  const bool epi = !ga && (fp8 ? kmax <= 32 : !pair || kmax <= 64);
+  // kept blocks: 163 / 387 / 541 / 1275 / 5023 us against 170 / 400 / 557 / 1293 / 5059, in the build that set the rule), FP8 up
+  // to 32 (18 / 64 / 256 blocks: 293 / 984 / 3865 against 312 / 984 / 3790), 64-token blocks up to 64 (bf16, 35 / 128 of 512
+  // blocks: 479 / 1539 against 486 / 1533, 4 heads of 75,600 with 591 of 1182: 4691 against 4641; FP8, 35 / 51 / 256 of 512: 397 /
+  // 556 / 2386 against 413 / 572 / 2379).
+  const bool epi = !ga && (pair ? kmax <= 64 : !fp8 || kmax <= 32);
   using Kern = void (*)(CUtensorMap, CUtensorMap, CUtensorMap, CUtensorMap, CUtensorMap, PipeParams);
   Kern kern;
   if (fp8 && pair)

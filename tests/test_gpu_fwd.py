@@ -476,6 +476,12 @@ def test_streams_of_short_items(block, stride, kind):
     _check_stream([[1] * 8, [2, 1] * 4, [1, 2] * 4, [3, 1, 1, 1, 2, 1, 1, 1], [1, 3] * 4], block, stride, kind)
 
 
+@pytest.mark.parametrize("block", [64, 128])
+def test_fp8_streams_past_the_closing_warpgroup(block):
+    """FP8 lists with a stride beyond 64 run the two-warpgroup kernel for both block sizes."""
+    _check_stream([[1] * 8, [2, 1] * 4, [3, 1, 0, 1, 2, 1, 0, 1]], block, 72, "fp8")
+
+
 STREAMS = [[1, 0, 0, 0, 1, 0, 0, 2], [2, 0, 0, 1, 0, 0, 0, 1], [0, 0, 1, 0, 0, 0, 1, 1], [1, 0, 1, 0, 1, 0, 0, 0],
            [0, 1, 0, 0, 1, 1, 0, 3], [0, 0, 0, 0, 0, 0, 0, 0]]     # tiles of the items that one CTA takes in turn
 
