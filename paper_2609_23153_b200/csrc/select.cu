@@ -697,7 +697,7 @@ int launch_select_pooled(const sparkattn_shape_t& s, int topk, int32_t* kept_idx
                          cudaStream_t stream) {
   const int nb = (s.N + s.block - 1) / s.block;
   if (nb > kSelectMaxBlocks) return SPARKATTN_E_UNSUPPORTED_SHAPE;
-  const int rc = launch_topk_any(s, topk, 0, 0, kept_idx, kept_cnt, workspace, false, stream);
+  const int rc = launch_topk_any(s, topk, 0, 0, kept_idx, kept_cnt, workspace, true, stream);
   if (rc != SPARKATTN_OK) return rc;
   return cudaGetLastError() == cudaSuccess ? SPARKATTN_OK : SPARKATTN_E_CUDA;
 }
