@@ -113,7 +113,9 @@ void* ptr(const at::Tensor& t) { return t.defined() ? t.data_ptr() : nullptr; }
 int32_t* iptr(const at::Tensor& t) { return static_cast<int32_t*>(ptr(t)); }
 float* fptr(const at::Tensor& t) { return static_cast<float*>(ptr(t)); }
 at::TensorOptions on(const at::Tensor& x, at::ScalarType type) { return at::TensorOptions().dtype(type).device(x.device()); }
-int64_t blocks(const sparkattn_shape_t& s) { return ((int64_t)s.N + s.block - 1) / s.block; }
+// Token blocks of a head.  Outputs are sized with it before the library has looked at the shape: a block size below 1,
+// which the library refuses, has none.
+int64_t blocks(const sparkattn_shape_t& s) { return s.block < 1 ? 0 : ((int64_t)s.N + s.block - 1) / s.block; }
 
 // The caller's workspace, or a new one; undefined when the library does not serve the shape.
 at::Tensor workspace_for(at::Tensor given, const sparkattn_shape_t& s, int32_t which, int32_t k, const at::Tensor& x) {

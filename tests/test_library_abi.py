@@ -340,3 +340,23 @@ def test_binding_refuses_what_it_refused(lib):
         with pytest.raises(sa.SparkAttnError) as e:
             call()
         assert e.value.status == sa.E_UNSUPPORTED_SHAPE
+
+
+class _DefaultStream:
+    cuda_stream = 0
+
+
+@pytest.mark.parametrize("block", [0, -1, -128, -(1 << 31)])
+def test_binding_leaves_block_sizes_to_the_library(lib, block):
+    """A block size below 1 is an unsupported shape like any other that the library does not serve: the binding sizes its
+    outputs by the number of blocks, which no such size has."""
+    q = torch.zeros((1, 2, 256, 128), dtype=torch.bfloat16)
+    idx, cnt = torch.zeros((1, 2, 2, 1), dtype=torch.int32), torch.ones((1, 2, 2), dtype=torch.int32)
+    ws = torch.zeros(1 << 16, dtype=torch.uint8)
+    kw = dict(stream=_DefaultStream)                 # refused before the stream is used
+    for call in (lambda: sa.select(q, q, block, 1, **kw), lambda: sa.select(q, q, block, 1, kept_idx=idx, kept_cnt=cnt, workspace=ws, **kw),
+                 lambda: sa.select_pooled(q, block, 1, ws, **kw), lambda: sa.select_pooled(q, block, 1, ws, kept_idx=idx, kept_cnt=cnt, **kw),
+                 lambda: sa.fwd(q, q, q, idx, cnt, block, **kw), lambda: sa.fwd(q, q, q, idx, cnt, block, workspace=ws, **kw)):
+        with pytest.raises(sa.SparkAttnError) as e:
+            call()
+        assert e.value.status == sa.E_UNSUPPORTED_SHAPE
