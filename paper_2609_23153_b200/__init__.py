@@ -242,7 +242,7 @@ def quant_fp8(x: torch.Tensor, block: int, *, codes: Optional[torch.Tensor] = No
               scales: Optional[torch.Tensor] = None, stream: Optional[torch.cuda.Stream] = None,
               ) -> Tuple[torch.Tensor, torch.Tensor]:
     """``sparkattn_quant_fp8``: x bf16 [B,H,N,d] -> (codes uint8, same strides; scales fp32 [B,H,nb])."""
-    rc, codes, scales = _calls().quant(x, block, -1, None, codes, scales, None if stream is None else stream.cuda_stream)
+    rc, codes, scales = _calls().quant_fp8(x, block, codes, scales, None if stream is None else stream.cuda_stream)
     _check(rc, "sparkattn_quant_fp8")
     return codes, scales
 
@@ -252,8 +252,8 @@ def quant_fp8_pooled(x: torch.Tensor, block: int, key_side: bool, select_workspa
                      stream: Optional[torch.cuda.Stream] = None) -> Tuple[torch.Tensor, torch.Tensor]:
     """``sparkattn_quant_fp8_pooled``: :func:`quant_fp8` that also leaves the pooled block means of ``x`` (the query
     tensor, or the key tensor with ``key_side``) in ``select_workspace`` for :func:`select_pooled`."""
-    rc, codes, scales = _calls().quant(x, block, 1 if key_side else 0, select_workspace, codes, scales,
-                                       None if stream is None else stream.cuda_stream)
+    rc, codes, scales = _calls().quant_fp8_pooled(x, block, key_side, select_workspace, codes, scales,
+                                                  None if stream is None else stream.cuda_stream)
     _check(rc, "sparkattn_quant_fp8_pooled")
     return codes, scales
 
@@ -273,7 +273,7 @@ def quant_fp8_per_token(x: torch.Tensor, *, codes: Optional[torch.Tensor] = None
                         scales: Optional[torch.Tensor] = None, stream: Optional[torch.cuda.Stream] = None,
                         ) -> Tuple[torch.Tensor, torch.Tensor]:
     """``sparkattn_quant_fp8_per_token``: x bf16 [B,H,N,d] -> (codes uint8, same strides; scales fp32 [B,H,N])."""
-    rc, codes, scales = _calls().quant(x, 0, -1, None, codes, scales, None if stream is None else stream.cuda_stream)
+    rc, codes, scales = _calls().quant_fp8_per_token(x, codes, scales, None if stream is None else stream.cuda_stream)
     _check(rc, "sparkattn_quant_fp8_per_token")
     return codes, scales
 

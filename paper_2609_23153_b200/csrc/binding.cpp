@@ -195,30 +195,57 @@ PyObject* select_pooled(PyObject*, PyObject* const* argv, Py_ssize_t n) {
   END_HANDLE_TH_ERRORS
 }
 
-// quant(x, block (0: a scale per token), pooled side (-1: no pooling, 0: query, 1: key), select workspace, codes, scales,
-// stream) -> rc, codes, scales
-PyObject* quant(PyObject*, PyObject* const* argv, Py_ssize_t n) {
-  HANDLE_TH_ERRORS
-  Args a(argv, n);
-  a.expect(7);
-  const at::Tensor x = a.tensor();
-  const int32_t block = a.i32(), side = a.i32();
-  const at::Tensor ws = a.optional_tensor();
-  at::Tensor codes = a.optional_tensor(), scales = a.optional_tensor();
-  const Stream stream = a.stream();
-  const bool per_token = block == 0;
-  const sparkattn_shape_t s = make_shape(x, per_token ? (x.size(-1) == 64 ? 64 : 128) : block);
+// What the three quantisation calls share: codes (laid out like x) and scales [B, H, per_head] where the caller brings none.
+template <typename Call>
+PyObject* quantise(const at::Tensor& x, const sparkattn_shape_t& s, int64_t per_head, at::Tensor codes, at::Tensor scales, Call call) {
   int rc;
   {
     pybind11::gil_scoped_release no_gil;
     if (!codes.defined()) codes = at::empty_strided(x.sizes(), x.strides(), on(x, at::kByte));
-    if (!scales.defined()) scales = at::empty({s.B, s.H, per_token ? (int64_t)s.N : blocks(s)}, on(x, at::kFloat));
-    uint8_t* out = static_cast<uint8_t*>(ptr(codes));
-    if (per_token) rc = g_lib.quant_fp8_per_token(&s, ptr(x), out, fptr(scales), stream);
-    else if (side >= 0) rc = g_lib.quant_fp8_pooled(&s, ptr(x), out, fptr(scales), side, ptr(ws), (size_t)ws.numel(), stream);
-    else rc = g_lib.quant_fp8(&s, ptr(x), out, fptr(scales), 0, stream);
+    if (!scales.defined()) scales = at::empty({s.B, s.H, per_head}, on(x, at::kFloat));
+    rc = call(&s, ptr(x), static_cast<uint8_t*>(ptr(codes)), fptr(scales));
   }
   return result(rc, {codes, scales});
+}
+
+// quant_fp8(x, block, codes, scales, stream) -> rc, codes, scales
+PyObject* quant_fp8(PyObject*, PyObject* const* argv, Py_ssize_t n) {
+  HANDLE_TH_ERRORS
+  Args a(argv, n);
+  a.expect(5);
+  const at::Tensor x = a.tensor();
+  const sparkattn_shape_t s = make_shape(x, a.i32());
+  const at::Tensor codes = a.optional_tensor(), scales = a.optional_tensor();
+  const Stream stream = a.stream();
+  return quantise(x, s, blocks(s), codes, scales, [&](auto... to) { return g_lib.quant_fp8(to..., 0, stream); });
+  END_HANDLE_TH_ERRORS
+}
+
+// quant_fp8_pooled(x, block, key side, select workspace, codes, scales, stream) -> rc, codes, scales
+PyObject* quant_fp8_pooled(PyObject*, PyObject* const* argv, Py_ssize_t n) {
+  HANDLE_TH_ERRORS
+  Args a(argv, n);
+  a.expect(7);
+  const at::Tensor x = a.tensor();
+  const sparkattn_shape_t s = make_shape(x, a.i32());
+  const bool key_side = a.truth();
+  const at::Tensor ws = a.tensor(), codes = a.optional_tensor(), scales = a.optional_tensor();
+  const Stream stream = a.stream();
+  return quantise(x, s, blocks(s), codes, scales,
+                  [&](auto... to) { return g_lib.quant_fp8_pooled(to..., key_side, ptr(ws), (size_t)ws.numel(), stream); });
+  END_HANDLE_TH_ERRORS
+}
+
+// quant_fp8_per_token(x, codes, scales, stream) -> rc, codes, scales
+PyObject* quant_fp8_per_token(PyObject*, PyObject* const* argv, Py_ssize_t n) {
+  HANDLE_TH_ERRORS
+  Args a(argv, n);
+  a.expect(4);
+  const at::Tensor x = a.tensor();
+  const sparkattn_shape_t s = make_shape(x, x.size(-1) == 64 ? 64 : 128);
+  const at::Tensor codes = a.optional_tensor(), scales = a.optional_tensor();
+  const Stream stream = a.stream();
+  return quantise(x, s, s.N, codes, scales, [&](auto... to) { return g_lib.quant_fp8_per_token(to..., stream); });
   END_HANDLE_TH_ERRORS
 }
 
@@ -410,7 +437,8 @@ PyObject* bind(PyObject*, PyObject* const* argv, Py_ssize_t n) {
 template <PyObject* (*F)(PyObject*, PyObject* const*, Py_ssize_t)>
 PyMethodDef method(const char* name) { return {name, reinterpret_cast<PyCFunction>(reinterpret_cast<void (*)()>(F)), METH_FASTCALL, nullptr}; }
 PyMethodDef g_methods[] = {method<bind>("bind"), method<select>("select"), method<select_pooled>("select_pooled"),
-                           method<quant>("quant"), method<fwd>("fwd"), method<gather_tokens>("gather_tokens"),
+                           method<quant_fp8>("quant_fp8"), method<quant_fp8_pooled>("quant_fp8_pooled"),
+                           method<quant_fp8_per_token>("quant_fp8_per_token"), method<fwd>("fwd"), method<gather_tokens>("gather_tokens"),
                            method<comp_state>("comp_state"), method<comp_apply>("comp_apply"), method<fwd_gated>("fwd_gated"), {nullptr, nullptr, 0, nullptr}};
 PyModuleDef g_module = {PyModuleDef_HEAD_INIT, "_sparkattn", nullptr, -1, g_methods, nullptr, nullptr, nullptr, nullptr};
 

@@ -360,3 +360,20 @@ def test_binding_leaves_block_sizes_to_the_library(lib, block):
         with pytest.raises(sa.SparkAttnError) as e:
             call()
         assert e.value.status == sa.E_UNSUPPORTED_SHAPE
+
+
+@pytest.mark.parametrize("block", [0, -1, -128])
+def test_block_quantisation_has_no_hidden_mode(lib, block):
+    """quant_fp8 and quant_fp8_pooled scale by token block: a block size that there is none of is refused, whatever
+    buffers come with it, and is not taken for the per-token call, which writes N scales per head."""
+    x = torch.zeros((1, 2, 256, 128), dtype=torch.bfloat16)
+    ws = torch.zeros(1 << 16, dtype=torch.uint8)
+    own = dict(codes=torch.full((1, 2, 256, 128), 7, dtype=torch.uint8), scales=torch.full((1, 2, 2), 7.0))
+    for kw in ({}, own):
+        for call in (lambda: sa.quant_fp8(x, block, stream=_DefaultStream, **kw),
+                     lambda: sa.quant_fp8_pooled(x, block, False, ws, stream=_DefaultStream, **kw),
+                     lambda: sa.quant_fp8_pooled(x, block, True, ws, stream=_DefaultStream, **kw)):
+            with pytest.raises(sa.SparkAttnError) as e:
+                call()
+            assert e.value.status == sa.E_UNSUPPORTED_SHAPE
+    assert torch.all(own["codes"] == 7) and torch.all(own["scales"] == 7)
