@@ -315,15 +315,21 @@ PyObject* gather_tokens(PyObject*, PyObject* const* argv, Py_ssize_t n) {
   END_HANDLE_TH_ERRORS
 }
 
-// What the calls of the compensation branch share: the grid and the rotary tables, on the host.
+// What the calls of the compensation branch share: the grid and the rotary tables.
 struct Rope {
   int32_t grid[3];
   at::Tensor axis, freq;
   explicit Rope(Args& a) {
     for (int32_t& g : grid) g = a.i32();
-    axis = a.tensor().detach().to(at::kCPU, at::kInt).contiguous();
-    freq = a.tensor().detach().to(at::kCPU, at::kFloat).contiguous();
+    axis = a.tensor();
+    freq = a.tensor();
     TORCH_CHECK_VALUE(axis.numel() == freq.numel(), "rope axis and frequency tables must have rank/2 entries each");
+  }
+  // The library reads the tables on the host.  A copy from the device waits for the stream's earlier work, so this is
+  // called without the interpreter lock.
+  void to_host() {
+    axis = axis.detach().to(at::kCPU, at::kInt).contiguous();
+    freq = freq.detach().to(at::kCPU, at::kFloat).contiguous();
   }
 };
 bool is_contiguous(const at::Tensor& t, at::IntArrayRef sizes) { return t.is_contiguous() && t.sizes() == sizes; }
@@ -346,13 +352,14 @@ PyObject* comp_state(PyObject*, PyObject* const* argv, Py_ssize_t n) {
   const at::Tensor k = a.tensor(), v = a.tensor(), pk = a.tensor();
   same_layout(k, v);
   const sparkattn_shape_t s = make_shape(k, 128);
-  const Rope rope(a);
+  Rope rope(a);
   const int32_t rank = check_projection(pk, s, "pk");
   at::Tensor state = a.optional_tensor(), ws = a.optional_tensor();
   const Stream stream = a.stream();
   int rc;
   {
     pybind11::gil_scoped_release no_gil;
+    rope.to_host();
     if (!state.defined()) state = at::empty({s.B, s.H, rank, s.d}, on(k, at::kFloat));
     if (!ws.defined()) ws = at_least_256(g_lib.comp_workspace_bytes(&s, rope.grid), k);
     rc = g_lib.comp_state(&s, ptr(k), ptr(v), ptr(pk), rank, rope.grid, iptr(rope.axis), fptr(rope.freq), fptr(state), ptr(ws),
@@ -370,7 +377,7 @@ PyObject* comp_apply(PyObject*, PyObject* const* argv, Py_ssize_t n) {
   const at::Tensor q = a.tensor(), pq = a.tensor(), state = a.tensor(), gate = a.tensor(), o_sparse = a.tensor();
   same_layout(q, o_sparse);
   const sparkattn_shape_t s = make_shape(q, 128);
-  const Rope rope(a);
+  Rope rope(a);
   const int32_t rank = check_projection(pq, s, "pq");
   check_gate_operands(state, gate, s, rank);
   const float eps = a.number();
@@ -379,6 +386,7 @@ PyObject* comp_apply(PyObject*, PyObject* const* argv, Py_ssize_t n) {
   int rc;
   {
     pybind11::gil_scoped_release no_gil;
+    rope.to_host();
     if (!out.defined()) out = at::empty_strided(q.sizes(), q.strides(), on(q, at::kBFloat16));
     if (!ws.defined()) ws = at_least_256(g_lib.comp_workspace_bytes(&s, rope.grid), q);
     rc = g_lib.comp_apply(&s, ptr(q), ptr(pq), rank, rope.grid, iptr(rope.axis), fptr(rope.freq), fptr(state), fptr(gate),
@@ -398,7 +406,7 @@ PyObject* fwd_gated(PyObject*, PyObject* const* argv, Py_ssize_t n) {
                    state = a.tensor(), gate = a.tensor();
   same_layout(q, k);
   same_layout(q, v);
-  const Rope rope(a);
+  Rope rope(a);
   const float eps = a.number(), softmax_scale = a.number();
   const sparkattn_shape_t s = make_shape(q, 128, softmax_scale);
   const int32_t rank = check_projection(pq, s, "pq"), kmax = (int32_t)idx.size(-1);
@@ -410,6 +418,7 @@ PyObject* fwd_gated(PyObject*, PyObject* const* argv, Py_ssize_t n) {
   int rc;
   {
     pybind11::gil_scoped_release no_gil;
+    rope.to_host();
     if (!out.defined()) out = at::empty_strided(q.sizes(), q.strides(), on(q, at::kBFloat16));
     if (return_lse) lse = at::empty({s.B, s.H, s.N}, on(q, at::kFloat));
     if (!ws.defined()) ws = at_least_256(g_lib.fwd_gated_workspace_bytes(&s, kmax, rope.grid), q);

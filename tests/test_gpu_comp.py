@@ -8,6 +8,8 @@ Tolerances.  State: sums of bf16-rounded features times bf16 values in fp32, rel
 <= 1e-2.  Fused output: relative RMS <= 1e-2; element-wise |err| <= 3e-2 + 2^-8 |ref| (the second
 term is the bf16 rounding of the stored output, whose magnitude follows O_s)."""
 import math
+import threading
+import time
 
 import pytest
 import torch
@@ -158,3 +160,40 @@ def test_argument_errors():
     with pytest.raises(sa.SparkAttnError) as e:
         sa.comp_state(k, v, pk, w.grid, axis, freq, workspace=torch.empty(256, dtype=torch.uint8, device=DEV))
     assert e.value.status == sa.E_WORKSPACE_TOO_SMALL
+
+
+@pytest.mark.parametrize("call", ["state", "apply", "gated"])
+def test_device_rope_tables_leave_other_threads_running(call):
+    """The rotary tables may be on the device: the call then waits for the stream's earlier work (here a third of a second
+    of it), and another Python thread goes on meanwhile."""
+    w = workloads.Workload("ropethread", 17, 1, 2, 128, (3, 10, 13), 128, 0.5)
+    q, k, v, osp, pq, pk, gate, axis, freq = _inputs(w)
+    idx, cnt = sa.select(q, k, w.block, 2)
+    state = sa.comp_state(k, v, pk, w.grid, axis, freq)
+
+    def run(a, f):
+        return {"state": lambda: sa.comp_state(k, v, pk, w.grid, a, f), "apply": lambda: sa.comp_apply(q, pq, state, gate, osp, w.grid, a, f),
+                "gated": lambda: sa.fwd_gated(q, k, v, idx, cnt, pq, state, gate, w.grid, a, f)}[call]()
+
+    want = run(axis, freq)
+    on_device = axis.to(DEV), freq.to(DEV)
+    got, stream = {}, torch.cuda.Stream()
+    torch.cuda.synchronize()
+
+    def work():
+        with torch.cuda.stream(stream):
+            torch.cuda._sleep(600_000_000)               # clocks: 0.3 s at the highest rate
+            start = time.perf_counter()
+            got["out"] = run(*on_device)
+            got["waited"] = time.perf_counter() - start
+
+    thread = threading.Thread(target=work)
+    thread.start()
+    longest, last = 0.0, time.perf_counter()
+    while thread.is_alive():
+        now = time.perf_counter()
+        longest, last = max(longest, now - last), now
+    thread.join()
+    torch.cuda.synchronize()
+    assert torch.equal(got["out"].view(torch.uint8), want.view(torch.uint8))
+    assert got["waited"] > 0.15 and longest < 0.5 * got["waited"], (got["waited"], longest)
