@@ -66,7 +66,6 @@ quant_fp8_kernel(const __nv_bfloat16* x, uint8_t* __restrict__ codes, float* __r
   constexpr int kPerThread = kChunks / kQuantThreads;       // 8 for (128,128), 2 for (64,64)
   static_assert(kChunks % kQuantThreads == 0, "block must split evenly over the CTA");
 
-  pdl_trigger();
   const int blk = blockIdx.x % nb;
   const int bh = blockIdx.x / nb;
   const int h = bh % H, b = bh / H;
@@ -199,7 +198,6 @@ quant_fp8_token_kernel(const __nv_bfloat16* x, uint8_t* __restrict__ codes, floa
   const int sub = lane / kTokenLanes, chunk = lane % kTokenLanes;
   const int64_t warp_id = (int64_t)blockIdx.x * (kQuantThreads / 32) + (threadIdx.x >> 5);
   const int64_t row0 = warp_id * (kTokenSteps * kTokenRows);
-  pdl_trigger();
   pdl_wait();
   uint4 v[kTokenSteps][CPL];
   int64_t off[kTokenSteps];
@@ -297,13 +295,14 @@ int launch_quant_fp8_pooled(const sparkattn_shape_t& s, const void* x, uint8_t* 
               : s.d == 128 && s.block == 64 ? quant_fp8_pool_kernel<128, 64>
               : s.d == 64 && s.block == 64 ? quant_fp8_pool_kernel<64, 64> : nullptr;
   if (kern == nullptr) return SPARKATTN_E_UNSUPPORTED_SHAPE;
-  // Launched early, and letting the next kernel in early, only where all of it fits the chip at once: 3 heads of 1,200 tokens
-  // 3.9 -> 3.6 us, but 40 of 75,600 217 -> 226.  The kernels without pooling always are (2.6 -> 2.45 and 172 -> 170 us there).
   const int sm_count = current_sm_count();
   if (sm_count < 1) return SPARKATTN_E_CUDA;
-  const bool overlap = items <= (long long)sm_count * quant_pool_ctas(s.d, s.block);
-  return launch_kernel(kern, (unsigned)items, kQuantThreads, 0, overlap, stream, static_cast<const __nv_bfloat16*>(x), codes, scales,
-                       s.H, s.N, nb, s.stride_b, s.stride_h, s.stride_n, pooled, key_side ? 1 : 0, nbp, overlap);
+  // It lets the next kernel in early, which by this call's contract is another quantisation or the top-k, while there are at most
+  // two of its CTAs per SM.  Pooled Q and K, V, selection, 128-token blocks: 30 of them 19.6 us without and 18.9 with that, 296
+  // 24.9 either way, 370 27.6 and 29.0, 444 27.8 and 29.3: beyond the line CTAs of the next kernel fill up some SMs of the chip unevenly.
+  const bool early = items <= 2 * sm_count;
+  return launch_kernel(kern, (unsigned)items, kQuantThreads, 0, true, stream, static_cast<const __nv_bfloat16*>(x), codes, scales,
+                       s.H, s.N, nb, s.stride_b, s.stride_h, s.stride_n, pooled, key_side ? 1 : 0, nbp, early);
 }
 
 }  // namespace sparkattn
