@@ -12,6 +12,8 @@ HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "libsparkattn.so")
 BINDING = os.path.join(HERE, "_sparkattn.so")
+OBJDIR = os.path.join(HERE, "build")
+BINDING_FOR = os.path.join(OBJDIR, "_sparkattn.for")      # what the binding was built against
 SOURCES = ["api.cu", "select.cu", "quant.cu", "fwd.cu", "noalloc.cu", "comp.cu", "fwd_pipe.cu", "reorder.cu"]
 NVCC_FLAGS = [
     "-std=c++17", "-O3", "-lineinfo", "-gencode", "arch=compute_100a,code=sm_100a",
@@ -26,8 +28,23 @@ def _nvcc() -> str:
     raise RuntimeError("nvcc not found")
 
 
+def _target() -> str:
+    """The torch and Python that a binding built now belongs to: it uses torch's C++ interface, which is another one in
+    every build of torch, and Python's."""
+    import torch
+    return f"torch {torch.__version__} {torch.version.git_version} python {sysconfig.get_config_var('SOABI')}"
+
+
+def _binding_target() -> str:
+    try:
+        with open(BINDING_FOR) as f:
+            return f.read()
+    except FileNotFoundError:
+        return ""
+
+
 def needs_build() -> bool:
-    if not os.path.exists(LIB) or not os.path.exists(BINDING):
+    if not os.path.exists(LIB) or not os.path.exists(BINDING) or _binding_target() != _target():
         return True
     t = min(os.path.getmtime(LIB), os.path.getmtime(BINDING))
     deps = [os.path.join(CSRC, f) for f in os.listdir(CSRC)] + [os.path.join(HERE, "..", "include", "sparkattn.h")]
@@ -38,11 +55,10 @@ def build(force: bool = False, verbose: bool = False) -> str:
     if not force and not needs_build():
         return LIB
     nvcc = _nvcc()
-    objdir = os.path.join(HERE, "build")
-    os.makedirs(objdir, exist_ok=True)
+    os.makedirs(OBJDIR, exist_ok=True)
 
     def compile_one(src: str) -> str:
-        obj = os.path.join(objdir, src.replace(".cu", ".o"))
+        obj = os.path.join(OBJDIR, src.replace(".cu", ".o"))
         cmd = [nvcc, *NVCC_FLAGS, "-c", os.path.join(CSRC, src), "-o", obj]
         r = subprocess.run(cmd, capture_output=True, text=True)
         if verbose or r.returncode != 0:
@@ -65,6 +81,8 @@ def build(force: bool = False, verbose: bool = False) -> str:
             sys.stderr.write(r.stdout + r.stderr)
         if r.returncode != 0:
             raise RuntimeError("g++ failed on binding.cpp")
+        with open(BINDING_FOR, "w") as f:
+            f.write(_target())
 
     with ThreadPoolExecutor(max_workers=5) as ex:
         binding = ex.submit(build_binding)

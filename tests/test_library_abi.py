@@ -20,6 +20,24 @@ def lib():
     return sa.lib()
 
 
+def test_binding_of_another_torch_or_python_is_rebuilt(lib, monkeypatch, tmp_path):
+    """The native marshalling belongs to the torch and the Python that it was built against; nothing in the source tree
+    changes when one of them does."""
+    from paper_2609_23153_b200 import build
+    assert not build.needs_build()
+    for module, name in ((torch, "__version__"), (torch.version, "git_version")):
+        with monkeypatch.context() as m:
+            m.setattr(module, name, "another")
+            assert build.needs_build()
+    with monkeypatch.context() as m:
+        m.setattr(build.sysconfig, "get_config_var", lambda name: "another")
+        assert build.needs_build()
+    with monkeypatch.context() as m:                          # built before this was recorded
+        m.setattr(build, "BINDING_FOR", str(tmp_path / "none"))
+        assert build.needs_build()
+    assert not build.needs_build()
+
+
 def _declared_symbols():
     text = open(os.path.join(ROOT, "include", "sparkattn.h")).read()
     text = re.sub(r"/\*.*?\*/", "", text, flags=re.S)
