@@ -331,7 +331,7 @@ fwd_pipe_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
   uint64_t* bar_gt = bars + 54;               // GATE [2]: the projection Q P_q^T of warpgroup g's closing is complete
   uint64_t* bar_gy = bars + 56;               // GATE [2]: y = q~ C is complete
   uint64_t* bar_pq = bars + 58;               // GATE [2]: P_q of a new head has landed
-  uint64_t* bar_s_full = bars + 14;    // [2] S of a tile complete in S buffer (tile & 1)
+  uint64_t* bar_s_full = bars + 14;    // [2] S of a tile complete in S buffer (tile & 1): the product's arrival and its issuer's
   uint64_t* bar_s_free = bars + 16;    // [2] 128 arrivals: the warpgroup holds that S row in registers
   uint64_t* bar_p_full = bars + 18;    // [2] 128 arrivals: P written to P buffer (tile & 1)
   uint64_t* bar_pv_done = bars + 20;   // [2] PV of a tile complete: P buffer free again
@@ -349,6 +349,13 @@ fwd_pipe_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
   // 30 and 31; FP8: K scale, log2 of the factor folded into P, its inverse.  PAIR: the same of the tile's second block.
   // Tile t's entry is overwritten with tile t + 8's: K of that tile is requested when S of tile t + 8 - RK is complete,
   // which needs the row of tile t + 6 - RK >= t + 2 in registers.
+  // A softmax warp sees the entry because every link from the store to its read is a release and an acquire of ordinary
+  // threads: the producer arrives on bar_k_full after the store, the S issuer waits for that and arrives on bar_s_full
+  // itself, the softmax warp waits for that.  (The tensor core's own arrival on bar_s_full, by tcgen05.commit, stands for the
+  // product; whether it also carries what its issuer has seen is not documented.  The second arrival is lost in
+  // the noise but once: 12 heads of 32,760 tokens, 26 of 256 blocks, bf16 529.1 us without it and 529.8 with, FP8 417.5 and
+  // 415.8; FP8 with 64-token blocks, 51 of 512, 558.6 and 561.6.)  The entry is read with ordinary loads, which stay between
+  // the wait before them and the arrival on bar_s_free behind them.
   // (Loading list entries two tiles and scales one tile ahead in every softmax thread, and the logarithm there, took 490 us
   // where this takes 472, FP8, 12 heads of 32,760 tokens, 26 of 256 blocks; 64-token blocks at 40 x 75,600, 97 %, 3602 -> 3513;
   // plain bf16 546 -> 542.)
@@ -363,7 +370,7 @@ fwd_pipe_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
     for (int i = 0; i < 2; ++i) {
       mbar_init(bar_q_full + i, 1); mbar_init(bar_q_free + i, 1);
       mbar_init(bar_tok + i, 128);
-      mbar_init(bar_s_full + i, 1); mbar_init(bar_s_free + i, 128);
+      mbar_init(bar_s_full + i, 2); mbar_init(bar_s_free + i, 128);
       mbar_init(bar_p_full + i, 128); mbar_init(bar_pv_done + i, 1);
     }
     if constexpr (GATE) {
@@ -574,6 +581,7 @@ fwd_pipe_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
               mma_ss<FP8>(tmem + sbuf * kPBLK, make_desc(qa + ((sl * (kTile / 2) + kk * 32) >> 4), q_hi),
                           make_desc(ka + ((sl * (kTile / 2) + kk * 32) >> 4), q_hi), idesc_qk, (sl | kk) != 0 ? 1u : 0u);
           tc_commit(bar_s_full + sbuf);
+          mbar_arrive(bar_s_full + sbuf);           // see s_desc
           tc_commit(bar_k_free + kslot);
         }
         __syncwarp();
@@ -706,18 +714,18 @@ fwd_pipe_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
 #pragma unroll
         for (int ch = 0; ch < kPBLK / 32; ++ch) tmem_ld32(tS + ch * 32, *reinterpret_cast<uint32_t(*)[32]>(&sr[ch * 32]));
         // the tile's descriptor (see s_desc)
-        const volatile int* desc = s_desc + (tt & (kTileRing - 1)) * 8;
+        const int* desc = s_desc + (tt & (kTileRing - 1)) * 8;
         int x0, x1 = 0;
         float c = p.scale_log2, p_off = 0.0f, p_inv = 1.0f;       // logit -> log2 units; log2 of the factor folded into P; its inverse
         float c1 = c, p_off1 = 0.0f, p_inv1 = 1.0f;               // PAIR + FP8: the second key block of the tile has its own scales
         if constexpr (FP8) {
-          const int4 e = *reinterpret_cast<const int4*>(const_cast<const int*>(desc));
+          const int4 e = *reinterpret_cast<const int4*>(desc);
           x0 = e.x;
           c *= q_sc * __int_as_float(e.y);
           p_off = __int_as_float(e.z);
           p_inv = __int_as_float(e.w);
           if constexpr (PAIR) {
-            const int4 f = *reinterpret_cast<const int4*>(const_cast<const int*>(desc + 4));
+            const int4 f = *reinterpret_cast<const int4*>(desc + 4);
             x1 = f.x;
             c1 *= q_sc * __int_as_float(f.y);
             p_off1 = __int_as_float(f.z);
