@@ -60,9 +60,9 @@
 // and order are those of comp.cu's apply pass, so the result equals the two separate calls bit for
 // bit.  Measured (720p shape, 97 % sparsity): the closing grows from ~1300 to ~7200 clocks per item
 // (two dependent tensor-core round trips, 128 special-function operations per row, three passes over
-// TMEM), during which the pipeline drains: the fused call takes 2 % longer than the two calls it replaces (3.44
-// against 3.37 ms after idle, in turn; 480p shape 0.623 against 0.610) and less only where launches are what
-// counts (3 heads of 1,200 tokens: 33 against 47 us).
+// TMEM), during which the pipeline drains: the fused call takes 1 % longer than the two calls it replaces, in turn (3.41
+// against 3.37 ms after idle, 3.98 against 3.94 back to back), as long at the 480p shape (0.611 against 0.610), and less
+// where launches are what counts (3 heads of 1,200 tokens: 21 against 27 us).
 #include <cuda.h>
 #include <cuda_fp8.h>
 
@@ -1405,11 +1405,15 @@ static int launch_pipe(const sparkattn_shape_t& s, bool fp8, const void* q, cons
                                  s.B * s.H, nb)) != SPARKATTN_OK)
     return rc;
   const bool win = frame_tokens > 0;
-  // The variant with a closing warpgroup: bf16 with 128-token blocks always (12 heads of 32,760 tokens; 6 / 18 / 26 / 64 / 256
-  // kept blocks: 163 / 387 / 541 / 1275 / 5023 us against 170 / 400 / 557 / 1293 / 5059, in the build that set the rule), FP8 up
-  // to 32 (18 / 64 / 256 blocks: 293 / 984 / 3865 against 312 / 984 / 3790), 64-token blocks up to 64 (bf16, 35 / 128 of 512
-  // blocks: 479 / 1539 against 486 / 1533, 4 heads of 75,600 with 591 of 1182: 4691 against 4641; FP8, 35 / 51 / 256 of 512: 397 /
-  // 556 / 2386 against 413 / 572 / 2379).
+  // The variant with a closing warpgroup: bf16 with 128-token blocks always, FP8 with 128-token blocks up to 32 kept blocks,
+  // 64-token blocks up to 64.  It gains a fixed time per item, and its tile loop is a little slower, so the lead shrinks with
+  // the list; the lines lie before the point where the two meet, at about twice as many blocks.  12 heads of 32,760
+  // tokens, after idle, us with / without:
+  //   bf16, 128-token blocks  6: 163 / 170, 18: 387 / 400, 26: 541 / 557, 64: 1275 / 1293, 256: 5023 / 5059 (an earlier build)
+  //   FP8, 128-token blocks   18: 298 / 317, 26: 420 / 436, 32: 511 / 524, 40: 632 / 643, 48: 755 / 761, 64: 997 / 997, 256: 3865 / 3790
+  //   bf16, 64-token blocks   35: 408 / 416, 48: 547 / 551, 64: 708 / 713, 80: 871 / 873, 96: 1034 / 1035, 128: 1358 / 1355
+  //   FP8, 64-token blocks    35: 347 / 360, 48: 462 / 473, 64: 600 / 609, 80: 739 / 746, 96: 874 / 880, 128: 1150 / 1151, 192: 1687 / 1680
+  // 40 heads of 75,600: FP8 18: 2163 / 2312, 32: 3753 / 3860, 48: 5576 / 5630; 64-token blocks 35: 2515 / 2615, 64: 4438 / 4509.
   const bool epi = !ga && (pair ? kmax <= 64 : !fp8 || kmax <= 32);
   using Kern = void (*)(CUtensorMap, CUtensorMap, CUtensorMap, CUtensorMap, CUtensorMap, PipeParams);
   Kern kern;
