@@ -133,12 +133,13 @@ __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_gr
 // Programmatic dependent launch.  A kernel that may be launched while the one before it on the stream is still
 // running (launch_kernel with overlap) calls pdl_wait before its first access to device memory: it returns when
 // everything earlier on the stream is complete and visible.  pdl_trigger lets the next such kernel be launched.  The last
-// kernel of a call has none, because it does not know what comes next: the selection's pooling kernel, two persistent CTAs per
-// SM with their blocks dealt out beforehand, comes to stand three deep on some SMs and alone on others when it is let in
-// while SMs become free one by one.  comp_state then select, 40 heads of 75,600 tokens: 698 us with a trigger at the start of the
-// state pass's last kernel, 641 without; comp_apply then select 904 and 850; three quant_fp8 then select, 444 64-token blocks 24.1
-// and 20.9, 40 heads of 75,600 999 and 947.  What it gives elsewhere is less: comp_state then comp_apply, 3 heads of 1,200 19.2 and
-// 18.3.  (quant.cu has the one exception, whose successors are known.)
+// kernel of a call has none unless the call's purpose says what comes next, because of the selection's pooling kernel: two
+// persistent CTAs per SM with their blocks dealt out beforehand, which come to stand three deep on some SMs and alone on
+// others when they are let in while SMs become free one by one.  comp_apply then select, 40 heads of 75,600 tokens: 880 us
+// with a trigger at the start of the apply pass, 837 without; three quant_fp8 then select, 444 64-token blocks 24.1 and 20.9, 40 heads
+// of 75,600 999 and 947.  The two exceptions are the pooling quantisation (quant.cu) and the state pass, whose state comp_apply
+// or fwd_gated takes next: selection, state and gated forward of 10 heads of 7,252 tokens 174 us with its trigger, 184 without;
+// state and apply of 3 heads of 1,200 18.2 and 19.2.  (launch_select has what that leaves for the pooling kernel to do.)
 // Such a kernel reads device memory with ordinary loads only: a read-only load (__ldg, or through a const __restrict__
 // parameter) is for data that nothing writes during the whole life of the kernel, and the compiler may move it ahead of
 // the wait.

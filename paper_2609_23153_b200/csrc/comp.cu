@@ -355,6 +355,7 @@ comp_state_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid_const
 // overlapped, 3 heads of 1,200 tokens 64 -> 7.7 us, of 32,760 203 -> 16, 12 heads of 32,760 97 -> 38, 40 of 75,600 270 -> 232.
 constexpr int kReduceChannels = 8, kReduceThreads = kReduceChannels * kRank / 4;
 __global__ void __launch_bounds__(kReduceThreads) comp_reduce_kernel(const float* partial, float* __restrict__ state, int nchunks) {
+  pdl_trigger();
   pdl_wait();
   constexpr int kGroups = kCD / kReduceChannels;
   const int bh = blockIdx.x / kGroups, c0 = blockIdx.x % kGroups * kReduceChannels;

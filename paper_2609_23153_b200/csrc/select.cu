@@ -721,7 +721,12 @@ int launch_select(const sparkattn_shape_t& s, const void* q, const void* k, int 
     return SPARKATTN_E_CUDA;
   const int64_t resident = (int64_t)sm_count * kPoolCtasPerSm * (65536 / (int)pool_smem);
   const int64_t pool_ctas = 2 * n_items < resident ? 2 * n_items : resident;
-  const int rc0 = launch_kernel(pool, (unsigned)pool_ctas, s.d / 2, pool_smem, true, stream, qb, kb, pq, pkT, s.H, s.N, s.block, nb,
+  // Launched early while a CTA has fewer than four blocks.  Beyond that the microsecond it saves is lost in the noise (256 blocks of 12
+  // heads 50.8 us either way), and behind a kernel that lets it in its CTAs are placed unevenly for their whole run (see pdl_wait):
+  // comp_state then select, 12 heads of 32,760 tokens 92.5 us let in, 88.4 not; 40 of 75,600 675 and 620.  Below the line it
+  // would be 0.2 us of a selection of 12 to 17 us, and that order of calls stays slower there (2 heads of 12,000 26.5 us, 24.2 if not let in).
+  const bool early = 2 * n_items < 4 * resident;
+  const int rc0 = launch_kernel(pool, (unsigned)pool_ctas, s.d / 2, pool_smem, early, stream, qb, kb, pq, pkT, s.H, s.N, s.block, nb,
                                 nbp, s.stride_b, s.stride_h, s.stride_n, n_items, block_valid, static_cast<int32_t*>(workspace));
   if (rc0 != SPARKATTN_OK) return rc0;
   const int rc = launch_topk_any(s, topk, frame_tokens, window, kept_idx, kept_cnt, workspace, true, stream);

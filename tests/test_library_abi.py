@@ -312,8 +312,8 @@ def test_early_launched_kernels_read_with_ordinary_loads():
 
 def test_only_kernels_inside_a_call_let_the_next_one_in_early():
     """A kernel that ends a call does not know what follows, and the pooling kernel of a selection that is let in while it
-    drains is placed unevenly for its whole run.  The pooling quantisation may (its successors are fixed by its contract),
-    and every other kernel with pdl_trigger is followed by another one of the same call."""
+    drains is placed unevenly for its whole run.  The pooling quantisation and the state pass may (what they are for says what
+    follows), and every other kernel with pdl_trigger is followed by another one of the same call."""
     src = os.path.join(ROOT, "paper_2609_23153_b200", "csrc")
     found = {}
     for name in sorted(f for f in os.listdir(src) if f.endswith(".cu")):
@@ -321,7 +321,7 @@ def test_only_kernels_inside_a_call_let_the_next_one_in_early():
         for kernel in re.split(r"\b__global__\b", text)[1:]:
             if "pdl_trigger" in kernel:
                 found[re.search(r"(\w+)\s*\((?=[^()]*(const|int))", kernel[kernel.index("void"):]).group(1)] = name
-    assert found == {"rope_table_kernel": "comp.cu", "comp_state_kernel": "comp.cu", "clear_header_kernel": "fwd.cu",
+    assert found == {"rope_table_kernel": "comp.cu", "comp_state_kernel": "comp.cu", "comp_reduce_kernel": "comp.cu", "clear_header_kernel": "fwd.cu",
                      "compact_lists_kernel": "fwd_pipe.cu", "pair_lists_kernel": "fwd_pipe.cu", "head_vmax_kernel": "fwd_pipe.cu",
                      "pool_kernel": "select.cu", "quant_fp8_pool_kernel": "quant.cu"}
 
