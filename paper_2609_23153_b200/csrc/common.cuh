@@ -140,7 +140,7 @@ __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_gr
 // of 75,600 999 and 947.  The two exceptions are the pooling quantisation (quant.cu) and the state pass, whose state comp_apply
 // or fwd_gated takes next: selection, state and gated forward of 10 heads of 7,252 tokens 174 us with its trigger, 184 without;
 // state and apply of 3 heads of 1,200 18.2 and 19.2.  (launch_select has what that leaves for the pooling kernel to do.)
-// Such a kernel reads device memory with ordinary loads only: a read-only load (__ldg, or through a const __restrict__
+// A kernel launched early reads device memory with ordinary loads only: a read-only load (__ldg, or through a const __restrict__
 // parameter) is for data that nothing writes during the whole life of the kernel, and the compiler may move it ahead of
 // the wait.
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
