@@ -5,25 +5,28 @@
 // softmax attention (Sec. 2, softmax(Q K^T / sqrt(d)) V) restricted, for every
 // query block, to the key blocks of its kept list.
 //
-// One CTA owns one (batch, head, query block) work item.  A tile's chain (S product, softmax, P V product) is a
-// string of latencies, 2800 clocks when a 64-key tile was taken in two halves by one chain, so the kept tiles are
-// dealt out to C independent chains, each with its own S / P and O columns in TMEM, K / V slots, running maximum and
-// row sum: chain c takes list positions c, c + C, ...  The chains are merged at the end: every warp can read the O
-// of every chain for its own rows.  C = 4 (the whole TMEM, one CTA per SM) when the items do not fill the device,
-// where the length of the chain is the whole time; else C = 2 with two CTAs per SM, which overlap one item's start and
-// end with the other's tiles.
-// 2 heads of 2,048 tokens, 16 tiles per item: 12.5 us (C = 2: 14.5; one chain in halves: 25); 12 heads of 8,000 tokens, 125
-// tiles: 513 us (C = 4: 531; before: 1036), 770 clocks per tile and SM.  What bounds it there is the softmax: 64 rows live
-// in two of the SM's four quarters, whose special-function units need 512 clocks for a tile's 4096 exponentials.
-//   warps 4c, 4c+1   softmax of chain c: thread r owns query row r (the other two warps of each four would own MMA
-//                    rows 64-127, which do not exist).  The row of S comes into registers in one pass, fp32 online
-//                    softmax with packed fp32x2 FMA / ADD and 3-input max (row max / row sum need no shuffles), P is
-//                    written back to TMEM over S as bf16, conditional rescale of O.
-//   warp 4c+2        TMA producer of chain c: its K / V tiles, two slots each (128-byte swizzle); the first one Q as well.
-//   warp 4c+3        MMA issuer of chain c: S = Q K_j^T (operands in shared memory) and O += P V_j (P from TMEM, V MN-major
-//                    from shared memory) as tcgen05.mma with fp32 accumulators in TMEM.  S of the next tile is issued
-//                    right behind the PV that reads P out of the same columns.  (One issuer for all chains takes
-//                    14.1 us for the 16 tiles with four chains as with two.)
+// One CTA owns one (batch, head, query block) work item.  A query block has 64 rows and the tensor core 128, each half of
+// them in two of the SM's four quarters, so the rows are there twice and the halves take different key blocks: [Q; Q] times
+// [K1; K2] has Q K1^T and Q K2^T on its diagonal, [P1; P2] times [V1 | V2] has P1 V1 and P2 V2.  What lies off the diagonal is
+// computed and never read: the products cost as much as two of half the size, and the softmax warps of all four
+// quarters have work (with 64 rows in two quarters the special-function units of the other two stood idle).
+// A chain takes pairs of kept blocks one after the other (S product, softmax, P V product), each half with its own running
+// maximum and row sum; S of the next pair runs under the softmax of this one.  C chains share the list (chain c takes pairs c,
+// c + C, ...), and the 2 C partial results of a row are merged through shared memory at the end.  C = 2 (the whole
+// TMEM, one CTA per SM) when the items do not fill the device; else C = 1 with two CTAs per SM, which overlap one
+// item's start and end with the other's tiles.
+//   warps 4c .. 4c+3     softmax of chain c: thread r owns query row r mod 64, warps 4c and 4c+1 the pair's first block, the other
+//                        two its second.  The row of S comes into registers in one pass, fp32 online softmax with packed
+//                        fp32x2 FMA / ADD and 3-input max (row max / row sum need no shuffles), P goes to shared memory as
+//                        bf16 (S may be overwritten as soon as it sits in registers), conditional rescale of O.
+//   warp 4C + c          TMA producer of chain c: its K / V pairs, two slots each (128-byte swizzle); the first one Q as well.
+//   warp 5C + c          MMA issuer of chain c: tcgen05.mma with fp32 accumulators in TMEM, all operands from shared memory.
+// An odd list's last pair has a block past the end for a second one: zeros from the copy, all of its columns masked.
+// Bound by the softmax warps: a pair's 8192 exponentials are 512 clocks of the SM's special-function units, 1,170 clocks per
+// pair and SM at 125 tiles per item, where one chain runs its short steps under the other's exponentials.  Against one query block
+// per CTA with its 64 rows in two quarters (four or two chains of single tiles), us: 2 heads of 2,048 tokens, 16 of 32 tiles 12.6 ->
+// 10.2; 16 heads, 32 of 32 59 -> 42; 6 heads of 6,479, 10 of 102 30.5 -> 26.0, in a window of three frames 48 -> 38.5; 12 heads of
+// 8,000, 125 of 125 520 -> 410; 40 heads of 32,760, 15 of 512 1020 -> 900.
 //
 // Every wait on an mbarrier is bounded (common.cuh); a kept index outside
 // [0, nb) is reported in the status word and its tile skipped by all roles.
@@ -43,14 +46,20 @@ constexpr float kLazyRescaleLog2 = 8.0f;
 constexpr int kD = 64, kBlk = 64;
 constexpr int kFwdTile = kBlk * kD * 2;                 // bytes of a K or V tile: 64 rows of 128 bytes
 
+constexpr int kFwdPair = 2 * kFwdTile;                  // of the two tiles of a pair
+
 template <int C>
 struct Fwd64Smem {
-  static constexpr int kQ = 0;                          // 128 MMA rows of 128 bytes, the first 64 loaded
-  static constexpr int kKV = 2 * kFwdTile;              // [C][2 slots][K, V]
-  static constexpr int kBars = kKV + C * 4 * kFwdTile;  // 12 barriers per chain, Q, flags
-  static constexpr int kSums = kBars + 512;             // [C][64] (reference maximum, row sum)
-  static constexpr int kList = kSums + C * 64 * 8;      // [kFwdMaxKept]
+  static constexpr int kQ = 0;                          // the 64 query rows twice
+  static constexpr int kP = kFwdPair;                   // [C] P of both halves
+  static constexpr int kKV = kP + C * kFwdPair;         // [C][2 slots][K, V]
+  static constexpr int kBars = kKV + C * 4 * kFwdPair;  // 12 barriers per chain, Q, flags
+  static constexpr int kSums = kBars + 512;             // [2 C][64] (reference maximum, row sum)
+  static constexpr int kList = kSums + 2 * C * 64 * 8;  // [kFwdMaxKept]
   static constexpr int kBytes = 1024 /*align slack*/ + kList + kFwdMaxKept * 4;
+  // after the last product the K / V slots hold the weighted O of the 2 C half chains, fp32, rows padded to 68
+  static constexpr int kORow = kD + 4;
+  static_assert(2 * C * 64 * kORow * 4 <= C * 4 * kFwdPair, "partial results fit the K / V slots");
 };
 
 struct FwdParams {
@@ -66,63 +75,69 @@ struct FwdParams {
 };
 
 template <int C, bool WINDOW>
-__global__ void __launch_bounds__(128 * C, C == 2 ? 2 : 1)
+__global__ void __launch_bounds__(192 * C, C == 1 ? 2 : 1)
 fwd_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant__ CUtensorMap tmap_k,
            const __grid_constant__ CUtensorMap tmap_v, const FwdParams p) {
   using Smem = Fwd64Smem<C>;
   extern __shared__ unsigned char smem_dyn[];
   unsigned char* smem = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_dyn) + 1023) & ~uintptr_t(1023));
   uint64_t* bars = reinterpret_cast<uint64_t*>(smem + Smem::kBars);
-  // per chain: [2] K landed, [2] K free, [2] V landed, [2] V free, S complete, P written (64 arrivals), PV complete
+  // per chain: [2] K landed, [2] K free, [2] V landed, [2] V free, S complete, S in registers (128 arrivals), P written (128
+  // arrivals), PV complete
   auto bar_k_full = [&](int c, int slot) { return bars + c * 12 + slot; };
   auto bar_k_free = [&](int c, int slot) { return bars + c * 12 + 2 + slot; };
   auto bar_v_full = [&](int c, int slot) { return bars + c * 12 + 4 + slot; };
   auto bar_v_free = [&](int c, int slot) { return bars + c * 12 + 6 + slot; };
   auto bar_s_full = [&](int c) { return bars + c * 12 + 8; };
-  auto bar_p_full = [&](int c) { return bars + c * 12 + 9; };
-  auto bar_pv_done = [&](int c) { return bars + c * 12 + 10; };
+  auto bar_s_free = [&](int c) { return bars + c * 12 + 9; };
+  auto bar_p_full = [&](int c) { return bars + c * 12 + 10; };
+  auto bar_pv_done = [&](int c) { return bars + c * 12 + 11; };
   uint64_t* bar_q_full = bars + 48;
-  uint64_t* bar_sums = bars + 49;     // 64 C arrivals: every chain's last PV is complete and its sums are published
-  uint32_t* s_tmem_base = reinterpret_cast<uint32_t*>(bars + 50);
-  volatile int* s_abort = reinterpret_cast<volatile int*>(bars + 51);
-  int* s_ntiles = reinterpret_cast<int*>(bars + 52);
+  uint64_t* bar_sums = bars + 49;     // 128 C arrivals: every chain's last PV is complete and its sums are published
+  uint64_t* bar_parts = bars + 50;    // 128 C arrivals: every half chain's weighted O is in shared memory
+  uint32_t* s_tmem_base = reinterpret_cast<uint32_t*>(bars + 51);
+  volatile int* s_abort = reinterpret_cast<volatile int*>(bars + 52);
+  int* s_ntiles = reinterpret_cast<int*>(bars + 53);
   float2* s_sums = reinterpret_cast<float2*>(smem + Smem::kSums);
   int32_t* s_list = reinterpret_cast<int32_t*>(smem + Smem::kList);   // validated kept block indices
-  auto tile_k = [&](int c, int slot) { return smem + Smem::kKV + (c * 4 + slot * 2) * kFwdTile; };
-  auto tile_v = [&](int c, int slot) { return smem + Smem::kKV + (c * 4 + slot * 2 + 1) * kFwdTile; };
+  auto tile_k = [&](int c, int slot) { return smem + Smem::kKV + (c * 4 + slot * 2) * kFwdPair; };
+  auto tile_v = [&](int c, int slot) { return smem + Smem::kKV + (c * 4 + slot * 2 + 1) * kFwdPair; };
 
   const int warp = threadIdx.x >> 5;
   const int lane = threadIdx.x & 31;
   const int qb = blockIdx.x % p.nb;
   const int bh = blockIdx.x / p.nb;
   const int h = bh % p.H, b = bh / p.H;
+  constexpr int kTmaWarp = 4 * C, kMmaWarp = 5 * C;
 
   if (threadIdx.x == 0) {
     mbar_init(bar_q_full, 1);
-    mbar_init(bar_sums, 64 * C);
+    mbar_init(bar_sums, 128 * C);
+    mbar_init(bar_parts, 128 * C);
 #pragma unroll
     for (int c = 0; c < C; ++c) {
 #pragma unroll
       for (int i = 0; i < 9; ++i) mbar_init(bars + c * 12 + i, 1);
-      mbar_init(bar_p_full(c), 64);
+      mbar_init(bar_s_free(c), 128);
+      mbar_init(bar_p_full(c), 128);
       mbar_init(bar_pv_done(c), 1);
     }
     mbar_fence_init();
   }
-  if (warp == 2) {
+  if (warp == kTmaWarp) {
     if (lane == 0) {
       tma_prefetch_desc(&tmap_q);
       tma_prefetch_desc(&tmap_k);
       tma_prefetch_desc(&tmap_v);
     }
     __syncwarp();
-    tmem_alloc(s_tmem_base, 128 * C);
+    tmem_alloc(s_tmem_base, 256 * C);
     tmem_relinquish();
   }
   pdl_wait();
   // a timeout recorded by an earlier CTA of this launch makes the rest of the grid drain at once
   if (threadIdx.x == 0) *s_abort = (*reinterpret_cast<volatile int32_t*>(p.status) == SPARKATTN_E_DEVICE_TIMEOUT) ? 1 : 0;
-  if (warp == 6) {
+  if (warp == kMmaWarp) {
     // Stage the kept list in shared memory, in order, dropping (and reporting) indices outside [0, nb).
     const int cnt = p.kept_cnt ? min(max(p.kept_cnt[(int64_t)bh * p.nb + qb], 0), p.kmax) : p.kmax;
     const int32_t* list = p.kept_idx + ((int64_t)bh * p.nb + qb) * p.kmax;
@@ -141,47 +156,33 @@ fwd_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant__ C
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
-  const uint32_t tmem = *s_tmem_base;      // chain c: S (P overlays its start) at columns [128 c, +64), O at [128 c + 64, +64)
+  const uint32_t tmem = *s_tmem_base;      // chain c: S at columns [256 c, +128), O at [256 c + 128, +128)
   const bool dead = *s_abort != 0;
   const int ntiles = *s_ntiles;
-  auto tiles_of = [&](int c) { return (ntiles - c + C - 1) / C; };
+  auto pairs_of = [&](int c) { return ((ntiles + 1) / 2 - c + C - 1) / C; };
+  // key block of half `half` of pair n of chain c; past the end of an odd list: the block behind the last one, which is empty
+  auto block_of = [&](int c, int n, int half) {
+    const int at = 2 * (n * C + c) + half;
+    return at < ntiles ? s_list[at] : p.nb;
+  };
 
   if (dead) {
     // nothing to do: fall through to the teardown
-  } else if ((warp & 3) == 2) {
-    // ------------------------------------------------------------ TMA producer of chain warp / 4 (the first one: Q as well)
-    const int c = warp >> 2, mine = tiles_of(c);
+  } else if (warp >= kMmaWarp) {
+    // -------------------------------------------------------------- MMA issuer of chain warp - 5 C (one thread; its MMAs execute in order)
+    const int c = warp - kMmaWarp, mine = pairs_of(c);
     if (lane == 0 && mine > 0) {
-      if (c == 0) {
-        mbar_expect_tx(bar_q_full, kFwdTile);
-        tma_load_4d(smem + Smem::kQ, &tmap_q, bar_q_full, 0, qb * kBlk, h, b);
-      }
-      for (int n = 0; n < mine; ++n) {
-        const int slot = n & 1;
-        const int kb = s_list[n * C + c];
-        if (n >= 2 && !mbar_wait(bar_k_free(c, slot), ((n >> 1) - 1) & 1, s_abort, p.status, 1)) break;
-        mbar_expect_tx(bar_k_full(c, slot), kFwdTile);
-        tma_load_4d(tile_k(c, slot), &tmap_k, bar_k_full(c, slot), 0, kb * kBlk, h, b);
-        if (n >= 2 && !mbar_wait(bar_v_free(c, slot), ((n >> 1) - 1) & 1, s_abort, p.status, 2)) break;
-        mbar_expect_tx(bar_v_full(c, slot), kFwdTile);
-        tma_load_4d(tile_v(c, slot), &tmap_v, bar_v_full(c, slot), 0, kb * kBlk, h, b);
-      }
-    }
-  } else if ((warp & 3) == 3) {
-    // -------------------------------------------------------------- MMA issuer of chain warp / 4 (one thread; its MMAs execute in order)
-    const int c = warp >> 2, mine = tiles_of(c);
-    if (lane == 0 && mine > 0) {
-      constexpr uint32_t idesc_qk = make_idesc(1u, 128, kBlk, false);
-      constexpr uint32_t idesc_pv = make_idesc(1u, 128, kD, true);
-      const uint32_t tS = tmem + c * 128;
+      constexpr uint32_t idesc_qk = make_idesc(1u, 128, 2 * kBlk, false);
+      constexpr uint32_t idesc_pv = make_idesc(1u, 128, 2 * kD, true);
+      const uint32_t tS = tmem + c * 256;
       const uint64_t dQ = make_smem_desc_sw128(smem_u32(smem + Smem::kQ), 16);
-      const uint32_t q_lo = (uint32_t)dQ, q_hi = (uint32_t)(dQ >> 32);
+      const uint64_t dP = make_smem_desc_sw128(smem_u32(smem + Smem::kP + c * kFwdPair), 16);
+      const uint32_t q_lo = (uint32_t)dQ, p_lo = (uint32_t)dP, q_hi = (uint32_t)(dQ >> 32);
       auto issue_s = [&](int n) {
-        const uint64_t dK = make_smem_desc_sw128(smem_u32(tile_k(c, n & 1)), 16);
-        const uint32_t k_lo = (uint32_t)dK, k_hi = (uint32_t)(dK >> 32);
+        const uint32_t k_lo = (uint32_t)make_smem_desc_sw128(smem_u32(tile_k(c, n & 1)), 16);
 #pragma unroll
         for (int kk = 0; kk < kD / 16; ++kk)
-          mma_ss<false>(tS, make_desc(q_lo + ((kk * 32) >> 4), q_hi), make_desc(k_lo + ((kk * 32) >> 4), k_hi), idesc_qk,
+          mma_ss<false>(tS, make_desc(q_lo + ((kk * 32) >> 4), q_hi), make_desc(k_lo + ((kk * 32) >> 4), q_hi), idesc_qk,
                         kk != 0 ? 1u : 0u);
         tc_commit(bar_s_full(c));
         tc_commit(bar_k_free(c, n & 1));
@@ -193,28 +194,54 @@ fwd_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant__ C
       }
       for (int n = 0; ok && n < mine; ++n) {
         const int slot = n & 1;
-        const bool more = n + 1 < mine;
-        // this V and the next K have normally landed long before P is written
+        if (n + 1 < mine) {
+          ok = mbar_wait(bar_k_full(c, slot ^ 1), ((n + 1) >> 1) & 1, s_abort, p.status, 5);
+          if (ok) ok = mbar_wait(bar_s_free(c), n & 1, s_abort, p.status, 4);
+          if (!ok) break;
+          tc_fence_after();
+          issue_s(n + 1);
+        }
         ok = mbar_wait(bar_v_full(c, slot), (n >> 1) & 1, s_abort, p.status, 6);
-        if (ok && more) ok = mbar_wait(bar_k_full(c, slot ^ 1), ((n + 1) >> 1) & 1, s_abort, p.status, 5);
         if (ok) ok = mbar_wait(bar_p_full(c), n & 1, s_abort, p.status, 7);
         if (!ok) break;
         tc_fence_after();
-        const uint64_t dV = make_smem_desc_sw128(smem_u32(tile_v(c, slot)), kFwdTile);
+        const uint64_t dV = make_smem_desc_sw128(smem_u32(tile_v(c, slot)), kFwdTile);      // the pair's tiles are two slabs of columns
         const uint32_t v_lo = (uint32_t)dV, v_hi = (uint32_t)(dV >> 32);
 #pragma unroll
         for (int kk = 0; kk < kBlk / 16; ++kk)
-          mma_ts<false>(tS + 64, tS + kk * 8, make_desc(v_lo + ((kk * 16 * 128) >> 4), v_hi), idesc_pv, (n | kk) != 0 ? 1u : 0u);
-        if (more) issue_s(n + 1);
+          mma_ss<false>(tS + 128, make_desc(p_lo + ((kk * 32) >> 4), q_hi), make_desc(v_lo + ((kk * 16 * 128) >> 4), v_hi), idesc_pv,
+                        (n | kk) != 0 ? 1u : 0u);
         tc_commit(bar_pv_done(c));
         tc_commit(bar_v_free(c, slot));
       }
     }
-  } else if ((warp & 2) == 0) {
+  } else if (warp >= kTmaWarp) {
+    // ------------------------------------------------------------ TMA producer of chain warp - 4 C (the first one: Q as well)
+    const int c = warp - kTmaWarp, mine = pairs_of(c);
+    if (lane == 0 && mine > 0) {
+      if (c == 0) {
+        mbar_expect_tx(bar_q_full, kFwdPair);
+        tma_load_4d(smem + Smem::kQ, &tmap_q, bar_q_full, 0, qb * kBlk, h, b);
+        tma_load_4d(smem + Smem::kQ + kFwdTile, &tmap_q, bar_q_full, 0, qb * kBlk, h, b);
+      }
+      for (int n = 0; n < mine; ++n) {
+        const int slot = n & 1;
+        const int k0 = block_of(c, n, 0) * kBlk, k1 = block_of(c, n, 1) * kBlk;
+        if (n >= 2 && !mbar_wait(bar_k_free(c, slot), ((n >> 1) - 1) & 1, s_abort, p.status, 1)) break;
+        mbar_expect_tx(bar_k_full(c, slot), kFwdPair);
+        tma_load_4d(tile_k(c, slot), &tmap_k, bar_k_full(c, slot), 0, k0, h, b);
+        tma_load_4d(tile_k(c, slot) + kFwdTile, &tmap_k, bar_k_full(c, slot), 0, k1, h, b);
+        if (n >= 2 && !mbar_wait(bar_v_free(c, slot), ((n >> 1) - 1) & 1, s_abort, p.status, 2)) break;
+        mbar_expect_tx(bar_v_full(c, slot), kFwdPair);
+        tma_load_4d(tile_v(c, slot), &tmap_v, bar_v_full(c, slot), 0, k0, h, b);
+        tma_load_4d(tile_v(c, slot) + kFwdTile, &tmap_v, bar_v_full(c, slot), 0, k1, h, b);
+      }
+    }
+  } else {
     // ----------------------------------------------------------------- softmax of chain warp / 4
-    const int chain = warp >> 2;
-    const int row = threadIdx.x & 127;                // query row inside the block = TMEM lane (0..63)
-    const uint32_t lane_off = (uint32_t)((warp & 1) * 32) << 16;
+    const int chain = warp >> 2, half = (warp >> 1) & 1;
+    const int row = threadIdx.x & 63;                 // query row inside the block
+    const uint32_t lane_off = (uint32_t)((warp & 3) * 32) << 16;
     const int q_row = qb * kBlk + row;
     const bool row_valid = q_row < p.N;
     // keys this row may attend to: [klo, khi) (everything up to N without a causal window)
@@ -224,13 +251,15 @@ fwd_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant__ C
       klo = max(fi - p.window + 1, 0) * p.frame_tokens;
       khi = (int)min((long long)(fi + 1) * p.frame_tokens, (long long)p.N);
     }
-    const uint32_t tS = tmem + chain * 128 + lane_off;
+    const uint32_t tS = tmem + chain * 256 + lane_off + half * kBlk;           // this half's columns of S and of O
+    const uint32_t tO = tmem + chain * 256 + 128 + lane_off + half * kD;
+    unsigned char* p_row = smem + Smem::kP + chain * kFwdPair + (half * kBlk + row) * 128;
     const float c = p.scale_log2;                     // logit -> log2 units
-    const int mine = tiles_of(chain);
+    const int mine = pairs_of(chain);
     float m_used = -INFINITY, l = 0.0f;
     bool ok = true;
     for (int n = 0; ok && n < mine; ++n) {
-      const int kb = s_list[n * C + chain];
+      const int kb = block_of(chain, n, half);
       const int c_lo = klo - kb * kBlk, c_hi = khi - kb * kBlk;      // this row's valid columns of the tile: [c_lo, c_hi)
       ok = __all_sync(0xffffffffu, mbar_wait(bar_s_full(chain), n & 1, s_abort, p.status, 8));
       if (!ok) break;
@@ -239,6 +268,8 @@ fwd_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant__ C
 #pragma unroll
       for (int ch = 0; ch < kBlk / 32; ++ch) tmem_ld32(tS + ch * 32, *reinterpret_cast<uint32_t(*)[32]>(&sr[ch * 32]));
       tc_wait_ld();
+      tc_fence_before();
+      mbar_arrive(bar_s_free(chain));             // the next pair's S may overwrite this one
       if ((WINDOW && c_lo > 0) || c_hi < kBlk) {  // ragged last key block / keys outside the causal window get weight 0
 #pragma unroll
         for (int i = 0; i < kBlk; ++i)
@@ -257,9 +288,15 @@ fwd_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant__ C
         m_used = m_new;
         need = true;
       }
-      if (__any_sync(0xffffffffu, need)) {
-        // O must be quiescent: the chain's last PV is the previous tile's
-        ok = __all_sync(0xffffffffu, mbar_wait(bar_pv_done(chain), (n - 1) & 1, s_abort, p.status, 10));
+      // The chain's last PV is the previous pair's: once it is complete P has been read and O is quiescent.  It is waited for behind
+      // the first kWaitAt pieces of eight columns.  Two of them where the length of the chain is all there is (C = 2: 64 items
+      // of 16 tiles 10.1 us, 10.3 with none); none where the stores of P should run under the exponentials (C = 1: 12 heads of
+      // 8,000 tokens 410 us, two 432, all eight 450).
+      constexpr int kWaitAt = C == 2 ? 2 : 0;
+      auto wait_pv = [&]() { return n == 0 || __all_sync(0xffffffffu, mbar_wait(bar_pv_done(chain), (n - 1) & 1, s_abort, p.status, 10)); };
+      const bool rescale = __any_sync(0xffffffffu, need);
+      if (rescale) {
+        ok = wait_pv();
         if (!ok) break;
         tc_fence_after();
         l *= alpha;
@@ -267,7 +304,7 @@ fwd_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant__ C
 #pragma unroll 1
         for (int ch = 0; ch < kD / 16; ++ch) {
           uint32_t r[16];
-          tmem_ld16(tS + 64 + ch * 16, r);
+          tmem_ld16(tO + ch * 16, r);
           tc_wait_ld();
 #pragma unroll
           for (int i = 0; i < 16; i += 2) {
@@ -275,90 +312,115 @@ fwd_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant__ C
             r[i] = __float_as_uint(o2.x);
             r[i + 1] = __float_as_uint(o2.y);
           }
-          tmem_st16(tS + 64 + ch * 16, r);
+          tmem_st16(tO + ch * 16, r);
         }
+        tc_wait_st();
       }
 
-      // P = exp2(S*c - m) as bf16, written over the start of S
+      // P = exp2(S*c - m) as bf16
       const float neg_m = m_used == -INFINITY ? 0.0f : -m_used;   // a fully masked row: exp2(-inf) = 0, not NaN
       const uint64_t c2 = pack_f32x2(c, c), nm2 = pack_f32x2(neg_m, neg_m);
       uint64_t lsum0 = pack_f32x2(0.0f, 0.0f), lsum1 = lsum0;
       uint32_t w[kBlk / 2];
+      auto store = [&](int j) {                   // 128-byte swizzle
+        *reinterpret_cast<uint4*>(p_row + ((j ^ (row & 7)) << 4)) = make_uint4(w[4 * j], w[4 * j + 1], w[4 * j + 2], w[4 * j + 3]);
+      };
 #pragma unroll
-      for (int i = 0; i < kBlk; i += 2) {
-        const float2 x = unpack_f32x2(ffma2(pack_f32x2(__uint_as_float(sr[i]), __uint_as_float(sr[i + 1])), c2, nm2));
-        const float e0 = fast_exp2(x.x), e1 = fast_exp2(x.y);
-        if ((i >> 1) & 1) lsum1 = fadd2(lsum1, pack_f32x2(e0, e1));
-        else lsum0 = fadd2(lsum0, pack_f32x2(e0, e1));
-        const __nv_bfloat162 h2 = __floats2bfloat162_rn(e0, e1);
-        w[i / 2] = *reinterpret_cast<const uint32_t*>(&h2);
+      for (int j = 0; j < kBlk / 8; ++j) {
+        if (j == kWaitAt) {
+          if (!rescale) ok = wait_pv();
+          if (!ok) break;
+#pragma unroll
+          for (int i = 0; i < j; ++i) store(i);
+        }
+#pragma unroll
+        for (int i = 8 * j; i < 8 * j + 8; i += 2) {
+          const float2 x = unpack_f32x2(ffma2(pack_f32x2(__uint_as_float(sr[i]), __uint_as_float(sr[i + 1])), c2, nm2));
+          const float e0 = fast_exp2(x.x), e1 = fast_exp2(x.y);
+          if ((i >> 1) & 1) lsum1 = fadd2(lsum1, pack_f32x2(e0, e1));
+          else lsum0 = fadd2(lsum0, pack_f32x2(e0, e1));
+          const __nv_bfloat162 h2 = __floats2bfloat162_rn(e0, e1);
+          w[i / 2] = *reinterpret_cast<const uint32_t*>(&h2);
+        }
+        if (j >= kWaitAt) store(j);
       }
-      tmem_st32(tS, *reinterpret_cast<const uint32_t(*)[32]>(&w[0]));
+      if (!ok) break;
       const float2 ls = unpack_f32x2(fadd2(lsum0, lsum1));
       l += ls.x + ls.y;
-      tc_wait_st();
       tc_fence_before();
+      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
       mbar_arrive(bar_p_full(chain));
     }
 
-    // ---------------------------------------------------------------- merge of the chains and epilogue
+    // ---------------------------------------------------------------- merge of the half chains and epilogue
     if (ok && mine > 0) ok = __all_sync(0xffffffffu, mbar_wait(bar_pv_done(chain), (mine - 1) & 1, s_abort, p.status, 9));
+    const int part = chain * 2 + half;
     if (ok) {
       tc_fence_after();
-      tc_fence_before();
-      s_sums[chain * 64 + row] = make_float2(m_used, l);
+      s_sums[part * 64 + row] = make_float2(m_used, l);
       mbar_arrive(bar_sums);
       ok = __all_sync(0xffffffffu, mbar_wait(bar_sums, 0, s_abort, p.status, 11));
     }
     if (ok) {
-      tc_fence_after();
-      float2 sums[C];
+      // every product of the CTA is complete: the K / V slots are free for the weighted O of the half chains
       float m = -INFINITY;
 #pragma unroll
-      for (int i = 0; i < C; ++i) {
-        sums[i] = s_sums[i * 64 + row];
-        if (sums[i].y != 0.0f) m = fmaxf(m, sums[i].x);
+      for (int i = 0; i < 2 * C; ++i) {
+        const float2 s = s_sums[i * 64 + row];
+        if (s.y != 0.0f) m = fmaxf(m, s.x);
       }
-      float w[C], total = 0.0f;
+      float total = 0.0f;
 #pragma unroll
-      for (int i = 0; i < C; ++i) {
-        w[i] = sums[i].y != 0.0f ? fast_exp2(sums[i].x - m) : 0.0f;
-        total += w[i] * sums[i].y;
+      for (int i = 0; i < 2 * C; ++i) {
+        const float2 s = s_sums[i * 64 + row];
+        if (s.y != 0.0f) total += fast_exp2(s.x - m) * s.y;
       }
       const float inv = total > 0.0f ? 1.0f / total : 0.0f;     // no admissible key at all: zero row, lse = -inf
-      // this chain's warps write columns [64 / C * chain, +64 / C) of the row
-      constexpr int kCols = kD / C;
-      float o[kCols];
+      const float w = l != 0.0f ? fast_exp2(m_used - m) : 0.0f;
+      constexpr int kORow = Smem::kORow;
+      float* parts = reinterpret_cast<float*>(smem + Smem::kKV);
+      float* mine_o = parts + (part * 64 + row) * kORow;
 #pragma unroll
-      for (int j = 0; j < kCols; ++j) o[j] = 0.0f;
+      for (int ch = 0; ch < kD / 16; ++ch) {
+        uint32_t r[16] = {};
+        if (mine > 0) {                                          // (a chain without a pair has no O)
+          tmem_ld16(tO + ch * 16, r);
+          tc_wait_ld();
+        }
 #pragma unroll
-      for (int i = 0; i < C; ++i) {
-        if (i < ntiles) {                                        // chains without a tile have no O
-#pragma unroll
-          for (int ch = 0; ch < kCols / 16; ++ch) {
-            uint32_t r[16];
-            tmem_ld16(tmem + i * 128 + 64 + lane_off + chain * kCols + ch * 16, r);
-            tc_wait_ld();
-            if (w[i] != 0.0f) {
-#pragma unroll
-              for (int j = 0; j < 16; ++j) o[ch * 16 + j] = fmaf(__uint_as_float(r[j]), w[i], o[ch * 16 + j]);
-            }
-          }
+        for (int j = 0; j < 16; j += 4) {
+          float4 v = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+          if (w != 0.0f)
+            v = make_float4(__uint_as_float(r[j]) * w, __uint_as_float(r[j + 1]) * w, __uint_as_float(r[j + 2]) * w, __uint_as_float(r[j + 3]) * w);
+          *reinterpret_cast<float4*>(mine_o + ch * 16 + j) = v;
         }
       }
-      if (row_valid) {
-        __nv_bfloat16* orow = p.out + b * p.stride_b + h * p.stride_h + (int64_t)q_row * p.stride_n + chain * kCols;
+      mbar_arrive(bar_parts);
+      ok = __all_sync(0xffffffffu, mbar_wait(bar_parts, 0, s_abort, p.status, 12));
+      if (ok && row_valid) {
+        // this half chain's threads write columns [64 / 2C * part, +64 / 2C) of the row
+        constexpr int kCols = kD / (2 * C);
+        __nv_bfloat16* orow = p.out + b * p.stride_b + h * p.stride_h + (int64_t)q_row * p.stride_n + part * kCols;
+        const float* src = parts + row * kORow + part * kCols;
 #pragma unroll
         for (int i = 0; i < kCols / 8; ++i) {
+          float o[8] = {};
+#pragma unroll
+          for (int k = 0; k < 2 * C; ++k) {
+            const float4 x = *reinterpret_cast<const float4*>(src + k * 64 * kORow + 8 * i);
+            const float4 y = *reinterpret_cast<const float4*>(src + k * 64 * kORow + 8 * i + 4);
+            o[0] += x.x; o[1] += x.y; o[2] += x.z; o[3] += x.w;
+            o[4] += y.x; o[5] += y.y; o[6] += y.z; o[7] += y.w;
+          }
           uint32_t ww[4];
 #pragma unroll
           for (int j = 0; j < 4; ++j) {
-            const __nv_bfloat162 h2 = __floats2bfloat162_rn(o[8 * i + 2 * j] * inv, o[8 * i + 2 * j + 1] * inv);
+            const __nv_bfloat162 h2 = __floats2bfloat162_rn(o[2 * j] * inv, o[2 * j + 1] * inv);
             ww[j] = *reinterpret_cast<const uint32_t*>(&h2);
           }
           reinterpret_cast<uint4*>(orow)[i] = make_uint4(ww[0], ww[1], ww[2], ww[3]);
         }
-        if (p.lse && chain == 0) p.lse[(int64_t)bh * p.N + q_row] = fmaf(m, 0.6931471805599453f, log2f(total) * 0.6931471805599453f);   // one rounding
+        if (p.lse && part == 0) p.lse[(int64_t)bh * p.N + q_row] = fmaf(m, 0.6931471805599453f, log2f(total) * 0.6931471805599453f);   // one rounding
       }
     }
   }
@@ -366,10 +428,10 @@ fwd_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant__ C
   // ------------------------------------------------------------------ teardown
   tc_fence_before();
   __syncthreads();
-  if (warp == 2) {
+  if (warp == kTmaWarp) {
     if (*s_abort) __nanosleep(200000);  // let copies / MMAs in flight land before the CTA's resources go
     tc_fence_after();
-    tmem_dealloc(tmem, 128 * C);
+    tmem_dealloc(tmem, 256 * C);
   }
 }
 
@@ -394,7 +456,7 @@ static int launch_fwd_t(const CUtensorMap& mq, const CUtensorMap& mk, const CUte
   auto kern = prm.frame_tokens > 0 ? fwd_kernel<C, true> : fwd_kernel<C, false>;
   if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, Fwd64Smem<C>::kBytes) != cudaSuccess)
     return SPARKATTN_E_CUDA;
-  return launch_kernel(kern, (unsigned)ctas, 128 * C, Fwd64Smem<C>::kBytes, true, stream, mq, mk, mv, prm);
+  return launch_kernel(kern, (unsigned)ctas, 192 * C, Fwd64Smem<C>::kBytes, true, stream, mq, mk, mv, prm);
 }
 
 int launch_fwd(const sparkattn_shape_t& s, int dtype, const void* q, const void* k, const void* v,
@@ -435,9 +497,9 @@ int launch_fwd(const sparkattn_shape_t& s, int dtype, const void* q, const void*
   const int sm_count = current_sm_count();
   if (sm_count < 1) return SPARKATTN_E_CUDA;
   if ((rc = launch_kernel(clear_header_kernel, 1, kWorkspaceHeaderBytes / 4, 0, true, stream, prm.status)) != SPARKATTN_OK) return rc;
-  // four chains while no SM gets a second item: 64 to 144 items of 16 tiles 12.5-13 us against 14.5-15 with two; 256 items
-  // of 3 tiles 11.3 against 7.9, 512 of 32 tiles 68 against 59
-  return ctas <= sm_count ? launch_fwd_t<4>(mq, mk, mv, prm, ctas, stream) : launch_fwd_t<2>(mq, mk, mv, prm, ctas, stream);
+  // two chains while no SM gets a second item, us against one chain and two CTAs per SM: 64 items of 16 tiles 10.3 / 11.5, 128 10.7 /
+  // 11.9; but 160 19.0 / 14.2, 256 items of 3 tiles 12.3 / 8.1, 512 of 32 56.5 / 42.4
+  return ctas <= sm_count ? launch_fwd_t<2>(mq, mk, mv, prm, ctas, stream) : launch_fwd_t<1>(mq, mk, mv, prm, ctas, stream);
 }
 
 }  // namespace sparkattn

@@ -499,6 +499,30 @@ def test_empty_lists_between_short_ones(block, stride, kind):
     _check_stream(STREAMS, block, stride, kind)
 
 
+@pytest.mark.parametrize("H", [2, 5])
+def test_d64_infinity_stays_where_it_belongs(H):
+    """d = 64: the halves of a product take two key blocks at a time, and what one half makes of the other's block is computed
+    but never read.  An infinite value in one key block (lists of one to six blocks, odd ones with half a pair left over)
+    makes its channel infinite for the query blocks that keep it and leaves everything else as it is: no NaN.  82
+    items run two chains each, 205 one."""
+    nb, d = 41, 64
+    N = nb * 64 - 7
+    g = torch.Generator().manual_seed(900 + H)
+    q, k, v = (0.3 * torch.randn((1, H, N, d), generator=g) for _ in range(3))
+    idx = torch.stack([torch.stack([torch.randperm(nb, generator=g)[:6] for _ in range(nb)]) for _ in range(H)]).to(torch.int32)
+    cnt = (1 + torch.arange(nb, dtype=torch.int32) % 6).expand(H, nb).contiguous()
+    kept = (idx == 3) & (torch.arange(6) < cnt[..., None])
+    assert 0 < int(kept.any(-1).sum()) < H * nb
+    q, k, v = (t.to(torch.bfloat16).to(DEV) for t in (q, k, v))
+    clean = sa.fwd(q, k, v, idx[None].to(DEV), cnt[None].to(DEV), 64, check_status=True)
+    v[:, :, 3 * 64 + 11, 5] = math.inf
+    out = sa.fwd(q, k, v, idx[None].to(DEV), cnt[None].to(DEV), 64, check_status=True)
+    rows = kept.any(-1).to(DEV).repeat_interleave(64, 1)[:, :N]             # [H, N]
+    assert torch.all(torch.isposinf(out[0, ..., 5]) == rows)
+    clean[0, ..., 5] = torch.where(rows, math.inf, clean[0, ..., 5])
+    assert torch.equal(out, clean)
+
+
 @pytest.mark.parametrize("H", [28, 56])
 def test_lse_of_merged_chains_is_rounded_once(H):
     """d = 64: scores that fp32 holds exactly and one key that outweighs the others, so that the log-sum-exp is off by its
