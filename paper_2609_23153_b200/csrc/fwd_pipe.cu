@@ -149,15 +149,8 @@ __device__ __forceinline__ void report_bad_index(const PipeParams& p, int item, 
 }
 
 // one warp per item: drop (and flag) kept indices outside [0, nb), clamp the count, own block first
-__global__ void compact_lists_kernel(const int32_t* kept_idx, const int32_t* kept_cnt,
-                                     int32_t* __restrict__ clean_cnt, int32_t* __restrict__ clean_list, int items,
-                                     int nb, int kmax, int32_t* status) {
-  pdl_trigger();
-  pdl_wait();
-  if (blockIdx.x == 0 && threadIdx.x < kWorkspaceHeaderBytes / 4) status[threadIdx.x] = 0;
-  const int item = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-  const int lane = threadIdx.x & 31;
-  if (item >= items) return;
+__device__ __forceinline__ void compact_list(const int32_t* kept_idx, const int32_t* kept_cnt, int32_t* clean_cnt, int32_t* clean_list,
+                                             int item, int nb, int kmax, int lane) {
   const int cnt = kept_cnt ? min(max(kept_cnt[item], 0), kmax) : kmax;
   const int32_t* src = kept_idx + (int64_t)item * kmax;
   int32_t* dst = clean_list + (int64_t)item * kmax;
@@ -199,6 +192,16 @@ __global__ void compact_lists_kernel(const int32_t* kept_idx, const int32_t* kep
     }
   }
 }
+constexpr int kCompactWarps = 8;
+__global__ void __launch_bounds__(kCompactWarps * 32)
+compact_lists_kernel(const int32_t* kept_idx, const int32_t* kept_cnt, int32_t* __restrict__ clean_cnt,
+                     int32_t* __restrict__ clean_list, int items, int nb, int kmax, int32_t* status) {
+  pdl_trigger();
+  pdl_wait();
+  if (blockIdx.x == 0 && threadIdx.x < kWorkspaceHeaderBytes / 4) status[threadIdx.x] = 0;
+  const int item = blockIdx.x * kCompactWarps + (threadIdx.x >> 5);
+  if (item < items) compact_list(kept_idx, kept_cnt, clean_cnt, clean_list, item, nb, kmax, threadIdx.x & 31);
+}
 
 // 64-token blocks: the kernel works on pairs of adjacent query blocks (128 query rows, the MMA's M) and on
 // tiles of two key blocks.  One warp per pair merges the two kept lists (range-checked, duplicates folded)
@@ -206,18 +209,10 @@ __global__ void compact_lists_kernel(const int32_t* kept_idx, const int32_t* kep
 // two entries per tile (an odd tail repeats its block with both flags clear).  clean_cnt = tiles.
 constexpr int kPairMaxBlocks = 16384;    // key blocks per head the merge can mark in shared memory
 constexpr int kPairWarps = 4;
-__global__ void __launch_bounds__(kPairWarps * 32)
-pair_lists_kernel(const int32_t* kept_idx, const int32_t* kept_cnt,
-                  int32_t* __restrict__ clean_cnt, int32_t* __restrict__ clean_list, int pairs, int nb, int nbq,
-                  int kmax, int32_t* status) {
-  pdl_trigger();
-  pdl_wait();
-  if (blockIdx.x == 0 && threadIdx.x < kWorkspaceHeaderBytes / 4) status[threadIdx.x] = 0;
+__device__ __forceinline__ void pair_list(const int32_t* kept_idx, const int32_t* kept_cnt, int32_t* clean_cnt, int32_t* clean_list,
+                                          int pair, int nb, int nbq, int kmax, int wl, int lane) {
   extern __shared__ uint32_t s_bits[];                      // [kPairWarps][2][words]
   const int words = (nb + 31) / 32;
-  const int wl = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int pair = blockIdx.x * kPairWarps + wl;
-  if (pair >= pairs) return;
   uint32_t* bits = s_bits + wl * 2 * words;
   for (int i = lane; i < 2 * words; i += 32) bits[i] = 0u;
   __syncwarp();
@@ -265,18 +260,40 @@ pair_lists_kernel(const int32_t* kept_idx, const int32_t* kept_cnt,
   }
 }
 
-// FP8: largest V block scale of every (batch, head); one warp each
-__global__ void head_vmax_kernel(const float* v_scale, float* __restrict__ v_max, int bh_count, int nb) {
+__global__ void __launch_bounds__(kPairWarps * 32)
+pair_lists_kernel(const int32_t* kept_idx, const int32_t* kept_cnt,
+                  int32_t* __restrict__ clean_cnt, int32_t* __restrict__ clean_list, int pairs, int nb, int nbq,
+                  int kmax, int32_t* status) {
   pdl_trigger();
   pdl_wait();
-  const int bh = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-  const int lane = threadIdx.x & 31;
-  if (bh >= bh_count) return;
+  if (blockIdx.x == 0 && threadIdx.x < kWorkspaceHeaderBytes / 4) status[threadIdx.x] = 0;
+  const int wl = threadIdx.x >> 5, pair = blockIdx.x * kPairWarps + wl;
+  if (pair < pairs) pair_list(kept_idx, kept_cnt, clean_cnt, clean_list, pair, nb, nbq, kmax, wl, threadIdx.x & 31);
+}
+
+// FP8: the largest V block scale of every (batch, head), one warp each, and behind these warps the list pre-pass of either block
+// size, as above.  One launch between the quantisation and the forward instead of two in a row: forward of 3 heads of 1,200 tokens
+// 10.1 -> 9.0 us, 6 of 6,479 32.3 -> 31.1, with 64-token blocks 30.3 -> 28.5, 20 of 6,479 39.7 -> 38.2.
+template <bool PAIR>
+__global__ void __launch_bounds__((PAIR ? kPairWarps : kCompactWarps) * 32)
+head_vmax_kernel(const float* v_scale, float* __restrict__ v_max, int heads, const int32_t* kept_idx, const int32_t* kept_cnt,
+                 int32_t* __restrict__ clean_cnt, int32_t* __restrict__ clean_list, int items, int nb, int nbq, int kmax, int32_t* status) {
+  pdl_trigger();
+  pdl_wait();
+  if (blockIdx.x == 0 && threadIdx.x < kWorkspaceHeaderBytes / 4) status[threadIdx.x] = 0;
+  const int wl = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int w = blockIdx.x * (PAIR ? kPairWarps : kCompactWarps) + wl;
+  if (w >= heads) {
+    if (w - heads >= items) return;
+    if constexpr (PAIR) pair_list(kept_idx, kept_cnt, clean_cnt, clean_list, w - heads, nb, nbq, kmax, wl, lane);
+    else compact_list(kept_idx, kept_cnt, clean_cnt, clean_list, w - heads, nb, kmax, lane);
+    return;
+  }
   float m = 0.0f;
-  for (int j = lane; j < nb; j += 32) m = fmaxf(m, v_scale[(int64_t)bh * nb + j]);
+  for (int j = lane; j < nb; j += 32) m = fmaxf(m, v_scale[(int64_t)w * nb + j]);
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
-  if (lane == 0) v_max[bh] = m;
+  if (lane == 0) v_max[w] = m;
 }
 
 __device__ __forceinline__ void pipe_tma_store_4d(const void* tmap, const void* smem_src, int c0, int c1, int c2, int c3) {
@@ -1392,18 +1409,19 @@ static int launch_pipe(const sparkattn_shape_t& s, bool fp8, const void* q, cons
     prm.rope_table = table;
     prm.state = ga->state; prm.gate = ga->gate; prm.eps = ga->eps;
   }
-  if (pair) {
-    const size_t bits = (size_t)kPairWarps * 2 * ((nb + 31) / 32) * sizeof(uint32_t);
-    rc = launch_kernel(pair_lists_kernel, (unsigned)((items + kPairWarps - 1) / kPairWarps), kPairWarps * 32, bits, true, stream,
-                       kept_idx, kept_cnt, clean_cnt, clean_list, (int)items, nb, nbq, kmax, prm.status);
-  } else {
-    rc = launch_kernel(compact_lists_kernel, (unsigned)((items + 7) / 8), 256, 0, true, stream, kept_idx, kept_cnt, clean_cnt,
-                       clean_list, (int)items, nb, kmax, prm.status);
-  }
+  const size_t bits = pair ? (size_t)kPairWarps * 2 * ((nb + 31) / 32) * sizeof(uint32_t) : 0;
+  const int warps = pair ? kPairWarps : kCompactWarps, heads = s.B * s.H;
+  if (fp8)
+    rc = launch_kernel(pair ? head_vmax_kernel<true> : head_vmax_kernel<false>, (unsigned)((items + heads + warps - 1) / warps), warps * 32,
+                       bits, true, stream, v_scale, v_max, heads, kept_idx, kept_cnt, clean_cnt, clean_list, (int)items, nb, nbq, kmax,
+                       prm.status);
+  else if (pair)
+    rc = launch_kernel(pair_lists_kernel, (unsigned)((items + warps - 1) / warps), warps * 32, bits, true, stream, kept_idx, kept_cnt,
+                       clean_cnt, clean_list, (int)items, nb, nbq, kmax, prm.status);
+  else
+    rc = launch_kernel(compact_lists_kernel, (unsigned)((items + warps - 1) / warps), warps * 32, 0, true, stream, kept_idx, kept_cnt,
+                       clean_cnt, clean_list, (int)items, nb, kmax, prm.status);
   if (rc != SPARKATTN_OK) return rc;
-  if (fp8 && (rc = launch_kernel(head_vmax_kernel, (unsigned)((s.B * s.H + 7) / 8), 256, 0, true, stream, v_scale, v_max,
-                                 s.B * s.H, nb)) != SPARKATTN_OK)
-    return rc;
   const bool win = frame_tokens > 0;
   // The variant with a closing warpgroup: bf16 with 128-token blocks always, FP8 with 128-token blocks up to 32 kept blocks,
   // 64-token blocks up to 64.  It gains a fixed time per item, and its tile loop is a little slower, so the lead shrinks with
