@@ -148,12 +148,48 @@ __device__ __forceinline__ void report_bad_index(const PipeParams& p, int item, 
   }
 }
 
-// one warp per item: drop (and flag) kept indices outside [0, nb), clamp the count, own block first
+// One warp per item: drop (and flag) kept indices outside [0, nb), clamp the count, and move the query block's own key block to the
+// front.  The result does not depend on the order of the tiles, the work does: a row's running maximum is usually set by its own
+// block, and when that block comes late (it is the last entry of an ascending list under a causal window) nearly every
+// row's maximum jumps past the lazy threshold there and the whole O tile is rescaled; with it first the later tiles stay
+// below the reference.
+// Nothing but latency: lists of up to 128 entries are requested together with their count and written once from registers
+// (forward of 3 heads of 1,200 tokens, 2 entries, 9.6 -> 9.0 us; 6 of 6,479, 10 entries, 35.0 -> 34.0); longer ones are written as
+// they come, and the part before the own block is shifted afterwards.
 __device__ __forceinline__ void compact_list(const int32_t* kept_idx, const int32_t* kept_cnt, int32_t* clean_cnt, int32_t* clean_list,
                                              int item, int nb, int kmax, int lane) {
-  const int cnt = kept_cnt ? min(max(kept_cnt[item], 0), kmax) : kmax;
+  constexpr int kChunks = 4;
   const int32_t* src = kept_idx + (int64_t)item * kmax;
   int32_t* dst = clean_list + (int64_t)item * kmax;
+  const uint32_t lt_mask = (1u << lane) - 1u;
+  const int qb = item % nb;
+  if (kmax <= 32 * kChunks) {
+    int kb[kChunks];
+#pragma unroll
+    for (int c = 0; c < kChunks; ++c) kb[c] = 32 * c + lane < kmax ? src[32 * c + lane] : -1;
+    const int cnt = kept_cnt ? min(max(kept_cnt[item], 0), kmax) : kmax;
+    uint32_t keep[kChunks];
+    int at[kChunks + 1], own = -1;                       // own: place of the own block among those kept
+    at[0] = 0;
+    bool bad = false;
+#pragma unroll
+    for (int c = 0; c < kChunks; ++c) {
+      const bool listed = 32 * c + lane < cnt, valid = listed && kb[c] >= 0 && kb[c] < nb;
+      bad = __any_sync(0xffffffffu, listed && !valid) || bad;
+      keep[c] = __ballot_sync(0xffffffffu, valid);
+      const uint32_t hit = __ballot_sync(0xffffffffu, valid && kb[c] == qb);
+      if (own < 0 && hit) own = at[c] + __popc(keep[c] & ((hit & (0u - hit)) - 1u));
+      at[c + 1] = at[c] + __popc(keep[c]);
+    }
+#pragma unroll
+    for (int c = 0; c < kChunks; ++c) {
+      const int r = at[c] + __popc(keep[c] & lt_mask);
+      if ((keep[c] >> lane) & 1u) dst[r == own ? 0 : r < own ? r + 1 : r] = kb[c];
+    }
+    if (lane == 0) clean_cnt[item] = at[kChunks] | (bad ? kBadFlag : 0);
+    return;
+  }
+  const int cnt = kept_cnt ? min(max(kept_cnt[item], 0), kmax) : kmax;
   int out = 0;
   bool bad = false;
   for (int base = 0; base < cnt; base += 32) {
@@ -162,18 +198,13 @@ __device__ __forceinline__ void compact_list(const int32_t* kept_idx, const int3
     const bool valid = (t < cnt) && kb >= 0 && kb < nb;
     bad = __any_sync(0xffffffffu, (t < cnt) && !valid) || bad;
     const uint32_t ballot = __ballot_sync(0xffffffffu, valid);
-    if (valid) dst[out + __popc(ballot & ((1u << lane) - 1u))] = kb;
+    if (valid) dst[out + __popc(ballot & lt_mask)] = kb;
     out += __popc(ballot);
   }
   if (lane == 0) clean_cnt[item] = out | (bad ? kBadFlag : 0);
-  // The query block's own key block goes first.  The result does not depend on the order of the tiles, the
-  // work does: a row's running maximum is usually set by its own block, and when that block comes late (it is
-  // the last entry of an ascending list under a causal window) nearly every row's maximum jumps past the lazy
-  // threshold there and the whole O tile is rescaled; with it first the later tiles stay below the reference.
   // (The list is read back past L1: the forward kernel may already be resident, and must find no line of it there that
   // was fetched before a neighbouring item's warp had written its part.)
   __syncwarp();
-  const int qb = item % nb;
   int p = -1;
   for (int base = 0; base < out && p < 0; base += 32) {
     const int t = base + lane;
@@ -217,17 +248,25 @@ __device__ __forceinline__ void pair_list(const int32_t* kept_idx, const int32_t
   for (int i = lane; i < 2 * words; i += 32) bits[i] = 0u;
   __syncwarp();
   const int bh = pair / nbq, qp = pair % nbq;
-  bool bad = false;
+  // both lists' counts and first entries are requested before anything waits for one of them
+  int cnt[2], first[2];
+  const int32_t* src[2];
+#pragma unroll
   for (int side = 0; side < 2; ++side) {
-    const int qb = 2 * qp + side;
-    if (qb >= nb) break;
-    const int64_t item = (int64_t)bh * nb + qb;
-    const int cnt = kept_cnt ? min(max(kept_cnt[item], 0), kmax) : kmax;
-    const int32_t* src = kept_idx + item * kmax;
-    for (int base = 0; base < cnt; base += 32) {
-      const int kb = base + lane < cnt ? src[base + lane] : 0;
+    const int64_t item = (int64_t)bh * nb + min(2 * qp + side, nb - 1);
+    src[side] = kept_idx + item * kmax;
+    first[side] = lane < kmax ? src[side][lane] : 0;
+    cnt[side] = kept_cnt ? min(max(kept_cnt[item], 0), kmax) : kmax;
+  }
+  if (2 * qp + 1 >= nb) cnt[1] = 0;
+  bool bad = false;
+#pragma unroll
+  for (int side = 0; side < 2; ++side) {
+    for (int base = 0; base < cnt[side]; base += 32) {
+      const bool listed = base + lane < cnt[side];
+      const int kb = !listed ? 0 : base == 0 ? first[side] : src[side][base + lane];
       const bool valid = kb >= 0 && kb < nb;
-      if (base + lane < cnt && valid) atomicOr(bits + side * words + (kb >> 5), 1u << (kb & 31));
+      if (listed && valid) atomicOr(bits + side * words + (kb >> 5), 1u << (kb & 31));
       bad = __any_sync(0xffffffffu, !valid) || bad;
     }
   }
