@@ -133,9 +133,7 @@ int sparkattn_select_pooled(const sparkattn_shape_t* shape, int32_t topk, int32_
   if (nb > kSelectMaxBlocks) return SPARKATTN_E_UNSUPPORTED_SHAPE;
   if (!aligned256(workspace)) return SPARKATTN_E_MISALIGNED;
   if (workspace_bytes < select_workspace_bytes(*shape)) return SPARKATTN_E_WORKSPACE_TOO_SMALL;
-  cudaStream_t stream = static_cast<cudaStream_t>(cuda_stream);
-  if (cudaMemsetAsync(workspace, 0, kWorkspaceHeaderBytes, stream) != cudaSuccess) return SPARKATTN_E_CUDA;
-  return launch_select_pooled(*shape, topk, kept_idx, kept_cnt, workspace, stream);
+  return launch_select_pooled(*shape, topk, kept_idx, kept_cnt, workspace, static_cast<cudaStream_t>(cuda_stream));
 }
 
 int sparkattn_quant_fp8_per_token(const sparkattn_shape_t* shape, const void* x_bf16, uint8_t* codes,
