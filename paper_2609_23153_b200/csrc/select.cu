@@ -18,6 +18,7 @@
 //                     shared memory, packed fp32x2 FMAs over row pairs), then a warp per query block (or two) selects
 //                     the topk largest keys exactly (keys in registers for nb <= 1280) and compacts them in order.
 //   topk_wide_kernel  nb > 256: 16 or 8 query blocks per CTA of ten warps, pooled K straight from L2.
+//   list_all_kernel   in place of all of them when every block is kept.
 // The second is launched before the first has drained (programmatic dependent launch) and waits inside.
 #include "common.cuh"
 #include "launch.h"
@@ -345,6 +346,16 @@ __device__ __forceinline__ void select_rows_regs(const uint32_t* const (&key)[NR
   }
 }
 
+// Causal frame window (Sec. 1, auto-regressive extension): only the key blocks that hold a key some row of query block i may
+// attend to are candidates, a contiguous run jlo..jhi.
+__device__ __forceinline__ void window_range(int i, int N, int blk_size, int frame_tokens, int window, int& jlo, int& jhi) {
+  const int r0 = i * blk_size, r1 = min((i + 1) * blk_size, N) - 1;
+  const int f0 = max(r0 / frame_tokens - window + 1, 0);
+  const int kend = (int)min((long long)(r1 / frame_tokens + 1) * frame_tokens, (long long)N);
+  jlo = (int)((long long)f0 * frame_tokens / blk_size);
+  jhi = (kend - 1) / blk_size;
+}
+
 // Selection of a CTA's rows from their keys in shared memory: a warp takes rows WARPS apart, NR of them at a time.
 // SHORT: nb <= 256, otherwise more.
 template <bool WINDOW, int WARPS, int NR, bool SHORT>
@@ -352,7 +363,6 @@ __device__ __forceinline__ void select_tile(const uint32_t* s_key, int nb, int n
                                             int blk_size, int frame_tokens, int window, int32_t* __restrict__ kept_idx,
                                             int32_t* __restrict__ kept_cnt) {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const bool all = topk >= nb;        // with all candidates kept there is nothing to compare
   for (int first = warp; first < nrows; first += WARPS * NR) {
     const uint32_t* key[NR];
     int32_t* dst[NR];
@@ -362,27 +372,17 @@ __device__ __forceinline__ void select_tile(const uint32_t* s_key, int nb, int n
       const int row = first + WARPS * r < nrows ? first + WARPS * r : first;        // (beyond the last row: the first one again)
       key[r] = s_key + (int64_t)row * nbp;
       dst[r] = kept_idx + (bh * nb + i0 + row) * (int64_t)topk;
-      // Causal frame window (Sec. 1, auto-regressive extension): only the key blocks that hold a key some
-      // row of this query block may attend to are candidates, a contiguous run jlo..jhi.
       jlo[r] = 0;
       jhi[r] = nb - 1;
       if constexpr (WINDOW) {
-        const int r0 = (i0 + row) * blk_size, r1 = min((i0 + row + 1) * blk_size, N) - 1;
-        const int f0 = max(r0 / frame_tokens - window + 1, 0);
-        const int kend = (int)min((long long)(r1 / frame_tokens + 1) * frame_tokens, (long long)N);
-        jlo[r] = (int)((long long)f0 * frame_tokens / blk_size);
-        jhi[r] = (kend - 1) / blk_size;
+        window_range(i0 + row, N, blk_size, frame_tokens, window, jlo[r], jhi[r]);
       }
       k_row[r] = min(topk, jhi[r] - jlo[r] + 1);
       if constexpr (WINDOW)
         for (int t = k_row[r] + lane; t < topk; t += 32) dst[r][t] = -1;    // unused tail of a list cut short by the window
       if (lane == 0 && kept_cnt != nullptr) kept_cnt[bh * nb + i0 + row] = k_row[r];
     }
-    if (all) {
-#pragma unroll
-      for (int r = 0; r < NR; ++r)
-        for (int t = lane; t < k_row[r]; t += 32) dst[r][t] = jlo[r] + t;
-    } else if constexpr (SHORT) {       // nb <= 256
+    if constexpr (SHORT) {       // nb <= 256
       select_rows_regs<8, WINDOW, NR>(key, nb, jlo, jhi, k_row, lane, dst);
     } else if (nb <= 32 * 20) {
       select_rows_regs<20, WINDOW, NR>(key, nb, jlo, jhi, k_row, lane, dst);
@@ -453,8 +453,6 @@ topk_kernel(const float* pq, const float* pkT, int32_t* __restrict__ kept_idx,
 
   constexpr int kSteps = D / KC;                                      // stages per sweep over JT key blocks
   const int steps = (nbp + JT - 1) / JT * kSteps;
-  // with all candidates kept there is nothing to compare
-  const bool all = topk >= nb;
   auto issue = [&](int step) {
     if (step < steps) {
       const int j0 = step / kSteps * JT, c0 = step % kSteps * KC;
@@ -472,66 +470,64 @@ topk_kernel(const float* pq, const float* pkT, int32_t* __restrict__ kept_idx,
 
   pdl_wait();
   clear_header(header);
-  if (!all) {
 #pragma unroll
-    for (int p = 0; p < NS - 1; ++p) issue(p);
-    for (int e = threadIdx.x; e < R * (D / 4); e += kTopkThreads) {
-      const int r = e % R, c = e / R * 4;
-      const float4 x = r < nrows ? *reinterpret_cast<const float4*>(pq + (bh * nb + i0 + r) * D + c)
-                                 : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-      s_pq[c * R + r] = x.x; s_pq[(c + 1) * R + r] = x.y; s_pq[(c + 2) * R + r] = x.z; s_pq[(c + 3) * R + r] = x.w;
-    }
+  for (int p = 0; p < NS - 1; ++p) issue(p);
+  for (int e = threadIdx.x; e < R * (D / 4); e += kTopkThreads) {
+    const int r = e % R, c = e / R * 4;
+    const float4 x = r < nrows ? *reinterpret_cast<const float4*>(pq + (bh * nb + i0 + r) * D + c)
+                               : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+    s_pq[c * R + r] = x.x; s_pq[(c + 1) * R + r] = x.y; s_pq[(c + 2) * R + r] = x.z; s_pq[(c + 3) * R + r] = x.w;
+  }
 
-    // scores: a thread owns 4 adjacent key blocks and RT query blocks and walks the channels in ascending order.
-    // fma.rn.f32x2 is a pair of IEEE fmaf over two rows, so every accumulator sees exactly the chain
-    // a = fmaf(pq[i,c], pk[j,c], a), c ascending.  Columns nb..nbp-1 of pooled K are padding whose scores are stored
-    // but never read.
-    constexpr int kPairs = RT / 2;
-    const int rg = warp % RG, jc = warp / RG * 128 + lane * 4;        // first row of the thread: rg * RT; its column in the sweep
-    for (int j0 = 0, step = 0; j0 < nbp; j0 += JT) {
-      uint64_t acc[4][kPairs];
+  // scores: a thread owns 4 adjacent key blocks and RT query blocks and walks the channels in ascending order.
+  // fma.rn.f32x2 is a pair of IEEE fmaf over two rows, so every accumulator sees exactly the chain
+  // a = fmaf(pq[i,c], pk[j,c], a), c ascending.  Columns nb..nbp-1 of pooled K are padding whose scores are stored
+  // but never read.
+  constexpr int kPairs = RT / 2;
+  const int rg = warp % RG, jc = warp / RG * 128 + lane * 4;        // first row of the thread: rg * RT; its column in the sweep
+  for (int j0 = 0, step = 0; j0 < nbp; j0 += JT) {
+    uint64_t acc[4][kPairs];
 #pragma unroll
-      for (int u = 0; u < 4; ++u)
+    for (int u = 0; u < 4; ++u)
 #pragma unroll
-        for (int r = 0; r < kPairs; ++r) acc[u][r] = pack_f32x2(0.0f, 0.0f);
-      const bool mine = j0 + warp / RG * 128 < nbp;                   // the warp has a key block in this sweep
+      for (int r = 0; r < kPairs; ++r) acc[u][r] = pack_f32x2(0.0f, 0.0f);
+    const bool mine = j0 + warp / RG * 128 < nbp;                   // the warp has a key block in this sweep
 #pragma unroll 1
-      for (int s = 0; s < kSteps; ++s, ++step) {
-        cp_async_wait<NS - 2>();
-        __syncthreads();                 // this stage has landed for everybody, and the slot of the last one is free
-        issue(step + NS - 1);
-        if (mine) {
-          const float* kst = s_ring + step % NS * Shape::kStageFloats + jc;
-          const float* qst = s_pq + s * KC * R + rg * RT;
+    for (int s = 0; s < kSteps; ++s, ++step) {
+      cp_async_wait<NS - 2>();
+      __syncthreads();                 // this stage has landed for everybody, and the slot of the last one is free
+      issue(step + NS - 1);
+      if (mine) {
+        const float* kst = s_ring + step % NS * Shape::kStageFloats + jc;
+        const float* qst = s_pq + s * KC * R + rg * RT;
 #pragma unroll
-          for (int cc = 0; cc < KC; ++cc) {
-            uint64_t q2[kPairs];
-            if constexpr (RT >= 4) {
+        for (int cc = 0; cc < KC; ++cc) {
+          uint64_t q2[kPairs];
+          if constexpr (RT >= 4) {
 #pragma unroll
-              for (int g = 0; g < RT / 4; ++g) {
-                const ulonglong2 t = *reinterpret_cast<const ulonglong2*>(qst + cc * R + 4 * g);   // rows (4g, 4g+1), (4g+2, 4g+3)
-                q2[2 * g] = t.x;
-                q2[2 * g + 1] = t.y;
-              }
-            } else {
-              q2[0] = *reinterpret_cast<const uint64_t*>(qst + cc * R);
+            for (int g = 0; g < RT / 4; ++g) {
+              const ulonglong2 t = *reinterpret_cast<const ulonglong2*>(qst + cc * R + 4 * g);   // rows (4g, 4g+1), (4g+2, 4g+3)
+              q2[2 * g] = t.x;
+              q2[2 * g + 1] = t.y;
             }
-            const float4 kv = *reinterpret_cast<const float4*>(kst + cc * JT);
-            const uint64_t k2[4] = {pack_f32x2(kv.x, kv.x), pack_f32x2(kv.y, kv.y), pack_f32x2(kv.z, kv.z),
-                                    pack_f32x2(kv.w, kv.w)};
-#pragma unroll
-            for (int u = 0; u < 4; ++u)
-#pragma unroll
-              for (int r = 0; r < kPairs; ++r) acc[u][r] = ffma2(q2[r], k2[u], acc[u][r]);
+          } else {
+            q2[0] = *reinterpret_cast<const uint64_t*>(qst + cc * R);
           }
+          const float4 kv = *reinterpret_cast<const float4*>(kst + cc * JT);
+          const uint64_t k2[4] = {pack_f32x2(kv.x, kv.x), pack_f32x2(kv.y, kv.y), pack_f32x2(kv.z, kv.z),
+                                  pack_f32x2(kv.w, kv.w)};
+#pragma unroll
+          for (int u = 0; u < 4; ++u)
+#pragma unroll
+            for (int r = 0; r < kPairs; ++r) acc[u][r] = ffma2(q2[r], k2[u], acc[u][r]);
         }
       }
-      if (j0 + jc < nbp) {
-        store_keys<kPairs>(acc, s_key + (int64_t)(rg * RT) * nbp + j0 + jc, nbp);
-      }
     }
-    __syncthreads();
+    if (j0 + jc < nbp) {
+      store_keys<kPairs>(acc, s_key + (int64_t)(rg * RT) * nbp + j0 + jc, nbp);
+    }
   }
+  __syncthreads();
 
   select_tile<WINDOW, 8, (R >= 16 ? 2 : 1), true>(s_key, nb, nbp, topk, bh, i0, nrows, N, blk_size, frame_tokens, window, kept_idx, kept_cnt);
 }
@@ -557,62 +553,79 @@ topk_wide_kernel(const float* pq, const float* pkT, int32_t* __restrict__ kept_i
 
   pdl_wait();
   clear_header(header);
-  if (topk < nb) {
-    for (int e = threadIdx.x; e < R * (D / 4); e += kThreads) {
-      const int r = e % R, c = e / R * 4;
-      const float4 x = r < nrows ? *reinterpret_cast<const float4*>(pq + (bh * nb + i0 + r) * D + c)
-                                 : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-      s_pq[c * R + r] = x.x; s_pq[(c + 1) * R + r] = x.y; s_pq[(c + 2) * R + r] = x.z; s_pq[(c + 3) * R + r] = x.w;
-    }
-    __syncthreads();
-    const float* kcol = pkT + bh * D * (int64_t)nbp;
-    const ulonglong2* s_pq2 = reinterpret_cast<const ulonglong2*>(s_pq);       // [D][R / 4]
-    constexpr int RG = R / RT, kPairs = RT / 2;
-    constexpr int kCB = 4;   // channels per batch of loads
-    const int rg = (threadIdx.x >> 5) % RG;
-    for (int j0 = (threadIdx.x / (32 * RG) * 32 + (threadIdx.x & 31)) * 4; j0 < nb; j0 += kThreads / RG * 4) {
-      uint64_t acc[4][kPairs];
-#pragma unroll
-      for (int u = 0; u < 4; ++u)
-#pragma unroll
-        for (int r = 0; r < kPairs; ++r) acc[u][r] = pack_f32x2(0.0f, 0.0f);
-      const float* kp = kcol + j0;
-      auto load_batch = [&](float4 (&kv)[kCB], int c0) {
-#pragma unroll
-        for (int cc = 0; cc < kCB; ++cc) kv[cc] = *reinterpret_cast<const float4*>(kp + (int64_t)(c0 + cc) * nbp);
-      };
-      auto fma_batch = [&](const float4 (&kv)[kCB], int c0) {
-#pragma unroll
-        for (int cc = 0; cc < kCB; ++cc) {
-          uint64_t q2[kPairs];
-#pragma unroll
-          for (int g = 0; g < RT / 4; ++g) {
-            const ulonglong2 t = s_pq2[(c0 + cc) * (R / 4) + rg * (RT / 4) + g];   // rows (4g, 4g+1), (4g+2, 4g+3)
-            q2[2 * g] = t.x;
-            q2[2 * g + 1] = t.y;
-          }
-          const uint64_t k2[4] = {pack_f32x2(kv[cc].x, kv[cc].x), pack_f32x2(kv[cc].y, kv[cc].y),
-                                  pack_f32x2(kv[cc].z, kv[cc].z), pack_f32x2(kv[cc].w, kv[cc].w)};
-#pragma unroll
-          for (int u = 0; u < 4; ++u)
-#pragma unroll
-            for (int r = 0; r < kPairs; ++r) acc[u][r] = ffma2(q2[r], k2[u], acc[u][r]);
-        }
-      };
-      float4 kva[kCB], kvb[kCB];
-      load_batch(kva, 0);
-#pragma unroll 1
-      for (int c0 = 0; c0 < D; c0 += 2 * kCB) {
-        load_batch(kvb, c0 + kCB);
-        fma_batch(kva, c0);
-        if (c0 + 2 * kCB < D) load_batch(kva, c0 + 2 * kCB);
-        fma_batch(kvb, c0 + kCB);
-      }
-      store_keys<kPairs>(acc, s_key + (int64_t)(rg * RT) * nbp + j0, nbp);
-    }
-    __syncthreads();
+  for (int e = threadIdx.x; e < R * (D / 4); e += kThreads) {
+    const int r = e % R, c = e / R * 4;
+    const float4 x = r < nrows ? *reinterpret_cast<const float4*>(pq + (bh * nb + i0 + r) * D + c)
+                               : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+    s_pq[c * R + r] = x.x; s_pq[(c + 1) * R + r] = x.y; s_pq[(c + 2) * R + r] = x.z; s_pq[(c + 3) * R + r] = x.w;
   }
+  __syncthreads();
+  const float* kcol = pkT + bh * D * (int64_t)nbp;
+  const ulonglong2* s_pq2 = reinterpret_cast<const ulonglong2*>(s_pq);       // [D][R / 4]
+  constexpr int RG = R / RT, kPairs = RT / 2;
+  constexpr int kCB = 4;   // channels per batch of loads
+  const int rg = (threadIdx.x >> 5) % RG;
+  for (int j0 = (threadIdx.x / (32 * RG) * 32 + (threadIdx.x & 31)) * 4; j0 < nb; j0 += kThreads / RG * 4) {
+    uint64_t acc[4][kPairs];
+#pragma unroll
+    for (int u = 0; u < 4; ++u)
+#pragma unroll
+      for (int r = 0; r < kPairs; ++r) acc[u][r] = pack_f32x2(0.0f, 0.0f);
+    const float* kp = kcol + j0;
+    auto load_batch = [&](float4 (&kv)[kCB], int c0) {
+#pragma unroll
+      for (int cc = 0; cc < kCB; ++cc) kv[cc] = *reinterpret_cast<const float4*>(kp + (int64_t)(c0 + cc) * nbp);
+    };
+    auto fma_batch = [&](const float4 (&kv)[kCB], int c0) {
+#pragma unroll
+      for (int cc = 0; cc < kCB; ++cc) {
+        uint64_t q2[kPairs];
+#pragma unroll
+        for (int g = 0; g < RT / 4; ++g) {
+          const ulonglong2 t = s_pq2[(c0 + cc) * (R / 4) + rg * (RT / 4) + g];   // rows (4g, 4g+1), (4g+2, 4g+3)
+          q2[2 * g] = t.x;
+          q2[2 * g + 1] = t.y;
+        }
+        const uint64_t k2[4] = {pack_f32x2(kv[cc].x, kv[cc].x), pack_f32x2(kv[cc].y, kv[cc].y),
+                                pack_f32x2(kv[cc].z, kv[cc].z), pack_f32x2(kv[cc].w, kv[cc].w)};
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+#pragma unroll
+          for (int r = 0; r < kPairs; ++r) acc[u][r] = ffma2(q2[r], k2[u], acc[u][r]);
+      }
+    };
+    float4 kva[kCB], kvb[kCB];
+    load_batch(kva, 0);
+#pragma unroll 1
+    for (int c0 = 0; c0 < D; c0 += 2 * kCB) {
+      load_batch(kvb, c0 + kCB);
+      fma_batch(kva, c0);
+      if (c0 + 2 * kCB < D) load_batch(kva, c0 + 2 * kCB);
+      fma_batch(kvb, c0 + kCB);
+    }
+    store_keys<kPairs>(acc, s_key + (int64_t)(rg * RT) * nbp + j0, nbp);
+  }
+  __syncthreads();
   select_tile<WINDOW, WARPS, 1, false>(s_key, nb, nbp, topk, bh, i0, nrows, N, blk_size, frame_tokens, window, kept_idx, kept_cnt);
+}
+
+// topk = nb: every candidate is kept whatever its score, so nothing is pooled and nothing compared.  A warp per list.
+// (Pooled and scored all the same, and then listed: attention over all blocks, 6 heads of 6,479 tokens, 150.2 us, now 143.0;
+// 3 heads in a causal window of three frames 36.2, now 31.1.)
+constexpr int kAllWarps = 8;
+__global__ void __launch_bounds__(kAllWarps * 32)
+list_all_kernel(int32_t* __restrict__ kept_idx, int32_t* __restrict__ kept_cnt, int64_t lists, int nb, int N, int blk_size,
+                int frame_tokens, int window, int32_t* __restrict__ header) {
+  pdl_wait();
+  clear_header(header);
+  const int lane = threadIdx.x & 31;
+  for (int64_t w = (int64_t)blockIdx.x * kAllWarps + (threadIdx.x >> 5); w < lists; w += (int64_t)gridDim.x * kAllWarps) {
+    int jlo = 0, jhi = nb - 1;
+    if (frame_tokens > 0) window_range((int)(w % nb), N, blk_size, frame_tokens, window, jlo, jhi);
+    int32_t* dst = kept_idx + w * nb;
+    for (int t = lane; t < nb; t += 32) dst[t] = jlo + t <= jhi ? jlo + t : -1;
+    if (lane == 0 && kept_cnt != nullptr) kept_cnt[w] = jhi - jlo + 1;
+  }
 }
 
 // The limit of a kernel's dynamic shared memory belongs to the kernel, not to a launch: it is always set to the most that any
@@ -694,6 +707,14 @@ static int launch_topk_d(const sparkattn_shape_t& s, int topk, int frame_tokens,
   return go(launch_topk<D, 2, 4, 16, 4>);
 }
 
+static int launch_list_all(const sparkattn_shape_t& s, int frame_tokens, int window, int32_t* kept_idx, int32_t* kept_cnt, int32_t* header,
+                           cudaStream_t stream) {
+  const int nb = (s.N + s.block - 1) / s.block;
+  const int64_t lists = (int64_t)s.B * s.H * nb, ctas = (lists + kAllWarps - 1) / kAllWarps;
+  return launch_kernel(list_all_kernel, (unsigned)(ctas < 4096 ? ctas : 4096), kAllWarps * 32, 0, true, stream, kept_idx, kept_cnt, lists, nb,
+                       s.N, s.block, frame_tokens, window, header);
+}
+
 static int launch_topk_any(const sparkattn_shape_t& s, int topk, int frame_tokens, int window, int32_t* kept_idx,
                            int32_t* kept_cnt, void* workspace, int32_t* header, cudaStream_t stream) {
   if (s.d == 128) return launch_topk_d<128>(s, topk, frame_tokens, window, kept_idx, kept_cnt, workspace, header, stream);
@@ -705,6 +726,8 @@ int launch_select_pooled(const sparkattn_shape_t& s, int topk, int32_t* kept_idx
                          cudaStream_t stream) {
   const int nb = (s.N + s.block - 1) / s.block;
   if (nb > kSelectMaxBlocks) return SPARKATTN_E_UNSUPPORTED_SHAPE;
+  if (s.d != 128 && s.d != 64) return SPARKATTN_E_UNSUPPORTED_SHAPE;
+  if (topk >= nb) return launch_list_all(s, 0, 0, kept_idx, kept_cnt, static_cast<int32_t*>(workspace), stream);
   const int rc = launch_topk_any(s, topk, 0, 0, kept_idx, kept_cnt, workspace, static_cast<int32_t*>(workspace), stream);
   if (rc != SPARKATTN_OK) return rc;
   return cudaGetLastError() == cudaSuccess ? SPARKATTN_OK : SPARKATTN_E_CUDA;
@@ -721,6 +744,7 @@ int launch_select(const sparkattn_shape_t& s, const void* q, const void* k, int 
   const __nv_bfloat16* qb = static_cast<const __nv_bfloat16*>(q);
   const __nv_bfloat16* kb = static_cast<const __nv_bfloat16*>(k);
   if (s.d != 128 && s.d != 64) return SPARKATTN_E_UNSUPPORTED_SHAPE;
+  if (topk >= nb) return launch_list_all(s, frame_tokens, window, kept_idx, kept_cnt, static_cast<int32_t*>(workspace), stream);
   const int sm_count = current_sm_count();
   if (sm_count < 1) return SPARKATTN_E_CUDA;
   const size_t pool_smem = (size_t)2 * s.block * s.d * 2;

@@ -21,6 +21,27 @@ def _relrms(got, ref):
     return math.sqrt(float(((got - ref) ** 2).sum()) / max(float((ref ** 2).sum()), 1e-300)), float((got - ref).abs().max())
 
 
+@pytest.mark.parametrize("block,d,N,F,window,pooled", [(128, 128, 1150, 230, 2, False), (64, 64, 64 * 9 + 1, 100, 1, False),
+                                                       (64, 128, 5, 5, 3, False), (128, 128, 128 * 33, 128, 40, False), (64, 128, 64 * 9 + 1, 0, 0, True)])
+def test_every_block_asked_for(block, d, N, F, window, pooled):
+    """topk = nb takes a kernel of its own, which lists the candidates without scores: those of the oracle under a
+    window (counts, unused tails), all blocks on means pooled by the quantisation; the status is clean in a workspace of any content."""
+    g = torch.Generator().manual_seed(N)
+    q, k = (torch.randn((1, 3, N, d), generator=g).to(torch.bfloat16).to(DEV) for _ in range(2))
+    nb = -(-N // block)
+    ws = sa.alloc_workspace(sa.make_shape(q, block), 0, nb, DEV)
+    ws.fill_(0xA5)
+    if pooled:
+        sa.quant_fp8_pooled(q, block, False, ws), sa.quant_fp8_pooled(k, block, True, ws)
+        idx, cnt = sa.select_pooled(q, block, nb, ws)
+        want, count = oracle.select(q[0].cpu(), k[0].cpu(), block, nb)
+    else:
+        idx, cnt = sa.select(q, k, block, nb, frame_tokens=F, window=window, workspace=ws)
+        want, count = oracle.select(q[0].cpu(), k[0].cpu(), block, nb, frame_tokens=F, window=window)
+    assert torch.equal(idx[0].cpu(), want) and torch.equal(cnt[0].cpu(), count)
+    assert sa.read_status(ws) == sa.OK
+
+
 @pytest.mark.parametrize("H,d,grid,block,topk,window", [
     (2, 128, (6, 10, 23), 128, 4, 2),      # frames of 230 tokens straddle the 128-token blocks; ragged tail
     (3, 128, (12, 12, 15), 128, 6, 3),     # 180-token frames, 17 blocks per head
