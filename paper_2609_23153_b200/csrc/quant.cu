@@ -142,11 +142,24 @@ quant_fp8_pool_kernel(const __nv_bfloat16* x, uint8_t* __restrict__ codes, float
   amax = block_absmax(amax, s_red);
   const float inv = __fdiv_rn(448.0f, amax);
   if (threadIdx.x == 0) scales[(int64_t)bh * nb + blk] = __fdiv_rn(amax, 448.0f);
+  if constexpr (BLK == 128) {
+    // The threads of the columns go straight to them, the others encode for them.  40 heads of 75,600 tokens, two boards: 209.8 ->
+    // 201.3 and 201.0 -> 196.9 us per tensor, 12 of 32,760 30.2 -> 29.7, 20 of 6,479 10.6 -> 10.2.  With 64-token blocks, whose
+    // columns are half as long, everybody encodes first (225 us, 239 the other way).
+    if (threadIdx.x >= D / 2) {
+#pragma unroll 4
+      for (int ci = threadIdx.x - D / 2; ci < nvalid * kChunksPerRow; ci += kQuantThreads - D / 2) {
+        const int r = ci / kChunksPerRow, cc = ci % kChunksPerRow;
+        *reinterpret_cast<uint2*>(codes + base + r * stride_n + cc * 8) = encode8(reinterpret_cast<const uint4*>(tile)[ci], inv);
+      }
+    }
+  } else {
 #pragma unroll
-  for (int i = 0; i < kPerThread; ++i) {
-    const int ci = threadIdx.x + i * kQuantThreads, r = ci / kChunksPerRow, cc = ci % kChunksPerRow;
-    if (r < nvalid)
-      *reinterpret_cast<uint2*>(codes + base + r * stride_n + cc * 8) = encode8(reinterpret_cast<const uint4*>(tile)[ci], inv);
+    for (int i = 0; i < kPerThread; ++i) {
+      const int ci = threadIdx.x + i * kQuantThreads, r = ci / kChunksPerRow, cc = ci % kChunksPerRow;
+      if (r < nvalid)
+        *reinterpret_cast<uint2*>(codes + base + r * stride_n + cc * 8) = encode8(reinterpret_cast<const uint4*>(tile)[ci], inv);
+    }
   }
   if (threadIdx.x < D / 2) {
     const uint32_t* col = reinterpret_cast<const uint32_t*>(tile) + threadIdx.x;      // channels 2t and 2t + 1
