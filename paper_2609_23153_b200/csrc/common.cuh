@@ -13,11 +13,33 @@ namespace sparkattn {
 // Layout of the 256-byte header at the start of every workspace.
 //   word 0: device status (0 = OK, else a negative sparkattn_status)
 //   word 1: detail (offending index, or an id of the wait that expired)
-//   word 2: dynamic work counter of the persistent forward kernel
+//   word 2: how often a kernel has cleared the first two by itself (see header_begin)
 constexpr int kWorkspaceHeaderBytes = 256;
+constexpr int kHeaderTurnWord = 2;
 
 __device__ __forceinline__ void report_status(int32_t* status, int code, int detail) {
   if (atomicCAS(status, 0, code) == 0) status[1] = detail;
+}
+
+// Every call starts with a clean status.  Mostly a small kernel in front sees to it; a kernel that fills the device once at most
+// can do it itself: its first CTA clears the words and counts up, every CTA notes the count when it starts, and one with
+// something to report waits until the count has moved since (or for a millisecond, if it had moved already).  One
+// thread each; the memory may hold anything before.
+__device__ __forceinline__ int32_t header_begin(int32_t* status, bool first_cta) {
+  volatile int32_t* turn = status + kHeaderTurnWord;
+  const int32_t before = *turn;
+  if (first_cta) {
+    status[0] = 0;
+    status[1] = 0;
+    __threadfence();
+    *turn = before + 1;
+  }
+  return before;
+}
+__device__ __forceinline__ void header_await(int32_t* status, int32_t before) {
+  const volatile int32_t* turn = status + kHeaderTurnWord;
+  for (int i = 0; i < 1000 && *turn == before; ++i) __nanosleep(1000);
+  __threadfence();
 }
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p) {

@@ -29,7 +29,7 @@
 // 8,000, 125 of 125 520 -> 410; 40 heads of 32,760, 15 of 512 1020 -> 900.
 //
 // Every wait on an mbarrier is bounded (common.cuh); a kept index outside
-// [0, nb) is reported in the status word and its tile skipped by all roles.
+// [0, nb) is skipped by all roles and reported in the status word when the CTA winds down.
 #include <cuda.h>
 
 #include "common.cuh"
@@ -98,6 +98,7 @@ fwd_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant__ C
   uint32_t* s_tmem_base = reinterpret_cast<uint32_t*>(bars + 51);
   volatile int* s_abort = reinterpret_cast<volatile int*>(bars + 52);
   int* s_ntiles = reinterpret_cast<int*>(bars + 53);
+  int* s_bad = s_ntiles + 1;          // place of an invalid index in the list, or -1
   float2* s_sums = reinterpret_cast<float2*>(smem + Smem::kSums);
   int32_t* s_list = reinterpret_cast<int32_t*>(smem + Smem::kList);   // validated kept block indices
   auto tile_k = [&](int c, int slot) { return smem + Smem::kKV + (c * 4 + slot * 2) * kFwdPair; };
@@ -135,23 +136,37 @@ fwd_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant__ C
     tmem_relinquish();
   }
   pdl_wait();
-  // a timeout recorded by an earlier CTA of this launch makes the rest of the grid drain at once
-  if (threadIdx.x == 0) *s_abort = (*reinterpret_cast<volatile int32_t*>(p.status) == SPARKATTN_E_DEVICE_TIMEOUT) ? 1 : 0;
+  // C = 2 is one wave of CTAs at most and clears the status itself (64 items of 16 tiles 9.5 us, 10.2 with a kernel in front for it;
+  // one launch less: of 3 tiles 6.1 and 8.4); C = 1 has it cleared, and a timeout recorded by an earlier
+  // CTA of the launch makes the rest of the grid drain at once
+  int32_t turn = 0;
+  if (threadIdx.x == 0) {
+    if constexpr (C == 2) {
+      turn = header_begin(p.status, blockIdx.x == 0);
+      *s_abort = 0;
+    } else {
+      *s_abort = (*reinterpret_cast<volatile int32_t*>(p.status) == SPARKATTN_E_DEVICE_TIMEOUT) ? 1 : 0;
+    }
+  }
   if (warp == kMmaWarp) {
-    // Stage the kept list in shared memory, in order, dropping (and reporting) indices outside [0, nb).
+    // Stage the kept list in shared memory, in order, dropping (and noting, for the report at the end) indices outside [0, nb).
     const int cnt = p.kept_cnt ? min(max(p.kept_cnt[(int64_t)bh * p.nb + qb], 0), p.kmax) : p.kmax;
     const int32_t* list = p.kept_idx + ((int64_t)bh * p.nb + qb) * p.kmax;
-    int out = 0;
+    int out = 0, bad = -1;                          // bad: place in the list of one of them
     for (int base = 0; base < cnt; base += 32) {
       const int t = base + lane;
       const int kb = (t < cnt) ? list[t] : 0;
       const bool valid = (t < cnt) && kb >= 0 && kb < p.nb;
-      if (t < cnt && !valid) report_status(p.status, SPARKATTN_E_BAD_INDEX, kb);
+      if (t < cnt && !valid) bad = t;
       const uint32_t ballot = __ballot_sync(0xffffffffu, valid);
       if (valid) s_list[out + __popc(ballot & ((1u << lane) - 1u))] = kb;
       out += __popc(ballot);
     }
-    if (lane == 0) *s_ntiles = out;
+    bad = __reduce_max_sync(0xffffffffu, bad);
+    if (lane == 0) {
+      *s_ntiles = out;
+      *s_bad = bad;
+    }
   }
   tc_fence_before();
   __syncthreads();
@@ -187,7 +202,7 @@ fwd_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant__ C
         tc_commit(bar_s_full(c));
         tc_commit(bar_k_free(c, n & 1));
       };
-      bool ok = mbar_wait(bar_q_full, 0, s_abort, p.status, 3) && mbar_wait(bar_k_full(c, 0), 0, s_abort, p.status, 5);
+      bool ok = pipe_wait(bar_q_full, 0, s_abort, 3) && pipe_wait(bar_k_full(c, 0), 0, s_abort, 5);
       if (ok) {
         tc_fence_after();
         issue_s(0);
@@ -195,14 +210,14 @@ fwd_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant__ C
       for (int n = 0; ok && n < mine; ++n) {
         const int slot = n & 1;
         if (n + 1 < mine) {
-          ok = mbar_wait(bar_k_full(c, slot ^ 1), ((n + 1) >> 1) & 1, s_abort, p.status, 5);
-          if (ok) ok = mbar_wait(bar_s_free(c), n & 1, s_abort, p.status, 4);
+          ok = pipe_wait(bar_k_full(c, slot ^ 1), ((n + 1) >> 1) & 1, s_abort, 5);
+          if (ok) ok = pipe_wait(bar_s_free(c), n & 1, s_abort, 4);
           if (!ok) break;
           tc_fence_after();
           issue_s(n + 1);
         }
-        ok = mbar_wait(bar_v_full(c, slot), (n >> 1) & 1, s_abort, p.status, 6);
-        if (ok) ok = mbar_wait(bar_p_full(c), n & 1, s_abort, p.status, 7);
+        ok = pipe_wait(bar_v_full(c, slot), (n >> 1) & 1, s_abort, 6);
+        if (ok) ok = pipe_wait(bar_p_full(c), n & 1, s_abort, 7);
         if (!ok) break;
         tc_fence_after();
         const uint64_t dV = make_smem_desc_sw128(smem_u32(tile_v(c, slot)), kFwdTile);      // the pair's tiles are two slabs of columns
@@ -227,11 +242,11 @@ fwd_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant__ C
       for (int n = 0; n < mine; ++n) {
         const int slot = n & 1;
         const int k0 = block_of(c, n, 0) * kBlk, k1 = block_of(c, n, 1) * kBlk;
-        if (n >= 2 && !mbar_wait(bar_k_free(c, slot), ((n >> 1) - 1) & 1, s_abort, p.status, 1)) break;
+        if (n >= 2 && !pipe_wait(bar_k_free(c, slot), ((n >> 1) - 1) & 1, s_abort, 1)) break;
         mbar_expect_tx(bar_k_full(c, slot), kFwdPair);
         tma_load_4d(tile_k(c, slot), &tmap_k, bar_k_full(c, slot), 0, k0, h, b);
         tma_load_4d(tile_k(c, slot) + kFwdTile, &tmap_k, bar_k_full(c, slot), 0, k1, h, b);
-        if (n >= 2 && !mbar_wait(bar_v_free(c, slot), ((n >> 1) - 1) & 1, s_abort, p.status, 2)) break;
+        if (n >= 2 && !pipe_wait(bar_v_free(c, slot), ((n >> 1) - 1) & 1, s_abort, 2)) break;
         mbar_expect_tx(bar_v_full(c, slot), kFwdPair);
         tma_load_4d(tile_v(c, slot), &tmap_v, bar_v_full(c, slot), 0, k0, h, b);
         tma_load_4d(tile_v(c, slot) + kFwdTile, &tmap_v, bar_v_full(c, slot), 0, k1, h, b);
@@ -261,7 +276,7 @@ fwd_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant__ C
     for (int n = 0; ok && n < mine; ++n) {
       const int kb = block_of(chain, n, half);
       const int c_lo = klo - kb * kBlk, c_hi = khi - kb * kBlk;      // this row's valid columns of the tile: [c_lo, c_hi)
-      ok = __all_sync(0xffffffffu, mbar_wait(bar_s_full(chain), n & 1, s_abort, p.status, 8));
+      ok = __all_sync(0xffffffffu, pipe_wait(bar_s_full(chain), n & 1, s_abort, 8));
       if (!ok) break;
       tc_fence_after();
       uint32_t sr[kBlk];
@@ -293,7 +308,7 @@ fwd_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant__ C
       // of 16 tiles 10.1 us, 10.3 with none); none where the stores of P should run under the exponentials (C = 1: 12 heads of
       // 8,000 tokens 410 us, two 432, all eight 450).
       constexpr int kWaitAt = C == 2 ? 2 : 0;
-      auto wait_pv = [&]() { return n == 0 || __all_sync(0xffffffffu, mbar_wait(bar_pv_done(chain), (n - 1) & 1, s_abort, p.status, 10)); };
+      auto wait_pv = [&]() { return n == 0 || __all_sync(0xffffffffu, pipe_wait(bar_pv_done(chain), (n - 1) & 1, s_abort, 10)); };
       const bool rescale = __any_sync(0xffffffffu, need);
       if (rescale) {
         ok = wait_pv();
@@ -353,13 +368,13 @@ fwd_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant__ C
     }
 
     // ---------------------------------------------------------------- merge of the half chains and epilogue
-    if (ok && mine > 0) ok = __all_sync(0xffffffffu, mbar_wait(bar_pv_done(chain), (mine - 1) & 1, s_abort, p.status, 9));
+    if (ok && mine > 0) ok = __all_sync(0xffffffffu, pipe_wait(bar_pv_done(chain), (mine - 1) & 1, s_abort, 9));
     const int part = chain * 2 + half;
     if (ok) {
       tc_fence_after();
       s_sums[part * 64 + row] = make_float2(m_used, l);
       mbar_arrive(bar_sums);
-      ok = __all_sync(0xffffffffu, mbar_wait(bar_sums, 0, s_abort, p.status, 11));
+      ok = __all_sync(0xffffffffu, pipe_wait(bar_sums, 0, s_abort, 11));
     }
     if (ok) {
       // every product of the CTA is complete: the K / V slots are free for the weighted O of the half chains
@@ -396,7 +411,7 @@ fwd_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant__ C
         }
       }
       mbar_arrive(bar_parts);
-      ok = __all_sync(0xffffffffu, mbar_wait(bar_parts, 0, s_abort, p.status, 12));
+      ok = __all_sync(0xffffffffu, pipe_wait(bar_parts, 0, s_abort, 12));
       if (ok && row_valid) {
         // this half chain's threads write columns [64 / 2C * part, +64 / 2C) of the row
         constexpr int kCols = kD / (2 * C);
@@ -428,6 +443,11 @@ fwd_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant__ C
   // ------------------------------------------------------------------ teardown
   tc_fence_before();
   __syncthreads();
+  if (threadIdx.x == 0 && (*s_abort >= kAbortTimeout || *s_bad >= 0)) {
+    if constexpr (C == 2) header_await(p.status, turn);
+    if (*s_bad >= 0) report_status(p.status, SPARKATTN_E_BAD_INDEX, p.kept_idx[((int64_t)bh * p.nb + qb) * p.kmax + *s_bad]);
+    report_abort(p.status, *s_abort);
+  }
   if (warp == kTmaWarp) {
     if (*s_abort) __nanosleep(200000);  // let copies / MMAs in flight land before the CTA's resources go
     tc_fence_after();
@@ -443,7 +463,7 @@ size_t fwd_workspace_bytes(const sparkattn_shape_t& s, int kmax) {
   return kWorkspaceHeaderBytes;
 }
 
-// clears the workspace header ahead of a kernel that reports into it
+// clears the workspace header ahead of a kernel that reports into it (C = 1, whose CTAs come in waves)
 __global__ void clear_header_kernel(int32_t* header) {
   pdl_trigger();
   pdl_wait();
@@ -496,10 +516,11 @@ int launch_fwd(const sparkattn_shape_t& s, int dtype, const void* q, const void*
   if (ctas > 0x7fffffffLL) return SPARKATTN_E_UNSUPPORTED_SHAPE;
   const int sm_count = current_sm_count();
   if (sm_count < 1) return SPARKATTN_E_CUDA;
-  if ((rc = launch_kernel(clear_header_kernel, 1, kWorkspaceHeaderBytes / 4, 0, true, stream, prm.status)) != SPARKATTN_OK) return rc;
   // two chains while no SM gets a second item, us against one chain and two CTAs per SM: 64 items of 16 tiles 10.3 / 11.5, 128 10.7 /
   // 11.9; but 160 19.0 / 14.2, 256 items of 3 tiles 12.3 / 8.1, 512 of 32 56.5 / 42.4
-  return ctas <= sm_count ? launch_fwd_t<2>(mq, mk, mv, prm, ctas, stream) : launch_fwd_t<1>(mq, mk, mv, prm, ctas, stream);
+  if (ctas <= sm_count) return launch_fwd_t<2>(mq, mk, mv, prm, ctas, stream);
+  if ((rc = launch_kernel(clear_header_kernel, 1, kWorkspaceHeaderBytes / 4, 0, true, stream, prm.status)) != SPARKATTN_OK) return rc;
+  return launch_fwd_t<1>(mq, mk, mv, prm, ctas, stream);
 }
 
 }  // namespace sparkattn

@@ -523,6 +523,23 @@ def test_d64_infinity_stays_where_it_belongs(H):
     assert torch.equal(out, clean)
 
 
+@pytest.mark.parametrize("H", [2, 5])
+def test_d64_status_in_a_workspace_of_any_content(H):
+    """d = 64: up to one item per SM (82 items) the forward clears its status itself, beyond (205) a kernel in front does.
+    Either way a call reports its own bad index and nothing that was in the workspace before."""
+    nb = 41
+    q = torch.randn((1, H, nb * 64, 64), generator=torch.Generator().manual_seed(H)).to(torch.bfloat16).to(DEV)
+    idx = torch.arange(nb, dtype=torch.int32, device=DEV)[None, None, :, None].expand(1, H, nb, 3).contiguous()
+    bad = idx.clone()
+    bad[0, H - 1, nb - 1, 1] = nb
+    for fill in (0x00, 0xA5, 0xFF):
+        ws = sa.alloc_workspace(sa.make_shape(q, 64), 1, 3, DEV)
+        ws.fill_(fill)
+        for lists, want in ((idx, sa.OK), (bad, sa.E_BAD_INDEX), (bad, sa.E_BAD_INDEX), (idx, sa.OK)):
+            sa.fwd(q, q, q, lists, None, 64, workspace=ws)
+            assert sa.read_status(ws) == want
+
+
 @pytest.mark.parametrize("H", [28, 56])
 def test_lse_of_merged_chains_is_rounded_once(H):
     """d = 64: scores that fp32 holds exactly and one key that outweighs the others, so that the log-sum-exp is off by its
