@@ -32,7 +32,8 @@
 //                    Both sleep in their barrier waits (everything a product needs is needed).
 // Work items (batch, head, query block) go to CTA c as c, c + grid, ... in head-major order, so
 // the CTAs running together read K/V of one head from L2.  Kept lists are range-checked and
-// compacted by a small pre-pass into the workspace; every role reads the clean lists from there.
+// compacted into the workspace, by a small pre-pass or, where a CTA has few items, by the CTA itself (launch_pipe has the
+// line); every role reads the clean lists from there.
 // Every wait is bounded; nothing here waits on another CTA.
 //
 // EPI variant (512 threads): warps 12-15 are a closing warpgroup.  At the end of an item the softmax warpgroups only
@@ -103,8 +104,8 @@ static FastDiv make_fast_div(uint32_t d) {
 __device__ __forceinline__ int fast_div(int x, FastDiv f) { return (int)((__umulhi((uint32_t)x, f.mul) + (uint32_t)x) >> f.shift); }
 
 struct PipeParams {
-  const int32_t* clean_cnt;    // [items] valid kept blocks per item
-  const int32_t* clean_list;   // [items][kmax] their indices, compacted in list order
+  int32_t* clean_cnt;          // [items] valid kept blocks per item
+  int32_t* clean_list;         // [items][kmax] their indices, compacted in list order
   const float* q_scale;        // FP8: [B*H*nb] dequantisation scales of the token blocks
   const float* k_scale;
   const float* v_scale;
@@ -119,6 +120,7 @@ struct PipeParams {
   FastDiv by_nbq, by_H;
   int nbq;                     // work items per (batch, head): query blocks, or pairs of 64-token query blocks
   int lstride;                 // list entries per item in clean_list
+  bool own_lists;              // there was no list pre-pass: every CTA cleans the lists of its items, and the status is cleared here
   int frame_tokens, window;    // causal frame window (0 = none): key frame in (query frame - window, query frame]
   const int32_t* blk_valid;    // [nb] real tokens per block (bricks padded to whole blocks), or NULL
   int64_t stride_b, stride_h, stride_n;
@@ -131,9 +133,10 @@ struct PipeParams {
   float eps;
 };
 
-// The list pre-passes are also what clears the workspace header, so they cannot report into it themselves (their CTAs
-// run in no order): an item with an index outside [0, nb) gets this flag in its count, and the forward kernel looks the
-// index up and reports it.
+// What cleans the lists also clears the workspace header, so it cannot report into it itself (its CTAs run in no order): an
+// item with an index outside [0, nb) gets this flag in its count, and the forward kernel looks the index up and reports
+// it when it winds down (out of the producers' loops, where the code for it took instruction cache from the tile loops: 40
+// heads of 75,600 tokens, 97 %, 0.995 of the time before, 64-token blocks 0.992).
 constexpr int32_t kBadFlag = 0x40000000;
 __device__ __forceinline__ int clean_count(const int32_t* clean_cnt, int item) { return clean_cnt[item] & ~kBadFlag; }
 __device__ __forceinline__ void report_bad_index(const PipeParams& p, int item, bool pair) {
@@ -400,6 +403,7 @@ fwd_pipe_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
   uint32_t* s_tmem = reinterpret_cast<uint32_t*>(s_lsum + 128);
   volatile int* s_abort = reinterpret_cast<volatile int*>(s_tmem + 1);
   volatile int* s_gate_bh = s_abort + 1;      // GATE: (batch, head) whose P_q and C are in shared memory
+  volatile int* s_bad = s_abort + 2;          // a list of this CTA's items held an invalid index
   // What the softmax warpgroups need to know of a tile, written by the K producer in the slot tile % 8 before it requests
   // the K tile: the number of real columns (WINDOW: the key block), PAIR with the flags of the two query blocks in bits
   // 30 and 31; FP8: K scale, log2 of the factor folded into P, its inverse.  PAIR: the same of the tile's second block.
@@ -435,6 +439,7 @@ fwd_pipe_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
       mbar_init(bar_cl, 128); mbar_init(bar_cl + 1, 128);
     }
     *s_gate_bh = -1;
+    *s_bad = 0;
     for (int i = 0; i < RK; ++i) { mbar_init(bar_k_full + i, 1); mbar_init(bar_k_free + i, 1); }
     for (int i = 0; i < RV; ++i) { mbar_init(bar_v_full + i, 1); mbar_init(bar_v_free + i, 1); }
     mbar_init(bar_o_free, 128); mbar_init(bar_lsum, 128); mbar_init(bar_lsum_ack, 128);
@@ -461,8 +466,19 @@ fwd_pipe_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
   // returns from this.  (The grid is one wave: there are no later CTAs that could look for a timeout of earlier ones.  With that look
   // and the line-up behind the wait: 3 heads of 1,200 tokens 9.0 us, 8.8 without, FP8 8.5 and 8.1, 40 of 6,479 106.6 and 105.3.)
   pdl_wait();
-  if (dead && threadIdx.x == 0) report_status(p.status, SPARKATTN_E_MISALIGNED, (int)(smem_u32(smem) & 1023u));
   const int first_item = blockIdx.x, item_step = gridDim.x;
+  int32_t turn = 0;
+  if constexpr (!FP8) {
+    if (p.own_lists) {
+      if (threadIdx.x == 0) turn = header_begin(p.status, blockIdx.x == 0);
+      for (int item = first_item + warp * item_step; item < p.items; item += (int)(blockDim.x >> 5) * item_step) {
+        if constexpr (PAIR) pair_list(p.kept_idx, p.kept_cnt, p.clean_cnt, p.clean_list, item, p.nb, p.nbq, p.kmax, warp, lane);
+        else compact_list(p.kept_idx, p.kept_cnt, p.clean_cnt, p.clean_list, item, p.nb, p.kmax, lane);
+      }
+      if constexpr (PAIR) asm volatile("fence.proxy.async.shared::cta;" ::: "memory");      // the lists' bitmaps lie where tiles go
+      __syncthreads();
+    }
+  }
   // A wait of a control warp.  bf16 with 128-token blocks runs at the chip's power limit: there one thread polls and
   // all learn of it (720p shape at 97 %: 2.86 ms, against 3.00 with 32 polling threads in 3 % fewer clocks).  The
   // others run at full clock and take the shorter way (the gated kernel: 8-11 % faster with it).
@@ -532,7 +548,7 @@ fwd_pipe_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
         cnt = uniform(cnt);
         if (cnt & kBadFlag) {
           cnt &= ~kBadFlag;
-          if (!is_v && lane == 0) report_bad_index(p, item, PAIR);
+          if (!is_v && lane == 0) *s_bad = 1;      // (reported when the CTA winds down: no code for it among the loops)
         }
         float inv_vmax = 1.0f;
         Desc d0{}, d1{};
@@ -1320,7 +1336,13 @@ fwd_pipe_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
   // ------------------------------------------------------------------ teardown
   tc_fence_before();
   __syncthreads();
-  if (threadIdx.x == 0) report_abort(p.status, *s_abort);
+  if (threadIdx.x == 0 && (dead || *s_abort || *s_bad)) {
+    if (!FP8 && p.own_lists) header_await(p.status, turn);
+    if (dead) report_status(p.status, SPARKATTN_E_MISALIGNED, (int)(smem_u32(smem) & 1023u));
+    for (int item = first_item; *s_bad && item < p.items; item += item_step)
+      if (p.clean_cnt[item] & kBadFlag) report_bad_index(p, item, PAIR);
+    report_abort(p.status, *s_abort);
+  }
   if (warp == 0) {
     if (*s_abort) __nanosleep(200000);  // let copies / MMAs in flight land before the CTA's resources go
     tc_fence_after();
@@ -1447,10 +1469,19 @@ static int launch_pipe(const sparkattn_shape_t& s, bool fp8, const void* q, cons
   }
   const size_t bits = pair ? (size_t)kPairWarps * 2 * ((nb + 31) / 32) * sizeof(uint32_t) : 0;
   const int warps = pair ? kPairWarps : kCompactWarps, heads = s.B * s.H;
+  // bf16, up to 16 items per CTA (a warp each, or two rounds of the warps): every CTA cleans the lists of its own items before it
+  // starts, and no kernel stands between the caller's last one and the forward.  Beyond, the pre-pass costs nothing that
+  // shows.  Attention, pre-pass / own lists, us: 3 heads of 1,200 tokens 17.9 / 17.5, 6 of 6,479 48.7 / 47.8 (64-token blocks 41.1 /
+  // 40.0, causal 50.2 / 49.4), 20 of 6,479 (6.9 items) 79.5 / 77.7, 40 of 6,479 (13.8) 148.2 / 147.2.  FP8 needs a kernel for the largest V
+  // scales all the same.
+  constexpr int kOwnItems = 16;
+  prm.own_lists = !fp8 && items <= (long long)kOwnItems * sm_count;
   if (fp8)
     rc = launch_kernel(pair ? head_vmax_kernel<true> : head_vmax_kernel<false>, (unsigned)((items + heads + warps - 1) / warps), warps * 32,
                        bits, true, stream, v_scale, v_max, heads, kept_idx, kept_cnt, clean_cnt, clean_list, (int)items, nb, nbq, kmax,
                        prm.status);
+  else if (prm.own_lists)
+    rc = SPARKATTN_OK;
   else if (pair)
     rc = launch_kernel(pair_lists_kernel, (unsigned)((items + warps - 1) / warps), warps * 32, bits, true, stream, kept_idx, kept_cnt,
                        clean_cnt, clean_list, (int)items, nb, nbq, kmax, prm.status);

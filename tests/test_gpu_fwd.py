@@ -226,6 +226,39 @@ def test_bad_indices_are_dropped_and_reported(block, kmax):
     assert torch.equal(out.view(torch.int16), ref.view(torch.int16))
 
 
+@pytest.mark.parametrize("block,kmax", [(128, 5), (128, 33), (128, 128), (128, 129), (64, 9), (64, 70)])
+def test_lists_cleaned_ahead_or_by_the_cta(block, kmax):
+    """bf16, d = 128: up to 16 items per CTA the forward's CTAs clean their lists themselves, beyond (18 heads of 140 items) a
+    pre-pass does.  Lists of every kind (own block first, in the middle, last, missing, twice; invalid indices; empty), strides
+    on both sides of a warp and of what is held in registers: the same output, lse and status bit for bit, in a
+    workspace of any content."""
+    nbk, H = 140 * 128 // block, 18
+    N = nbk * block - 5
+    g = torch.Generator().manual_seed(block + kmax)
+    q, k, v = (torch.randn((1, H, N, 128), generator=g).to(torch.bfloat16).to(DEV) for _ in range(3))
+    idx = torch.randint(0, nbk, (1, H, nbk, kmax), generator=g, dtype=torch.int32)
+    cnt = torch.randint(0, 7, (1, H, nbk), generator=g, dtype=torch.int32).clamp(max=kmax)
+    at = torch.randint(0, 8, (1, H, nbk, 1), generator=g).clamp(max=kmax - 1)
+    idx.scatter_(-1, at, torch.arange(nbk, dtype=torch.int32)[None, None, :, None].expand(1, H, nbk, 1).contiguous())
+    cnt[0, :, 7], cnt[0, :, 11] = kmax, kmax                      # (a few full ones)
+    bad = idx.clone()
+    bad[0, ::3, 3, 0], bad[0, ::3, 7, kmax - 1], bad[0, ::3, 11, kmax // 2] = -1, nbk, 1 << 30
+    cnt[0, ::3, 3] = cnt[0, ::3, 3].clamp(min=1)
+    halves = (slice(0, 9), slice(9, 18))
+    for lists, want in ((idx, sa.OK), (bad, sa.E_BAD_INDEX)):
+        ws = sa.alloc_workspace(sa.make_shape(q, block), 1, kmax, DEV)
+        ws.fill_(0xA5)
+        out, lse = sa.fwd(q, k, v, lists.to(DEV), cnt.to(DEV), block, return_lse=True, workspace=ws)
+        assert sa.read_status(ws) == want
+        ws.fill_(0x5A)
+        for h in halves:
+            one, lse_one = sa.fwd(q[:, h], k[:, h], v[:, h], lists[:, h].contiguous().to(DEV), cnt[:, h].contiguous().to(DEV), block,
+                                  return_lse=True, workspace=ws)
+            assert sa.read_status(ws) == want
+            assert torch.equal(out[:, h].view(torch.int16), one.view(torch.int16))
+            assert torch.equal(lse[:, h].view(torch.int32), lse_one.view(torch.int32))
+
+
 @pytest.mark.parametrize("H,window", [(3, 0), (7, 0), (3, 2)])
 def test_d64_chains_of_every_length(H, window):
     """d = 64: the tiles of an item go to four chains (H = 3: 123 items, no SM gets a second one) or two (H = 7), so lists
