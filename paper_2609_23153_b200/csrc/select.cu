@@ -13,6 +13,7 @@
 //                     memory in one go (asynchronous copies into one of two buffers) while thread c adds up two
 //                     channels of the block before.  The only HBM-heavy step (2 bytes per element); writes pooled Q
 //                     [BH][nb][d] and pooled K transposed [BH][d][nbp].
+//   topk_small_kernel nb <= 64: one CTA per 8 query blocks, a warp each, all of the head's pooled K in shared memory.
 //   topk_kernel       nb <= 256: one CTA per 8, 16 or 32 query blocks of one (batch, head): scores against all key
 //                     blocks as an RT x 4 register tile per thread (pooled K through a ring of asynchronous copies in
 //                     shared memory, packed fp32x2 FMAs over row pairs), then a warp per query block (or two) selects
@@ -27,6 +28,7 @@
 namespace sparkattn {
 
 constexpr int kTopkThreads = 256;
+constexpr int kSmallBlocks = 64;      // key blocks up to which topk_small_kernel scores and selects
 
 static inline int round_up(int x, int m) { return (x + m - 1) / m * m; }
 
@@ -357,8 +359,8 @@ __device__ __forceinline__ void window_range(int i, int N, int blk_size, int fra
 }
 
 // Selection of a CTA's rows from their keys in shared memory: a warp takes rows WARPS apart, NR of them at a time.
-// SHORT: nb <= 256, otherwise more.
-template <bool WINDOW, int WARPS, int NR, bool SHORT>
+// KR: keys per lane, nb <= 32 KR; 0: more than 256 blocks, by their number.
+template <bool WINDOW, int WARPS, int NR, int KR>
 __device__ __forceinline__ void select_tile(const uint32_t* s_key, int nb, int nbp, int topk, int64_t bh, int i0, int nrows, int N,
                                             int blk_size, int frame_tokens, int window, int32_t* __restrict__ kept_idx,
                                             int32_t* __restrict__ kept_cnt) {
@@ -382,8 +384,8 @@ __device__ __forceinline__ void select_tile(const uint32_t* s_key, int nb, int n
         for (int t = k_row[r] + lane; t < topk; t += 32) dst[r][t] = -1;    // unused tail of a list cut short by the window
       if (lane == 0 && kept_cnt != nullptr) kept_cnt[bh * nb + i0 + row] = k_row[r];
     }
-    if constexpr (SHORT) {       // nb <= 256
-      select_rows_regs<8, WINDOW, NR>(key, nb, jlo, jhi, k_row, lane, dst);
+    if constexpr (KR > 0) {
+      select_rows_regs<KR, WINDOW, NR>(key, nb, jlo, jhi, k_row, lane, dst);
     } else if (nb <= 32 * 20) {
       select_rows_regs<20, WINDOW, NR>(key, nb, jlo, jhi, k_row, lane, dst);
     } else if (nb <= 32 * 40) {
@@ -529,7 +531,7 @@ topk_kernel(const float* pq, const float* pkT, int32_t* __restrict__ kept_idx,
   }
   __syncthreads();
 
-  select_tile<WINDOW, 8, (R >= 16 ? 2 : 1), true>(s_key, nb, nbp, topk, bh, i0, nrows, N, blk_size, frame_tokens, window, kept_idx, kept_cnt);
+  select_tile<WINDOW, 8, (R >= 16 ? 2 : 1), 8>(s_key, nb, nbp, topk, bh, i0, nrows, N, blk_size, frame_tokens, window, kept_idx, kept_cnt);
 }
 
 // The same for long rows of key blocks: a CTA of WARPS warps takes R query blocks, a thread owns an RT x 4 register tile
@@ -606,7 +608,55 @@ topk_wide_kernel(const float* pq, const float* pkT, int32_t* __restrict__ kept_i
     store_keys<kPairs>(acc, s_key + (int64_t)(rg * RT) * nbp + j0, nbp);
   }
   __syncthreads();
-  select_tile<WINDOW, WARPS, 1, false>(s_key, nb, nbp, topk, bh, i0, nrows, N, blk_size, frame_tokens, window, kept_idx, kept_cnt);
+  select_tile<WINDOW, WARPS, 1, 0>(s_key, nb, nbp, topk, bh, i0, nrows, N, blk_size, frame_tokens, window, kept_idx, kept_cnt);
+}
+
+// Up to 64 key blocks: latency is all there is.  The pooled K of the (batch, head) comes into shared memory in one go, not
+// through a ring, a warp takes a query block, a lane one or two key blocks (lane, lane + 32) with their chains in registers,
+// and the selection holds one or two keys per lane instead of eight.  38 KB of shared memory at most, so that its CTAs are
+// on the SMs while the pooling kernel drains.  Whole selection against topk_kernel, us: 3 heads of 10 blocks 8.4 -> 5.9, 8 of 25 10.3 -> 7.7,
+// 6 of 51 13.3 -> 10.0, 20 of 51 20.0 -> 16.2, 40 of 51 35.0 -> 33.6; the same for up to 128 blocks (72 KB): 6 of 94 15.8 -> 19.1.  Two query
+// blocks per warp: 6 of 51 21.4.
+template <int D, int KPL, bool WINDOW>
+__global__ void __launch_bounds__(kTopkThreads)
+topk_small_kernel(const float* pq, const float* pkT, int32_t* __restrict__ kept_idx, int32_t* __restrict__ kept_cnt, int nb, int nbp,
+                  int topk, int groups_per_bh, int N, int blk_size, int frame_tokens, int window, int32_t* __restrict__ header) {
+  constexpr int W = 32 * KPL, R = kTopkThreads / 32;                  // nbp = W
+  __shared__ __align__(16) float s_k[D * W];                          // [D][W]
+  __shared__ __align__(16) float s_q[R * D];                          // [R][D]
+  __shared__ uint32_t s_key[R * W];                                   // [R][W]
+  const int64_t bh = blockIdx.x / groups_per_bh;
+  const int i0 = (blockIdx.x % groups_per_bh) * R;
+  const int nrows = min(R, nb - i0);
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const float* kcol = pkT + bh * D * (int64_t)W;
+  const float* qrow = pq + (bh * nb + i0) * D;
+  pdl_wait();
+  clear_header(header);
+  for (int e = threadIdx.x; e < D * W / 4; e += kTopkThreads) cp_async16(smem_u32(s_k + 4 * e), kcol + 4 * e);
+  for (int e = threadIdx.x; e < nrows * (D / 4); e += kTopkThreads) cp_async16(smem_u32(s_q + 4 * e), qrow + 4 * e);
+  cp_async_commit();
+  cp_async_wait<0>();
+  __syncthreads();
+  if (warp < nrows) {
+    float acc[KPL] = {};
+#pragma unroll 4
+    for (int c = 0; c < D; c += 4) {
+      const float4 q = *reinterpret_cast<const float4*>(s_q + warp * D + c);
+#pragma unroll
+      for (int u = 0; u < KPL; ++u) {                                 // each its own chain, channels in ascending order
+        const float* k = s_k + c * W + 32 * u + lane;
+        acc[u] = fmaf(q.x, k[0], acc[u]);
+        acc[u] = fmaf(q.y, k[W], acc[u]);
+        acc[u] = fmaf(q.z, k[2 * W], acc[u]);
+        acc[u] = fmaf(q.w, k[3 * W], acc[u]);
+      }
+    }
+#pragma unroll
+    for (int u = 0; u < KPL; ++u) s_key[warp * W + 32 * u + lane] = score_key(acc[u]);
+  }
+  __syncwarp();                        // (a warp reads the keys of its own row)
+  select_tile<WINDOW, R, 1, KPL>(s_key, nb, W, topk, bh, i0, nrows, N, blk_size, frame_tokens, window, kept_idx, kept_cnt);
 }
 
 // topk = nb: every candidate is kept whatever its score, so nothing is pooled and nothing compared.  A warp per list.
@@ -646,6 +696,18 @@ static int launch_topk(const float* pq, const float* pkT, int32_t* kept_idx, int
     return SPARKATTN_E_CUDA;
   return launch_kernel(kern, (unsigned)ctas, kTopkThreads, smem, true, stream, pq, pkT, kept_idx, kept_cnt, nb, nbp, topk,
                        groups, N, block, frame_tokens, window, header);
+}
+
+template <int D, int KPL>
+static int launch_topk_small(const float* pq, const float* pkT, int32_t* kept_idx, int32_t* kept_cnt, int nb, int nbp, int topk,
+                             int64_t bh, int N, int block, int frame_tokens, int window, int32_t* header, cudaStream_t stream) {
+  constexpr int R = kTopkThreads / 32;
+  const int groups = (nb + R - 1) / R;
+  const int64_t ctas = bh * groups;
+  if (ctas > 0x7fffffffLL) return SPARKATTN_E_UNSUPPORTED_SHAPE;
+  auto kern = frame_tokens > 0 ? topk_small_kernel<D, KPL, true> : topk_small_kernel<D, KPL, false>;
+  return launch_kernel(kern, (unsigned)ctas, kTopkThreads, 0, true, stream, pq, pkT, kept_idx, kept_cnt, nb, nbp, topk, groups, N, block,
+                       frame_tokens, window, header);
 }
 
 static size_t wide_smem(int rows, int d, int nbp) { return (size_t)rows * (d + nbp) * sizeof(float); }
@@ -697,6 +759,7 @@ static int launch_topk_d(const sparkattn_shape_t& s, int topk, int frame_tokens,
   // 65 against 9.1 / 20.8 / 59), with as many rows per CTA as still leave 1.5 CTAs (32 rows) or one CTA (16) per SM:
   // 80 heads of 250 blocks 63.9 us with 32 rows, 69.9 with 16, 94.6 with 8; 12 heads of 256 22.0 / 20.8 / 22.2; 3 heads
   // of 50 16.9 / 12.5 / 10.4.
+  if (nb <= kSmallBlocks) return nbp == 32 ? go(launch_topk_small<D, 1>) : go(launch_topk_small<D, 2>);
   if (nb > 256) {
     if (ctas16 > kNumSMs && wide_smem(16, D, nbp) <= kSmemOfTwo) return go(launch_topk_wide<D, 16, 8, 10, 2>);
     return go(launch_topk_wide<D, 8, 8, 10, 2>);               // at most 132 KB

@@ -126,6 +126,24 @@ def test_select_kernel_variants_match_oracle(H, nb, tail, block, d):
     assert sa.read_status(ws) == sa.OK
 
 
+@pytest.mark.parametrize("nb", [2, 7, 8, 9, 31, 32, 33, 63, 64, 65])
+@pytest.mark.parametrize("d,block,window", [(64, 64, 0), (128, 64, 0), (128, 64, 2), (64, 64, 3)])
+def test_select_few_blocks(nb, d, block, window):
+    """Up to 64 key blocks have a kernel of their own: 8 query blocks per CTA, one or two key blocks per lane.  Both sides of those
+    lines against the oracle, with key blocks that repeat (ties to the lowest index) and under a causal window."""
+    g = torch.Generator().manual_seed(nb * d + window)
+    N = nb * block - 3
+    q, k = (torch.randn((2, 3, N, d), generator=g).to(torch.bfloat16) for _ in range(2))
+    if nb > 7:
+        k[1, :, 5 * block: 6 * block], k[1, :, (nb - 2) * block: (nb - 1) * block] = k[1, :, :block], k[1, :, :block]
+    kw = dict(frame_tokens=100, window=window) if window else {}
+    for topk in sorted({1, nb // 2, nb - 1}):
+        idx, cnt = sa.select(q.to(DEV), k.to(DEV), block, topk, **kw)
+        for b in range(2):
+            want, count = oracle.select(q[b], k[b], block, topk, **kw)
+            assert torch.equal(idx[b].cpu(), want) and torch.equal(cnt[b].cpu(), count), topk
+
+
 def test_select_strided_layout_and_batch():
     # [B, N, H, d] storage viewed as [B, H, N, d]; two batches
     w = workloads.small_structured(H=2, d=128, grid=(2, 10, 26), block=128, sparsity=0.75, cfg_id=16)
