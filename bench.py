@@ -483,7 +483,7 @@ def run_ours(args, w):
         fp8["chain_fused_ms_quantpool_topk_fwd"] = ms8f
         fp8["fused_quantpool_plus_topk_ms"] = ms_pre
         fp8["separate_select_plus_quant_ms"] = ms_sel + ms_q
-        fp8["fused_launches_per_step"] = 4 + (3 if pipelined else 1)
+        fp8["fused_launches_per_step"] = 4 + (2 if pipelined else 1)
         # per-token activation quantisation (the paper's fused scale-and-cast kernel), one tensor, outside the step
         tok_scales = torch.empty((w.B, Hl, w.N), dtype=torch.float32, device=dev)
         tok_codes = torch.empty(q.shape, dtype=torch.uint8, device=dev)    # (its own buffer: codes[] feed the later FP8 legs)
