@@ -98,6 +98,7 @@ __device__ __forceinline__ void rope_factors(float2 (&cs)[kRank / 2], const Rope
 // One token row of T (64 fp32 columns at `taddr`) -> silu -> rank-truncated rotary rotation of the
 // adjacent pairs -> bf16 -> row `row` of a [128 rows x 128 B] tile with 128-byte swizzle.
 // Done in two halves of 32 columns to bound the live registers.
+template <bool TMEM>
 __device__ __forceinline__ void feature_row(uint32_t taddr, unsigned char* tile, int row, const float2 (&cs)[kRank / 2]) {
 #pragma unroll
   for (int half = 0; half < 2; ++half) {
@@ -117,11 +118,16 @@ __device__ __forceinline__ void feature_row(uint32_t taddr, unsigned char* tile,
       const __nv_bfloat162 h2 = __floats2bfloat162_rn(o0, o1);
       w[j] = *reinterpret_cast<const uint32_t*>(&h2);
     }
+    if constexpr (TMEM) {
+      tmem_st16(taddr + half * 16, w);
+    } else {
 #pragma unroll
-    for (int c = 0; c < 4; ++c)
-      *reinterpret_cast<uint4*>(tile + row * 128 + (((half * 4 + c) ^ (row & 7)) << 4)) =
-          make_uint4(w[4 * c], w[4 * c + 1], w[4 * c + 2], w[4 * c + 3]);
+      for (int c = 0; c < 4; ++c)
+        *reinterpret_cast<uint4*>(tile + row * 128 + (((half * 4 + c) ^ (row & 7)) << 4)) =
+            make_uint4(w[4 * c], w[4 * c + 1], w[4 * c + 2], w[4 * c + 3]);
+    }
   }
+  if constexpr (TMEM) tc_wait_st();
 }
 
 // instruction descriptor with both major bits explicit (bf16 in, fp32 accumulate)
@@ -167,9 +173,10 @@ struct IdleGuard {
 constexpr int kStateOffK = 16384, kStateOffV = kStateOffK + 2 * 32768, kStateOffF = kStateOffV + 2 * 32768;
 constexpr int kStateOffBar = kStateOffF + kFeatWGs * 16384;
 constexpr int kStateSmem = 1024 + kStateOffBar + 256;
-// apply kernel shared memory: P | C | Q ring (3) | q~ tiles | barriers
-constexpr int kApplyOffC = 16384, kApplyOffQ = 32768, kApplyOffF = kApplyOffQ + kFeatWGs * 32768;
-constexpr int kApplyOffBar = kApplyOffF + kFeatWGs * 16384;
+// apply kernel shared memory: P | C | Q ring (2) | O_s slots (3) | barriers
+constexpr int kApplyQ = 2;
+constexpr int kApplyOffC = 16384, kApplyOffQ = 32768, kApplyOffO = kApplyOffQ + kApplyQ * 32768;
+constexpr int kApplyOffBar = kApplyOffO + kFeatWGs * 32768;
 constexpr int kApplySmem = 1024 + kApplyOffBar + 256;
 
 __global__ void __launch_bounds__(kCompThreads, 1)
@@ -314,7 +321,7 @@ comp_state_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid_const
         if (!ok) break;
       }
       tc_fence_after();
-      feature_row(tmem + g * 64 + lane_off, tileF, row, cs);
+      feature_row<false>(tmem + g * 64 + lane_off, tileF, row, cs);
       fence_proxy_async_smem();
       tc_fence_before();
       mbar_arrive(bar_f_full + g);
@@ -394,9 +401,13 @@ __device__ __forceinline__ void named_bar_sync(int id, int count) {
   asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(count) : "memory");
 }
 
-// A ring slot of the apply kernel lives through: Q tile (TMA) -> projection MMAs -> sparse-branch
-// tile O_s (TMA into the same bytes) -> fused output written in place by the warpgroup -> TMA
-// store -> free.  Slot = warpgroup = tile % 3, so all global traffic of the tile is bulk copies.
+// Bound by HBM, and with one slot per tile that took Q, then O_s, by the latency of the two reads in a row.  Q has a ring of its own
+// now and is requested while the tiles before are being worked on; a warpgroup's O_s slot, which becomes the output in
+// place, is filled as soon as its last store has read it.  q~ goes to the second product from TMEM instead of shared memory,
+// which makes the room.  40 heads of 75,600 tokens 472 -> 440 us, 12 of 32,760 69.3 -> 66.8, 20 of 6,479 28.2 -> 26.8, 1 of 75,600 17.4 -> 16.4,
+// 6 of 6,479 12.9 -> 12.8.  (A slot for Q per warpgroup: 426, 66.2, 27.8, 16.6, 13.0; it leaves 26 KB of L1 for the rotary factors.)
+// A warpgroup's TMEM columns: T (64), q~ over the first 32 of them, Y behind these (128).
+constexpr int kApplyCols = 160, kApplyColY = 32;
 __global__ void __launch_bounds__(kCompThreads, 1)
 comp_apply_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant__ CUtensorMap tmap_p,
                   const __grid_constant__ CUtensorMap tmap_os, const __grid_constant__ CUtensorMap tmap_out,
@@ -405,20 +416,21 @@ comp_apply_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_const
   unsigned char* smem = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_dyn) + 1023) & ~uintptr_t(1023));
   unsigned char* sP = smem;
   unsigned char* sC = smem + kApplyOffC;           // C as bf16, [64 r rows][128 d], two 64-column slabs of 8 KB
-  unsigned char* sQ = smem + kApplyOffQ;           // ring of 3 slots (Q, then O_s / O), slot = tile % 3
-  unsigned char* sF = smem + kApplyOffF;           // q~ tiles, one per warpgroup
+  unsigned char* sQ = smem + kApplyOffQ;           // [kApplyQ] ring of Q tiles
+  unsigned char* sO = smem + kApplyOffO;           // [3] O_s, then O: slot = warpgroup = tile % 3
   uint64_t* bars = reinterpret_cast<uint64_t*>(smem + kApplyOffBar);
   uint64_t* bar_p_full = bars + 0;
   uint64_t* bar_c_full = bars + 1;                 // C staged (128 arrivals)
-  uint64_t* bar_q_full = bars + 2;                 // [3] Q tile landed
-  uint64_t* bar_q_empty = bars + 5;                // [3] projection MMAs done: slot may take O_s
+  uint64_t* bar_q_full = bars + 2;                 // [kApplyQ] Q tile landed
+  uint64_t* bar_q_empty = bars + 5;                // [kApplyQ] projection MMAs done: the slot may take the next Q
   uint64_t* bar_os_full = bars + 8;                // [3] O_s tile landed
   uint64_t* bar_t_full = bars + 11;                // [3]
   uint64_t* bar_f_full = bars + 14;                // [3] q~ tile written (128 arrivals)
   uint64_t* bar_y_full = bars + 17;                // [3] Y = q~ C done
-  uint64_t* bar_slot_free = bars + 20;             // [3] output store has read the slot; Y has been read
-  uint32_t* s_tmem = reinterpret_cast<uint32_t*>(bars + 24);
-  volatile int* s_abort = reinterpret_cast<volatile int*>(bars + 25);
+  uint64_t* bar_slot_free = bars + 20;             // [3] output store has read the slot
+  uint64_t* bar_t_free = bars + 23;                // [3] Y has been read (128 arrivals): the columns may take the next T
+  uint32_t* s_tmem = reinterpret_cast<uint32_t*>(bars + 26);
+  volatile int* s_abort = reinterpret_cast<volatile int*>(bars + 27);
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int bh = blockIdx.y;
@@ -432,7 +444,7 @@ comp_apply_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_const
     for (int g = 0; g < kFeatWGs; ++g) {
       mbar_init(bar_q_full + g, 1); mbar_init(bar_q_empty + g, 1); mbar_init(bar_os_full + g, 1);
       mbar_init(bar_t_full + g, 1); mbar_init(bar_f_full + g, 128); mbar_init(bar_y_full + g, 1);
-      mbar_init(bar_slot_free + g, 1);
+      mbar_init(bar_slot_free + g, 1); mbar_init(bar_t_free + g, 128);
     }
     *s_abort = 0;
     mbar_fence_init();
@@ -445,7 +457,7 @@ comp_apply_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_const
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
-  const uint32_t tmem = *s_tmem;                   // warpgroup g: columns [128 g, 128 g + 128): T in the first 64, then Y over all
+  const uint32_t tmem = *s_tmem;                   // warpgroup g: columns [160 g, 160 g + 160)
 
   if (warp >= kProducerWarp) reg_dec<kCtrlRegs>();
   if (warp == kProducerWarp) {
@@ -460,23 +472,24 @@ comp_apply_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_const
       while (ok && io < ntiles) {
         bool progressed = false;
         if (iq < ntiles) {
-          const int g = iq % kFeatWGs, n = iq / kFeatWGs;
-          if (n == 0 || mbar_try_wait(bar_slot_free + g, (n - 1) & 1)) {
+          const int c = iq % kApplyQ, n = iq / kApplyQ;
+          if (n == 0 || mbar_try_wait(bar_q_empty + c, (n - 1) & 1)) {
             const int row = (tile0 + iq) * kTileTok;
-            mbar_expect_tx(bar_q_full + g, 32768);
-            tma_load_4d(sQ + g * 32768, &tmap_q, bar_q_full + g, 0, row, h, b);
-            tma_load_4d(sQ + g * 32768 + 16384, &tmap_q, bar_q_full + g, 64, row, h, b);
+            mbar_expect_tx(bar_q_full + c, 32768);
+            tma_load_4d(sQ + c * 32768, &tmap_q, bar_q_full + c, 0, row, h, b);
+            tma_load_4d(sQ + c * 32768 + 16384, &tmap_q, bar_q_full + c, 64, row, h, b);
             ++iq;
-            progressed = true;
+            guard.reset();
+            continue;                              // (a Q is waited for before its O_s)
           }
         }
         if (io < iq) {
-          const int g = io % kFeatWGs;
-          if (mbar_try_wait(bar_q_empty + g, (io / kFeatWGs) & 1)) {
+          const int g = io % kFeatWGs, n = io / kFeatWGs;
+          if (n == 0 || mbar_try_wait(bar_slot_free + g, (n - 1) & 1)) {
             const int row = (tile0 + io) * kTileTok;
             mbar_expect_tx(bar_os_full + g, 32768);
-            tma_load_4d(sQ + g * 32768, &tmap_os, bar_os_full + g, 0, row, h, b);
-            tma_load_4d(sQ + g * 32768 + 16384, &tmap_os, bar_os_full + g, 64, row, h, b);
+            tma_load_4d(sO + g * 32768, &tmap_os, bar_os_full + g, 0, row, h, b);
+            tma_load_4d(sO + g * 32768 + 16384, &tmap_os, bar_os_full + g, 64, row, h, b);
             ++io;
             progressed = true;
           }
@@ -487,7 +500,7 @@ comp_apply_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_const
     }
   } else if (warp == kMmaWarp) {
     if (lane == 0 && ntiles > 0) {
-      // Y[128 tokens x 128 d] = q~ C : A = q~ tile (K-major: r contiguous), B = C (MN-major: d contiguous, two slabs)
+      // Y[128 tokens x 128 d] = q~ C : A = q~ (TMEM), B = C (MN-major: d contiguous, two slabs)
       const uint64_t dC = make_smem_desc_sw128(smem_u32(sC), 8192);
       const uint32_t c_lo = (uint32_t)dC, c_hi = (uint32_t)(dC >> 32);
       constexpr uint32_t idesc_y = comp_idesc(128, kCD, false, true);
@@ -497,25 +510,22 @@ comp_apply_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_const
       guard.reset();
       while (ok && s2 < ntiles) {
         bool progressed = false;
-        const int g1 = s1 % kFeatWGs;
-        // a landed Q tile implies its slot (and with it the TMEM columns of the warpgroup) was released
-        if (s1 < ntiles && mbar_try_wait(bar_q_full + g1, (s1 / kFeatWGs) & 1)) {
+        const int g1 = s1 % kFeatWGs, n1 = s1 / kFeatWGs, c1 = s1 % kApplyQ;
+        if (s1 < ntiles && mbar_try_wait(bar_q_full + c1, (s1 / kApplyQ) & 1) && (n1 == 0 || mbar_try_wait(bar_t_free + g1, (n1 - 1) & 1))) {
           tc_fence_after();
-          issue_projection(tmem + g1 * 128, smem_u32(sQ + g1 * 32768), smem_u32(sP));
+          issue_projection(tmem + g1 * kApplyCols, smem_u32(sQ + c1 * 32768), smem_u32(sP));
           tc_commit(bar_t_full + g1);
-          tc_commit(bar_q_empty + g1);
+          tc_commit(bar_q_empty + c1);
           ++s1;
           progressed = true;
         }
         const int g2 = s2 % kFeatWGs;
         if (s2 < s1 && mbar_try_wait(bar_f_full + g2, (s2 / kFeatWGs) & 1)) {
           tc_fence_after();
-          const uint64_t dF = make_smem_desc_sw128(smem_u32(sF + g2 * 16384), 16);
-          const uint32_t f_lo = (uint32_t)dF, f_hi = (uint32_t)(dF >> 32);
+          const uint32_t tF = tmem + g2 * kApplyCols;
 #pragma unroll
           for (int kk = 0; kk < 4; ++kk)
-            mma_ss<false>(tmem + g2 * 128, make_desc(f_lo + ((kk * 32) >> 4), f_hi),
-                          make_desc(c_lo + ((kk * 2048) >> 4), c_hi), idesc_y, kk != 0 ? 1u : 0u);
+            mma_ts<false>(tF + kApplyColY, tF + kk * 8, make_desc(c_lo + ((kk * 2048) >> 4), c_hi), idesc_y, kk != 0 ? 1u : 0u);
           tc_commit(bar_y_full + g2);
           ++s2;
           progressed = true;
@@ -529,9 +539,8 @@ comp_apply_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_const
     const int g = warp >> 2;
     const int row = threadIdx.x & 127;
     const uint32_t lane_off = (uint32_t)((warp & 3) * 32) << 16;
-    unsigned char* tileF = sF + g * 16384;
-    unsigned char* slot = sQ + g * 32768;
-    const uint32_t tmem_g = tmem + g * 128 + lane_off;
+    unsigned char* slot = sO + g * 32768;
+    const uint32_t tmem_g = tmem + g * kApplyCols + lane_off, tmem_y = tmem_g + kApplyColY;
     if (g == 0) {
       if (ntiles > 0) {
         // stage C: thread j converts row a = j/2, columns [64*(j%2), +64) of the fp32 state to bf16
@@ -561,9 +570,7 @@ comp_apply_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_const
       ok = __all_sync(0xffffffffu, mbar_wait(bar_t_full + g, u & 1, s_abort, p.status, 64));
       if (!ok) break;
       tc_fence_after();
-      // the previous tile of this warpgroup has passed its Y wait, so the q~ tile is free
-      feature_row(tmem_g, tileF, row, cs);
-      fence_proxy_async_smem();
+      feature_row<true>(tmem_g, nullptr, row, cs);
       tc_fence_before();
       mbar_arrive(bar_f_full + g);
 
@@ -589,7 +596,7 @@ comp_apply_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_const
 #pragma unroll
       for (int ch = 0; ch < 4; ++ch) {
         uint32_t r[32];
-        tmem_ld32(tmem_g + ch * 32, r);
+        tmem_ld32(tmem_y + ch * 32, r);
         tc_wait_ld();
 #pragma unroll
         for (int j = 0; j < 32; ++j) ss = fmaf(__uint_as_float(r[j]), __uint_as_float(r[j]), ss);
@@ -598,7 +605,7 @@ comp_apply_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_const
 #pragma unroll
       for (int ch = 0; ch < 4; ++ch) {
         uint32_t r[32];
-        tmem_ld32(tmem_g + ch * 32, r);
+        tmem_ld32(tmem_y + ch * 32, r);
         tc_wait_ld();
 #pragma unroll
         for (int c = 0; c < 4; ++c) {
@@ -619,6 +626,7 @@ comp_apply_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_const
       }
       fence_proxy_async_smem();
       tc_fence_before();
+      mbar_arrive(bar_t_free + g);
       named_bar_sync(1 + g, 128);
       if (row == 0) {
         tma_store_4d(&tmap_out, slot, 0, tile_row, h, b);
