@@ -21,6 +21,8 @@
 //   topk_wide_kernel  nb > 256: 16 or 8 query blocks per CTA of ten warps, pooled K straight from L2.
 //   list_all_kernel   in place of all of them when every block is kept.
 // The second is launched before the first has drained (programmatic dependent launch) and waits inside.
+#include <atomic>
+
 #include "common.cuh"
 #include "launch.h"
 #include "tmap.h"
@@ -678,6 +680,22 @@ list_all_kernel(int32_t* __restrict__ kept_idx, int32_t* __restrict__ kept_cnt, 
   }
 }
 
+// The kernels of a selection stand by while the one before them drains, so they have to agree on how an SM's memory is split between
+// L1 and shared memory.  Left to itself the runtime picks a split for each kernel, and a CTA that needs another one waits until
+// the SM is empty.  Selection with the runtime's splits / with the most shared memory for all, us: 3 heads of 192 blocks 18.8 /
+// 15.2, 6 of 94 15.6 / 13.8, 35 of 48 29.0 / 25.0, 40 of 48 31.8 / 27.8, elsewhere the same.  A preference of the kernel, told once per device.
+template <auto Kern>
+static bool max_shared_memory() {
+  static std::atomic<uint64_t> told{0};
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess) return false;
+  const uint64_t bit = 1ull << (dev & 63);
+  if (told.load(std::memory_order_relaxed) & bit) return true;
+  if (cudaFuncSetAttribute(Kern, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared) != cudaSuccess) return false;
+  if (dev < 64) told.fetch_or(bit, std::memory_order_relaxed);
+  return true;
+}
+
 // The limit of a kernel's dynamic shared memory belongs to the kernel, not to a launch: it is always set to the most that any
 // launch of the kernel asks for.  Set to what this launch needs, it could be lowered by another thread before the
 // launch, which then fails.
@@ -692,7 +710,8 @@ static int launch_topk(const float* pq, const float* pkT, int32_t* kept_idx, int
   if (ctas > 0x7fffffffLL) return SPARKATTN_E_UNSUPPORTED_SHAPE;
   const size_t smem = Shape::smem_bytes(D, nbp);
   auto kern = frame_tokens > 0 ? topk_kernel<D, RT, RG, KC, NS, true> : topk_kernel<D, RT, RG, KC, NS, false>;
-  if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Shape::smem_bytes(D, 256)) != cudaSuccess)
+  if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Shape::smem_bytes(D, 256)) != cudaSuccess ||
+      !(frame_tokens > 0 ? max_shared_memory<topk_kernel<D, RT, RG, KC, NS, true>>() : max_shared_memory<topk_kernel<D, RT, RG, KC, NS, false>>()))
     return SPARKATTN_E_CUDA;
   return launch_kernel(kern, (unsigned)ctas, kTopkThreads, smem, true, stream, pq, pkT, kept_idx, kept_cnt, nb, nbp, topk,
                        groups, N, block, frame_tokens, window, header);
@@ -706,6 +725,8 @@ static int launch_topk_small(const float* pq, const float* pkT, int32_t* kept_id
   const int64_t ctas = bh * groups;
   if (ctas > 0x7fffffffLL) return SPARKATTN_E_UNSUPPORTED_SHAPE;
   auto kern = frame_tokens > 0 ? topk_small_kernel<D, KPL, true> : topk_small_kernel<D, KPL, false>;
+  if (!(frame_tokens > 0 ? max_shared_memory<topk_small_kernel<D, KPL, true>>() : max_shared_memory<topk_small_kernel<D, KPL, false>>()))
+    return SPARKATTN_E_CUDA;
   return launch_kernel(kern, (unsigned)ctas, kTopkThreads, 0, true, stream, pq, pkT, kept_idx, kept_cnt, nb, nbp, topk, groups, N, block,
                        frame_tokens, window, header);
 }
@@ -720,7 +741,9 @@ static int launch_topk_wide(const float* pq, const float* pkT, int32_t* kept_idx
   if (ctas > 0x7fffffffLL) return SPARKATTN_E_UNSUPPORTED_SHAPE;
   const size_t smem = wide_smem(R, D, nbp);
   auto kern = frame_tokens > 0 ? topk_wide_kernel<D, R, RT, WARPS, CTAS, true> : topk_wide_kernel<D, R, RT, WARPS, CTAS, false>;
-  if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, CTAS == 2 && R == 16 ? kSmemOfTwo : kSmemOfOne) != cudaSuccess)
+  if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, CTAS == 2 && R == 16 ? kSmemOfTwo : kSmemOfOne) != cudaSuccess ||
+      !(frame_tokens > 0 ? max_shared_memory<topk_wide_kernel<D, R, RT, WARPS, CTAS, true>>()
+                         : max_shared_memory<topk_wide_kernel<D, R, RT, WARPS, CTAS, false>>()))
     return SPARKATTN_E_CUDA;
   return launch_kernel(kern, (unsigned)ctas, WARPS * 32, smem, true, stream, pq, pkT, kept_idx, kept_cnt, nb, nbp, topk,
                        groups, N, block, frame_tokens, window, header);
@@ -814,6 +837,7 @@ int launch_select(const sparkattn_shape_t& s, const void* q, const void* k, int 
   auto pool = s.d == 128 ? pool_kernel<128> : pool_kernel<64>;
   if (cudaFuncSetAttribute(pool, cudaFuncAttributeMaxDynamicSharedMemorySize, 2 * 128 * s.d * 2) != cudaSuccess)    // (see kSmemOfOne)
     return SPARKATTN_E_CUDA;
+  if (!(s.d == 128 ? max_shared_memory<pool_kernel<128>>() : max_shared_memory<pool_kernel<64>>())) return SPARKATTN_E_CUDA;
   const int64_t resident = (int64_t)sm_count * kPoolCtasPerSm * (65536 / (int)pool_smem);
   const int64_t pool_ctas = 2 * n_items < resident ? 2 * n_items : resident;
   // Launched early while a CTA has fewer than four blocks.  Beyond that the microsecond it saves is lost in the noise (256 blocks of 12
