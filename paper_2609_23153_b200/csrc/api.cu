@@ -322,7 +322,6 @@ int sparkattn_gather_tokens(const sparkattn_shape_t* src_shape, const void* x_bf
   if (!aligned16(x_bf16) || !aligned16(out_bf16) || !aligned256(workspace)) return SPARKATTN_E_MISALIGNED;
   if (workspace_bytes < (size_t)kWorkspaceHeaderBytes) return SPARKATTN_E_WORKSPACE_TOO_SMALL;
   cudaStream_t stream = static_cast<cudaStream_t>(cuda_stream);
-  if (cudaMemsetAsync(workspace, 0, kWorkspaceHeaderBytes, stream) != cudaSuccess) return SPARKATTN_E_CUDA;
   return launch_gather_tokens(*src_shape, x_bf16, *dst_shape, index, out_bf16, workspace, stream);
 }
 

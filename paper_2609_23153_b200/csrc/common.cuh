@@ -21,10 +21,10 @@ __device__ __forceinline__ void report_status(int32_t* status, int code, int det
   if (atomicCAS(status, 0, code) == 0) status[1] = detail;
 }
 
-// Every call starts with a clean status.  Mostly a small kernel in front sees to it; a kernel that fills the device once at most
-// can do it itself: its first CTA clears the words and counts up, every CTA notes the count when it starts, and one with
-// something to report waits until the count has moved since (or for a millisecond, if it had moved already).  One
-// thread each; the memory may hold anything before.
+// Every call starts with a clean status.  A small kernel in front can see to it; a kernel whose CTAs report nothing before their
+// end can do it itself: its first CTA clears the words and counts up, every CTA notes the count when it starts, and one
+// with something to report waits until the count has moved since (or for a millisecond, if it had moved already).
+// The memory may hold anything before.
 __device__ __forceinline__ int32_t header_begin(int32_t* status, bool first_cta) {
   volatile int32_t* turn = status + kHeaderTurnWord;
   const int32_t before = *turn;

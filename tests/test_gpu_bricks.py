@@ -51,6 +51,24 @@ def test_gather_moves_rows_exactly(d):
     assert torch.all(out[:, :, 3] == 0)
 
 
+@pytest.mark.parametrize("d,rows", [(64, 1), (64, 513), (128, 130), (128, 40000)])
+def test_gather_status_in_a_workspace_of_any_content(d, rows):
+    """The gather clears its status itself, in a grid of one CTA or of several waves: a call reports its own bad index and
+    nothing that was in the workspace before."""
+    x = torch.randn((1, 3, 700, d), generator=torch.Generator().manual_seed(rows)).to(torch.bfloat16).to(DEV)
+    index = (torch.arange(rows, dtype=torch.int32, device=DEV) * 7) % 700
+    bad = index.clone()
+    bad[rows - 1] = -2
+    want = x[:, :, index.long()]
+    for fill in (0x00, 0xA5, 0xFF):
+        ws = torch.full((256,), fill, dtype=torch.uint8, device=DEV)
+        for i, status in ((index, sa.OK), (bad, sa.E_BAD_INDEX), (index, sa.OK)):
+            out = sa.gather_tokens(x, i, workspace=ws)
+            assert sa.read_status(ws) == status
+            assert torch.equal(out[:, :, : rows - 1], want[:, :, : rows - 1])
+            assert torch.equal(out[:, :, rows - 1], want[:, :, rows - 1] * (1 if status == sa.OK else 0))
+
+
 def _to_bricks(x, gather):
     return sa.gather_tokens(x, gather)
 
