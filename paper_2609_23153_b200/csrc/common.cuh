@@ -13,33 +13,55 @@ namespace sparkattn {
 // Layout of the 256-byte header at the start of every workspace.
 //   word 0: device status (0 = OK, else a negative sparkattn_status)
 //   word 1: detail (offending index, or an id of the wait that expired)
-//   word 2: how often a kernel has cleared the first two by itself (see header_begin)
 constexpr int kWorkspaceHeaderBytes = 256;
-constexpr int kHeaderTurnWord = 2;
 
 __device__ __forceinline__ void report_status(int32_t* status, int code, int detail) {
   if (atomicCAS(status, 0, code) == 0) status[1] = detail;
 }
 
-// Every call starts with a clean status.  A small kernel in front can see to it; a kernel whose CTAs report nothing before their
-// end can do it itself: its first CTA clears the words and counts up, every CTA notes the count when it starts, and one
-// with something to report waits until the count has moved since (or for a millisecond, if it had moved already).
-// The memory may hold anything before.
-__device__ __forceinline__ int32_t header_begin(int32_t* status, bool first_cta) {
-  volatile int32_t* turn = status + kHeaderTurnWord;
-  const int32_t before = *turn;
-  if (first_cta) {
-    status[0] = 0;
-    status[1] = 0;
-    __threadfence();
-    *turn = before + 1;
-  }
-  return before;
+// Every call starts with a clean status, in memory of any content.  A small kernel in front can see to it (report_status above
+// relies on that), or the kernel does it itself: its first CTA takes the two words in one exchange.  CTAs run in no order, so
+// a report may come before that, and nobody waits to find out: report_early puts its code over everything but
+// another code, and a first CTA that has taken a code, which may be one of this launch or what an earlier call left, looks
+// through all of the call's indices itself (recheck_lists; the gather has its own) and reports again what it finds.  A bad index
+// is reported whatever the order; it costs what the CTAs that hold it need for an atomic each, and the next call on
+// that workspace the first CTA's look.  (A wait that runs out can't be looked up again.  It is reported two seconds after
+// its CTA began, and lost only if the first CTA begins later than that.)  Having waited for the first CTA, for a millisecond
+// where it could have begun before, cost one bad index among the 75,600 of 40 heads 1,256 us instead of 235.
+__device__ __forceinline__ bool is_status_code(unsigned long long header) {
+  const int32_t code = (int32_t)(uint32_t)header;
+  return code < 0 && code >= SPARKATTN_E_NO_DEVICE;
 }
-__device__ __forceinline__ void header_await(int32_t* status, int32_t before) {
-  const volatile int32_t* turn = status + kHeaderTurnWord;
-  for (int i = 0; i < 1000 && *turn == before; ++i) __nanosleep(1000);
-  __threadfence();
+__device__ __forceinline__ bool take_header(int32_t* status) {
+  return is_status_code(atomicExch(reinterpret_cast<unsigned long long*>(status), 0ull));
+}
+__device__ __forceinline__ void report_early(int32_t* status, int code, int detail) {
+  unsigned long long* header = reinterpret_cast<unsigned long long*>(status);
+  const unsigned long long mine = (unsigned long long)(uint32_t)detail << 32 | (uint32_t)code;
+  unsigned long long seen = 0;
+  for (int i = 0; i < 8; ++i) {          // (what is no code changes once at most, into the zero of the first CTA)
+    const unsigned long long found = atomicCAS(header, seen, mine);
+    if (found == seen || is_status_code(found)) return;
+    seen = found;
+  }
+}
+// warp `warp` of the `warps` of the first CTA that look the kept lists up again; each reports one bad index.  (Called behind
+// everything else, so that the compiler keeps it away from the tile loops: in front of them, 40 heads of 75,600 tokens 2974 us instead of
+// 2954, 64-token blocks 3408 and 3344.)
+static __device__ __noinline__ void recheck_lists(const int32_t* kept_idx, const int32_t* kept_cnt, int64_t lists, int nb, int kmax, int32_t* status,
+                                                  int warp, int warps) {
+  const int lane = threadIdx.x & 31;
+  for (int64_t l = warp; l < lists; l += warps) {
+    const int cnt = kept_cnt ? min(max(kept_cnt[l], 0), kmax) : kmax;
+    for (int base = 0; base < cnt; base += 32) {
+      const int kb = base + lane < cnt ? kept_idx[l * kmax + base + lane] : 0;
+      const bool bad = kb < 0 || kb >= nb;
+      const uint32_t who = __ballot_sync(0xffffffffu, bad);
+      if (who == 0) continue;
+      if (lane == __ffs(who) - 1) report_early(status, SPARKATTN_E_BAD_INDEX, kb);
+      return;
+    }
+  }
 }
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p) {
@@ -141,7 +163,7 @@ __device__ __forceinline__ bool pipe_wait(uint64_t* bar, uint32_t parity, volati
   }
 }
 __device__ __forceinline__ void report_abort(int32_t* status, int abort_flag) {
-  if (abort_flag >= kAbortTimeout) report_status(status, SPARKATTN_E_DEVICE_TIMEOUT, abort_flag - kAbortTimeout);
+  if (abort_flag >= kAbortTimeout) report_early(status, SPARKATTN_E_DEVICE_TIMEOUT, abort_flag - kAbortTimeout);
 }
 
 // Asynchronous 16-byte copies global -> shared (both sides 16-byte aligned) and their groups.

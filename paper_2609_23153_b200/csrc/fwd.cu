@@ -99,6 +99,7 @@ fwd_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant__ C
   volatile int* s_abort = reinterpret_cast<volatile int*>(bars + 52);
   int* s_ntiles = reinterpret_cast<int*>(bars + 53);
   int* s_bad = s_ntiles + 1;          // place of an invalid index in the list, or -1
+  int* s_code = s_ntiles + 2;         // first CTA, C = 2: there was a code in the header it has taken
   float2* s_sums = reinterpret_cast<float2*>(smem + Smem::kSums);
   int32_t* s_list = reinterpret_cast<int32_t*>(smem + Smem::kList);   // validated kept block indices
   auto tile_k = [&](int c, int slot) { return smem + Smem::kKV + (c * 4 + slot * 2) * kFwdPair; };
@@ -139,10 +140,9 @@ fwd_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant__ C
   // C = 2 is one wave of CTAs at most and clears the status itself (64 items of 16 tiles 9.5 us, 10.2 with a kernel in front for it;
   // one launch less: of 3 tiles 6.1 and 8.4); C = 1 has it cleared, and a timeout recorded by an earlier
   // CTA of the launch makes the rest of the grid drain at once
-  int32_t turn = 0;
   if (threadIdx.x == 0) {
     if constexpr (C == 2) {
-      turn = header_begin(p.status, blockIdx.x == 0);
+      if (blockIdx.x == 0) *s_code = take_header(p.status);
       *s_abort = 0;
     } else {
       *s_abort = (*reinterpret_cast<volatile int32_t*>(p.status) == SPARKATTN_E_DEVICE_TIMEOUT) ? 1 : 0;
@@ -444,9 +444,11 @@ fwd_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant__ C
   tc_fence_before();
   __syncthreads();
   if (threadIdx.x == 0 && (*s_abort >= kAbortTimeout || *s_bad >= 0)) {
-    if constexpr (C == 2) header_await(p.status, turn);
-    if (*s_bad >= 0) report_status(p.status, SPARKATTN_E_BAD_INDEX, p.kept_idx[((int64_t)bh * p.nb + qb) * p.kmax + *s_bad]);
+    if (*s_bad >= 0) report_early(p.status, SPARKATTN_E_BAD_INDEX, p.kept_idx[((int64_t)bh * p.nb + qb) * p.kmax + *s_bad]);
     report_abort(p.status, *s_abort);
+  }
+  if constexpr (C == 2) {
+    if (blockIdx.x == 0 && *s_code) recheck_lists(p.kept_idx, p.kept_cnt, gridDim.x, p.nb, p.kmax, p.status, warp, 6 * C);
   }
   if (warp == kTmaWarp) {
     if (*s_abort) __nanosleep(200000);  // let copies / MMAs in flight land before the CTA's resources go

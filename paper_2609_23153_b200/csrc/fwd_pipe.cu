@@ -146,7 +146,7 @@ __device__ __forceinline__ void report_bad_index(const PipeParams& p, int item, 
     const int cnt = p.kept_cnt ? min(max(p.kept_cnt[list], 0), p.kmax) : p.kmax;
     for (int t = 0; t < cnt; ++t) {
       const int kb = p.kept_idx[list * p.kmax + t];
-      if (kb < 0 || kb >= p.nb) report_status(p.status, SPARKATTN_E_BAD_INDEX, kb);
+      if (kb < 0 || kb >= p.nb) report_early(p.status, SPARKATTN_E_BAD_INDEX, kb);
     }
   }
 }
@@ -404,6 +404,7 @@ fwd_pipe_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
   volatile int* s_abort = reinterpret_cast<volatile int*>(s_tmem + 1);
   volatile int* s_gate_bh = s_abort + 1;      // GATE: (batch, head) whose P_q and C are in shared memory
   volatile int* s_bad = s_abort + 2;          // a list of this CTA's items held an invalid index
+  volatile int* s_code = s_abort + 3;         // first CTA, own lists: there was a code in the header it has taken
   // What the softmax warpgroups need to know of a tile, written by the K producer in the slot tile % 8 before it requests
   // the K tile: the number of real columns (WINDOW: the key block), PAIR with the flags of the two query blocks in bits
   // 30 and 31; FP8: K scale, log2 of the factor folded into P, its inverse.  PAIR: the same of the tile's second block.
@@ -467,10 +468,9 @@ fwd_pipe_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
   // and the line-up behind the wait: 3 heads of 1,200 tokens 9.0 us, 8.8 without, FP8 8.5 and 8.1, 40 of 6,479 106.6 and 105.3.)
   pdl_wait();
   const int first_item = blockIdx.x, item_step = gridDim.x;
-  int32_t turn = 0;
   if constexpr (!FP8) {
     if (p.own_lists) {
-      if (threadIdx.x == 0) turn = header_begin(p.status, blockIdx.x == 0);
+      if (blockIdx.x == 0 && threadIdx.x == 0) *s_code = take_header(p.status);
       for (int item = first_item + warp * item_step; item < p.items; item += (int)(blockDim.x >> 5) * item_step) {
         if constexpr (PAIR) pair_list(p.kept_idx, p.kept_cnt, p.clean_cnt, p.clean_list, item, p.nb, p.nbq, p.kmax, warp, lane);
         else compact_list(p.kept_idx, p.kept_cnt, p.clean_cnt, p.clean_list, item, p.nb, p.kmax, lane);
@@ -1337,11 +1337,14 @@ fwd_pipe_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
   tc_fence_before();
   __syncthreads();
   if (threadIdx.x == 0 && (dead || *s_abort || *s_bad)) {
-    if (!FP8 && p.own_lists) header_await(p.status, turn);
-    if (dead) report_status(p.status, SPARKATTN_E_MISALIGNED, (int)(smem_u32(smem) & 1023u));
+    if (dead) report_early(p.status, SPARKATTN_E_MISALIGNED, (int)(smem_u32(smem) & 1023u));
     for (int item = first_item; *s_bad && item < p.items; item += item_step)
       if (p.clean_cnt[item] & kBadFlag) report_bad_index(p, item, PAIR);
     report_abort(p.status, *s_abort);
+  }
+  if constexpr (!FP8) {            // (by the softmax warps, which have the registers of any code)
+    if (p.own_lists && blockIdx.x == 0 && *s_code && warp >= 4 && warp < 12)
+      recheck_lists(p.kept_idx, p.kept_cnt, (int64_t)(p.items / p.nbq) * p.nb, p.nb, p.kmax, p.status, warp - 4, 8);
   }
   if (warp == 0) {
     if (*s_abort) __nanosleep(200000);  // let copies / MMAs in flight land before the CTA's resources go

@@ -47,9 +47,9 @@ constexpr int kGatherThreads = 256, kGatherUnroll = 8;
 // (between the loads it kept them from being in flight together).  Launched while the kernel before it drains, and it
 // clears its status itself; a memset in front and a plain launch were a third of a small call.  6 heads of 6,479 tokens 8.2 -> 5.5 us, 40 of
 // 6,479 34.5 -> 26.3, 12 of 28,050 43.2 -> 32.9 (bricks of 3 x 5 x 8); attention in brick order with its four gathers 82.1 -> 61.7, 340.6 ->
-// 299.3, 955.8 -> 924.0.
+// 299.3, 955.8 -> 924.0.  (Four CTAs per SM: left to itself the compiler takes registers for three.)
 template <int PIECES>   // 16-byte pieces per token row: 16 (d = 128) or 8 (d = 64)
-__global__ void __launch_bounds__(kGatherThreads)
+__global__ void __launch_bounds__(kGatherThreads, 4)
 gather_tokens_kernel(const uint4* x, const int32_t* index, uint4* __restrict__ out, int H,
                      int n_src, int n_dst, int64_t src_b, int64_t src_h, int64_t src_n, int64_t dst_b, int64_t dst_h,
                      int64_t dst_n /* strides in 16-byte pieces */, int chunks_per_bh, int32_t* __restrict__ status) {
@@ -62,7 +62,8 @@ gather_tokens_kernel(const uint4* x, const int32_t* index, uint4* __restrict__ o
   const uint4* xs = x + b * src_b + h * src_h + piece;
   uint4* os = out + b * dst_b + h * dst_h + piece;
   pdl_wait();
-  const int32_t turn = header_begin(status, blockIdx.x == 0 && threadIdx.x == 0);
+  bool code_there = false;
+  if (blockIdx.x == 0 && threadIdx.x == 0) code_there = take_header(status);
   int src[kGatherUnroll];
   uint4 v[kGatherUnroll];
 #pragma unroll
@@ -78,13 +79,21 @@ gather_tokens_kernel(const uint4* x, const int32_t* index, uint4* __restrict__ o
     const int i = row0 + u * kRowsPerPass;
     if (i < n_dst) os[(int64_t)i * dst_n] = v[u];
   }
-  int bad = -1;                                            // (such a row is written as zeros)
+  // a bad index (its rows are written as zeros) is reported by one thread of one (batch, head)
+  auto is_bad = [&](int i) { return (unsigned)i >= (unsigned)n_src && i != -1; };
+  if (bh == 0 && piece == 0) {
+    int bad = -1;
 #pragma unroll
-  for (int u = 0; u < kGatherUnroll; ++u)
-    if ((unsigned)src[u] >= (unsigned)n_src && src[u] != -1) bad = src[u];
-  if (bad != -1) {
-    header_await(status, turn);
-    report_status(status, SPARKATTN_E_BAD_INDEX, bad);
+    for (int u = 0; u < kGatherUnroll; ++u)
+      if (is_bad(src[u])) bad = src[u];
+    if (bad != -1) report_early(status, SPARKATTN_E_BAD_INDEX, bad);
+  }
+  if (blockIdx.x == 0 && __syncthreads_or(code_there)) {
+    int bad = -1;
+#pragma unroll 1
+    for (int i = threadIdx.x; i < n_dst; i += kGatherThreads)
+      if (is_bad(index[i])) bad = index[i];
+    if (bad != -1) report_early(status, SPARKATTN_E_BAD_INDEX, bad);
   }
 }
 

@@ -51,6 +51,28 @@ extern "C" int timeout_probe(void* workspace, unsigned long long limit_ns, int w
   return cudaGetLastError() == cudaSuccess ? 0 : -1;
 }
 
+// The status header of a kernel that clears it itself: the first of two CTAs takes the header and looks the two lists up again
+// when a code was in it, the second reports the bad index of its list, if it has one.  Whichever is not `early` begins some
+// milliseconds late (neither waits for the other).
+__global__ void header_probe_kernel(int32_t* status, const int32_t* lists, int nb, int kmax, int early) {
+  if ((int)blockIdx.x != early)
+    for (int i = 0; i < 5000; ++i) __nanosleep(1000);
+  if (blockIdx.x == 0) {
+    bool code_there = false;
+    if (threadIdx.x == 0) code_there = take_header(status);
+    if (__syncthreads_or(code_there)) recheck_lists(lists, nullptr, 2, nb, kmax, status, threadIdx.x >> 5, 2);
+  } else if (threadIdx.x < kmax) {
+    const int32_t kb = lists[kmax + threadIdx.x];
+    if (kb < 0 || kb >= nb) report_early(status, SPARKATTN_E_BAD_INDEX, kb);
+  }
+}
+
+extern "C" int header_probe(void* workspace, const void* lists, int nb, int kmax, int early, void* stream) {
+  header_probe_kernel<<<2, 64, 0, static_cast<cudaStream_t>(stream)>>>(static_cast<int32_t*>(workspace), static_cast<const int32_t*>(lists), nb,
+                                                                      kmax, early);
+  return cudaGetLastError() == cudaSuccess ? 0 : -1;
+}
+
 // A launch without blocks, which the runtime refuses on the host, through the library's launch helper.  Bit 0: the helper
 // did not report it; bit 1: the runtime still holds the error.
 __global__ void never_run_kernel(int) {}

@@ -69,6 +69,27 @@ def test_gather_status_in_a_workspace_of_any_content(d, rows):
             assert torch.equal(out[:, :, rows - 1], want[:, :, rows - 1] * (1 if status == sa.OK else 0))
 
 
+def test_gather_bad_index_holds_nothing_up():
+    """A grid of several waves (10 heads of 591 CTAs, 60 us): a bad index in the last row, in every row and in none take
+    the same time; a CTA that waited for another to report would need a millisecond."""
+    N = 75_600
+    x = torch.randn((1, 10, N, 128), device=DEV).to(torch.bfloat16)
+    good = torch.arange(N, dtype=torch.int32, device=DEV).flip(0)
+    one, every = good.clone(), torch.full_like(good, N)
+    one[N - 1] = -7
+    ws = torch.zeros(256, dtype=torch.uint8, device=DEV)
+    for index, want in ((good, sa.OK), (one, sa.E_BAD_INDEX), (every, sa.E_BAD_INDEX), (good, sa.OK)):
+        times = []
+        for _ in range(5):
+            start, end = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            start.record()
+            sa.gather_tokens(x, index, workspace=ws)
+            end.record()
+            assert sa.read_status(ws) == want
+            times.append(start.elapsed_time(end))
+        assert min(times) < 0.5, times
+
+
 def _to_bricks(x, gather):
     return sa.gather_tokens(x, gather)
 

@@ -54,3 +54,22 @@ def test_failed_launch_is_reported_once(probe, overlap):
     """A launch that the runtime refuses on the host: the library's launch helper reports it and takes the runtime's
     last error with it, so that the check after a later, unrelated launch does not find it again."""
     assert probe.launch_probe(overlap) == 0
+
+
+@pytest.mark.parametrize("early", [0, 1])
+@pytest.mark.parametrize("words", [(0, 0), (0, 5), (0x5A5A5A5A, 1), (-1515870811, -1515870811), (-1, -1), (sa.E_BAD_INDEX, 3), (sa.E_DEVICE_TIMEOUT, 9), (-9, 0)])
+def test_bad_index_is_reported_in_any_order(probe, early, words):
+    """A kernel that clears the status itself: a report made milliseconds before the first CTA begins is kept, whatever the
+    memory held (nothing, anything, an earlier call's code), and what an earlier call left is gone."""
+    probe.header_probe.argtypes = [ctypes.c_void_p, ctypes.c_void_p, ctypes.c_int, ctypes.c_int, ctypes.c_int, ctypes.c_void_p]
+    nb, kmax = 7, 40
+    good = torch.arange(2 * kmax, dtype=torch.int32, device="cuda:0") % nb
+    bad = good.clone()
+    bad[2 * kmax - 3] = nb + 4
+    stream = ctypes.c_void_p(torch.cuda.current_stream().cuda_stream)
+    for lists, status, detail in ((good, sa.OK, 0), (bad, sa.E_BAD_INDEX, nb + 4)):
+        ws = torch.zeros(64, dtype=torch.int32)
+        ws[0], ws[1] = words
+        ws = ws.cuda()
+        assert probe.header_probe(ctypes.c_void_p(ws.data_ptr()), ctypes.c_void_p(lists.data_ptr()), nb, kmax, early, stream) == 0
+        assert ws[:2].tolist() == [status, detail]
