@@ -281,6 +281,26 @@ def test_quant_with_pooling_at_every_tail(d, block, tail):
         assert torch.equal(pooled.view(torch.int32), want)
 
 
+@pytest.mark.parametrize("nb,H", [(65, 2), (65, 30), (65, 74), (250, 2), (250, 10), (250, 28), (257, 1), (257, 9)])
+@pytest.mark.parametrize("d", [64, 128])
+def test_select_from_pooled_clears_the_status(nb, H, d):
+    """Scores + top-k on pooled means clear the status themselves.  More than 64 key blocks: 8, 16 and 32 query blocks per CTA
+    (2, 30 or 10, 74 or 28 heads), beyond 256 blocks 8 and 16 (1 and 9 heads); in a workspace of any content, twice in the
+    same one, and with the lists of the selection that pools for itself."""
+    q, k = (torch.randn((1, H, nb * 64 - 3, d), generator=torch.Generator().manual_seed(nb + H + i)).to(torch.bfloat16).to(DEV) for i in (0, 1))
+    topk = nb // 3
+    want, count = sa.select(q, k, 64, topk)
+    ws = sa.alloc_workspace(sa.make_shape(q, 64), 0, topk, DEV)
+    for fill in (0xA5, 0xFF):
+        ws.fill_(fill)
+        sa.quant_fp8_pooled(q, 64, False, ws), sa.quant_fp8_pooled(k, 64, True, ws)
+        for _ in range(2):
+            idx, cnt = sa.select_pooled(q, 64, topk, ws)
+            assert sa.read_status(ws) == sa.OK
+            assert torch.equal(idx, want) and torch.equal(cnt, count)
+            ws[:256] = fill
+
+
 def test_quant_with_pooling_strided_batch_equals_separate_calls():
     """[B, N, H, d] buffers viewed as [B, H, N, d], two batch entries: the fused pass must reproduce the separate
     sparkattn_quant_fp8 / sparkattn_select calls bit for bit."""
