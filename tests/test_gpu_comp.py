@@ -73,6 +73,29 @@ def test_state_over_chunk_counts(tiles, H):
     assert _relrms(state[0].cpu(), ref) <= 1e-2
 
 
+@pytest.mark.parametrize("tiles", range(1, 8))
+def test_apply_over_tiles_per_cta(tiles):
+    """148 heads, a CTA each: 1 to 7 tiles of one CTA, so that the two Q slots and the three output slots go once round and
+    again, with a ragged last tile.  Against the oracle for some heads; one head at a time (its tiles spread over as many
+    CTAs) and in place bit for bit."""
+    H = 148
+    w = workloads.Workload("comptiles", 61 + tiles, 1, H, 128, (1, 1, tiles * 128 - 5), 128, 0.5)
+    q, k, v, osp, pq, pk, gate, axis, freq = _inputs(w)
+    state = sa.comp_state(k, v, pk, w.grid, axis, freq)
+    out = sa.comp_apply(q, pq, state, gate, osp, w.grid, axis, freq, check_status=True)
+    buf = osp.clone()
+    sa.comp_apply(q, pq, state, gate, buf, w.grid, axis, freq, out=buf)
+    assert torch.equal(out, buf)
+    for h in (0, 73, 147):
+        one = slice(h, h + 1)
+        part = [t[:, one].contiguous() for t in (q, state, gate, osp)]
+        alone = sa.comp_apply(part[0], pq[one].contiguous(), part[1], part[2], part[3], w.grid, axis, freq)
+        assert torch.equal(out[:, one].view(torch.int16), alone.view(torch.int16))
+        ref = oracle.comp_apply(part[0][0].cpu(), pq[one].cpu().contiguous(), part[1][0].cpu().double(), part[2][0].cpu(), part[3][0].cpu(), w.grid,
+                                axis, freq, [(0, i) for i in range(w.N)]).reshape(1, w.N, w.d)
+        _check_out(out[0, one].cpu(), ref)
+
+
 def test_state_is_deterministic_and_apply_in_place():
     w = workloads.Workload("compdet", 17, 1, 2, 128, (4, 10, 16), 128, 0.5)
     q, k, v, osp, pq, pk, gate, axis, freq = _inputs(w)
