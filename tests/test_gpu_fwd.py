@@ -259,10 +259,50 @@ def test_lists_cleaned_ahead_or_by_the_cta(block, kmax):
             assert torch.equal(lse[:, h].view(torch.int32), lse_one.view(torch.int32))
 
 
+@pytest.mark.parametrize("form,block,kmax", [("window", 128, 9), ("window", 128, 129), ("window", 64, 9), ("window", 64, 70), ("padded", 128, 9),
+                                             ("padded", 64, 9), ("gated", 128, 9), ("gated", 128, 129)])
+def test_lists_cleaned_ahead_or_by_the_cta_in_every_form(form, block, kmax):
+    """The same for the windowed, padded and gated forwards: 18 heads at once take the pre-pass, 9 and 9 clean their own
+    lists (64-token blocks up to 64 entries in the variant with a closing warpgroup, beyond in the other).  Bad indices in some of
+    the lists, then good lists in the workspace that a bad call has left and in memory that reads as a status code."""
+    nbk, H = 140 * 128 // block, 18
+    N, grid = nbk * block, (7, 40, 64)
+    g = torch.Generator().manual_seed(block + kmax)
+    q, k, v = (torch.randn((1, H, N, 128), generator=g).to(torch.bfloat16).to(DEV) for _ in range(3))
+    idx = torch.randint(0, nbk, (1, H, nbk, kmax), generator=g, dtype=torch.int32)
+    cnt = torch.randint(0, 7, (1, H, nbk), generator=g, dtype=torch.int32)
+    cnt[0, :, 7] = kmax
+    bad = idx.clone()
+    bad[0, ::3, 7, kmax - 1] = nbk
+    valid = torch.randint(1, block + 1, (nbk,), generator=g, dtype=torch.int32).to(DEV)
+    if form == "gated":
+        pq = (torch.randn((H, 64, 128), generator=g) / 128 ** 0.5).to(torch.bfloat16).to(DEV)
+        state, gate = torch.randn((1, H, 64, 128), generator=g).to(DEV), torch.rand((1, H, N), generator=g).to(DEV)
+        axis, freq = workloads.rope_schedule(128, 64)
+
+    def run(lists, h, ws):
+        args = [t[:, h] for t in (q, k, v)] + [t[:, h].contiguous().to(DEV) for t in (lists, cnt)]
+        kw = dict(return_lse=True, workspace=ws)
+        if form == "gated":
+            return sa.fwd_gated(*args, pq[h].contiguous(), state[:, h].contiguous(), gate[:, h].contiguous(), grid, axis, freq, **kw)
+        return sa.fwd(*args, block, **kw, **(dict(frame_tokens=450, window=20) if form == "window" else dict(block_valid=valid)))
+
+    shape = sa.make_shape(q, block)
+    size = sa.fwd_gated_workspace_bytes(shape, kmax, grid) if form == "gated" else sa.workspace_bytes(shape, 1, kmax)
+    ws = torch.full((size,), 0xFF, dtype=torch.uint8, device=DEV)
+    for lists, want in ((idx, sa.OK), (bad, sa.E_BAD_INDEX), (idx, sa.OK)):
+        out, lse = run(lists, slice(0, H), torch.full_like(ws, 0xA5) if lists is bad else ws)
+        for h in (slice(0, 9), slice(9, 18)):
+            one, lse_one = run(lists, h, ws)
+            assert sa.read_status(ws) == want
+            assert torch.equal(out[:, h].view(torch.int16), one.view(torch.int16))
+            assert torch.equal(lse[:, h].view(torch.int32), lse_one.view(torch.int32))
+
+
 @pytest.mark.parametrize("H,window", [(3, 0), (7, 0), (3, 2)])
 def test_d64_chains_of_every_length(H, window):
-    """d = 64: the tiles of an item go to four chains (H = 3: 123 items, no SM gets a second one) or two (H = 7), so lists
-    of 0 .. 9 blocks leave chains empty, level and one tile apart; ragged last block, and rows whose tiles are all
+    """d = 64: the pairs of blocks of an item go to two chains (H = 3: 123 items, no SM gets a second one) or one (H = 7), so lists
+    of 0 .. 9 blocks leave chains empty, level, a pair and half a pair apart; ragged last block, and rows whose tiles are all
     masked in some chains (causal window).  Scores large enough that references are raised on the way."""
     nbk, block, frame = 41, 64, 300
     N = nbk * block - 21
@@ -577,7 +617,7 @@ def test_d64_status_in_a_workspace_of_any_content(H):
 def test_lse_of_merged_chains_is_rounded_once(H):
     """d = 64: scores that fp32 holds exactly and one key that outweighs the others, so that the log-sum-exp is off by its
     own rounding (at most 2^-24 of it) and by what ln 2 and log2 e lose as fp32 constants (1.1e-8 together).  112 items
-    run four chains each, 224 two."""
+    run two chains each, 224 one."""
     N, nb = 256, 4
     a = 128 + torch.arange(N) % 128
     b = (200 + torch.arange(H))[:, None] - 16 * torch.ones((H, N), dtype=torch.int64)
