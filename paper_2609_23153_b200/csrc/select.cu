@@ -616,9 +616,10 @@ topk_wide_kernel(const float* pq, const float* pkT, int32_t* __restrict__ kept_i
 // Up to 64 key blocks: latency is all there is.  The pooled K of the (batch, head) comes into shared memory in one go, not
 // through a ring, a warp takes a query block, a lane one or two key blocks (lane, lane + 32) with their chains in registers,
 // and the selection holds one or two keys per lane instead of eight.  38 KB of shared memory at most, so that its CTAs are
-// on the SMs while the pooling kernel drains.  Whole selection against topk_kernel, us: 3 heads of 10 blocks 8.4 -> 5.9, 8 of 25 10.3 -> 7.7,
-// 6 of 51 13.3 -> 10.0, 20 of 51 20.0 -> 16.2, 40 of 51 35.0 -> 33.6; the same for up to 128 blocks (72 KB): 6 of 94 15.8 -> 19.1.  Two query
-// blocks per warp: 6 of 51 21.4.
+// on the SMs while the pooling kernel drains.  Whole selection against topk_kernel, us, d = 128: 3 heads of 10 blocks 8.3 -> 5.6, 8 of 25 9.9 ->
+// 7.1, 6 of 51 11.5 -> 9.4, 20 of 51 17.5 -> 15.4, 40 of 51 34.4 -> 28.4, 80 of 64 71.5 -> 62.6; d = 64: 3 of 10 6.4 -> 5.1, 6 of 51 6.9 -> 5.8, 40 of 33
+// 10.8 -> 9.1, 40 of 51 15.0 -> 10.8, 80 of 64 26.7 -> 21.4.  The same for up to 128 blocks (72 KB): 6 of 94 15.8 -> 19.1.  Two query blocks per
+// warp: 6 of 51 21.4.
 template <int D, int KPL, bool WINDOW>
 __global__ void __launch_bounds__(kTopkThreads)
 topk_small_kernel(const float* pq, const float* pkT, int32_t* __restrict__ kept_idx, int32_t* __restrict__ kept_cnt, int nb, int nbp,
@@ -781,7 +782,7 @@ static int launch_topk_d(const sparkattn_shape_t& s, int topk, int frame_tokens,
   // no warp idle there; wide with 16 rows: 1 / 12 / 40 heads of 256 20.6 / 54 / 158 against 12.8 / 51 / 143, d = 64 14.7 / 23.9 /
   // 65 against 9.1 / 20.8 / 59), with as many rows per CTA as still leave 1.5 CTAs (32 rows) or one CTA (16) per SM:
   // 80 heads of 250 blocks 63.9 us with 32 rows, 69.9 with 16, 94.6 with 8; 12 heads of 256 22.0 / 20.8 / 22.2; 3 heads
-  // of 50 16.9 / 12.5 / 10.4.
+  // of 100 19.8 / 14.3 / 11.5.  Up to 64 blocks: the small kernel, which has both sides.
   if (nb <= kSmallBlocks) return nbp == 32 ? go(launch_topk_small<D, 1>) : go(launch_topk_small<D, 2>);
   if (nb > 256) {
     if (ctas16 > kNumSMs && wide_smem(16, D, nbp) <= kSmemOfTwo) return go(launch_topk_wide<D, 16, 8, 10, 2>);
