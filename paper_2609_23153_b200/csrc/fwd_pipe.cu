@@ -1473,10 +1473,12 @@ static int launch_pipe(const sparkattn_shape_t& s, bool fp8, const void* q, cons
   const size_t bits = pair ? (size_t)kPairWarps * 2 * ((nb + 31) / 32) * sizeof(uint32_t) : 0;
   const int warps = pair ? kPairWarps : kCompactWarps, heads = s.B * s.H;
   // bf16, up to 16 items per CTA (a warp each, or two rounds of the warps): every CTA cleans the lists of its own items before it
-  // starts, and no kernel stands between the caller's last one and the forward.  Beyond, the pre-pass costs nothing that
-  // shows.  Attention, pre-pass / own lists, us: 3 heads of 1,200 tokens 17.9 / 17.5, 6 of 6,479 48.7 / 47.8 (64-token blocks 41.1 /
-  // 40.0, causal 50.2 / 49.4), 20 of 6,479 (6.9 items) 79.5 / 77.7, 40 of 6,479 (13.8) 148.2 / 147.2.  FP8 needs a kernel for the largest V
-  // scales all the same.
+  // starts, and no kernel stands between the caller's last one and the forward.  Attention, pre-pass / own lists, us: 3 heads of
+  // 1,200 tokens 17.9 / 17.5, 6 of 6,479 48.7 / 47.8 (64-token blocks 41.1 / 40.0, causal 50.2 / 49.4), 20 of 6,479 (6.9 items) 79.5 / 77.7, 40
+  // of 6,479 (13.8) 148.2 / 147.2.  Beyond, it makes no difference that shows and the tile loops start at once: 50 heads of 6,479 (17.2)
+  // 263.4 / 265.8, 80 (27.6) 411.8 / 410.8, 100 with 64-token blocks (34.5) 468.5 / 469.3.  Long lists take no harm within the line, forward alone:
+  // 192 of 256 blocks (15.6 items) 3282 / 3266, 300 of 591 (8.0) 2606 / 2569, 64-token blocks 200 of 512 (6.9) 1113 / 1107, 1024 of 2048 (13.8)
+  // 15,493 / 15,496; 10 entries in lists of 300 195.5 / 193.9, of 2048 169.7 / 168.2.  FP8 needs a kernel for the largest V scales all the same.
   constexpr int kOwnItems = 16;
   prm.own_lists = !fp8 && items <= (long long)kOwnItems * sm_count;
   if (fp8)
