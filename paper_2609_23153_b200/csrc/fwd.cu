@@ -25,7 +25,7 @@
 // Bound by the softmax warps: a pair's 8192 exponentials are 512 clocks of the SM's special-function units, 1,170 clocks per
 // pair and SM at 125 tiles per item, where one chain runs its short steps under the other's exponentials.  Against one query block
 // per CTA with its 64 rows in two quarters (four or two chains of single tiles), us: 2 heads of 2,048 tokens, 16 of 32 tiles 12.6 ->
-// 10.2; 16 heads, 32 of 32 59 -> 42; 6 heads of 6,479, 10 of 102 30.5 -> 26.0, in a window of three frames 48 -> 38.5; 12 heads of
+// 10.2 (9.5 since it clears the status itself); 16 heads, 32 of 32 59 -> 42; 6 heads of 6,479, 10 of 102 30.5 -> 26.0, in a window of three frames 48 -> 38.5; 12 heads of
 // 8,000, 125 of 125 520 -> 410; 40 heads of 32,760, 15 of 512 1020 -> 900.
 //
 // Every wait on an mbarrier is bounded (common.cuh); a kept index outside
@@ -305,7 +305,7 @@ fwd_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant__ C
       }
       // The chain's last PV is the previous pair's: once it is complete P has been read and O is quiescent.  It is waited for behind
       // the first kWaitAt pieces of eight columns.  Two of them where the length of the chain is all there is (C = 2: 64 items
-      // of 16 tiles 10.1 us, 10.3 with none); none where the stores of P should run under the exponentials (C = 1: 12 heads of
+      // of 16 tiles 0.2 us less than with none); none where the stores of P should run under the exponentials (C = 1: 12 heads of
       // 8,000 tokens 410 us, two 432, all eight 450).
       constexpr int kWaitAt = C == 2 ? 2 : 0;
       auto wait_pv = [&]() { return n == 0 || __all_sync(0xffffffffu, pipe_wait(bar_pv_done(chain), (n - 1) & 1, s_abort, 10)); };
@@ -489,7 +489,7 @@ int launch_fwd(const sparkattn_shape_t& s, int dtype, const void* q, const void*
   if (fwd_pipe_supported(s))
     return launch_fwd_pipe(s, fp8, q, k, v, q_scale, k_scale, v_scale, kept_idx, kept_cnt, kmax, frame_tokens, window,
                            block_valid, out, lse, workspace, stream);
-  // d = 128 always runs the persistent kernel; a sequence too long for its list pre-pass is not served
+  // d = 128 always runs the persistent kernel; a sequence too long for its merged lists is not served
   if (s.d != 64 || s.block != 64 || fp8 || block_valid != nullptr) return SPARKATTN_E_UNSUPPORTED_SHAPE;
   const int elt = 2;
   CUtensorMap mq, mk, mv;
@@ -518,7 +518,7 @@ int launch_fwd(const sparkattn_shape_t& s, int dtype, const void* q, const void*
   if (ctas > 0x7fffffffLL) return SPARKATTN_E_UNSUPPORTED_SHAPE;
   const int sm_count = current_sm_count();
   if (sm_count < 1) return SPARKATTN_E_CUDA;
-  // two chains while no SM gets a second item, us against one chain and two CTAs per SM: 64 items of 16 tiles 10.3 / 11.5, 128 10.7 /
+  // two chains while no SM gets a second item, us against one chain and two CTAs per SM (the status cleared in front of both): 64 items of 16 tiles 10.3 / 11.5, 128 10.7 /
   // 11.9; but 160 19.0 / 14.2, 256 items of 3 tiles 12.3 / 8.1, 512 of 32 56.5 / 42.4
   if (ctas <= sm_count) return launch_fwd_t<2>(mq, mk, mv, prm, ctas, stream);
   if ((rc = launch_kernel(clear_header_kernel, 1, kWorkspaceHeaderBytes / 4, 0, true, stream, prm.status)) != SPARKATTN_OK) return rc;

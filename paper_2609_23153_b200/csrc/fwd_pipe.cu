@@ -245,7 +245,7 @@ constexpr int kPairMaxBlocks = 16384;    // key blocks per head the merge can ma
 constexpr int kPairWarps = 4;
 __device__ __forceinline__ void pair_list(const int32_t* kept_idx, const int32_t* kept_cnt, int32_t* clean_cnt, int32_t* clean_list,
                                           int pair, int nb, int nbq, int kmax, int wl, int lane) {
-  extern __shared__ uint32_t s_bits[];                      // [kPairWarps][2][words]
+  extern __shared__ uint32_t s_bits[];                      // two bitmaps per calling warp: [warps][2][words]
   const int words = (nb + 31) / 32;
   uint32_t* bits = s_bits + wl * 2 * words;
   for (int i = lane; i < 2 * words; i += 32) bits[i] = 0u;
@@ -276,7 +276,7 @@ __device__ __forceinline__ void pair_list(const int32_t* kept_idx, const int32_t
   __syncwarp();
   int32_t* dst = clean_list + (int64_t)pair * (2 * kmax);
   int out = 0;
-  // the pair's own two key blocks first (see compact_lists_kernel), then the rest in ascending order
+  // the pair's own two key blocks first (see compact_list), then the rest in ascending order
   const int own0 = 2 * qp;
   for (int kb = own0; kb <= own0 + 1 && kb < nb; ++kb) {
     const bool ina = (bits[kb >> 5] >> (kb & 31)) & 1u, inb = (bits[words + (kb >> 5)] >> (kb & 31)) & 1u;
@@ -358,7 +358,7 @@ struct Const {
 };
 __device__ __forceinline__ int uniform(int x) { return __shfl_sync(0xffffffffu, x, 0); }
 
-// PAIR: 64-token blocks; a work item is a pair of query blocks, a tile two key blocks (see pair_lists_kernel).
+// PAIR: 64-token blocks; a work item is a pair of query blocks, a tile two key blocks (see pair_list).
 // GATE (bf16, 128-token blocks, no window): the closing warpgroup of an item also computes the low-rank branch
 // of its 128 query rows and writes O = O_s + g * r * RMSNorm(q~ C) instead of O_s: the item's Q tile is still in
 // shared memory and its normalised output row in registers, so the separate pass that would read Q and O_s

@@ -205,7 +205,7 @@ def test_persistent_path_short_and_empty_lists(seed, kmax, block):
 
 @pytest.mark.parametrize("block,kmax", [(128, 33), (128, 4), (64, 5), (64, 40)])
 def test_bad_indices_are_dropped_and_reported(block, kmax):
-    """d = 128: an index outside [0, nb) is dropped by the list pre-pass and reported by the forward kernel (64-token
+    """d = 128: an index outside [0, nb) is dropped where the lists are cleaned and reported at the end of the CTA (64-token
     blocks: pairs of lists, one with a bad index, an odd number of blocks left).  The output is that of the lists
     without it, bit for bit; the next call's status is clean."""
     nbk, H = 41, 5
@@ -325,7 +325,7 @@ def test_d64_chains_of_every_length(H, window):
 
 @pytest.mark.parametrize("block,fp8", [(128, False), (128, True), (64, False)])
 def test_long_permuted_lists_own_block_anywhere(block, fp8):
-    """Kept lists of 70-100 entries in random order: the forward's list pre-pass moves the query block's own
+    """Kept lists of 70-100 entries in random order: cleaning them moves the query block's own
     key block to the front, wherever it stands (first, inside the first 32 entries, beyond them, at a
     multiple of 32, last, absent), and must keep every other entry exactly once.  Compared with the oracle,
     which walks the lists as given."""
