@@ -341,6 +341,13 @@ def time_region(fn, steps, warmup, stream, dist_on):
     return max_over_ranks(e0.elapsed_time(e1), "cuda")
 
 
+def launches_per_step(w, heads, sm_count):
+    """Kernels of one selection and of one bf16 forward: a selection that keeps every block only lists them; the forward has a kernel
+    in front of it only where a CTA has more than 16 work items (d = 64: an SM more than one)."""
+    items = w.B * heads * ((w.nb + 1) // 2 if (w.d, w.block) == (128, 64) else w.nb)
+    return 1 if w.topk == w.nb else 2, 1 if items <= (16 if w.d == 128 else 1) * sm_count else 2
+
+
 def run_ours(args, w):
     import paper_2609_23153_b200 as sa
     from paper_2609_23153_b200 import build as sa_build
@@ -413,12 +420,13 @@ def run_ours(args, w):
     fwd_tflops = flops / (ms_fwd * 1e-3) / 1e12
     elems = q.numel()
     sel_bytes = 2 * elems * 2 + kept_idx.numel() * 4 + kept_cnt.numel() * 4
+    sel_launches, fwd_launches = launches_per_step(w, Hl, torch.cuda.get_device_properties(dev).multi_processor_count)
     kernels = {
-        "select": {"ms": ms_sel, "launches_per_step": 2, "algorithmic_bytes": sel_bytes,
+        "select": {"ms": ms_sel, "launches_per_step": sel_launches, "algorithmic_bytes": sel_bytes,
                    "GBps": sel_bytes / (ms_sel * 1e-3) / 1e9, "frac_of_hbm_peak": sel_bytes / (ms_sel * 1e-3) / 1e9 / peaks["hbm"]},
-        "fwd_bf16": {"ms": ms_fwd, "launches_per_step": 2, "TFLOPs": fwd_tflops},
+        "fwd_bf16": {"ms": ms_fwd, "launches_per_step": fwd_launches, "TFLOPs": fwd_tflops},
     }
-    pipelined = w.d == 128 and w.block in (64, 128)   # d = 128 runs the persistent pipelined kernel (+ list pre-pass)
+    pipelined = w.d == 128 and w.block in (64, 128)   # d = 128 runs the persistent pipelined kernel
     roofline = {"kernel": f"fwd_pipe_kernel (bf16, d=128, {w.block}x{w.block} blocks)" if pipelined else f"fwd_kernel<{w.d},{w.block},bf16>", "bound": "tensor", "achieved": fwd_tflops, "peak": peaks["bf16"],
                 "unit": "TFLOP/s", "frac": fwd_tflops / peaks["bf16"], "traffic": FWD_DRAM_TRAFFIC_BYTES.get(w.name) if w.sparsity == 0.97 else None,
                 "peak_source": f"{peaks['source']} bf16 burst (sustained {peaks['bf16_sustained']})",
@@ -483,7 +491,7 @@ def run_ours(args, w):
         fp8["chain_fused_ms_quantpool_topk_fwd"] = ms8f
         fp8["fused_quantpool_plus_topk_ms"] = ms_pre
         fp8["separate_select_plus_quant_ms"] = ms_sel + ms_q
-        fp8["fused_launches_per_step"] = 4 + (2 if pipelined else 1)
+        fp8["fused_launches_per_step"] = 4 + 2                # (FP8 is d = 128; its list kernel runs at every size)
         # per-token activation quantisation (the paper's fused scale-and-cast kernel), one tensor, outside the step
         tok_scales = torch.empty((w.B, Hl, w.N), dtype=torch.float32, device=dev)
         tok_codes = torch.empty(q.shape, dtype=torch.uint8, device=dev)    # (its own buffer: codes[] feed the later FP8 legs)
@@ -719,7 +727,7 @@ def run_ours(args, w):
             "metric": METRIC, "value": value, "unit": UNIT, "n_gpus": world, "steps": K, "warmup": args.warmup,
             "ms_per_step": ms_step, "higher_is_better": True, "scaling": "strong" if shard_heads else "weak", "vs_baseline": None,
             "dtype": "bf16", "data": "synthetic", "config": config_dict(w, "bf16", shard_heads, world),
-            "kept_flops_per_step_per_gpu": flops, "clocks": clocks, "gpu_launches": 4 * K,
+            "kept_flops_per_step_per_gpu": flops, "clocks": clocks, "gpu_launches": (sel_launches + fwd_launches) * K,
             "kernels": kernels, "roofline": roofline, "fp8": fp8, "sweep": sweep, "second_workload": second,
             "compensation": comp, "bricks": bricks, "e2e": e2e, "cpu_baseline": cpu, "peaks_in_run": run_peaks,
         }

@@ -411,3 +411,20 @@ def test_block_quantisation_has_no_hidden_mode(lib, block):
                 call()
             assert e.value.status == sa.E_UNSUPPORTED_SHAPE
     assert torch.all(own["codes"] == 7) and torch.all(own["scales"] == 7)
+
+
+def test_bench_counts_the_launches_that_the_launchers_make():
+    """The benchmark's launch counts take the forward's lines from its source, on both sides of each."""
+    import bench
+    import workloads
+    text = open(os.path.join(ROOT, "paper_2609_23153_b200", "csrc", "fwd_pipe.cu")).read()
+    own = int(re.search(r"constexpr int kOwnItems = (\d+);", text).group(1))
+    make = lambda H, blocks, d, block, sparsity: workloads.Workload("launches", 1, 1, H, d, (1, blocks, block), block, sparsity)
+    for d, block, per_sm, items in ((128, 128, own, 37), (128, 64, own, 37), (64, 64, 1, 37)):
+        blocks = 2 * items if (d, block) == (128, 64) else items
+        edge = per_sm * 148 // items                          # 4 heads of 37 items fill 148 SMs, 64 of them 16 times over
+        assert edge * items == per_sm * 148
+        for H, fwd in ((edge, 1), (edge + 1, 2)):
+            assert bench.launches_per_step(make(H, blocks, d, block, 0.5), H, 148) == (2, fwd)
+            assert bench.launches_per_step(make(H, blocks, d, block, 0.0), H, 148) == (1, fwd)
+    assert bench.launches_per_step(workloads.WORKLOADS["wan14b"], 40, 148) == (2, 2)
