@@ -557,7 +557,7 @@ def run_ours(args, w):
                 "state_frac_of_hbm_peak": sbytes / (ms_s * 1e-3) / 1e9 / peaks["hbm"],
                 "apply_ms": ms_a, "apply_GBps": abytes / (ms_a * 1e-3) / 1e9,
                 "apply_frac_of_hbm_peak": abytes / (ms_a * 1e-3) / 1e9 / peaks["hbm"],
-                "launches_per_step": 3}
+                "launches_per_step": 5}          # rotary table, state, its sum over chunks; rotary table, apply
         # the same module output from one call: the forward whose epilogue adds the gated term (bf16, 128-token blocks),
         # against the forward followed by the apply pass, each timed alone after an idle second
         if w.block == 128 and not args.block:
