@@ -38,27 +38,30 @@ __device__ __forceinline__ bool take_header(int32_t* status) {
 __device__ __forceinline__ void report_early(int32_t* status, int code, int detail) {
   unsigned long long* header = reinterpret_cast<unsigned long long*>(status);
   const unsigned long long mine = (unsigned long long)(uint32_t)detail << 32 | (uint32_t)code;
-  unsigned long long seen = 0;
-  for (int i = 0; i < 8; ++i) {          // (what is no code changes once at most, into the zero of the first CTA)
-    const unsigned long long found = atomicCAS(header, seen, mine);
-    if (found == seen || is_status_code(found)) return;
-    seen = found;
-  }
+  const unsigned long long found = atomicCAS(header, 0ull, mine);
+  if (found != 0 && !is_status_code(found)) atomicExch(header, mine);      // (nothing of this launch, unless the first CTA came in between)
 }
-// warp `warp` of the `warps` of the first CTA that look the kept lists up again; each reports one bad index.  (Called behind
-// everything else, so that the compiler keeps it away from the tile loops: in front of them, 40 heads of 75,600 tokens 2974 us instead of
-// 2954, 64-token blocks 3408 and 3344.)
-static __device__ __noinline__ void recheck_lists(const int32_t* kept_idx, const int32_t* kept_cnt, int64_t lists, int nb, int kmax, int32_t* status,
-                                                  int warp, int warps) {
-  const int lane = threadIdx.x & 31;
-  for (int64_t l = warp; l < lists; l += warps) {
-    const int cnt = kept_cnt ? min(max(kept_cnt[l], 0), kmax) : kmax;
-    for (int base = 0; base < cnt; base += 32) {
-      const int kb = base + lane < cnt ? kept_idx[l * kmax + base + lane] : 0;
-      const bool bad = kb < 0 || kb >= nb;
-      const uint32_t who = __ballot_sync(0xffffffffu, bad);
-      if (who == 0) continue;
-      if (lane == __ffs(who) - 1) report_early(status, SPARKATTN_E_BAD_INDEX, kb);
+// Thread `thread` of the `threads` of the first CTA that look the kept lists up again, up to 2048 entries of a few thousand lists;
+// each reports one bad index.  All entries are asked for eight at a time, those behind a list's count as well, and only one that is out of
+// range is looked at closely: 2040 lists of 10 add 30 us to the call (list by list 125).  (Behind everything else in the kernel: in front of the tile
+// loops, 40 heads of 75,600 tokens took 2974 us instead of 2954, 64-token blocks 3408 and 3344.)
+__device__ __forceinline__ void recheck_lists(const int32_t* kept_idx, const int32_t* kept_cnt, int lists, int nb, int kmax, int32_t* status,
+                                              int thread, int threads) {
+  const uint32_t n = (uint32_t)lists * (uint32_t)kmax;
+#pragma unroll 1
+  for (uint32_t first = thread; first < n; first += 8 * threads) {
+    bool odd = false;
+#pragma unroll
+    for (int u = 0; u < 8; ++u) {
+      const uint32_t e = first + u * threads;
+      odd = odd || (uint32_t)(e < n ? kept_idx[e] : 0) >= (uint32_t)nb;
+    }
+    if (!odd) continue;
+#pragma unroll 1
+    for (uint32_t e = first; e < n && e < first + 8 * threads; e += threads) {
+      const int kb = kept_idx[e], list = (int)(e / (uint32_t)kmax), at = (int)(e - (uint32_t)list * (uint32_t)kmax);
+      if ((uint32_t)kb < (uint32_t)nb || at >= (kept_cnt ? kept_cnt[list] : kmax)) continue;
+      report_early(status, SPARKATTN_E_BAD_INDEX, kb);
       return;
     }
   }

@@ -443,17 +443,17 @@ fwd_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant__ C
   // ------------------------------------------------------------------ teardown
   tc_fence_before();
   __syncthreads();
+  if (warp == kTmaWarp) {
+    if (*s_abort) __nanosleep(200000);  // let copies / MMAs in flight land before the CTA's resources go
+    tc_fence_after();
+    tmem_dealloc(tmem, 256 * C);
+  }
   if (threadIdx.x == 0 && (*s_abort >= kAbortTimeout || *s_bad >= 0)) {
     if (*s_bad >= 0) report_early(p.status, SPARKATTN_E_BAD_INDEX, p.kept_idx[((int64_t)bh * p.nb + qb) * p.kmax + *s_bad]);
     report_abort(p.status, *s_abort);
   }
   if constexpr (C == 2) {
-    if (blockIdx.x == 0 && *s_code) recheck_lists(p.kept_idx, p.kept_cnt, gridDim.x, p.nb, p.kmax, p.status, warp, 6 * C);
-  }
-  if (warp == kTmaWarp) {
-    if (*s_abort) __nanosleep(200000);  // let copies / MMAs in flight land before the CTA's resources go
-    tc_fence_after();
-    tmem_dealloc(tmem, 256 * C);
+    if (blockIdx.x == 0 && *s_code) recheck_lists(p.kept_idx, p.kept_cnt, (int)gridDim.x, p.nb, p.kmax, p.status, threadIdx.x, 192 * C);
   }
 }
 

@@ -138,6 +138,12 @@ struct PipeParams {
 // it when it winds down (out of the producers' loops, where the code for it took instruction cache from the tile loops: 40
 // heads of 75,600 tokens, 97 %, 0.995 of the time before, 64-token blocks 0.992, both builds in turn in one process).
 constexpr int32_t kBadFlag = 0x40000000;
+// recheck_lists as a function of its own: inlined, 12 heads of 28,050 tokens in padded bricks 668 us, called 662; 6 heads of 6,479, lists given,
+// 33.2 and 33.1
+static __device__ __noinline__ void recheck_called(const int32_t* kept_idx, const int32_t* kept_cnt, int lists, int nb, int kmax, int32_t* status,
+                                                   int thread, int threads) {
+  recheck_lists(kept_idx, kept_cnt, lists, nb, kmax, status, thread, threads);
+}
 __device__ __forceinline__ int clean_count(const int32_t* clean_cnt, int item) { return clean_cnt[item] & ~kBadFlag; }
 __device__ __forceinline__ void report_bad_index(const PipeParams& p, int item, bool pair) {
   const int bh = item / p.nbq, first = pair ? 2 * (item % p.nbq) : item % p.nbq;
@@ -1344,7 +1350,7 @@ fwd_pipe_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constan
   }
   if constexpr (!FP8) {            // (by the softmax warps, which have the registers of any code)
     if (p.own_lists && blockIdx.x == 0 && *s_code && warp >= 4 && warp < 12)
-      recheck_lists(p.kept_idx, p.kept_cnt, (int64_t)(p.items / p.nbq) * p.nb, p.nb, p.kmax, p.status, warp - 4, 8);
+      recheck_called(p.kept_idx, p.kept_cnt, p.items / p.nbq * p.nb, p.nb, p.kmax, p.status, (int)threadIdx.x - 128, 256);
   }
   if (warp == 0) {
     if (*s_abort) __nanosleep(200000);  // let copies / MMAs in flight land before the CTA's resources go

@@ -60,7 +60,7 @@ __global__ void header_probe_kernel(int32_t* status, const int32_t* lists, int n
   if (blockIdx.x == 0) {
     bool code_there = false;
     if (threadIdx.x == 0) code_there = take_header(status);
-    if (__syncthreads_or(code_there)) recheck_lists(lists, nullptr, 2, nb, kmax, status, threadIdx.x >> 5, 2);
+    if (__syncthreads_or(code_there)) recheck_lists(lists, nullptr, 2, nb, kmax, status, threadIdx.x, 64);
   } else if (threadIdx.x < kmax) {
     const int32_t kb = lists[kmax + threadIdx.x];
     if (kb < 0 || kb >= nb) report_early(status, SPARKATTN_E_BAD_INDEX, kb);
